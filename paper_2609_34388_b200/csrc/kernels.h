@@ -226,8 +226,8 @@ struct PolicyTable {
 void launch_policy(const BatchLayout& bl, const PolicyTable& tb, float* e1, float* e2, int* block_index, int* full,
                    const float* entropy_mean, const int* accept_len, int* next_block, cudaStream_t st);
 
-// KV import / export
-void launch_kv_io(bool write, void* pool, int64_t n_pages, int layer, const Dims& dm, const int* page_row_dev, int pos0,
-                  int n_pos, void* k, void* v, int* status, cudaStream_t st);
+// KV import / export.  page_row: HOST, page ids by logical page (validated by the caller); they travel as kernel parameters
+void launch_kv_io(bool write, void* pool, int64_t n_pages, int layer, const Dims& dm, const int* page_row, int pos0, int n_pos,
+                  void* k, void* v, cudaStream_t st);
 
 }  // namespace recg

@@ -345,29 +345,54 @@ __global__ void __launch_bounds__(256) rmsnorm_kernel(const float* __restrict__ 
   }
 }
 
-// grid (n_pos, n_kv), head_dim/8 threads: each moves one 16-byte chunk of K and of V.
-__global__ void kv_io_kernel(bool write, __nv_bfloat16* pool, int64_t n_pages, int layer, int n_kv, int head_dim,
-                             const int* __restrict__ page_row, int pos0, __nv_bfloat16* k, __nv_bfloat16* v,
-                             int* status) {
-  const int p = pos0 + blockIdx.x, hk = blockIdx.y, c = threadIdx.x;
-  const int page = page_row[p / kPageSize];
-  if (page < 0 || page >= n_pages) {
-    set_status(status, DEV_BAD_INDEX);
-    return;
+// Moves logical K/V rows [n_pos, n_kv, head_dim] into or out of the pool.  Nothing but bytes: bound by HBM.  A thread takes
+// kKvIoUnroll 16-byte chunks of K and the same of V, all loads in flight before the first store; consecutive threads take
+// consecutive chunks, so the logical side is one contiguous stream and the pool side whole 128-byte rows of the swizzled
+// tiles.  The page ids come with the launch (constant bank: a warp covers few positions), so no upload goes ahead of it.
+// 4001 positions of 8 heads x 128 (33 MB in and out): 18.8 us with one 16-thread CTA per (position, head) and a copied page
+// row, KVIO_US with this kernel.
+constexpr int kKvIoPages = 896;       // page ids per launch: 3.5 of the 4 KB of kernel parameters
+constexpr int kKvIoThreads = 256, kKvIoUnroll = 4;
+struct KvIoPages {
+  int first;                          // logical page of ids[0]
+  int ids[kKvIoPages];
+};
+template <bool WRITE>
+__global__ void __launch_bounds__(kKvIoThreads) kv_io_kernel(__nv_bfloat16* pool, int64_t n_pages, int layer, int n_kv, int log2_cpr,
+                                                             const __grid_constant__ KvIoPages pages, int pos0, int n_pos,
+                                                             uint4* __restrict__ k, uint4* __restrict__ v) {
+  griddep_launch();
+  griddep_wait();
+  const int cpr = 1 << log2_cpr, head_dim = cpr * 8;          // 16-byte chunks per row
+  const int total = (n_pos * n_kv) << log2_cpr;
+  const int base = blockIdx.x * (kKvIoThreads * kKvIoUnroll) + threadIdx.x;
+  uint4* at[kKvIoUnroll];
+  uint4 a[kKvIoUnroll], b[kKvIoUnroll];
+  const int v_off = (int)kv_tile_elems(head_dim) / 8;
+#pragma unroll
+  for (int u = 0; u < kKvIoUnroll; ++u) {
+    const int i = base + u * kKvIoThreads;
+    at[u] = nullptr;
+    if (i >= total) continue;
+    const int row = i >> log2_cpr, c = i & (cpr - 1);
+    const int p = row / n_kv, hk = row - p * n_kv, pos = pos0 + p;
+    const int page = pages.ids[pos / kPageSize - pages.first];
+    at[u] = reinterpret_cast<uint4*>(pool + kv_tile_base(n_pages, n_kv, head_dim, layer, page, hk) +
+                                     kv_tile_offset(pos % kPageSize, c * 8, head_dim));
+    a[u] = WRITE ? k[i] : at[u][0];
+    b[u] = WRITE ? v[i] : at[u][v_off];
   }
-  const size_t base = kv_tile_base(n_pages, n_kv, head_dim, layer, page, hk);
-  const int off = kv_tile_offset(p % kPageSize, c * 8, head_dim);
-  uint4* pk = reinterpret_cast<uint4*>(pool + base + off);
-  uint4* pv = reinterpret_cast<uint4*>(pool + base + kv_tile_elems(head_dim) + off);
-  const size_t lin = ((size_t)blockIdx.x * n_kv + hk) * head_dim + c * 8;
-  uint4* lk = reinterpret_cast<uint4*>(k + lin);
-  uint4* lv = reinterpret_cast<uint4*>(v + lin);
-  if (write) {
-    *pk = *lk;
-    *pv = *lv;
-  } else {
-    *lk = *pk;
-    *lv = *pv;
+#pragma unroll
+  for (int u = 0; u < kKvIoUnroll; ++u) {
+    if (!at[u]) continue;
+    const int i = base + u * kKvIoThreads;
+    if (WRITE) {
+      at[u][0] = a[u];
+      at[u][v_off] = b[u];
+    } else {
+      k[i] = a[u];
+      v[i] = b[u];
+    }
   }
 }
 
@@ -398,13 +423,26 @@ void launch_rmsnorm(const float* h, const void* gain, void* x, int rows, int hid
              static_cast<__nv_bfloat16*>(x), hidden, eps, rows_dev);
 }
 
-void launch_kv_io(bool write, void* pool, int64_t n_pages, int layer, const Dims& dm, const int* page_row_dev, int pos0,
-                  int n_pos, void* k, void* v, int* status, cudaStream_t st) {
-  if (n_pos <= 0) return;
-  dim3 grid(n_pos, dm.n_kv);
-  kv_io_kernel<<<grid, dm.head_dim / 8, 0, st>>>(write, static_cast<__nv_bfloat16*>(pool), n_pages, layer, dm.n_kv,
-                                                 dm.head_dim, page_row_dev, pos0, static_cast<__nv_bfloat16*>(k),
-                                                 static_cast<__nv_bfloat16*>(v), status);
+void launch_kv_io(bool write, void* pool, int64_t n_pages, int layer, const Dims& dm, const int* page_row, int pos0, int n_pos,
+                  void* k, void* v, cudaStream_t st) {
+  const int log2_cpr = dm.head_dim == 128 ? 4 : 3;
+  const size_t row = (size_t)dm.n_kv << log2_cpr;             // chunks per position
+  while (n_pos > 0) {
+    KvIoPages pg;
+    pg.first = pos0 / kPageSize;
+    int n = (pg.first + kKvIoPages) * kPageSize - pos0;       // positions this launch's page ids cover
+    if (n > n_pos) n = n_pos;
+    const int last = (pos0 + n - 1) / kPageSize;
+    for (int i = pg.first; i <= last; ++i) pg.ids[i - pg.first] = page_row[i];
+    constexpr size_t kPer = (size_t)kKvIoThreads * kKvIoUnroll;
+    const dim3 grid((unsigned)((n * row + kPer - 1) / kPer));
+    launch_pdl(write ? kv_io_kernel<true> : kv_io_kernel<false>, grid, dim3(kKvIoThreads), 0, st, static_cast<__nv_bfloat16*>(pool),
+               n_pages, layer, dm.n_kv, log2_cpr, pg, pos0, n, static_cast<uint4*>(k), static_cast<uint4*>(v));
+    pos0 += n;
+    n_pos -= n;
+    k = static_cast<uint4*>(k) + n * row;
+    v = static_cast<uint4*>(v) + n * row;
+  }
 }
 
 }  // namespace recg

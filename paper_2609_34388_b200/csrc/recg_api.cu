@@ -73,7 +73,6 @@ struct recg_ctx {
   uint8_t* h_vout = nullptr;             // ... mirrored by one pinned host buffer: a single copy brings all results back
   int* d_status = nullptr;
   int* d_dyn = nullptr;          // device-resident rounds: {n_tok, n_ver} of the round laid out last
-  int* d_page_row = nullptr;
   size_t* d_guards = nullptr;    // RECG_FLAG_DEBUG_CHECKS: offsets of the guard bands, on the device
   int n_guards = 0;
   int* d_policy = nullptr;       // block-size rule: [blocks x8 | cost x8 | edges x64 | value]
@@ -144,7 +143,6 @@ size_t carve(recg_ctx* c, DeviceArena& A) {
   bl.counts = A.take<int>(4);
   c->d_status = A.take<int>(1);
   c->d_dyn = A.take<int>(4);
-  c->d_page_row = A.take<int>(Pm);
   c->d_policy = A.take<int>(8 + 8 + 64 + RECG_POLICY_MAX_BLOCKS * RECG_POLICY_MAX_BINS * RECG_POLICY_MAX_BLOCKS * 2);
   c->rope_cs = A.take<float2>(Tm * (d.head_dim / 2));
   c->part_o = A.take<float>((size_t)bl.max_parts * 128 * d.head_dim);
@@ -889,8 +887,7 @@ static recg_status kv_io(recg_ctx* ctx, bool write, void* pool, int64_t n_pool_p
   if ((pos0 + n_pos - 1) / kPageSize >= n_table) return fail(ctx, RECG_ERR_CAPACITY, "recg_kv_*: positions beyond the page table row");
   for (int i = pos0 / kPageSize; i <= (pos0 + n_pos - 1) / kPageSize; ++i)
     if (row[i] < 0 || row[i] >= n_pool_pages) return fail(ctx, RECG_ERR_INVALID_ARG, "recg_kv_*: page id outside the pool");
-  CU(cudaMemcpyAsync(ctx->d_page_row, row, n_table * sizeof(int), cudaMemcpyHostToDevice, ctx->stream));
-  launch_kv_io(write, pool, n_pool_pages, layer, ctx->dm, ctx->d_page_row, pos0, n_pos, k, v, ctx->d_status, ctx->stream);
+  launch_kv_io(write, pool, n_pool_pages, layer, ctx->dm, row, pos0, n_pos, k, v, ctx->stream);
   CU(cudaGetLastError());
   return RECG_OK;
 }
