@@ -1,6 +1,7 @@
 // Internal launcher interface between the C ABI (recg_api.cu) and the kernel files.
 #pragma once
 #include <cuda_runtime.h>
+#include <stddef.h>
 #include <stdint.h>
 
 namespace recg {
@@ -44,7 +45,7 @@ struct BatchLayout {
   int* tok_id;
   int* tok_req;
   int* tok_pos;     // rotary position (a branch token: the position its branch hypothesises)
-  int* tok_slot;    // page*16 + offset of cache position L + (row within the request), -1 without a page table
+  int* tok_slot;    // page*16 + offset of cache position L + (row within the request)
   int* tok_climit;  // sees every cache position <= climit ...
   int* tok_lo;      // ... and every cache position in [lo, hi)
   int* tok_hi;
@@ -58,7 +59,7 @@ struct BatchLayout {
   int max_items, max_parts;
 };
 
-// S1: per-token arrays and the attention work list.
+// S1: per-token arrays and the attention work list (batches with a page table: a verify-only batch needs neither).
 void launch_layout(const BatchLayout& bl, const Dims& dm, int tok_per_tile, int n_ctas, int64_t n_pages,
                    int* status, cudaStream_t st);
 // the layout kernel keeps eight ints per request in shared memory: requests per step are bounded by this
@@ -208,13 +209,15 @@ struct VerifyBuffers {   // DEVICE outputs (library workspace or caller buffers)
   int *corr_hit, *risky_n, *risky_index, *risky_token;
   int *freed_page_ids;
 };
+// mirror: byte distance from every output array to its copy in mapped host memory (0: no copy is wanted)
 struct RowPartial {      // per (row, vocab chunk)
   float m1, m2;          // largest and second-largest logit of the chunk
   int i1, i2;
   float s, t;            // sum exp(x - m1), sum x exp(x - m1)
 };
 void launch_verify(const BatchLayout& bl, const void* logits, int logits_dtype, int vocab, RowPartial* partials,
-                   int max_chunks_total, const VerifyBuffers& vb, int n_sm, cudaStream_t st);   // (bl.dyn: rows from the device)
+                   int max_chunks_total, const VerifyBuffers& vb, int n_sm, cudaStream_t st,
+                   ptrdiff_t mirror = 0);   // (bl.dyn: rows from the device)
 int verify_chunks_per_row(int rows, int vocab, int n_sm);
 
 // Block-size rule (Eq. 2-3): table = [blocks (int) x8 | cost x8 | edges x64 | value n_blocks*n_bins*n_blocks*2]

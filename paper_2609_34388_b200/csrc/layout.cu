@@ -349,8 +349,8 @@ __global__ void __launch_bounds__(256) rmsnorm_kernel(const float* __restrict__ 
 // kKvIoUnroll 16-byte chunks of K and the same of V, all loads in flight before the first store; consecutive threads take
 // consecutive chunks, so the logical side is one contiguous stream and the pool side whole 128-byte rows of the swizzled
 // tiles.  The page ids come with the launch (constant bank: a warp covers few positions), so no upload goes ahead of it.
-// 4001 positions of 8 heads x 128 (33 MB in and out): 18.8 us with one 16-thread CTA per (position, head) and a copied page
-// row, KVIO_US with this kernel.
+// 4001 positions of 8 heads x 128 (33 MB in and out): 22.5 us a call with one 16-thread CTA per (position, head) and a page
+// row copied ahead of it, 9.2 us with this kernel.
 constexpr int kKvIoPages = 896;       // page ids per launch: 3.5 of the 4 KB of kernel parameters
 constexpr int kKvIoThreads = 256, kKvIoUnroll = 4;
 struct KvIoPages {

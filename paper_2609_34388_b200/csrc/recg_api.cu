@@ -13,7 +13,7 @@ using namespace recg;
 namespace {
 
 thread_local std::string g_init_error;
-constexpr size_t kVoutMirrorMax = 1 << 20;   // verify outputs up to this size come back to the host in one copy
+constexpr size_t kVoutMirrorMax = 1 << 20;   // verify outputs up to this size have a mirror in mapped host memory
 
 // One cudaMalloc, carved with 256-byte alignment.  With guard = true (RECG_FLAG_DEBUG_CHECKS) every region is followed
 // by a 256-byte guard band; the offsets of the bands are recorded so that they can be filled with a pattern at init
@@ -70,7 +70,8 @@ struct recg_ctx {
   int max_chunks_total = 0;
   VerifyBuffers vws{};
   size_t vout_off = 0, vout_bytes = 0;   // the verify outputs are one contiguous region of the arena ...
-  uint8_t* h_vout = nullptr;             // ... mirrored by one pinned host buffer: a single copy brings all results back
+  uint8_t* h_vout = nullptr;             // ... mirrored by one mapped pinned host buffer, which the kernel writes as well:
+  uint8_t* h_vout_dev = nullptr;         // no copy has to follow it (h_vout_dev: the buffer's device address)
   int* d_status = nullptr;
   int* d_dyn = nullptr;          // device-resident rounds: {n_tok, n_ver} of the round laid out last
   size_t* d_guards = nullptr;    // RECG_FLAG_DEBUG_CHECKS: offsets of the guard bands, on the device
@@ -323,8 +324,10 @@ recg_status upload_and_layout(recg_ctx* ctx, const recg_batch* b, bool need_page
   if (s != RECG_OK) return s;
   CU(cudaMemcpyAsync(ctx->d_desc, ctx->h_desc.data(), ctx->h_desc.size() * sizeof(int), cudaMemcpyHostToDevice,
                      ctx->stream));
-  const int64_t n_pages = b->page_table ? (b->kv_pool ? b->kv_pool_pages : (int64_t)1 << 40) : 0;
-  launch_layout(ctx->bl, ctx->dm, ctx->tok_per_tile, ctx->target_items, n_pages, ctx->d_status, ctx->stream);
+  if (b->page_table) {       // (a verify-only batch without pages has neither slots nor attention work)
+    const int64_t n_pages = b->kv_pool ? b->kv_pool_pages : (int64_t)1 << 40;
+    launch_layout(ctx->bl, ctx->dm, ctx->tok_per_tile, ctx->target_items, n_pages, ctx->d_status, ctx->stream);
+  }
   CU(cudaGetLastError());
   ctx->layout_valid = true;
   ctx->layout_has_pages = b->page_table != nullptr;
@@ -436,8 +439,11 @@ recg_status recg_init(recg_ctx** out, const recg_config* cfg, const recg_weights
     }
     launch_guard_fill(ctx->arena.base, ctx->d_guards, ctx->n_guards, ctx->stream);
   }
-  if (ctx->vout_bytes <= kVoutMirrorMax && cudaMallocHost(reinterpret_cast<void**>(&ctx->h_vout), ctx->vout_bytes) != cudaSuccess) {
+  if (ctx->vout_bytes <= kVoutMirrorMax &&
+      (cudaHostAlloc(reinterpret_cast<void**>(&ctx->h_vout), ctx->vout_bytes, cudaHostAllocMapped) != cudaSuccess ||
+       cudaHostGetDevicePointer(reinterpret_cast<void**>(&ctx->h_vout_dev), ctx->h_vout, 0) != cudaSuccess)) {
     cudaGetLastError();
+    if (ctx->h_vout) cudaFreeHost(ctx->h_vout);
     ctx->h_vout = nullptr;   // fall back to one copy per output array
   }
   cudaMemsetAsync(ctx->d_status, 0, sizeof(int), ctx->stream);
@@ -784,15 +790,15 @@ recg_status recg_verify(recg_ctx* ctx, const recg_batch* batch, const void* logi
 #undef PICK
   }
   ctx->mark(-1);
-  launch_verify(bl, logits, logits_dtype, ctx->dm.vocab, ctx->vpart, ctx->max_chunks_total, vb, ctx->n_sm, ctx->stream);
+  uint8_t* region = ctx->arena.base + ctx->vout_off;
+  launch_verify(bl, logits, logits_dtype, ctx->dm.vocab, ctx->vpart, ctx->max_chunks_total, vb, ctx->n_sm, ctx->stream,
+                !dev && ctx->h_vout ? ctx->h_vout_dev - region : 0);
   CU(cudaGetLastError());
   ctx->mark(8, 2);
   if (!dev) {
     const size_t C = bl.n_req, T = bl.n_tok, Tv = bl.n_ver, Tb = T - Tv;
     if (ctx->h_vout) {
-      // one copy of the whole output region into pinned memory, then plain host copies into the caller's arrays
-      const uint8_t* region = ctx->arena.base + ctx->vout_off;
-      CU(cudaMemcpyAsync(ctx->h_vout, region, ctx->vout_bytes, cudaMemcpyDeviceToHost, ctx->stream));
+      // the kernel has written the mirror in pinned memory: plain host copies from there into the caller's arrays
       CU(cudaStreamSynchronize(ctx->stream));
 #define OUT(f, n) if (out->f && (n)) memcpy(out->f, ctx->h_vout + (reinterpret_cast<const uint8_t*>(vb.f) - region), (n) * 4)
       OUT(accept_len, C); OUT(n_emitted, C); OUT(emitted, Tv); OUT(new_ctx_len, C); OUT(slot_state, T);
