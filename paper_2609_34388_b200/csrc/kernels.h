@@ -54,7 +54,6 @@ struct BatchLayout {
   AttnTile* tiles;
   int* tile_off;    // [C+1] first tile entry of each request
   int* cta_off;     // [4 n_ctas] per CTA of the persistent attention grid: the two item index ranges [b0, e0), [b1, e1) it walks
-  int* item_cta;    // [max_items] owning CTA of each item (scratch of the layout kernel)
   int* counts;      // [0] number of items, [1] number of tiles, [2], [3] cost units per CTA / per CTA pair
   int max_items, max_parts;
 };
@@ -62,17 +61,18 @@ struct BatchLayout {
 // S1: per-token arrays and the attention work list (batches with a page table: a verify-only batch needs neither).
 void launch_layout(const BatchLayout& bl, const Dims& dm, int tok_per_tile, int n_ctas, int64_t n_pages,
                    int* status, cudaStream_t st);
-// the layout kernel keeps eight ints per request in shared memory: requests per step are bounded by this
+// the layout kernel keeps six ints per request in shared memory: requests per step are bounded by this
 constexpr int kMaxLayoutRequests = 4096;
 size_t layout_smem_bytes(int n_req, int n_ctas);
 // debug checks
 void launch_guard_fill(void* base, const size_t* offs_dev, int n, cudaStream_t st);
 void launch_guard_check(const void* base, const size_t* offs_dev, int n, int* status, cudaStream_t st);
 void launch_wait_timeout(uint32_t max_polls, int* status, cudaStream_t st);
-// S2: h[t] = embed[tok_id[t]] (fp32 residual stream).  With gain != null also the input of the first normalised
-// projection: x[t] = bf16(h[t] * gain) and ss[t] = sum h[t]^2 (one slot).
+// S2: h[t] = embed[tok_id[t]] (fp32 residual stream), the rotary table (cos, sin) of pos * base^(-2i/d) as float2
+// [head_dim/2][T] (frequency-major), and the input of the first normalised projection: x[t] = rmsnorm(h[t]) * gain, or with
+// ss != null (folded RMSNorm) x[t] = bf16(h[t] * gain) and ss[t] = sum h[t]^2 (one slot).
 void launch_embed(const BatchLayout& bl, const Dims& dm, const void* embed, float* h, const void* gain, void* x, float* ss,
-                  cudaStream_t st);
+                  void* rope_cs, cudaStream_t st);
 // x = rmsnorm(h) * g, bf16 out.  rows_dev (may be null): the true row count on the device (rows is then the capacity).
 void launch_rmsnorm(const float* h, const void* gain, void* x, int rows, int hidden, float eps, cudaStream_t st,
                     const int* rows_dev = nullptr);
@@ -100,10 +100,6 @@ struct RoundLog {
 };
 void launch_next_round(const DeviceRound& dr, const BatchLayout& bl, const VerifyBuffers& vb, const int* next_block,
                        const int* planted_emitted, const RoundLog& log, int round, int* status, cudaStream_t st);
-
-// (cos, sin) of pos * base^(-2i/d), angles evaluated in double: cs float2 [head_dim/2][T] (frequency-major).
-void launch_rope_table(const int* tok_pos, int n_tok, int head_dim, float rope_base, void* cs, cudaStream_t st,
-                       const int* n_tok_dev = nullptr);
 
 // Projection epilogues.
 enum Epilogue : int {

@@ -16,12 +16,14 @@ __device__ __forceinline__ int upper_request(const int* cu, int n_req, int t) {
   return lo;
 }
 
-// One CTA.  Shared: 8 arrays of n_req+1 ints, then n_ctas/2 + 1 and n_ctas + 1 ints.
+// CTA 0 builds the attention work list, every further CTA the per-token arrays of kLayoutThreads tokens.
 //
 // Attention work list.  A request with n new tokens has ceil(n / tok_per_tile) row tiles per kv head.  Row tiles
-// 2 j and 2 j + 1 of a kv head are "siblings": they read the same K/V.  Two lines of 64-token KV blocks are built,
-// every tile preceded by kItemCost virtual blocks that stand for the fixed cost of starting an item (fetching Q,
-// refilling and draining the pipeline):
+// 2 j and 2 j + 1 of a kv head are "siblings": they read the same K/V.  A tile reads the 64-token KV blocks up to the last
+// position that one of its rows may see (verify rows are causal, so the early tiles of a long chunk of prompt need fewer
+// blocks than the late ones; siblings share the range of the later one).  Two lines of KV blocks are built, every tile
+// preceded by kItemCost virtual blocks that stand for the fixed cost of starting an item (fetching Q, refilling and draining
+// the pipeline):
 //   line A holds one segment per sibling PAIR and is cut into equal contiguous ranges, one per pair of CTAs
 //          (2 p, 2 p + 1): the even CTA works on the first sibling and the odd CTA on the second sibling of the SAME
 //          block ranges, at the same time, so that the second reader of a K/V block finds it in L2;
@@ -31,264 +33,357 @@ __device__ __forceinline__ int upper_request(const int* cu, int n_req, int t) {
 // a tile whose blocks are cut by range boundaries gets one partial slot per piece.
 // Items: [line A, first siblings | line A, second siblings (same order) | line B]; cta_off holds, per CTA, two
 // index ranges it walks one after the other (the second one is empty in this division).
+//
+// The kernel is a chain of dependent steps on little data, so it is bound by latency: one thread handles one segment (all
+// per-request sums are block-wide scans), and descriptors are read into shared memory once.  Measured before, with one
+// thread per request and sums over the requests in one thread: 5.6 us for one request, 13 us with its attention work list,
+// 58 us for 8448 rows of 256 requests.
 constexpr int kItemCost = 4;
+constexpr int kLayoutThreads = 1024;
 
-__global__ void __launch_bounds__(1024) layout_kernel(BatchLayout bl, int n_kv, int mask_id, int tok_per_tile,
-                                                      int n_ctas, int64_t n_pages, int* status) {
+// exclusive prefix sums over the threads of the CTA, and the totals; `carry` scratch: 3 x 33 ints of shared memory
+struct Scan3 { int a, b, c; };
+__device__ __forceinline__ Scan3 block_scan(Scan3 x, Scan3* total, int (*sm)[33]) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  Scan3 s = x;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int ya = __shfl_up_sync(0xffffffffu, s.a, o), yb = __shfl_up_sync(0xffffffffu, s.b, o), yc = __shfl_up_sync(0xffffffffu, s.c, o);
+    if (lane >= o) { s.a += ya; s.b += yb; s.c += yc; }
+  }
+  if (lane == 31) { sm[0][warp] = s.a; sm[1][warp] = s.b; sm[2][warp] = s.c; }
+  __syncthreads();
+  if (warp < 3) {                       // warp k scans the warps' sums of component k
+    const int v = sm[warp][lane];
+    int t = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, t, o);
+      if (lane >= o) t += y;
+    }
+    sm[warp][lane] = t - v;
+    if (lane == 31) sm[warp][32] = t;
+  }
+  __syncthreads();
+  s.a += sm[0][warp] - x.a;
+  s.b += sm[1][warp] - x.b;
+  s.c += sm[2][warp] - x.c;
+  *total = Scan3{sm[0][32], sm[1][32], sm[2][32]};
+  __syncthreads();                      // the scratch may be reused
+  return s;
+}
+
+__device__ __forceinline__ void layout_tokens(const BatchLayout& bl, const int* cu_tok, int mask_id, int t, int64_t n_pages, int* status) {
+  const int r = upper_request(cu_tok, bl.n_req, t);
+  const int j = t - cu_tok[r];
+  const int L = bl.ctx_len[r], v = bl.verify_len[r], b = bl.block_size[r];
+  const int idx = L + j;   // cache position of the token's K/V
+  int pos, id, climit, lo, hi;
+  if (j < v) {             // verifier: causal
+    pos = idx; id = bl.verify_tokens[bl.cu_ver[r] + j]; climit = idx; lo = 0; hi = 0;
+  } else if (j < v + b) {  // continuation block: the whole prefix and the block
+    pos = idx; id = mask_id; climit = L + v - 1; lo = L + v; hi = L + v + b;
+  } else {                 // correction branch k: replacement token, then its mask tokens
+    const int* cr = bl.corr + 6 * r;
+    const int span = 1 + cr[1], jj = j - v - b, k = jj / span, q = jj - k * span;
+    const int i = cr[2 + k], first = L + v + b + k * span;
+    pos = L + i + q;
+    id = q == 0 ? cr[4 + k] : mask_id;
+    climit = L + i - 1;
+    lo = first;
+    hi = q == 0 ? first + 1 : first + span;
+  }
+  bl.tok_req[t] = r;
+  bl.tok_pos[t] = pos;
+  bl.tok_id[t] = id;
+  bl.tok_climit[t] = climit;
+  bl.tok_lo[t] = lo;
+  bl.tok_hi[t] = hi;
+  const int page = bl.page_table[(size_t)r * bl.pt_stride + idx / kPageSize];
+  int slot = -1;
+  if (page < 0 || page >= n_pages) set_status(status, DEV_BAD_INDEX);
+  else slot = page * kPageSize + idx % kPageSize;
+  bl.tok_slot[t] = slot;
+}
+
+__global__ void __launch_bounds__(kLayoutThreads) layout_kernel(BatchLayout bl, int n_kv, int mask_id, int tok_per_tile,
+                                                                int n_ctas, int64_t n_pages, int* status) {
   extern __shared__ int sm[];
   const int C = bl.n_req;
   const int max_pairs = n_ctas / 2;
-  int* off_a = sm;                       // first cost unit of request r in line A
-  int* off_b = sm + (C + 1);             // ... in line B
-  int* tile_off = sm + 2 * (C + 1);      // first tile entry of request r
-  int* item_a = sm + 3 * (C + 1);        // first line-A piece of request r
-  int* item_b = sm + 4 * (C + 1);        // first line-B piece of request r
-  int* part_off = sm + 5 * (C + 1);      // first partial slot of request r
-  int* req_nb = sm + 6 * (C + 1);        // blocks per tile of request r
-  int* req_rt = sm + 7 * (C + 1);        // row tiles per kv head of request r
-  int* a_off = sm + 8 * (C + 1);         // [max_pairs + 1] first line-A piece of every CTA pair
+  int* cu_tok = sm;                      // [C + 1] rows of the batch in front of request r
+  int* seg_a = sm + (C + 1);             // [C + 1] line-A segments in front of request r
+  int* seg_b = sm + 2 * (C + 1);         // [C + 1] line-B segments
+  int* tile_off = sm + 3 * (C + 1);      // [C + 1] first tile entry
+  int* ctx = sm + 4 * (C + 1);           // [C]
+  int* vis = sm + 5 * (C + 1);           // [C] verify rows (causal) of request r
+  int* a_off = sm + 6 * (C + 1);         // [max_pairs + 1] first line-A piece of every CTA pair
   int* b_off = a_off + (max_pairs + 1);  // [n_ctas + 1]  first line-B piece of every line-B CTA
-  __shared__ int s_per_a, s_per_b, s_pairs_a;
-  const int tid = threadIdx.x, nth = blockDim.x;
+  __shared__ int scratch[3][33];
+  __shared__ long long s_cost[2];
+  const int tid = threadIdx.x;
   griddep_launch();
   griddep_wait();   // the previous step's kernels may still be reading the arrays this kernel rewrites
-  const int n_tok = bl.dyn ? bl.dyn[0] : bl.n_tok;
+  for (int r = tid; r <= C; r += kLayoutThreads) cu_tok[r] = bl.cu_tok[r];
 
   // ---- per-token arrays ----
-  for (int t = tid; t < n_tok; t += nth) {
-    const int r = upper_request(bl.cu_tok, C, t);
-    const int j = t - bl.cu_tok[r];
-    const int L = bl.ctx_len[r], v = bl.verify_len[r], b = bl.block_size[r];
-    const int idx = L + j;   // cache position of the token's K/V
-    int pos, id, climit, lo, hi;
-    if (j < v) {             // verifier: causal
-      pos = idx; id = bl.verify_tokens[bl.cu_ver[r] + j]; climit = idx; lo = 0; hi = 0;
-    } else if (j < v + b) {  // continuation block: the whole prefix and the block
-      pos = idx; id = mask_id; climit = L + v - 1; lo = L + v; hi = L + v + b;
-    } else {                 // correction branch k: replacement token, then its mask tokens
-      const int* cr = bl.corr + 6 * r;
-      const int span = 1 + cr[1], jj = j - v - b, k = jj / span, q = jj - k * span;
-      const int i = cr[2 + k], first = L + v + b + k * span;
-      pos = L + i + q;
-      id = q == 0 ? cr[4 + k] : mask_id;
-      climit = L + i - 1;
-      lo = first;
-      hi = q == 0 ? first + 1 : first + span;
-    }
-    bl.tok_req[t] = r;
-    bl.tok_pos[t] = pos;
-    bl.tok_id[t] = id;
-    bl.tok_climit[t] = climit;
-    bl.tok_lo[t] = lo;
-    bl.tok_hi[t] = hi;
-    int slot = -1;
-    if (bl.page_table) {
-      const int page = bl.page_table[(size_t)r * bl.pt_stride + idx / kPageSize];
-      if (page < 0 || page >= n_pages) set_status(status, DEV_BAD_INDEX);
-      else slot = page * kPageSize + idx % kPageSize;
-    }
-    bl.tok_slot[t] = slot;
+  if (blockIdx.x > 0) {
+    __syncthreads();
+    const int t = (blockIdx.x - 1) * kLayoutThreads + tid;
+    if (t < cu_tok[C]) layout_tokens(bl, cu_tok, mask_id, t, n_pages, status);
+    return;
   }
 
   // ---- attention work list ----
-  for (int r = tid; r < C; r += nth) {
-    const int n = bl.cu_tok[r + 1] - bl.cu_tok[r];
-    req_nb[r] = (bl.ctx_len[r] + n + 63) / 64;
-    req_rt[r] = (n + tok_per_tile - 1) / tok_per_tile;
+  for (int r = tid; r < C; r += kLayoutThreads) {
+    ctx[r] = bl.ctx_len[r];
+    vis[r] = bl.verify_len[r];
   }
+  if (tid < 2) s_cost[tid] = 0;
   __syncthreads();
+  Scan3 carry{0, 0, 0};
+  for (int r0 = 0; r0 < C; r0 += kLayoutThreads) {
+    const int r = r0 + tid;
+    const int rt = r < C ? (cu_tok[r + 1] - cu_tok[r] + tok_per_tile - 1) / tok_per_tile : 0;
+    Scan3 tot;
+    const Scan3 e = block_scan(Scan3{n_kv * (rt / 2), n_kv * (rt & 1), n_kv * rt}, &tot, scratch);
+    if (r < C) {
+      seg_a[r] = carry.a + e.a;
+      seg_b[r] = carry.b + e.b;
+      tile_off[r] = carry.c + e.c;
+      bl.tile_off[r] = carry.c + e.c;
+    }
+    carry.a += tot.a;
+    carry.b += tot.b;
+    carry.c += tot.c;
+  }
+  const int n_seg_a = carry.a, n_seg_b = carry.b, n_tiles = carry.c;
   if (tid == 0) {
-    off_a[0] = off_b[0] = tile_off[0] = 0;
-    long long wa = 0, wb = 0;
-    for (int r = 0; r < C; ++r) {
-      const int rt = req_rt[r], seg = req_nb[r] + kItemCost;
-      wa += (long long)n_kv * (rt / 2) * seg;
-      wb += (long long)n_kv * (rt & 1) * seg;
-      if (wa > 0x3fffffff) wa = 0x3fffffff;   // far beyond any pool; keeps the arithmetic in int
-      if (wb > 0x3fffffff) wb = 0x3fffffff;
-      off_a[r + 1] = (int)wa;
-      off_b[r + 1] = (int)wb;
-      tile_off[r + 1] = tile_off[r] + n_kv * rt;
-    }
-    // CTAs for line A in proportion to its CTA time (two CTAs work on every unit of it)
-    int pairs_a = (2 * wa + wb) > 0 ? (int)(0.5 * n_ctas * (2.0 * wa) / (2.0 * wa + wb) + 0.5) : 0;
-    if (wa > 0 && pairs_a < 1) pairs_a = 1;
-    if (pairs_a > max_pairs) pairs_a = max_pairs;
-    if (wb > 0 && n_ctas - 2 * pairs_a < 1) pairs_a = (n_ctas - 1) / 2;
-    if (wa == 0) pairs_a = 0;
-    const int ctas_b = n_ctas - 2 * pairs_a;
-    const int pa = pairs_a > 0 ? (int)((wa + pairs_a - 1) / pairs_a) : 0x3fffffff;
-    const int pb = ctas_b > 0 ? (int)((wb + ctas_b - 1) / ctas_b) : 0x3fffffff;
-    s_per_a = pa < 1 ? 1 : pa;
-    s_per_b = pb < 1 ? 1 : pb;
-    s_pairs_a = pairs_a;
+    seg_a[C] = n_seg_a;
+    seg_b[C] = n_seg_b;
+    tile_off[C] = n_tiles;
+    bl.tile_off[C] = n_tiles;
   }
   __syncthreads();
-  const int per_a = s_per_a, per_b = s_per_b;
-  const int n_pairs = s_pairs_a, n_ctas_b = n_ctas - 2 * s_pairs_a;
-  // pieces of a segment whose real blocks occupy the cost range [g0, g0 + nb)
-  auto n_pieces = [](int g0, int nb, int per) { return (g0 + nb - 1) / per - g0 / per + 1; };
-  for (int r = tid; r < C; r += nth) {
-    const int nb = req_nb[r], rt = req_rt[r], seg = nb + kItemCost;
-    int ia = 0, ib = 0, parts = 0;
-    for (int kvh = 0; kvh < n_kv; ++kvh) {
-      for (int j = 0; j < rt / 2; ++j) {
-        const int np = n_pieces(off_a[r] + (kvh * (rt / 2) + j) * seg + kItemCost, nb, per_a);
-        ia += np;
-        if (np > 1) parts += 2 * np;
-      }
-      if (rt & 1) {
-        const int np = n_pieces(off_b[r] + kvh * seg + kItemCost, nb, per_b);
-        ib += np;
-        if (np > 1) parts += np;
-      }
+  // segment s of a line: its request, kv head, (first) tile and KV blocks
+  struct Seg { int r, kvh, tile, nb; };
+  auto segment = [&](const int* first, int s, bool pair) {
+    Seg g;
+    g.r = upper_request(first, C, s);
+    const int n = cu_tok[g.r + 1] - cu_tok[g.r], rt = (n + tok_per_tile - 1) / tok_per_tile;
+    const int per_head = pair ? rt / 2 : 1, i = s - first[g.r];
+    g.kvh = i / per_head;
+    g.tile = pair ? 2 * (i - g.kvh * per_head) : rt - 1;
+    // the last of the segment's rows: causal up to itself if it is a verify row, else anything up to the request's end
+    const int last_row = min(n, (g.tile + (pair ? 2 : 1)) * tok_per_tile);
+    g.nb = (ctx[g.r] + (last_row <= vis[g.r] ? last_row : n) + 63) / 64;
+    return g;
+  };
+  for (int line = 0; line < 2; ++line) {
+    const int n_seg = line ? n_seg_b : n_seg_a;
+    for (int s0 = 0; s0 < n_seg; s0 += kLayoutThreads) {
+      const int s = s0 + tid;
+      int cost = 0;
+      if (s < n_seg) cost = (line ? segment(seg_b, s, false) : segment(seg_a, s, true)).nb + kItemCost;
+      cost = __reduce_add_sync(0xffffffffu, cost);
+      if ((tid & 31) == 0 && cost) atomicAdd(reinterpret_cast<unsigned long long*>(&s_cost[line]), (unsigned long long)cost);
     }
-    item_a[r + 1] = ia;
-    item_b[r + 1] = ib;
-    part_off[r + 1] = parts;
   }
   __syncthreads();
+  const long long wa = s_cost[0], wb = s_cost[1];
+  const bool too_long = wa > 0x3fffffff || wb > 0x3fffffff;      // far beyond any pool; the arithmetic below is in int
+  // CTAs for line A in proportion to its CTA time (two CTAs work on every unit of it)
+  int pairs_a = (2 * wa + wb) > 0 ? (int)(0.5 * n_ctas * (2.0 * wa) / (2.0 * wa + wb) + 0.5) : 0;
+  if (wa > 0 && pairs_a < 1) pairs_a = 1;
+  if (pairs_a > max_pairs) pairs_a = max_pairs;
+  if (wb > 0 && n_ctas - 2 * pairs_a < 1) pairs_a = (n_ctas - 1) / 2;
+  if (wa == 0) pairs_a = 0;
+  const int n_ctas_b = n_ctas - 2 * pairs_a;
+  const int per_a = pairs_a > 0 && wa > 0 ? (int)((wa + pairs_a - 1) / pairs_a) : 0x3fffffff;
+  const int per_b = n_ctas_b > 0 && wb > 0 ? (int)((wb + n_ctas_b - 1) / n_ctas_b) : 0x3fffffff;
+
+  // Lines A, then B: offsets by scans over the segments, then every thread emits the pieces of its segment.
+  int n_pieces_a = 0, n_pieces_b = 0, parts = 0;
+  bool overflow = too_long;
+  // pass 0 counts line A's pieces (the second siblings' items lie behind all first ones), passes 1 and 2 emit
+  for (int pass = too_long ? 3 : 0; pass < 3; ++pass) {
+    const bool pair = pass < 2;
+    const int n_seg = pair ? n_seg_a : n_seg_b, per = pair ? per_a : per_b;
+    const int* first = pair ? seg_a : seg_b;
+    int* owner_off = pair ? a_off : b_off;
+    const int n_owners = pair ? max_pairs : n_ctas;
+    int off = 0, pieces = 0;             // cost units and pieces of the line so far
+    for (int s0 = 0; s0 < n_seg; s0 += kLayoutThreads) {
+      const int s = s0 + tid;
+      Seg g{0, 0, 0, 0};
+      if (s < n_seg) g = segment(first, s, pair);
+      Scan3 tot;
+      const Scan3 e1 = block_scan(Scan3{s < n_seg ? g.nb + kItemCost : 0, 0, 0}, &tot, scratch);
+      const int g0 = off + e1.a + kItemCost;              // cost range of the real blocks: [g0, g0 + nb)
+      off += tot.a;
+      const int c_first = g0 / per, c_last = (g0 + g.nb - 1) / per;
+      const int np = s < n_seg ? c_last - c_first + 1 : 0;
+      const Scan3 e2 = block_scan(Scan3{np, np > 1 ? (pair ? 2 * np : np) : 0, 0}, &tot, scratch);
+      const int item0 = pieces + e2.a;
+      int part = parts + e2.b;
+      pieces += tot.a;
+      if (pass > 0) parts += tot.b;
+      if (pass == 0 || s >= n_seg) continue;
+      // first piece of every owner: an owner without pieces starts where the next one does
+      const int c_prev = s == 0 ? -1 : (g0 - kItemCost - 1) / per;     // owner of the last block of the segment before
+      for (int c = c_prev + 1; c <= c_last && c <= n_owners; ++c) owner_off[c] = c <= c_first ? item0 : item0 + (c - c_first);
+      if (s == n_seg - 1)
+        for (int c = c_last + 1; c <= n_owners; ++c) owner_off[c] = item0 + np;
+      const int n = cu_tok[g.r + 1] - cu_tok[g.r], kv_len = ctx[g.r] + n, rt = (n + tok_per_tile - 1) / tok_per_tile;
+      for (int sib = 0; sib < (pair ? 2 : 1); ++sib) {
+        AttnTile tl;
+        tl.part_begin = np > 1 ? part : -1;
+        tl.n_parts = np;
+        tl.tok0 = cu_tok[g.r] + (g.tile + sib) * tok_per_tile;
+        tl.ntok = min(tok_per_tile, n - (g.tile + sib) * tok_per_tile);
+        tl.kv_head = g.kvh;
+        bl.tiles[tile_off[g.r] + g.kvh * rt + g.tile + sib] = tl;
+        const int at = pair ? (sib ? n_pieces_a : 0) + item0 : 2 * n_pieces_a + item0;
+        for (int c = c_first; c <= c_last; ++c) {
+          AttnItem a;
+          a.req = g.r;
+          a.kv_head = g.kvh;
+          a.tok0 = tl.tok0;
+          a.ntok = tl.ntok;
+          a.blk_begin = max(g0, c * per) - g0;
+          a.blk_end = min(g0 + g.nb, (c + 1) * per) - g0;
+          a.part = np > 1 ? part++ : -1;
+          a.kv_len = kv_len;
+          if (at + (c - c_first) < bl.max_items && a.part < bl.max_parts) bl.items[at + (c - c_first)] = a;
+        }
+      }
+    }
+    if (pass == 0) n_pieces_a = pieces;
+    if (pass == 2) n_pieces_b = pieces;
+    if (pass > 0 && n_seg == 0)
+      for (int c = tid; c <= n_owners; c += kLayoutThreads) owner_off[c] = 0;
+  }
+  overflow = overflow || 2 * n_pieces_a + n_pieces_b > bl.max_items || parts > bl.max_parts;
   if (tid == 0) {
-    item_a[0] = item_b[0] = part_off[0] = 0;
-    for (int r = 0; r < C; ++r) {
-      item_a[r + 1] += item_a[r];
-      item_b[r + 1] += item_b[r];
-      part_off[r + 1] += part_off[r];
-    }
-    int n_items = 2 * item_a[C] + item_b[C];
-    if (n_items > bl.max_items || part_off[C] > bl.max_parts) {
-      set_status(status, DEV_BAD_INDEX);
-      n_items = 0;
-    }
-    bl.counts[0] = n_items;
-    bl.counts[1] = tile_off[C];
+    if (overflow) set_status(status, DEV_BAD_INDEX);
+    bl.counts[0] = overflow ? 0 : 2 * n_pieces_a + n_pieces_b;
+    bl.counts[1] = n_tiles;
     bl.counts[2] = per_b;
     bl.counts[3] = per_a;
   }
   __syncthreads();
-  const int n_items = bl.counts[0];
-  const int na = n_items ? item_a[C] : 0, n_b = n_items ? item_b[C] : 0;
-  for (int r = tid; r <= C; r += nth) bl.tile_off[r] = tile_off[r];
-  for (int p = tid; p <= max_pairs; p += nth) a_off[p] = na;   // pairs after the last owner; the rest is filled below
-  for (int c = tid; c <= n_ctas; c += nth) b_off[c] = n_b;
-  __syncthreads();
-  if (n_items) {
-    for (int r = tid; r < C; r += nth) {
-      const int n = bl.cu_tok[r + 1] - bl.cu_tok[r];
-      const int kv_len = bl.ctx_len[r] + n;
-      const int nb = req_nb[r], rt = req_rt[r], seg = nb + kItemCost;
-      int ia = item_a[r], ib = item_b[r], part = part_off[r];
-      // one tile's entry, and its items on one line: pieces [c_first, c_last] of the cost range [g0, g0 + nb)
-      auto emit = [&](int kvh, int tile, int g0, int per, int item0, int* owner, int owner_base) {
-        const int c_first = g0 / per, c_last = (g0 + nb - 1) / per;
-        const int parts = c_last - c_first + 1;
-        AttnTile tl;
-        tl.part_begin = parts > 1 ? part : -1;
-        tl.n_parts = parts;
-        tl.tok0 = bl.cu_tok[r] + tile * tok_per_tile;
-        tl.ntok = min(tok_per_tile, n - tile * tok_per_tile);
-        tl.kv_head = kvh;
-        bl.tiles[tile_off[r] + kvh * rt + tile] = tl;
-        for (int c = c_first; c <= c_last; ++c) {
-          const int gs = max(g0, c * per), ge = min(g0 + nb, (c + 1) * per);
-          AttnItem a;
-          a.req = r;
-          a.kv_head = kvh;
-          a.tok0 = tl.tok0;
-          a.ntok = tl.ntok;
-          a.blk_begin = gs - g0;
-          a.blk_end = ge - g0;
-          a.part = parts > 1 ? part++ : -1;
-          a.kv_len = kv_len;
-          bl.items[item0 + (c - c_first)] = a;
-          if (owner) owner[owner_base + (c - c_first)] = c;
-        }
-        return parts;
-      };
-      for (int kvh = 0; kvh < n_kv; ++kvh) {
-        for (int j = 0; j < rt / 2; ++j) {
-          const int g0 = off_a[r] + (kvh * (rt / 2) + j) * seg + kItemCost;
-          const int np = emit(kvh, 2 * j, g0, per_a, ia, bl.item_cta, ia);       // first sibling: even CTA of the pair
-          emit(kvh, 2 * j + 1, g0, per_a, na + ia, nullptr, 0);                  // second sibling: odd CTA, same ranges
-          ia += np;
-        }
-        if (rt & 1) {
-          const int g0 = off_b[r] + kvh * seg + kItemCost;
-          ib += emit(kvh, rt - 1, g0, per_b, 2 * na + ib, bl.item_cta, 2 * na + ib);
-        }
-      }
-    }
-    // first piece of every owner: pieces are in line order, so an owner's range starts where the owner changes
-    __syncthreads();
-    for (int it = tid; it < na; it += nth) {
-      const int p = bl.item_cta[it];
-      const int prev = it ? bl.item_cta[it - 1] : -1;
-      for (int pp = prev + 1; pp <= p && pp <= max_pairs; ++pp) a_off[pp] = it;   // pairs between two owners have no items
-    }
-    for (int it = tid; it < n_b; it += nth) {
-      const int c = bl.item_cta[2 * na + it];
-      const int prev = it ? bl.item_cta[2 * na + it - 1] : -1;
-      for (int cc = prev + 1; cc <= c && cc <= n_ctas; ++cc) b_off[cc] = it;
-    }
-  }
-  __syncthreads();
   // the ranges of item indices every CTA walks: a CTA of line A its pair's pieces (first or second siblings), a CTA of
   // line B its own pieces
-  for (int c = tid; c < n_ctas; c += nth) {
+  for (int c = tid; c < n_ctas; c += kLayoutThreads) {
     int a0 = 0, a1 = 0, b0 = 0, b1 = 0;
-    if (c < 2 * n_pairs) {
-      const int p = c >> 1;
-      a0 = ((c & 1) ? na : 0) + a_off[p];
-      a1 = ((c & 1) ? na : 0) + a_off[p + 1];
-    } else if (c - 2 * n_pairs < n_ctas_b) {
-      b0 = 2 * na + b_off[c - 2 * n_pairs];
-      b1 = 2 * na + b_off[c - 2 * n_pairs + 1];
+    if (!overflow) {
+      if (c < 2 * pairs_a) {
+        const int p = c >> 1;
+        a0 = ((c & 1) ? n_pieces_a : 0) + a_off[p];
+        a1 = ((c & 1) ? n_pieces_a : 0) + a_off[p + 1];
+      } else if (c - 2 * pairs_a < n_ctas_b) {
+        b0 = 2 * n_pieces_a + b_off[c - 2 * pairs_a];
+        b1 = 2 * n_pieces_a + b_off[c - 2 * pairs_a + 1];
+      }
     }
-    bl.cta_off[4 * c + 0] = a0;
-    bl.cta_off[4 * c + 1] = a1;
-    bl.cta_off[4 * c + 2] = b0;
-    bl.cta_off[4 * c + 3] = b1;
-  }
-}
-
-__global__ void __launch_bounds__(256) embed_kernel(const int* __restrict__ tok_id, const __nv_bfloat16* __restrict__ embed,
-                                                    float* __restrict__ h, int hidden, int vocab,
-                                                    const __nv_bfloat16* __restrict__ gain, __nv_bfloat16* __restrict__ x,
-                                                    float* __restrict__ ss, const int* __restrict__ rows_dev) {
-  griddep_launch();
-  griddep_wait();
-  const int t = blockIdx.x;
-  if (rows_dev && t >= rows_dev[0]) return;
-  int id = tok_id[t];
-  id = id < 0 ? 0 : (id >= vocab ? vocab - 1 : id);
-  const __nv_bfloat162* src = reinterpret_cast<const __nv_bfloat162*>(embed + (size_t)id * hidden);
-  float2* dst = reinterpret_cast<float2*>(h + (size_t)t * hidden);
-  float sq = 0.f;
-  for (int i = threadIdx.x; i < hidden / 2; i += blockDim.x) {
-    const float2 v = __bfloat1622float2(src[i]);
-    dst[i] = v;
-    if (gain) {
-      const float2 g = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(gain)[i]);
-      reinterpret_cast<uint32_t*>(x + (size_t)t * hidden)[i] = pack_bf16(v.x * g.x, v.y * g.y);
-      sq += v.x * v.x + v.y * v.y;
-    }
-  }
-  if (gain) {
-    __shared__ float red[8];
-    for (int o = 16; o; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sq;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      float tot = 0.f;
-      for (int i = 0; i < 8; ++i) tot += red[i];
-      ss[t] = tot;
-    }
+    *reinterpret_cast<int4*>(bl.cta_off + 4 * c) = make_int4(a0, a1, b0, b1);
   }
 }
 
 // One CTA per row; fp32 in, bf16 out.  hidden a multiple of 4.  The row is read once and kept in registers
 // when it fits (hidden <= 256 threads x kRegVecs float4), otherwise it is read a second time.
 constexpr int kRegVecs = 8;
+__device__ __forceinline__ float row_sum(float ss) {     // over the 256 threads of the CTA, the same bits in every thread
+  __shared__ float red[8];
+  for (int o = 16; o; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
+  __syncthreads();
+  float tot = 0.f;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) tot += red[i];
+  return tot;
+}
+// four elements of x = bf16(h * rstd * gain); rstd = 1: x = bf16(h * gain)
+__device__ __forceinline__ uint2 norm_vec(const float4& t, float rstd, const uint2* __restrict__ gain, int i) {
+  const uint2 gv = __ldg(gain + i);
+  const float2 g0 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&gv.x));
+  const float2 g1 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&gv.y));
+  uint2 o;
+  o.x = pack_bf16(t.x * rstd * g0.x, t.y * rstd * g0.y);
+  o.y = pack_bf16(t.z * rstd * g1.x, t.w * rstd * g1.y);
+  return o;
+}
+
+// One CTA per token: the residual row h = embed[tok_id], the rotary table's column of the token, and the input of the first
+// projection: x = rmsnorm(h) * gain, or (ss given: folded RMSNorm) x = h * gain and the row's sum of squares.  All of it
+// follows from the token alone and each part by itself is one launch latency (2.5 us each at any size up to a few hundred
+// rows), so one launch does the three.
+__global__ void __launch_bounds__(256) embed_kernel(const int* __restrict__ tok_id, const int* __restrict__ tok_pos,
+                                                    const __nv_bfloat16* __restrict__ embed, float* __restrict__ h, int hidden,
+                                                    int vocab, const __nv_bfloat16* __restrict__ gain,
+                                                    __nv_bfloat16* __restrict__ x, float* __restrict__ ss, float eps,
+                                                    float2* __restrict__ cs, int half, double log_base, int n_tok,
+                                                    const int* __restrict__ rows_dev) {
+  griddep_launch();
+  griddep_wait();
+  const int t = blockIdx.x;
+  if (rows_dev) n_tok = rows_dev[0];       // (the grid was sized for the capacity)
+  if (t >= n_tok) return;
+  int id = tok_id[t];
+  const int pos = tok_pos[t];
+  id = id < 0 ? 0 : (id >= vocab ? vocab - 1 : id);
+  const uint2* src = reinterpret_cast<const uint2*>(embed + (size_t)id * hidden);
+  float4* dst = reinterpret_cast<float4*>(h + (size_t)t * hidden);
+  const int nvec = hidden / 4;
+  auto load = [&](int i) {
+    const uint2 u = __ldg(src + i);
+    return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u), __uint_as_float(u.y << 16),
+                       __uint_as_float(u.y & 0xffff0000u));
+  };
+  const bool in_regs = nvec <= 256 * kRegVecs;
+  float4 v[kRegVecs];
+  float sq = 0.f;
+  if (in_regs) {
+#pragma unroll
+    for (int u = 0; u < kRegVecs; ++u) {
+      const int i = threadIdx.x + u * 256;
+      v[u] = i < nvec ? load(i) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+#pragma unroll
+    for (int u = 0; u < kRegVecs; ++u) {
+      const int i = threadIdx.x + u * 256;
+      if (i < nvec) dst[i] = v[u];
+      sq += v[u].x * v[u].x + v[u].y * v[u].y + v[u].z * v[u].z + v[u].w * v[u].w;
+    }
+  } else {
+    for (int i = threadIdx.x; i < nvec; i += 256) {
+      const float4 f = load(i);
+      dst[i] = f;
+      sq += f.x * f.x + f.y * f.y + f.z * f.z + f.w * f.w;
+    }
+  }
+  // rotary factors, frequency-major [half][n_tok]: the projection epilogue has one token per thread, so a warp reads 32
+  // consecutive tokens of one frequency in one 256-byte request.  Angles in double.
+  for (int i = threadIdx.x; i < half; i += 256) {
+    const double ang = (double)pos * exp(-log_base * (double)i / (double)half);  // pos * base^(-2i/d)
+    cs[(size_t)i * n_tok + t] = make_float2((float)cos(ang), (float)sin(ang));
+  }
+  const float tot = row_sum(sq);
+  const float rstd = ss ? 1.f : rsqrtf(tot / hidden + eps);
+  if (ss && threadIdx.x == 0) ss[t] = tot;
+  uint2* xo = reinterpret_cast<uint2*>(x + (size_t)t * hidden);
+  const uint2* gg = reinterpret_cast<const uint2*>(gain);
+  if (in_regs) {
+#pragma unroll
+    for (int u = 0; u < kRegVecs; ++u) {
+      const int i = threadIdx.x + u * 256;
+      if (i < nvec) xo[i] = norm_vec(v[u], rstd, gg, i);
+    }
+  } else {
+    for (int i = threadIdx.x; i < nvec; i += 256) xo[i] = norm_vec(load(i), rstd, gg, i);
+  }
+}
+
 __global__ void __launch_bounds__(256) rmsnorm_kernel(const float* __restrict__ h, const __nv_bfloat16* __restrict__ g,
                                                       __nv_bfloat16* __restrict__ x, int hidden, float eps,
                                                       const int* __restrict__ rows_dev) {
@@ -315,33 +410,17 @@ __global__ void __launch_bounds__(256) rmsnorm_kernel(const float* __restrict__ 
       ss += t.x * t.x + t.y * t.y + t.z * t.z + t.w * t.w;
     }
   }
-  __shared__ float red[8];
-  for (int o = 16; o; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
-  __syncthreads();
-  float tot = 0.f;
-#pragma unroll
-  for (int i = 0; i < 8; ++i) tot += red[i];
-  const float rstd = rsqrtf(tot / hidden + eps);
+  const float rstd = rsqrtf(row_sum(ss) / hidden + eps);
   uint2* dst = reinterpret_cast<uint2*>(x + (size_t)row * hidden);
   const uint2* gg = reinterpret_cast<const uint2*>(g);
-  auto emit = [&](int i, const float4& t) {
-    const uint2 gv = __ldg(gg + i);
-    const float2 g0 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&gv.x));
-    const float2 g1 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&gv.y));
-    uint2 o;
-    o.x = pack_bf16(t.x * rstd * g0.x, t.y * rstd * g0.y);
-    o.y = pack_bf16(t.z * rstd * g1.x, t.w * rstd * g1.y);
-    dst[i] = o;
-  };
   if (in_regs) {
 #pragma unroll
     for (int u = 0; u < kRegVecs; ++u) {
       const int i = threadIdx.x + u * 256;
-      if (i < nvec) emit(i, v[u]);
+      if (i < nvec) dst[i] = norm_vec(v[u], rstd, gg, i);
     }
   } else {
-    for (int i = threadIdx.x; i < nvec; i += 256) emit(i, src[i]);
+    for (int i = threadIdx.x; i < nvec; i += 256) dst[i] = norm_vec(src[i], rstd, gg, i);
   }
 }
 
@@ -399,7 +478,7 @@ __global__ void __launch_bounds__(kKvIoThreads) kv_io_kernel(__nv_bfloat16* pool
 }  // namespace
 
 size_t layout_smem_bytes(int n_req, int n_ctas) {
-  return (8 * (size_t)(n_req + 1) + (size_t)(n_ctas / 2 + 1) + (size_t)(n_ctas + 1)) * sizeof(int);
+  return (6 * (size_t)(n_req + 1) + (size_t)(n_ctas / 2 + 1) + (size_t)(n_ctas + 1)) * sizeof(int);
 }
 
 void launch_layout(const BatchLayout& bl, const Dims& dm, int tok_per_tile, int n_ctas, int64_t n_pages,
@@ -408,13 +487,15 @@ void launch_layout(const BatchLayout& bl, const Dims& dm, int tok_per_tile, int 
   static bool configured[kMaxDevices] = {false};
   if (first_use_on_device(configured))    // room for kMaxLayoutRequests requests (the default limit is 48 KB)
     cudaFuncSetAttribute(layout_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)layout_smem_bytes(kMaxLayoutRequests, 1024));
-  launch_pdl(layout_kernel, dim3(1), dim3(1024), smem, st, bl, dm.n_kv, dm.mask_id, tok_per_tile, n_ctas, n_pages, status);
+  launch_pdl(layout_kernel, dim3(1 + (bl.n_tok + kLayoutThreads - 1) / kLayoutThreads), dim3(kLayoutThreads), smem, st, bl, dm.n_kv, dm.mask_id, tok_per_tile, n_ctas, n_pages, status);
 }
 
 void launch_embed(const BatchLayout& bl, const Dims& dm, const void* embed, float* h, const void* gain, void* x, float* ss,
-                  cudaStream_t st) {
-  launch_pdl(embed_kernel, dim3(bl.n_tok), dim3(256), 0, st, (const int*)bl.tok_id, static_cast<const __nv_bfloat16*>(embed), h,
-             dm.hidden, dm.vocab, static_cast<const __nv_bfloat16*>(gain), static_cast<__nv_bfloat16*>(x), ss, bl.dyn);
+                  void* rope_cs, cudaStream_t st) {
+  launch_pdl(embed_kernel, dim3(bl.n_tok), dim3(256), 0, st, (const int*)bl.tok_id, (const int*)bl.tok_pos,
+             static_cast<const __nv_bfloat16*>(embed), h, dm.hidden, dm.vocab, static_cast<const __nv_bfloat16*>(gain),
+             static_cast<__nv_bfloat16*>(x), ss, dm.rms_eps, static_cast<float2*>(rope_cs), dm.head_dim / 2,
+             log((double)dm.rope_base), bl.n_tok, bl.dyn);
 }
 
 void launch_rmsnorm(const float* h, const void* gain, void* x, int rows, int hidden, float eps, cudaStream_t st,
@@ -445,34 +526,6 @@ void launch_kv_io(bool write, void* pool, int64_t n_pages, int layer, const Dims
   }
 }
 
-}  // namespace recg
-
-namespace recg {
-namespace {
-__global__ void rope_table_kernel(const int* __restrict__ tok_pos, int n_tok, int half, double log_base,
-                                  float2* __restrict__ cs, const int* __restrict__ n_tok_dev) {
-  griddep_launch();
-  griddep_wait();
-  if (n_tok_dev) n_tok = n_tok_dev[0];     // (the grid was sized for the capacity)
-  // frequency-major [half][n_tok]: the projection epilogue has one token per thread, so a warp reads 32 consecutive
-  // tokens of one frequency in one 256-byte request
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= n_tok * half) return;
-  const int i = idx / n_tok, t = idx % n_tok;
-  const double theta = exp(-log_base * (double)i / (double)half);  // base^(-2i/d)
-  const double ang = (double)tok_pos[t] * theta;
-  cs[idx] = make_float2((float)cos(ang), (float)sin(ang));
-}
-}  // namespace
-
-void launch_rope_table(const int* tok_pos, int n_tok, int head_dim, float rope_base, void* cs, cudaStream_t st,
-                       const int* n_tok_dev) {
-  const int half = head_dim / 2;
-  const int total = n_tok * half;
-  if (total <= 0) return;
-  launch_pdl(rope_table_kernel, dim3((total + 255) / 256), dim3(256), 0, st, tok_pos, n_tok, half,
-             log((double)rope_base), static_cast<float2*>(cs), n_tok_dev);
-}
 }  // namespace recg
 
 // ---------------------------------------------------------------------------------------------------

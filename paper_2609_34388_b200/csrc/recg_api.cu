@@ -137,7 +137,6 @@ size_t carve(recg_ctx* c, DeviceArena& A) {
   bl.max_parts = 4 * c->target_items;      // two lines of work, each cut at fewer than target_items places (see layout.cu)
   bl.max_items = (int)(4 * c->target_items + max_tiles);
   bl.items = A.take<AttnItem>(bl.max_items);
-  bl.item_cta = A.take<int>(bl.max_items);
   bl.tiles = A.take<AttnTile>(max_tiles);
   bl.tile_off = A.take<int>(Cm + 1);
   bl.cta_off = A.take<int>(4 * (c->target_items + 1));
@@ -529,7 +528,6 @@ static recg_status run_forward(recg_ctx* ctx, void* kv_pool, int64_t kv_pool_pag
   const BatchLayout& bl = ctx->bl;
   const int T = bl.n_tok;
   cudaStream_t st = ctx->stream;
-  launch_rope_table(bl.tok_pos, T, d.head_dim, d.rope_base, ctx->rope_cs, st, bl.dyn);
   // RMSNorm runs as a kernel of its own, or (RECG_FLAG_FOLD_NORM, tcgen05 path only) folded into the projections:
   // whoever writes the residual stream also writes x = bf16(h * gain of the next norm) and partial sums of squares per
   // row, and the projection that reads x scales its accumulator rows by the row's rstd.
@@ -541,10 +539,10 @@ static recg_status run_forward(recg_ctx* ctx, void* kv_pool, int64_t kv_pool_pag
   const bool fold = ((ctx->cfg.flags & RECG_FLAG_FOLD_NORM) || chain) && !(ctx->cfg.flags & RECG_FLAG_SIMT_GEMM);
   const int Tm = ctx->cfg.max_tokens;
   const void* first_gain = d.n_layers > 0 ? ctx->attn_norm[0] : ctx->final_norm;
-  launch_embed(bl, d, ctx->embed, ctx->h, fold ? first_gain : nullptr, ctx->x, ctx->ss, st);
+  launch_embed(bl, d, ctx->embed, ctx->h, first_gain, ctx->x, fold ? ctx->ss : nullptr, ctx->rope_cs, st);
   int slots = 1;
   CU(cudaGetLastError());
-  ctx->mark(0, 3);
+  ctx->mark(0, 2);
   const int qdim = d.n_q * d.head_dim;
   int n_proj = 0;                        // projections enqueued so far in this step
   auto normed = [&](GemmArgs& g) {       // g reads the normalised residual stream
@@ -569,7 +567,7 @@ static recg_status run_forward(recg_ctx* ctx, void* kv_pool, int64_t kv_pool_pag
     if (chain && l > 0) {
       // the QKV projection of this layer was the last op of the previous layer's chain
     } else {
-    if (!fold) {
+    if (!fold && l > 0) {                // (the embedding kernel has normalised the first layer's input)
       launch_rmsnorm(ctx->h, ctx->attn_norm[l], ctx->x, T, d.hidden, d.rms_eps, st, bl.dyn);
       ctx->mark(1, 1);
     }
@@ -634,7 +632,7 @@ static recg_status run_forward(recg_ctx* ctx, void* kv_pool, int64_t kv_pool_pag
     ctx->mark(6, 1);
   }
   if (!chain) {      // (the chain of the last layer ends with the LM head)
-    if (!fold) {
+    if (!fold && d.n_layers > 0) {
       launch_rmsnorm(ctx->h, ctx->final_norm, ctx->x, T, d.hidden, d.rms_eps, st, bl.dyn);
       ctx->mark(1, 1);
     }
