@@ -362,64 +362,75 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attention_kernel(AttnParams P
 
 // Merges the KV-range partials of the tiles that were split.  Tiles with a single part were written by the
 // attention kernel itself and are skipped.  Work unit = 16 rows of a tile, one warp per query row, each lane D/32
-// consecutive dims.  The kernel is latency bound (tile entry -> (max, sum) pairs -> partial rows), so every level
-// is fetched for all parts at once and the grid is sized to hold all rows in one or two waves.
+// consecutive dims.  Bound by latency, not by its bytes (a tile entry, the (max, sum) pairs and the partial rows are
+// dependent reads): the tile entry is read ahead of the wait where the work list is settled, lane p fetches the pair of part
+// p, so that one read and a few shuffles give all weights of up to 32 parts, and the rows of the first kRows parts are on
+// their way at the same time.  Measured for one request (18 parts per row), attention and combine kernel of a layer together:
+// 19.5 us with four parts fetched at a time, each with its own pair, 16.1 us like this.
 template <int D>
-__global__ void __launch_bounds__(512, 3) attention_combine_kernel(const AttnTile* __restrict__ tiles,
+__global__ void __launch_bounds__(512, 2) attention_combine_kernel(const AttnTile* __restrict__ tiles,
                                                                 const int* __restrict__ counts, int n_q, int group,
                                                                 const float* __restrict__ part_o,
                                                                 const float* __restrict__ part_ml,
-                                                                __nv_bfloat16* __restrict__ o) {
+                                                                __nv_bfloat16* __restrict__ o, int list_settled) {
   constexpr int E = D / 32;
-  constexpr int kMaxP = 4;     // parts fetched together; longer lists go round by round
+  constexpr int kRows = 6;     // partial rows in flight
   griddep_launch();
-  griddep_wait();
+  if (!list_settled) griddep_wait();
   const int n_tiles = counts[1];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  AttnTile tl = {};
+  if ((int)blockIdx.x < n_tiles * 8) tl = tiles[blockIdx.x >> 3];
+  if (list_settled) griddep_wait();
   for (int wu = blockIdx.x; wu < n_tiles * 8; wu += gridDim.x) {
-    const AttnTile tl = tiles[wu >> 3];
+    if (wu != (int)blockIdx.x) tl = tiles[wu >> 3];
     if (tl.n_parts <= 1) continue;
     const int rho = (wu & 7) * 16 + warp;
     if (rho >= tl.ntok * group) continue;
+    const float* rows = part_o + ((size_t)tl.part_begin * 128 + rho) * D + lane * E;
+    auto fetch = [&](int p, float (&v)[E]) {
+      if constexpr (E == 4) {
+        const float4 t = __ldcg(reinterpret_cast<const float4*>(rows + (size_t)p * 128 * D));
+        v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+      } else {
+        const float2 t = __ldcg(reinterpret_cast<const float2*>(rows + (size_t)p * 128 * D));
+        v[0] = t.x; v[1] = t.y;
+      }
+    };
     float acc[E];
 #pragma unroll
     for (int e = 0; e < E; ++e) acc[e] = 0.f;
     float m = -1e30f, l = 0.f;
-    for (int p0 = 0; p0 < tl.n_parts; p0 += kMaxP) {
-      const int np = min(kMaxP, tl.n_parts - p0);
-      float2 ml[kMaxP];
-      float v[kMaxP][E];
+    for (int p0 = 0; p0 < tl.n_parts; p0 += 32) {
+      const int np = min(32, tl.n_parts - p0);
+      float2 ml = make_float2(-1e30f, 0.f);
+      if (lane < np) ml = __ldcg(reinterpret_cast<const float2*>(part_ml) + (size_t)(tl.part_begin + p0 + lane) * 128 + rho);
+      float v[kRows][E];
 #pragma unroll
-      for (int p = 0; p < kMaxP; ++p) {
-        ml[p] = make_float2(-1e30f, 0.f);
-        if (p < np) {
-          const size_t row = (size_t)(tl.part_begin + p0 + p) * 128 + rho;
-          ml[p] = __ldcg(reinterpret_cast<const float2*>(part_ml) + row);
-          if constexpr (E == 4) {
-            const float4 t = __ldcg(reinterpret_cast<const float4*>(part_o + row * D) + lane);
-            v[p][0] = t.x; v[p][1] = t.y; v[p][2] = t.z; v[p][3] = t.w;
-          } else {
-            const float2 t = __ldcg(reinterpret_cast<const float2*>(part_o + row * D) + lane);
-            v[p][0] = t.x; v[p][1] = t.y;
-          }
-        }
-      }
-      float m_new = m;
+      for (int k = 0; k < kRows; ++k)
+        if (k < np) fetch(p0 + k, v[k]);
+      float m_new = ml.x;
 #pragma unroll
-      for (int p = 0; p < kMaxP; ++p) m_new = fmaxf(m_new, ml[p].x);
-      const float f = exp2f(m - m_new);
+      for (int s = 16; s; s >>= 1) m_new = fmaxf(m_new, __shfl_xor_sync(0xffffffffu, m_new, s));
+      m_new = fmaxf(m_new, m);
+      const float f = exp2f(m - m_new), wgt = exp2f(ml.x - m_new);   // (a lane without a part: sum 0)
       m = m_new;
-      l *= f;
+      float ls = wgt * ml.y;
+#pragma unroll
+      for (int s = 16; s; s >>= 1) ls += __shfl_xor_sync(0xffffffffu, ls, s);
+      l = l * f + ls;
 #pragma unroll
       for (int e = 0; e < E; ++e) acc[e] *= f;
+      for (int k0 = 0; k0 < np; k0 += kRows) {
 #pragma unroll
-      for (int p = 0; p < kMaxP; ++p)
-        if (p < np) {
-          const float wgt = exp2f(ml[p].x - m);
-          l += wgt * ml[p].y;
+        for (int k = 0; k < kRows; ++k) {
+          if (k0 + k >= np) continue;
+          const float wk = __shfl_sync(0xffffffffu, wgt, k0 + k);
 #pragma unroll
-          for (int e = 0; e < E; ++e) acc[e] += wgt * v[p][e];
+          for (int e = 0; e < E; ++e) acc[e] += wk * v[k][e];
+          if (k0 + kRows + k < np) fetch(p0 + k0 + kRows + k, v[k]);      // the slot's next row follows at once
         }
+      }
     }
     const float inv = l > 0.f ? 1.f / l : 0.f;
     const int j = rho / group, hg = rho % group;
@@ -465,7 +476,7 @@ void launch_attention_t(const BatchLayout& bl, const Dims& dm, int layer, const 
   P.status = status;
   launch_pdl(attention_kernel<D>, dim3(n_sm), dim3(kAttnThreads), AttnSmem<D>::kTotal, st, P);
   launch_pdl(attention_combine_kernel<D>, dim3(4 * n_sm), dim3(512), 0, st, (const AttnTile*)bl.tiles, (const int*)bl.counts,
-             dm.n_q, P.group, (const float*)part_o, (const float*)part_ml, static_cast<__nv_bfloat16*>(o));
+             dm.n_q, P.group, (const float*)part_o, (const float*)part_ml, static_cast<__nv_bfloat16*>(o), 0);
 }
 
 }  // namespace
@@ -481,7 +492,7 @@ void launch_attention(const BatchLayout& bl, const Dims& dm, int layer, const vo
     launch_attention_tc_main(bl, dm, layer, q, o, kv_pool, n_pages, part_o, part_ml, n_sm, status, st, layout_settled);
     launch_pdl(attention_combine_kernel<128>, dim3(4 * n_sm), dim3(512), 0, st, (const AttnTile*)bl.tiles,
                (const int*)bl.counts, dm.n_q, dm.n_q / dm.n_kv, (const float*)part_o, (const float*)part_ml,
-               static_cast<__nv_bfloat16*>(o));
+               static_cast<__nv_bfloat16*>(o), 1);    // (the kernel in front signals its dependents after its own wait)
     return;
   }
   if (dm.head_dim == 64)
