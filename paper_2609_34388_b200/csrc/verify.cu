@@ -59,40 +59,92 @@ __device__ __forceinline__ void mass_merge(Mass& a, const Mass& b) {
   a.t += bb.t;
 }
 
+// One 16-byte vector of logits as words; fill = -inf in every element.
 template <typename T> struct Vec;
 template <> struct Vec<__nv_bfloat16> {
   static constexpr int N = 8;
-  __device__ static void load(const __nv_bfloat16* p, float (&x)[8]) {
-    uint4 u;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(u.x), "=r"(u.y), "=r"(u.z), "=r"(u.w)
-                 : "l"(p));
-    const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+  static constexpr uint32_t kFill = 0xff80ff80u;
+  __device__ static float one(const __nv_bfloat16* p) { return __bfloat162float(*p); }
+  // largest element of four vectors
+  __device__ static float max_of(const uint4 (&r)[4]) {
+    __nv_bfloat162 m = word(r[0].x);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) m = __hmax2(__hmax2(m, __hmax2(word(r[u].x), word(r[u].y))), __hmax2(word(r[u].z), word(r[u].w)));
+    return fmaxf(__low2float(m), __high2float(m));
+  }
+  __device__ static __nv_bfloat162 word(uint32_t w) { return *reinterpret_cast<__nv_bfloat162*>(&w); }
+  __device__ static void elements(const uint4& r, float (&x)[8]) {
+    const uint32_t w[4] = {r.x, r.y, r.z, r.w};
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       x[2 * i] = __uint_as_float(w[i] << 16);
       x[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
     }
   }
-  __device__ static float one(const __nv_bfloat16* p) { return __bfloat162float(*p); }
+  static constexpr int kPairs = 4;       // pairs of elements per vector
+  __device__ static float2 pair(const uint4& r, int i) {
+    const uint32_t w = i == 0 ? r.x : (i == 1 ? r.y : (i == 2 ? r.z : r.w));
+    const __nv_bfloat162 c = __hmax2(word(w), word(0xff7fff7fu));      // -inf -> the lowest finite value
+    const uint32_t cw = *reinterpret_cast<const uint32_t*>(&c);
+    return make_float2(__uint_as_float(cw << 16), __uint_as_float(cw & 0xffff0000u));
+  }
 };
 template <> struct Vec<float> {
   static constexpr int N = 4;
-  __device__ static void load(const float* p, float (&x)[4]) {
-    float4 u = __ldg(reinterpret_cast<const float4*>(p));
-    x[0] = u.x; x[1] = u.y; x[2] = u.z; x[3] = u.w;
-  }
+  static constexpr uint32_t kFill = 0xff800000u;
   __device__ static float one(const float* p) { return *p; }
+  __device__ static float max_of(const uint4 (&r)[4]) {
+    float m = -INFINITY;
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      m = fmaxf(m, fmaxf(fmaxf(__uint_as_float(r[u].x), __uint_as_float(r[u].y)), fmaxf(__uint_as_float(r[u].z), __uint_as_float(r[u].w))));
+    return m;
+  }
+  __device__ static void elements(const uint4& r, float (&x)[4]) {
+    x[0] = __uint_as_float(r.x); x[1] = __uint_as_float(r.y); x[2] = __uint_as_float(r.z); x[3] = __uint_as_float(r.w);
+  }
+  static constexpr int kPairs = 2;
+  __device__ static float2 pair(const uint4& r, int i) {
+    return i == 0 ? make_float2(fmaxf(__uint_as_float(r.x), -3.0e38f), fmaxf(__uint_as_float(r.y), -3.0e38f))
+                  : make_float2(fmaxf(__uint_as_float(r.z), -3.0e38f), fmaxf(__uint_as_float(r.w), -3.0e38f));
+  }
 };
+__device__ __forceinline__ uint4 ld_stream(const void* p) {
+  uint4 u;
+  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(u.x), "=r"(u.y), "=r"(u.z), "=r"(u.w) : "l"(p));
+  return u;
+}
+// two fp32 operations per instruction
+__device__ __forceinline__ float2 fma2(const float2& a, const float2& b, const float2& c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;"
+      : "=l"(d)
+      : "l"(reinterpret_cast<const uint64_t&>(a)), "l"(reinterpret_cast<const uint64_t&>(b)), "l"(reinterpret_cast<const uint64_t&>(c)));
+  return reinterpret_cast<float2&>(d);
+}
+__device__ __forceinline__ float2 add2(const float2& a, const float2& b) {
+  uint64_t d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(reinterpret_cast<const uint64_t&>(a)), "l"(reinterpret_cast<const uint64_t&>(b)));
+  return reinterpret_cast<float2&>(d);
+}
 
 // One-dimensional grid of rows x chunks_per_row CTAs, chunk-fastest (consecutive CTAs read consecutive memory; the
 // row count is not bound by the 65535 limit of the other grid dimensions).  Each CTA scans [c0, c1) of one row.
+// Bound by HBM for bf16 logits only if little else is done per element (6.4 TB/s is 22 elements per SM and clock, the 2^x
+// unit gives 16 of them, the issue slots 128): vectors stay packed (maxima and the clamp of -inf on two bf16 at a time), sums
+// use two-element instructions, the next four vectors of a thread are on their way while it works on four, and the search
+// for the two largest elements remembers only the two best GROUPS of four vectors per thread, of which the CTA afterwards
+// re-reads those that reach its second-largest group maximum (two, as a rule).  8448 rows x 128256 bf16, the kernel: 435 us
+// with unpacked arithmetic, loads behind the arithmetic and a search per thread, 358 us (6.05 TB/s) like this.
 template <typename T>
-__global__ void __launch_bounds__(kVerifyThreads) verify_partial_kernel(const T* __restrict__ logits, int vocab,
-                                                                        int chunk_len, int chunks_per_row,
-                                                                        RowPartial* __restrict__ partials,
-                                                                        const int* __restrict__ rows_dev) {
-  constexpr int N = Vec<T>::N;
+__global__ void __launch_bounds__(kVerifyThreads, 4) verify_partial_kernel(const T* __restrict__ logits, int vocab,
+                                                                           int chunk_len, int chunks_per_row,
+                                                                           RowPartial* __restrict__ partials,
+                                                                           const int* __restrict__ rows_dev) {
+  constexpr int N = Vec<T>::N, kWarps = kVerifyThreads / 32;
+  __shared__ float2 s_g[kWarps];
+  __shared__ Top2 s_tp[kWarps];
+  __shared__ float2 s_st[kWarps];
   griddep_launch();
   griddep_wait();
   const int row = blockIdx.x / chunks_per_row, chunk = blockIdx.x - row * chunks_per_row;
@@ -100,113 +152,131 @@ __global__ void __launch_bounds__(kVerifyThreads) verify_partial_kernel(const T*
   const T* base = logits + (size_t)row * vocab;
   const int c0 = chunk * chunk_len;
   const int c1 = min(vocab, c0 + chunk_len);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const bool vec_ok = ((reinterpret_cast<uintptr_t>(base + c0) & 15) == 0);
+  const int nvec = vec_ok ? (c1 - c0) / N : 0;
   Top2 tp = {-INFINITY, -INFINITY, 0x7fffffff, 0x7fffffff};
   Mass ms = {-INFINITY, 0.f, 0.f};
-  const bool vec_ok = ((reinterpret_cast<uintptr_t>(base + c0) & 15) == 0);
-  int done = c0;
-  if (vec_ok) {
-    const int nvec = (c1 - c0) / N;
-    // Four 16-byte loads in flight per thread.  In the loop the top-2 bookkeeping is branch-free and per VECTOR:
-    // each thread remembers its two vectors with the largest maximum (the two largest elements it has seen lie
-    // in those two vectors; strict comparisons keep the earlier vector on ties), and only after the loop are
-    // these two vectors re-read and searched element by element.  A per-element test would diverge in nearly
-    // every warp and cost more issue slots than the arithmetic.
-    float bv1 = -INFINITY, bv2 = -INFINITY;   // two largest vector maxima of this thread
-    int bi1 = -1, bi2 = -1;                   // their vector indices
-    auto track = [&](float vmax, int vec) {
-      const bool g1 = vmax > bv1, g2 = vmax > bv2;
-      bi2 = g1 ? bi1 : (g2 ? vec : bi2);
-      bv2 = g1 ? bv1 : (g2 ? vmax : bv2);
-      bi1 = g1 ? vec : bi1;
-      bv1 = g1 ? vmax : bv1;
-    };
-    int i = threadIdx.x;
-    for (; i + 3 * kVerifyThreads < nvec; i += 4 * kVerifyThreads) {
-      float x[4][N];
+  float g1 = -INFINITY, g2 = -INFINITY;      // the two largest group maxima of this thread ...
+  int i1 = -1, i2 = -1;                      // ... and the first vector of those groups (the earlier one on ties)
+  const uint4* vec = reinterpret_cast<const uint4*>(base + c0);
+  auto fetch = [&](int i, uint4 (&r)[4]) {
 #pragma unroll
-      for (int u = 0; u < 4; ++u) Vec<T>::load(base + c0 + (size_t)(i + u * kVerifyThreads) * N, x[u]);
-      float vm[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        vm[u] = x[u][0];
-#pragma unroll
-        for (int k = 1; k < N; ++k) vm[u] = fmaxf(vm[u], x[u][k]);
+    for (int u = 0; u < 4; ++u) {
+      const int k = i + u * kVerifyThreads;
+      r[u] = k < nvec ? ld_stream(vec + k) : make_uint4(Vec<T>::kFill, Vec<T>::kFill, Vec<T>::kFill, Vec<T>::kFill);
+    }
+  };
+  if (nvec > 0) {
+    uint4 cur[4], nxt[4];
+    float2 s2 = make_float2(0.f, 0.f), t2 = make_float2(0.f, 0.f);
+    const float2 log2e = make_float2(kLog2e, kLog2e);
+    fetch(tid, cur);
+    for (int i = tid; i < nvec; i += 4 * kVerifyThreads) {
+      fetch(i + 4 * kVerifyThreads, nxt);
+      const float gm = Vec<T>::max_of(cur);
+      if (gm > ms.m) {
+        const float f = exp2f((ms.m - gm) * kLog2e);      // 0 the first time
+        s2.x *= f; s2.y *= f; t2.x *= f; t2.y *= f;
+        ms.m = gm;
       }
-      mass_rebase(ms, fmaxf(fmaxf(vm[0], vm[1]), fmaxf(vm[2], vm[3])));
+      const bool b1 = gm > g1, b2 = gm > g2;
+      i2 = b1 ? i1 : (b2 ? i : i2);
+      g2 = b1 ? g1 : (b2 ? gm : g2);
+      i1 = b1 ? i : i1;
+      g1 = b1 ? gm : g1;
       const float neg = ms.m > -INFINITY ? -ms.m * kLog2e : 0.f;   // all -inf so far: every term underflows to 0
+      const float2 neg2 = make_float2(neg, neg);
 #pragma unroll
-      for (int k = 0; k < N; ++k) {
+      for (int u = 0; u < 4; ++u)
 #pragma unroll
-        for (int u = 0; u < 4; ++u) mass_add(ms, x[u][k], neg);
-      }
+        for (int k = 0; k < Vec<T>::kPairs; ++k) {
+          const float2 x = Vec<T>::pair(cur[u], k);
+          const float2 y = fma2(x, log2e, neg2);
+          const float2 e = make_float2(exp2f(y.x), exp2f(y.y));
+          s2 = add2(s2, e);
+          t2 = fma2(x, e, t2);
+        }
 #pragma unroll
-      for (int u = 0; u < 4; ++u) track(vm[u], i + u * kVerifyThreads);
+      for (int u = 0; u < 4; ++u) cur[u] = nxt[u];
     }
-    for (; i < nvec; i += kVerifyThreads) {
-      float x[N];
-      Vec<T>::load(base + c0 + (size_t)i * N, x);
-      float vm = x[0];
-#pragma unroll
-      for (int k = 1; k < N; ++k) vm = fmaxf(vm, x[k]);
-      mass_rebase(ms, vm);
-      const float neg = ms.m > -INFINITY ? -ms.m * kLog2e : 0.f;   // all -inf so far: every term underflows to 0
-#pragma unroll
-      for (int k = 0; k < N; ++k) mass_add(ms, x[k], neg);
-      track(vm, i);
-    }
-    // element-level search of the two remembered vectors (in index order, so that ties resolve to the lowest index)
-    const int lo_vec = bi2 < 0 ? bi1 : min(bi1, bi2), hi_vec = bi2 < 0 ? -1 : max(bi1, bi2);
-    const int cand[2] = {lo_vec, hi_vec};
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      if (cand[q] < 0) continue;
-      float x[N];
-      Vec<T>::load(base + c0 + (size_t)cand[q] * N, x);
-#pragma unroll
-      for (int k = 0; k < N; ++k) top2_insert(tp, x[k], c0 + cand[q] * N + k);
-    }
-    done = c0 + nvec * N;
+    ms.s = s2.x + s2.y;
+    ms.t = t2.x + t2.y;
   }
-  for (int i = done + threadIdx.x; i < c1; i += kVerifyThreads) {
+  // elements outside whole vectors (unaligned rows: all of them)
+  for (int i = c0 + nvec * N + tid; i < c1; i += kVerifyThreads) {
     const float x = Vec<T>::one(base + i);
     mass_rebase(ms, x);
     mass_add(ms, x, ms.m > -INFINITY ? -ms.m * kLog2e : 0.f);
     if (x >= tp.m2) top2_insert(tp, x, i);
   }
-  // warp reduce, then across warps through shared memory
+  const float e1 = tp.m1, e2 = tp.m2;
+  // the CTA's largest and second-largest of the groups' maxima and the single elements
+  float h1 = fmaxf(g1, e1), h2 = fmaxf(fminf(g1, e1), fmaxf(g2, e2));
 #pragma unroll
   for (int o = 16; o; o >>= 1) {
-    Top2 ot;
-    ot.m1 = __shfl_xor_sync(0xffffffffu, tp.m1, o);
-    ot.i1 = __shfl_xor_sync(0xffffffffu, tp.i1, o);
-    ot.m2 = __shfl_xor_sync(0xffffffffu, tp.m2, o);
-    ot.i2 = __shfl_xor_sync(0xffffffffu, tp.i2, o);
+    const float a = __shfl_xor_sync(0xffffffffu, h1, o), b = __shfl_xor_sync(0xffffffffu, h2, o);
+    h2 = fmaxf(fminf(h1, a), fmaxf(h2, b));
+    h1 = fmaxf(h1, a);
+  }
+  if (lane == 0) s_g[warp] = make_float2(h1, h2);
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w) {
+    const float2 g = s_g[w];
+    if (w == 0) { h1 = g.x; h2 = g.y; continue; }
+    h2 = fmaxf(fminf(h1, g.x), fmaxf(h2, g.y));
+    h1 = fmaxf(h1, g.x);
+  }
+  // The two largest elements are not below the second-largest group maximum: only groups that reach it are searched element
+  // by element (in index order; ties resolve to the lowest index).
+  const int lo = i2 < 0 ? i1 : min(i1, i2), hi = i2 < 0 ? -1 : max(i1, i2);
+  const float g_lo = lo == i1 ? g1 : g2, g_hi = hi == i2 ? g2 : g1;
+#pragma unroll 1
+  for (int q = 0; q < 2; ++q) {
+    const int i = q ? hi : lo;
+    if (i < 0 || (q ? g_hi : g_lo) < h2) continue;
+    uint4 r[4];
+    fetch(i, r);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      float x[N];
+      Vec<T>::elements(r[u], x);
+      if (i + u * kVerifyThreads < nvec)
+#pragma unroll
+        for (int k = 0; k < N; ++k)
+          if (x[k] >= tp.m2) top2_insert(tp, x[k], c0 + (i + u * kVerifyThreads) * N + k);
+    }
+  }
+  const float f = ms.m > -INFINITY ? exp2f((ms.m - h1) * kLog2e) : 0.f;
+  ms.s *= f;
+  ms.t *= f;
+  const bool any = __any_sync(0xffffffffu, tp.i1 != 0x7fffffff);
+#pragma unroll
+  for (int o = 16; o; o >>= 1) {
+    ms.s += __shfl_xor_sync(0xffffffffu, ms.s, o);
+    ms.t += __shfl_xor_sync(0xffffffffu, ms.t, o);
+    if (!any) continue;
+    const Top2 ot = {__shfl_xor_sync(0xffffffffu, tp.m1, o), __shfl_xor_sync(0xffffffffu, tp.m2, o),
+                     __shfl_xor_sync(0xffffffffu, tp.i1, o), __shfl_xor_sync(0xffffffffu, tp.i2, o)};
     top2_insert(tp, ot.m1, ot.i1);
     top2_insert(tp, ot.m2, ot.i2);
-    Mass om;
-    om.m = __shfl_xor_sync(0xffffffffu, ms.m, o);
-    om.s = __shfl_xor_sync(0xffffffffu, ms.s, o);
-    om.t = __shfl_xor_sync(0xffffffffu, ms.t, o);
-    mass_merge(ms, om);
   }
-  __shared__ Top2 s_tp[kVerifyThreads / 32];
-  __shared__ Mass s_ms[kVerifyThreads / 32];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (lane == 0) {
     s_tp[warp] = tp;
-    s_ms[warp] = ms;
+    s_st[warp] = make_float2(ms.s, ms.t);
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < kVerifyThreads / 32; ++w) {
+  if (tid == 0) {
+    for (int w = 1; w < kWarps; ++w) {
       top2_insert(tp, s_tp[w].m1, s_tp[w].i1);
       top2_insert(tp, s_tp[w].m2, s_tp[w].i2);
-      mass_merge(ms, s_ms[w]);
+      ms.s += s_st[w].x;
+      ms.t += s_st[w].y;
     }
-    // express the mass relative to the chunk maximum m1 (== ms.m unless the chunk is empty)
     RowPartial p;
     p.m1 = tp.m1; p.m2 = tp.m2; p.i1 = tp.i1; p.i2 = tp.i2;
-    p.s = ms.s; p.t = ms.t;
+    p.s = ms.s; p.t = ms.t;               // relative to the chunk's maximum
     partials[(size_t)row * chunks_per_row + chunk] = p;
   }
 }
