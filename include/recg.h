@@ -50,12 +50,10 @@ enum {
   RECG_FLAG_LOGITS_BF16 = 1, /* recg_step() stores logits as bf16 instead of fp32               */
   RECG_FLAG_SIMT_GEMM = 2,   /* run the projections on the legacy mma.sync kernel (A/B checks)  */
   RECG_FLAG_SIMT_ATTENTION = 4, /* run attention on the legacy mma.sync kernel (A/B checks)     */
-  RECG_FLAG_FOLD_NORM = 16,  /* fold every RMSNorm into the projections around it instead of running it as a kernel of
-                                its own: the projection that updates the residual stream also writes x = bf16(h * gain)
-                                and per-row partial sums of squares, the projection that reads x scales its rows by the
-                                row's rstd.  Same results within bf16 rounding (x is rounded before the division instead
-                                of after it); measured 3 % slower than the separate kernel, which hides behind the next
-                                projection's weight prefetch, hence off by default                            */
+  RECG_FLAG_FOLD_NORM = 16,  /* fold every RMSNorm into the projections around it: the projection that updates the residual
+                                stream also writes x = bf16(h * gain) and per-row partial sums of squares, the projection
+                                that reads x scales its rows by the row's rstd.  This is what the tcgen05 projections do
+                                in any case; the flag is kept for callers that set it                         */
   RECG_FLAG_CHAIN = 32,      /* steps of at most 128 rows (low concurrency): run the projections between two attention
                                 calls (output projection, gate|up, down, the next layer's QKV projection or the LM head)
                                 as ONE persistent kernel with grid-wide barriers, so that the weight stream does not stop
@@ -261,12 +259,11 @@ recg_status recg_debug_buffer(recg_ctx *ctx, int32_t which, const void **ptr, in
 /*
  * Debugging aids (the paper has no counterpart).
  * recg_debug_gemm_config(): force the tile configuration of the projection launches that follow on this context,
- *   instead of the cost model's choice: tile = 64, 128 or 256 (single CTAs, 128-row tiles of that width), 384 (CTA
- *   pairs, 256 x 128 tiles), 512 (CTA pairs, 256 x 256 tiles), 0 = back to the cost model; stream_k = 1 cuts the
- *   K range of the tiles evenly over the SMs, stream_k = 2 does the same and also (with any tile value, 0 included)
- *   keeps problems of at most 128 rows from handing their partial tiles over inside thread-block clusters: they go
- *   through the partial-tile workspace like everything else; stream_k = 0: whole tiles.  A configuration that does not
- *   fit a shape is ignored for that launch.
+ *   instead of the cost model's choice: tile = 64, 128 or 256 (single CTAs, 128 output features x at most that many rows),
+ *   384 or 512 (CTA pairs, 256 output features x at most 128 or 256 rows), 0 = back to the cost model; stream_k = 1 cuts the
+ *   K range of the tiles over the SMs, stream_k = 2 does the same and also (with any tile value, 0 included) keeps
+ *   partial tiles from being handed over inside thread-block clusters: they go through the partial-tile workspace;
+ *   stream_k = 0: whole tiles.  A configuration that does not fit a shape is ignored for that launch.
  * recg_debug_wait_timeout(): enqueue a one-thread kernel that waits on a barrier nobody arrives on, bounded by
  *   max_polls polls (1 .. 1048576) exactly like the waits inside the kernels; it gives up, records the timeout in the
  *   device status word and returns.  The next recg_sync() then reports RECG_ERR_TIMEOUT and clears the word; the

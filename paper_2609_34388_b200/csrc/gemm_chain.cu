@@ -443,10 +443,10 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_chain_kernel(const __grid_co
             const int head = tile;             // one head per tile: head_dim = 128
             const bool is_q = head < P.n_q, is_v = head >= P.n_q + P.n_kv;
             if (!is_v) {
-              const float2* cs = P.rope_cs + (size_t)(16 * pc) * P.M + m;      // [frequency][token]
+              const float2* cs = P.rope_cs + (size_t)m * 64 + 16 * pc;      // [token][frequency]
 #pragma unroll
               for (int i = 0; i < 16; ++i) {
-                const float2 t = cs[(size_t)i * P.M];
+                const float2 t = cs[i];
                 const float a = lo[i] * t.x - hi[i] * t.y, b = hi[i] * t.x + lo[i] * t.y;
                 lo[i] = a;
                 hi[i] = b;

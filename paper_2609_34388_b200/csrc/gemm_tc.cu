@@ -1,19 +1,32 @@
 // Projection GEMM on the 5th-generation tensor cores: y = x . w^T, bf16 in, fp32 accumulate in TMEM.
 //
+// The WEIGHTS are the M operand (128 output features per CTA) and the tokens the N operand of the tensor core: the N extent
+// of an instruction is any multiple of 16 up to 256, so a batch of T rows is cut into ceil(T / 256) or a few more equal token
+// tiles and next to nothing is computed for padding (with the tokens on the M side 376 rows cost as much as 512), and an
+// accumulator tile is spread over all four epilogue warps however few tokens there are (TMEM lane = output feature).
+//
 // Persistent, warp-specialised CTA of 6 warps:
-//   warp 0   producer: TMA tiled loads (128B swizzle) of the x tile [128 x 64] and the w tile [BN x 64]
-//            into a shared-memory ring, completion on mbarriers;
-//   warp 1   one elected lane issues tcgen05.mma (M = 128, N = BN, K = 16) from shared-memory descriptors
+//   warp 0   producer: TMA loads (128-byte swizzle) of the w tile [128 x 64] and the x tile [tokens x 64] into a
+//            shared-memory ring, completion on mbarriers;
+//   warp 1   one elected lane issues tcgen05.mma (M = 128, N = tokens, K = 16) from shared-memory descriptors
 //            into one of two TMEM accumulators and commits to the ring's empty barriers;
-//   warps 2-5  epilogue: tcgen05.ld of the finished accumulator (each warp its 32-lane quadrant), then the
-//            fused epilogue straight from registers (residual add, SwiGLU, rotary + paged KV append, or
-//            plain store) while the MMA warp already fills the other accumulator; output rows leave through
-//            TMA box stores (add-reductions for the residual stream) from a small swizzled staging area.
-// Tiles are walked m-fastest so that CTAs running together share the same weight tile through L2.
-// Tiles can be cut over K (stream-K): partial tiles are parked in a workspace and reduced by the last part to arrive; for
-// problems of one row tile (at most 128 rows) the parts of a tile form a thread-block cluster instead and hand their
-// partial tiles to the cluster's leader through distributed shared memory.
+//   warps 2-5  epilogue: tcgen05.ld of the finished accumulator (each warp its 32 lanes = features, 32 tokens at a time),
+//            then the fused epilogue straight from registers (residual add with the next norm's input, SwiGLU, rotary +
+//            paged KV append, or plain store) while the MMA warp already fills the other accumulator.  One warp per
+//            scheduler runs it, so what counts is its instructions: the 16x256b form of tcgen05.ld hands out 8 x 8 fragments,
+//            stmatrix.trans turns them into rows of tokens, and stores are whole 32-byte sectors.
+// Operands of an epilogue that belong together sit in the same thread: the tensor map over w lists its rows 16 by 16 in the
+// order the tile wants them (16 gate rows, their 16 up rows, ...; 16 low dims of a head, their 16 rotation partners, ...), and
+// a thread holds the same row of both halves of a 32-row quadrant.
+// Tiles are walked token-fastest so that CTAs running together share the same weight tile through L2.
+// Tiles can be cut over K: stream-K (partial tiles are parked in a workspace and reduced by the last part to arrive), or the
+// parts of a tile form a thread-block cluster and reduce it through distributed shared memory, each member finishing its share
+// of the tokens.
 // Every wait is bounded; on a timeout the kernel records a status code, drains and frees TMEM.
+//
+// What bounds it (B200): a k-block (64 of K) costs max(operand bytes / 115 GB/s per SM (64 bytes per clock from L2), token
+// columns x 1.5 ns (the tensor pipe at the clock that the power cap leaves), weight bytes / its share of HBM).  Figures at
+// the choice of the configuration (choose_config below).
 #include <cuda.h>
 
 #include <cstdio>
@@ -32,54 +45,38 @@ namespace recg {
 
 namespace {
 
-constexpr int BM = 128, BK = 64;
+constexpr int FT = 128, BK = 64;            // output features per CTA, k-block
 constexpr int kTcThreads = 192;
-constexpr int kSmemBudget = 192 * 1024;     // operand ring (every configuration's stage size divides it)
-constexpr int kStageOutBytes = 4 * 4096;      // per epilogue warp: two 2 KB boxes of output on their way to the TMA unit
-// EPI_RESIDUAL_NORM kernels also stage the OLD residual rows (two 4 KB chunks per epilogue warp, fetched by the TMA unit
-// ahead of their use) and the gains of the tile's columns (512 bytes per warp); their operand ring is that much shorter
-constexpr int kNormHBytes = 4 * 2 * 4096;
-constexpr int kNormGBytes = 4 * 512;
-constexpr int kNormBytes = kNormHBytes + kNormGBytes + 6 * 1024;   // (rounded so that the ring budget stays a multiple of 8 KB)
+constexpr int kMaxTok = 256;                // widest token tile
+constexpr int kRingBytes = 210 * 1024;      // operand ring
+constexpr int kMaxStages = 16;
+constexpr int kABytes = FT * BK * 2;
+constexpr int kChunkBytes = 32 * FT * 4;    // 32 tokens of a partial tile
+constexpr int kAccStride = kMaxTok;         // TMEM columns between the two accumulators
+constexpr int kTmemCols = 2 * kMaxTok;
+constexpr int kOffBar = kRingBytes;
+constexpr int kBarBytes = (2 * kMaxStages + 2 + 2 + 1 + 1) * 8 + 16;
+constexpr int kOffRstd = kOffBar + ((kBarBytes + 15) & ~15);      // float [256] row factors of the token tile
+constexpr int kOffSlot = kOffRstd + kMaxTok * 4;                   // int [256] cache slots of the token tile
+constexpr int kOffSs = kOffSlot + kMaxTok * 4;                     // float [4][256] sums of squares per epilogue warp
+constexpr int kOffStage = kOffSs + 4 * kMaxTok * 4;                // per epilogue warp: 32 tokens x 32 bf16 on their way out
+constexpr int kSmemBytes = kOffStage + 4 * 2048 + 1024;            // + slack for 1024-byte alignment
+static_assert(kSmemBytes <= 227 * 1024, "shared memory budget");
 constexpr uint32_t kSpin = 1u << 22;
-
-template <int BN, bool PAIR = false, bool NORM = false> struct TcCfg {
-  static constexpr int kBudget = NORM ? kSmemBudget - kNormBytes : kSmemBudget;
-  static constexpr int kABytes = BM * BK * 2;
-  static constexpr int kBBytes = (PAIR ? BN / 2 : BN) * BK * 2;     // per CTA: a pair splits the weight tile
-  static constexpr int kStageBytes = kABytes + kBBytes;
-  static constexpr int kStages = (kBudget / kStageBytes) > 8 ? 8 : (kBudget / kStageBytes);
-  static constexpr int kMaxStages = 16;
-  // thin problems (M <= 32) load only 32 rows of x per stage: the stage shrinks and more stages fit.  The MMA
-  // still reads 128 rows; rows 32.. alias the bytes that follow (harmless: those accumulator rows are never
-  // stored), so the ring is followed by a pad that keeps the last stage's read inside the allocation.
-  static constexpr int kThinABytes = 32 * BK * 2;
-  static constexpr int kThinStageBytes = kThinABytes + kBBytes;
-  static constexpr int kThinStages =
-      (kBudget / kThinStageBytes) > kMaxStages ? kMaxStages : (kBudget / kThinStageBytes);
-  static constexpr int kRingBytes = kBudget + kABytes;     // either ring plus the pad
-  static constexpr int kBarBytes = (2 * kMaxStages + 5 + 8) * 8 + 16;
-  static constexpr int kNormOff = kRingBytes + kStageOutBytes;             // old residual rows, then gains (NORM only)
-  static constexpr int kBarOff = kNormOff + (NORM ? kNormHBytes + kNormGBytes : 0);
-  static constexpr int kSmemBytes = kBarOff + kBarBytes + 1024;  // + slack for 1024-byte alignment
-  static constexpr int kTmemCols = 2 * BN < 32 ? 32 : 2 * BN;                  // power of two: 128, 256, 512
-};
 
 using namespace tc;   // the tcgen05 / TMA wrappers (tc_ptx.cuh)
 
 // ---- CTA pairs (tcgen05 cta_group::2) ----------------------------------------------------------------
-// With PAIR a cluster of two CTAs computes tiles of 256 rows: each CTA loads its own 128 rows of x and its own
-// half of the weight tile per k-block (32 KB per stage instead of the 48 KB a single CTA needs for 128 x 256, so
-// six stages fit and a third fewer operand bytes cross L2 -> shared memory per flop); the tensor cores of the
-// pair read both halves of the weight tile, each CTA accumulates its 128 rows in its own TMEM.  Only the leader
-// CTA (cluster rank 0) issues MMAs.
+// With PAIR two CTAs of a cluster compute tiles of 256 features: each CTA loads its own 128 rows of w and its own half of the
+// token tile per k-block (28 KB for 192 tokens instead of the 40 KB of a single CTA, so more stages fit and fewer operand
+// bytes cross L2 -> shared memory per flop); the tensor cores of the pair read both halves of the token tile, each CTA
+// accumulates its 128 features in its own TMEM.  Only the pair's leader (even cluster rank) issues MMAs.
 //   full barrier  (leader's):   the leader's producer arrives with the byte count of BOTH CTAs' loads; both CTAs'
 //                               TMA loads (cta_group::2 form, no multicast) complete on it
 //   empty barrier (per CTA):    tcgen05.commit multicast to both CTAs frees the stage in each
 //   accumulator full (per CTA): commit multicast; accumulator empty (leader's): all eight epilogue warps of the
-//                               pair arrive (the peer's remotely)
-// The scheduling unit is the cluster; the two CTAs of a cluster park and reduce their halves of a cut tile
-// independently (own slots, own counters).
+//                               pair arrive (the other CTA's remotely)
+// The scheduling unit becomes the pair; its two CTAs park, hand over and reduce their halves of a cut tile independently.
 __device__ __forceinline__ uint32_t cluster_ctarank() {
   uint32_t r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
@@ -100,6 +97,22 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t smem_dst, const CUtens
                : "r"(smem_dst), "l"(map), "r"(bar_cluster), "r"(x), "r"(y)
                : "memory");
 }
+__device__ __forceinline__ void tma_load_w_pair(uint32_t smem_dst, const CUtensorMap* map, int k, int c3, int c4, uint32_t bar_cluster) {
+  const int z = 0;
+  asm volatile(
+      "cp.async.bulk.tensor.5d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %6, %6, %4, %5}], [%2];"
+      :
+      : "r"(smem_dst), "l"(map), "r"(bar_cluster), "r"(k), "r"(c3), "r"(c4), "r"(z)
+      : "memory");
+}
+__device__ __forceinline__ void tma_load_w(uint32_t smem_dst, const CUtensorMap* map, int k, int c3, int c4, uint64_t* bar) {
+  const int z = 0;
+  asm volatile(
+      "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %6, %6, %4, %5}], [%2];"
+      :
+      : "r"(smem_dst), "l"(map), "r"(smem_u32(bar)), "r"(k), "r"(c3), "r"(c4), "r"(z)
+      : "memory");
+}
 __device__ __forceinline__ void umma_bf16_pair(uint32_t tmem_d, uint64_t desc_a, uint64_t desc_b, uint32_t idesc,
                                                uint32_t accumulate) {
   const uint32_t z = 0;
@@ -110,8 +123,8 @@ __device__ __forceinline__ void umma_bf16_pair(uint32_t tmem_d, uint64_t desc_a,
       : "r"(tmem_d), "l"(desc_a), "l"(desc_b), "r"(idesc), "r"(accumulate), "r"(z)
       : "memory");
 }
-__device__ __forceinline__ void umma_commit_pair(uint64_t* bar) {   // arrives on this barrier in both CTAs
-  const uint16_t mask = 3;
+// arrives on this barrier in both CTAs of the pair (mask: their cluster ranks)
+__device__ __forceinline__ void umma_commit_pair(uint64_t* bar, uint16_t mask) {
   asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
                    smem_u32(bar)),
                "h"(mask)
@@ -130,108 +143,54 @@ __device__ __forceinline__ void tmem_dealloc_pair(uint32_t addr, uint32_t cols) 
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar_cluster) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster) : "memory");
 }
+__device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+               : "=r"(ok)
+               : "r"(smem_u32(bar)), "r"(parity)
+               : "memory");
+  return ok != 0;
+}
 __device__ __forceinline__ void st_cluster_f4(uint32_t addr_cluster, const float4& v) {
   asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr_cluster), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
                : "memory");
 }
 
-// ---- register epilogue: one thread owns one output row -------------------------------------------
-
-// ---- epilogue through the TMA unit --------------------------------------------------------------------------------
-// A warp's chunk (lane = row, 64 bytes per row: 32 bf16 or 16 fp32 columns) goes to one of the warp's two 2 KB staging
-// buffers in the 64-byte-swizzle order of the output tensor map (16-byte piece c of row r at piece c ^ ((r >> 1) & 3):
-// conflict free), and one lane hands it to the TMA unit as a 32-row box: the unit clips rows beyond M and columns
-// beyond N, writes whole row segments, and with add = true adds into the fp32 destination (one addend per element and
-// launch, hence the same single rounding as a load-add-store).  OutStage counts the boxes of the warp so that a
-// buffer is only rewritten after the unit has read it.
-struct OutStage {
-  uint8_t* buf;     // this warp's 4 KB (two buffers)
-  uint32_t k;       // boxes issued so far
-};
-__device__ __forceinline__ void tma_store_box(const CUtensorMap* map, OutStage& os, const uint4 (&piece)[4], int col, int row,
-                                              bool add, bool active, int lane) {
-  if (os.k >= 2) {
-    if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");   // the box before the last one has been read
-    __syncwarp();
-  }
-  uint4* dst = reinterpret_cast<uint4*>(os.buf + (os.k & 1) * 2048) + lane * 4;
-  const int x = (lane >> 1) & 3;
+// ---- where the epilogue takes its accumulator values (32 features x 32 tokens per warp) from --------------------------------
+// Thread `lane` holds features rg + 8 q (rg = lane / 4, q = 0 .. 3 within the warp's 32) of tokens 8 k + 2 (lane % 4) + e (k = 0 .. 3,
+// e = 0, 1) of the chunk: value (q, k, e) at index 16 (q / 2) + 4 k + 2 (q % 2) + e.
+__device__ __forceinline__ int vidx(int q, int k, int e) { return 16 * (q >> 1) + 4 * k + 2 * (q & 1) + e; }
+__device__ __forceinline__ void tmem_ld_chunk(uint32_t taddr, float (&v)[32]) {   // taddr: (lane quadrant, first column)
+  uint32_t r[32];
 #pragma unroll
-  for (int c = 0; c < 4; ++c) dst[c ^ x] = piece[c];
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  __syncwarp();
-  if (lane == 0) {
-    const uint32_t src = smem_u32(os.buf + (os.k & 1) * 2048);
-    if (active) {
-      if (add)
-        asm volatile("cp.reduce.async.bulk.tensor.2d.global.shared::cta.add.tile.bulk_group [%0, {%2, %3}], [%1];" ::"l"(map),
-                     "r"(src), "r"(col), "r"(row)
-                     : "memory");
-      else
-        asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%2, %3}], [%1];" ::"l"(map), "r"(src),
-                     "r"(col), "r"(row)
-                     : "memory");
-    }
-    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-  }
-  ++os.k;
-}
-// 32 columns of the thread's row as bf16 (one box) or fp32 (two boxes of 16 columns)
-__device__ __forceinline__ void tma_store_rows_bf16(const CUtensorMap* map, OutStage& os, const float (&v)[32], int col, int row,
-                                                    bool active, int lane) {
-  uint4 piece[4];
+  for (int h = 0; h < 2; ++h)
+    asm volatile(
+        "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(r[16 * h]), "=r"(r[16 * h + 1]), "=r"(r[16 * h + 2]), "=r"(r[16 * h + 3]), "=r"(r[16 * h + 4]), "=r"(r[16 * h + 5]),
+          "=r"(r[16 * h + 6]), "=r"(r[16 * h + 7]), "=r"(r[16 * h + 8]), "=r"(r[16 * h + 9]), "=r"(r[16 * h + 10]),
+          "=r"(r[16 * h + 11]), "=r"(r[16 * h + 12]), "=r"(r[16 * h + 13]), "=r"(r[16 * h + 14]), "=r"(r[16 * h + 15])
+        : "r"(taddr + ((uint32_t)(16 * h) << 16)));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    piece[q].x = pack_bf16(v[8 * q], v[8 * q + 1]);
-    piece[q].y = pack_bf16(v[8 * q + 2], v[8 * q + 3]);
-    piece[q].z = pack_bf16(v[8 * q + 4], v[8 * q + 5]);
-    piece[q].w = pack_bf16(v[8 * q + 6], v[8 * q + 7]);
-  }
-  tma_store_box(map, os, piece, col, row, false, active, lane);
+  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
-__device__ __forceinline__ void tma_store_rows_f32(const CUtensorMap* map, OutStage& os, const float (&v)[32], int col, int row,
-                                                   bool add, bool active, int lane) {
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    uint4 piece[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-      piece[q] = make_uint4(__float_as_uint(v[16 * h + 4 * q]), __float_as_uint(v[16 * h + 4 * q + 1]),
-                            __float_as_uint(v[16 * h + 4 * q + 2]), __float_as_uint(v[16 * h + 4 * q + 3]));
-    tma_store_box(map, os, piece, col + 16 * h, row, add, active, lane);
-  }
-}
-// the unit has read every box of the warp (its staging may be rewritten) / has written them all
-__device__ __forceinline__ void tma_store_drain_reads(int lane) {
-  if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-  __syncwarp();
-}
-__device__ __forceinline__ void tma_store_drain_all(int lane) {
-  if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
-  __syncwarp();
-}
-
-// Where the epilogue takes the thread's accumulator row from: TMEM, or the sum over the K splits' partial tiles.
+// Partial tiles hold the values as the threads hold them, [chunk][8][128 threads][4] fp32: a warp's access is 512 contiguous
+// bytes.  Parts are added in part order starting from zero, so the result does not depend on who arrived last.
 struct TmemLoader {
   uint32_t tacc;   // TMEM address of (lane quadrant, column 0)
-  __device__ __forceinline__ void operator()(int col, float (&v)[32]) const { tmem_ld32(tacc + col, v); }
+  __device__ __forceinline__ void operator()(int c, float (&v)[32]) const { tmem_ld_chunk(tacc + c * 32, v); }
 };
 struct SplitLoader {
-  const float* ws;        // partial-tile workspace; slot s holds a [BM][bn] fp32 tile
-  int bn, row;            // tile width, this thread's row in the tile
+  const float4* ws;       // partial-tile workspace + this thread
+  int part_f4;            // float4 x 128 threads per part (8 per chunk)
   int slot0;              // slot of part 0
   int slot_next;          // slot of part 1; part p >= 1 is in slot_next + slot_stride (p - 1)
   int slot_stride;
   int n_parts;
-  bool valid;             // rows beyond M were never parked
-  __device__ __forceinline__ void operator()(int col, float (&v)[32]) const {
+  __device__ __forceinline__ void operator()(int c, float (&v)[32]) const {
 #pragma unroll
     for (int i = 0; i < 32; ++i) v[i] = 0.f;
-    if (!valid) return;
-    // partial tiles are stored [column / 4][row][4]: a warp's 32 rows of one float4 column are 512 contiguous
-    // bytes.  Parts are added in part order (the result does not depend on who arrived last); the loads of two
-    // parts are issued together so that their latencies overlap.
-    const float4* base = reinterpret_cast<const float4*>(ws) + (size_t)(col / 4) * BM + row;
+    // the loads of two parts are issued together so that their latencies overlap
     for (int p = 0; p < n_parts; p += 2) {
       const int sa = p == 0 ? slot0 : slot_next + slot_stride * (p - 1);
       const bool two = p + 1 < n_parts;
@@ -239,8 +198,8 @@ struct SplitLoader {
       float4 a[8], b[8];
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
-        a[i] = __ldcg(base + ((size_t)sa * (bn / 4) + i) * BM);
-        b[i] = two ? __ldcg(base + ((size_t)sb * (bn / 4) + i) * BM) : make_float4(0.f, 0.f, 0.f, 0.f);
+        a[i] = __ldcg(ws + ((size_t)sa * part_f4 + c * 8 + i) * FT);
+        b[i] = two ? __ldcg(ws + ((size_t)sb * part_f4 + c * 8 + i) * FT) : make_float4(0.f, 0.f, 0.f, 0.f);
       }
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
@@ -250,33 +209,31 @@ struct SplitLoader {
     }
   }
 };
-
-// The reducing CTA's own part comes from its TMEM accumulator, the other parts from copies in shared memory (the
-// idle operand ring, one [BN/4][rows] float4 tile after the other in part order without the own part; rows = BM, or
-// 32 for the parts that the CTAs of a cluster hand to their leader).  Parts are added in part order starting from
-// zero, exactly like SplitLoader, so both give the same bits.
+// The finishing CTA's own part comes from its TMEM accumulator, the other parts from copies in shared memory (the idle operand
+// ring or a reserve at its top), one part after the other in part order without the own one.  Every lane takes part (the TMEM
+// load is a warp-wide instruction).
 struct RingLoader {
   uint32_t tacc;
-  const float4* ring;     // + row
-  int bn, own, n_parts, rows;
-  // Every lane takes part, also those whose row lies beyond M (the TMEM load is a warp-wide instruction; their
-  // sums are never stored).
-  __device__ __forceinline__ void operator()(int col, float (&v)[32]) const {
+  const float4* ring;     // + this thread
+  int part_f4;            // float4 x 128 threads per part
+  int own, n_parts;
+  int c_off;              // token chunk the copies begin with
+  __device__ __forceinline__ void operator()(int c, float (&v)[32]) const {
 #pragma unroll
     for (int i = 0; i < 32; ++i) v[i] = 0.f;
     int k = 0;
     for (int p = 0; p < n_parts; ++p) {
       if (p == own) {
         float t[32];
-        tmem_ld32(tacc + col, t);
+        tmem_ld_chunk(tacc + c * 32, t);
 #pragma unroll
         for (int i = 0; i < 32; ++i) v[i] += t[i];
       } else {
-        const float4* src = ring + ((size_t)k * (bn / 4) + col / 4) * rows;
+        const float4* src = ring + ((size_t)k * part_f4 + (c - c_off) * 8) * FT;
         ++k;
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-          const float4 a = src[(size_t)i * rows];
+          const float4 a = src[(size_t)i * FT];
           v[4 * i] += a.x; v[4 * i + 1] += a.y; v[4 * i + 2] += a.z; v[4 * i + 3] += a.w;
         }
       }
@@ -284,18 +241,24 @@ struct RingLoader {
   }
 };
 
-// Work decomposition ("stream-K"), done per COLUMN of output tiles (the mt row tiles that share one weight tile):
-// the k-blocks of the columns form one line of n_cols * KB units, column after column; a TEAM of mt CTAs (CTA
-// team * mt + i works on row tile i) owns the contiguous range [team * per, (team + 1) * per) and walks it in
-// step, so that the members read the same weight k-blocks at the same time and share them through L2, exactly
-// like the CTAs of a wave of whole tiles.  A column may be cut by team boundaries; each owner computes its K range
-// of its row tile ("part").  Part p >= 1 of a tile is always the FIRST piece of its CTA, part 0 the last piece (or
-// the first, when the range starts exactly at the column): that decides the workspace slot,
-// 2 * cta + (first piece ? 0 : 1).
-// The stream-K division of a problem of mt x (n_tiles / mt) tiles with KB k-blocks each over n_units scheduling units:
-// all but the last one-to-two waves stay whole tiles (dp_tiles of them, done after the cut ones), the k-blocks of the
-// remaining tile columns are spread evenly over teams of mt units.  Computed on the host, or in the kernel when the row
-// count (hence mt) is only known on the device.  Needs mt <= n_units.
+// ---- work decomposition -----------------------------------------------------------------------------------------------------
+// The rows of the batch in equal token tiles: as few as tmax allows, each a multiple of gran wide (tmax is one too).
+__host__ __device__ inline void token_tiles(int M, int tmax, int gran, int* width, int* count) {
+  const int n = (M + tmax - 1) / tmax;
+  const int per = (M + n - 1) / n;
+  *width = (per + gran - 1) / gran * gran;
+  *count = (M + *width - 1) / *width;
+}
+
+// "Stream-K", done per COLUMN of output tiles (the mt token tiles that share one weight tile): the k-blocks of the columns
+// form one line of n_cols * KB units, column after column; a TEAM of mt units (unit team * mt + i works on token tile i) owns
+// the contiguous range [team * per, (team + 1) * per) and walks it in step, so that the members read the same weight k-blocks
+// at the same time and share them through L2, exactly like the CTAs of a wave of whole tiles.  A column may be cut by team
+// boundaries; each owner computes its K range of its token tile ("part").  Part p >= 1 of a tile is always the FIRST piece of
+// its unit, part 0 the last piece (or the first, when the range starts exactly at the column): that decides the workspace
+// slot, 2 * unit + (first piece ? 0 : 1).
+// All but the last one-to-two waves stay whole tiles (dp_tiles of them, done after the cut ones).  Computed on the host, or in
+// the kernel when the row count (hence mt) is only known on the device.  Needs mt <= n_units.
 __host__ __device__ inline void stream_k_schedule(int n_tiles, int mt, int KB, int n_units, int* dp_tiles, long long* per,
                                                   int* used_units) {
   const int n_teams = n_units / mt;
@@ -317,14 +280,14 @@ struct Piece {
   int slot;               // workspace slot if n_parts > 1
   int slot0, slot_next;   // slots of part 0 and part 1 (for the reducing CTA)
 };
-// Next piece of this CTA: first its range of the stream-K line (pos advances by reference), then its whole tiles
+// Next piece of this unit: first its range of the stream-K line (pos advances by reference), then its whole tiles
 // (jd counts them).  The cut tiles come first so that parking and reducing their partials overlaps the main loop
 // of the whole tiles that follow, instead of happening in every CTA at once at the end of the kernel.
 __device__ __forceinline__ Piece make_piece(int& jd, int dp_tiles, long long& pos, long long hi, int KB,
-                                            long long per, int cta, int grid, int mt) {
+                                            long long per, int unit, int n_units, int mt) {
   Piece p;
   if (pos >= hi) {
-    p.tile = cta + jd * grid;
+    p.tile = unit + jd * n_units;
     ++jd;
     p.kb0 = 0;
     p.kb1 = KB;
@@ -333,7 +296,7 @@ __device__ __forceinline__ Piece make_piece(int& jd, int dp_tiles, long long& po
     p.slot = p.slot0 = p.slot_next = 0;
     return p;
   }
-  const int team = cta / mt, member = cta % mt;
+  const int team = unit / mt, member = unit % mt;
   const int col = (int)(pos / KB);
   p.kb0 = (int)(pos - (long long)col * KB);
   const long long room = hi - pos;
@@ -343,7 +306,7 @@ __device__ __forceinline__ Piece make_piece(int& jd, int dp_tiles, long long& po
   p.n_parts = c_last - c_first + 1;
   p.part = team - c_first;
   const bool first_piece = pos == (long long)team * per;
-  p.slot = 2 * cta + (first_piece ? 0 : 1);
+  p.slot = 2 * unit + (first_piece ? 0 : 1);
   p.slot0 = 2 * (c_first * mt + member) + (((long long)c_first * per >= t0) ? 0 : 1);
   p.slot_next = 2 * ((c_first + 1) * mt + member);
   p.tile = dp_tiles + col * mt + member;
@@ -351,241 +314,314 @@ __device__ __forceinline__ Piece make_piece(int& jd, int dp_tiles, long long& po
   return p;
 }
 
-// EPI_RESIDUAL_NORM: besides the accumulator a thread needs its row of the OLD residual stream and the gains of the
-// next norm.  Both come through shared memory: the TMA unit fetches the old rows of a 32-column chunk as two boxes (the
-// boxes of the output map: 32 rows x 16 columns, 64-byte swizzle) two chunks ahead of their use, completing on one
-// mbarrier per slot, and the tile's gains are staged once per tile.  (Plain global loads in flight would be waited for
-// by the proxy fence of every output box.)
-struct NormStage {
-  uint8_t* h;        // this warp's two 4 KB slots
-  uint4* g;          // this warp's 32 x 16 bytes of gains
-  uint64_t* bar;     // this warp's two barriers
-  uint32_t count;    // chunks fetched so far by this warp (slot = count & 1, phase = (count >> 1) & 1)
+// ---- epilogues --------------------------------------------------------------------------------------------------------------
+struct TileOut {
+  int tile;              // 128-feature tile
+  int t0, nv;            // first token, tokens of the tile that exist
+  int quad, lane;
+  const float* rstd;     // shared: row factors (ss_in given)
+  const int* slot;       // shared: cache slots (rotary epilogue)
+  float* ss;             // shared: [4][256]
+  uint8_t* stage;        // shared: this warp's 2 KB
 };
-__device__ __forceinline__ void norm_issue(NormStage& ns, const CUtensorMap* omap, uint32_t idx, int n, int m_base, int lane) {
-  if (lane == 0) {
-    uint64_t* bar = &ns.bar[idx & 1];
-    uint8_t* dst = ns.h + (idx & 1) * 4096;
-    mbar_arrive_expect_tx(bar, 4096);
-    tma_load_2d(dst, omap, n, m_base, bar);
-    tma_load_2d(dst + 2048, omap, n + 16, m_base, bar);
+// What the epilogue of a chunk reads besides the accumulator: the old residual values (index as the accumulator's), or the
+// rotary factors: (cos, sin) of (q = 0 / 1, k, e) at 2 vidx(q, k, e).  Fetched ahead: for the first chunk while the accumulator is
+// still being computed.
+__device__ __forceinline__ void prefetch_chunk(const EpiParams& ep, const TileOut& o, int c, float (&pre)[32]) {
+  const int rg = o.lane >> 2, tok = c * 32 + 2 * (o.lane & 3), nv = o.nv;
+  if (ep.epi == EPI_RESIDUAL || ep.epi == EPI_RESIDUAL_NORM) {
+    const int f = o.tile * FT + o.quad * 32 + rg;
+    const float* h = static_cast<const float*>(ep.out) + (size_t)(o.t0 + tok) * ep.N + f;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+      for (int e = 0; e < 2; ++e)
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          pre[vidx(q, k, e)] = (tok + 8 * k + e < nv && f + 8 * q < ep.N) ? __ldcg(h + (size_t)(8 * k + e) * ep.N + 8 * q) : 0.f;
+  } else if (ep.epi == EPI_QKV_ROPE) {
+    const int half = ep.head_dim / 2, g = ep.head_dim == 128 ? o.quad : (o.quad & 1);
+    const float2* tab = ep.rope_cs + (size_t)(o.t0 + tok) * half + g * 16 + rg;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+      for (int e = 0; e < 2; ++e)
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          const float2 cs = tok + 8 * k + e < nv ? __ldcg(tab + (size_t)(8 * k + e) * half + 8 * q) : make_float2(1.f, 0.f);
+          pre[2 * vidx(q, k, e)] = cs.x;
+          pre[2 * vidx(q, k, e) + 1] = cs.y;
+        }
   }
 }
-// gains of the tile's columns and the first two chunks of old rows; returns the chunks the tile has
-__device__ __forceinline__ int norm_prepare(const EpiParams& ep, NormStage& ns, const CUtensorMap* omap, int n0, int bn, int m_base,
-                                            int lane) {
-  const int left = ep.N - n0;
-  const int nch = left <= 0 ? 0 : ((left < bn ? left : bn) + 31) / 32;
-  if (lane * 8 < bn && n0 + lane * 8 < ep.N) ns.g[lane] = __ldg(reinterpret_cast<const uint4*>(ep.gain + n0) + lane);
-  __syncwarp();
-  for (int c = 0; c < 2 && c < nch; ++c) norm_issue(ns, omap, ns.count + c, n0 + c * 32, m_base, lane);
-  return nch;
+__device__ __forceinline__ void stmatrix_x4_trans(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+  asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d)
+               : "memory");
 }
-
-// Epilogue of one accumulator tile for the calling thread's row.
-// stg: this warp's 4 KB of output staging (two boxes).  All 32 lanes of the warp call together.
-// rstd: factor of this thread's row when the input of the projection was a residual stream that is normalised on the
-// fly (1 otherwise); xmap: the tensor map over x_out of EPI_RESIDUAL_NORM; tile_col: index of the tile's column.
-template <int BN, bool NORM, typename Loader>
-__device__ __forceinline__ void row_epilogue(const EpiParams& ep, const Loader& load, int m, int n0, float* stg,
-                                             const CUtensorMap* omap, const CUtensorMap* xmap, float rstd, int tile_col,
-                                             NormStage& ns, bool prepared) {
-  const bool row_ok = m < ep.M;
-  const int lane = threadIdx.x & 31;
-  const int m_base = m - lane;                                  // first row of this warp
-  const int valid_rows = ep.M - m_base < 0 ? 0 : (ep.M - m_base > 32 ? 32 : ep.M - m_base);
-  OutStage os{reinterpret_cast<uint8_t*>(stg), 0u};
-  const bool active = valid_rows > 0;      // a box that starts beyond the last row is not issued at all
-  if constexpr (NORM) {
-    // The residual stream itself is updated by the TMA unit's add-reduction (one addend per element and launch: the
-    // rounding of a load-add-store).  The new value is formed here as well, from the old rows staged in shared memory,
-    // for the next norm's input x = bf16(h * gain) and the row's sum of squares over this tile's columns.
-    const int nch = prepared ? (ep.N - n0 <= 0 ? 0 : ((ep.N - n0 < BN ? ep.N - n0 : BN) + 31) / 32)
-                             : norm_prepare(ep, ns, omap, n0, BN, m_base, lane);
-    const int sw = (lane >> 1) & 3;
-    float ss = 0.f;
-#pragma unroll 1
-    for (int c = 0; c < nch; ++c) {
-      const uint32_t idx = ns.count + c;
-      if (!mbar_wait(&ns.bar[idx & 1], (idx >> 1) & 1, kSpin)) set_status(ep.status, DEV_TIMEOUT_FULL);
-      float hv[32];
-      const uint8_t* slot = ns.h + (idx & 1) * 4096 + lane * 64;
+// The chunk as bf16 rows [32 tokens][32 features] in the warp's staging: 16-byte piece p of token t at piece p ^ ((t >> 1) & 3)
+// of its 64 bytes (conflict free both ways).
+__device__ __forceinline__ void stage_rows32(const TileOut& o, const float (&v)[32]) {
+  const int m = o.lane >> 3;             // this lane gives the address of row lane % 8 of matrix m = 8 features
+  __syncwarp();                          // the previous chunk has been read
 #pragma unroll
-      for (int b = 0; b < 2; ++b)
+  for (int k = 0; k < 4; ++k) {
+    const int t = 8 * k + (o.lane & 7);
+    stmatrix_x4_trans(smem_u32(o.stage) + t * 64 + ((m ^ ((t >> 1) & 3)) << 4), pack_bf16(v[vidx(0, k, 0)], v[vidx(0, k, 1)]),
+                      pack_bf16(v[vidx(1, k, 0)], v[vidx(1, k, 1)]), pack_bf16(v[vidx(2, k, 0)], v[vidx(2, k, 1)]),
+                      pack_bf16(v[vidx(3, k, 0)], v[vidx(3, k, 1)]));
+  }
+  __syncwarp();
+}
+// ... and the pieces handed to put(token, piece, 16 bytes), eight tokens x four pieces at a time
+template <typename Put>
+__device__ __forceinline__ void unstage_rows32(const TileOut& o, int nv, const Put& put) {
+  const int p = o.lane & 3;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const float4 t = *reinterpret_cast<const float4*>(slot + b * 2048 + ((q ^ sw) << 4));
-          hv[16 * b + 4 * q] = t.x; hv[16 * b + 4 * q + 1] = t.y; hv[16 * b + 4 * q + 2] = t.z; hv[16 * b + 4 * q + 3] = t.w;
-        }
-      __syncwarp();                 // every lane has read the slot: it may be refilled
-      if (c + 2 < nch) norm_issue(ns, omap, idx + 2, n0 + (c + 2) * 32, m_base, lane);
-      float v[32];
-      load(c * 32, v);
-      const int n = n0 + c * 32;
-      tma_store_rows_f32(omap, os, v, n, m_base, true, active, lane);
+  for (int i = 0; i < 4; ++i) {
+    const int t = 8 * i + (o.lane >> 2);
+    const uint4 w = *reinterpret_cast<const uint4*>(o.stage + t * 64 + ((p ^ ((t >> 1) & 3)) << 4));
+    if (t < nv) put(t, p, w);
+  }
+}
+// Epilogue of token chunks [c0, c1) (32 tokens each) of an accumulator tile; all 32 lanes of the warp call together.
+// pre: what prefetch_chunk brings for chunk c0.
+template <typename Loader>
+__device__ __forceinline__ void tile_out(const EpiParams& ep, const Loader& load, const TileOut& o, int c0, int c1, float (&pre)[32]) {
+  const int lane = o.lane, rg = lane >> 2, tq = lane & 3;
+  const int f0 = o.tile * FT + o.quad * 32;    // first feature of the warp (not of SwiGLU and the rotary epilogue)
+  auto scale = [&](int c, float (&v)[32]) {    // the row factors of a normalised input
+    if (!ep.ss_in) return;
 #pragma unroll
-      for (int i = 0; i < 32; ++i) {
-        v[i] += hv[i];
-        ss = fmaf(v[i], v[i], ss);
-      }
+    for (int k = 0; k < 4; ++k) {
+      const float2 s = *reinterpret_cast<const float2*>(o.rstd + c * 32 + 8 * k + 2 * tq);
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        const uint4 gq = ns.g[c * 4 + q];
-        const uint32_t w[4] = {gq.x, gq.y, gq.z, gq.w};
+        v[vidx(q, k, 0)] *= s.x;
+        v[vidx(q, k, 1)] *= s.y;
+      }
+    }
+  };
+  if (ep.epi == EPI_RESIDUAL || ep.epi == EPI_RESIDUAL_NORM) {
+    // every element has one writer, so the residual add is a load (ahead of the accumulator) and a store; the new value also
+    // gives the next norm's input x = bf16(h * gain) and the row's sum of squares over this tile's features
+    const bool norm = ep.epi == EPI_RESIDUAL_NORM;
+    float gain[4] = {0.f, 0.f, 0.f, 0.f};
+    if (norm) {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          v[8 * q + 2 * j] *= __uint_as_float(w[j] << 16);
-          v[8 * q + 2 * j + 1] *= __uint_as_float(w[j] & 0xffff0000u);
+      for (int q = 0; q < 4; ++q)
+        if (f0 + rg + 8 * q < ep.N) gain[q] = __bfloat162float(ep.gain[f0 + rg + 8 * q]);
+    }
+#pragma unroll 1
+    for (int c = c0; c < c1; ++c) {
+      const int nv = o.nv - c * 32;
+      float* h = static_cast<float*>(ep.out) + (size_t)(o.t0 + c * 32 + 2 * tq) * ep.N + f0 + rg;
+      float v[32], sq[8];
+      load(c, v);
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          float s = 0.f;
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            float& x = v[vidx(q, k, e)];
+            x += pre[vidx(q, k, e)];
+            if (2 * tq + 8 * k + e < nv && f0 + rg + 8 * q < ep.N) h[(size_t)(8 * k + e) * ep.N + 8 * q] = x;
+            else x = 0.f;
+            s = fmaf(x, x, s);
+            x *= gain[q];
+          }
+          sq[2 * k + e] = s;
+        }
+      if (c + 1 < c1) prefetch_chunk(ep, o, c + 1, pre);
+      if (!norm) continue;
+      stage_rows32(o, v);
+      __nv_bfloat16* xp = ep.x_out + (size_t)(o.t0 + c * 32) * ep.N + f0;
+      unstage_rows32(o, nv, [&](int t, int p, const uint4& w) {
+        if (f0 + 8 * p < ep.N) *reinterpret_cast<uint4*>(xp + (size_t)t * ep.N + 8 * p) = w;
+      });
+      // sums of squares over the warp's 32 features: the eight lanes of a token column (lane / 4) halve the tokens at each step
+#pragma unroll
+      for (int s = 4; s; s >>= 1) {           // lane bits 4, 3, 2 <-> token index bits 2, 1, 0 of the thread's eight
+        const bool up = lane & (4 * s);
+#pragma unroll
+        for (int j = 0; j < s; ++j) {
+          const float keep = up ? sq[j + s] : sq[j], send = up ? sq[j] : sq[j + s];
+          sq[j] = keep + __shfl_xor_sync(0xffffffffu, send, 4 * s);
         }
       }
-      tma_store_rows_bf16(xmap, os, v, n, m_base, active, lane);
+      // thread holds index rg = 2 k + e
+      o.ss[o.quad * kMaxTok + c * 32 + 8 * (rg >> 1) + 2 * tq + (rg & 1)] = sq[0];
     }
-    ns.count += nch;
-    if (row_ok) ep.ss_out[(size_t)tile_col * ep.ss_stride + m] = ss;
-    tma_store_drain_reads(lane);
+    if (norm) {
+      asm volatile("bar.sync 1, 128;" ::: "memory");
+      for (int t = c0 * 32 + o.quad * 32 + lane; t < o.nv && t < c1 * 32; t += 128)
+        ep.ss_out[(size_t)o.tile * ep.ss_stride + o.t0 + t] =
+            (o.ss[t] + o.ss[kMaxTok + t]) + (o.ss[2 * kMaxTok + t] + o.ss[3 * kMaxTok + t]);
+      asm volatile("bar.sync 1, 128;" ::: "memory");      // (the sums may be overwritten)
+    }
     return;
   }
   if (ep.epi == EPI_SWIGLU) {
-    // accumulator columns [0, BN/2) are gate, [BN/2, BN) up; n0 is the first output column
+    // features 0-15 of the warp: gate, 16-31: the up features that belong to them
+    const int fo = o.tile * (FT / 2) + o.quad * 16;
+    __nv_bfloat16* out = static_cast<__nv_bfloat16*>(ep.out) + (size_t)o.t0 * ep.N + fo;
 #pragma unroll 1
-    for (int c = 0; c < BN / 64; ++c) {
-      float g[32], u[32];
-      load(c * 32, g);
-      load(BN / 2 + c * 32, u);
-      if (n0 + c * 32 < ep.N) {
+    for (int c = c0; c < c1; ++c) {
+      float v[32];
+      load(c, v);
+      scale(c, v);
 #pragma unroll
-        for (int i = 0; i < 32; ++i) g[i] = silu_f(g[i] * rstd) * (u[i] * rstd);
-        tma_store_rows_bf16(omap, os, g, n0 + c * 32, m_base, active, lane);
+      for (int i = 0; i < 16; ++i) v[i] = silu_f(v[i]) * v[16 + i];
+      // rows [32 tokens][16 features] of 32 bytes
+      __syncwarp();
+#pragma unroll
+      for (int k = 0; k < 4; k += 2) {
+        const int m = lane >> 3, t = 8 * (k + (m >> 1)) + (lane & 7);
+        stmatrix_x4_trans(smem_u32(o.stage) + t * 32 + (m & 1) * 16, pack_bf16(v[vidx(0, k, 0)], v[vidx(0, k, 1)]),
+                          pack_bf16(v[vidx(1, k, 0)], v[vidx(1, k, 1)]), pack_bf16(v[vidx(0, k + 1, 0)], v[vidx(0, k + 1, 1)]),
+                          pack_bf16(v[vidx(1, k + 1, 0)], v[vidx(1, k + 1, 1)]));
+      }
+      __syncwarp();
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const int t = 16 * i + (lane >> 1);
+        const uint4 w = *reinterpret_cast<const uint4*>(o.stage + t * 32 + (lane & 1) * 16);
+        if (fo < ep.N && c * 32 + t < o.nv) *reinterpret_cast<uint4*>(out + (size_t)(c * 32 + t) * ep.N + (lane & 1) * 8) = w;
       }
     }
-    tma_store_drain_reads(lane);
     return;
   }
   if (ep.epi == EPI_QKV_ROPE) {
+    // features 0-15 of the warp: 16 low dims of a head, 16-31: their rotation partners half a head away
     const int D = ep.head_dim, half = D / 2;
-    const int slot = row_ok ? ep.tok_slot[m] : -1;
+    const int head = D == 128 ? o.tile : 2 * o.tile + (o.quad >> 1), g = D == 128 ? o.quad : (o.quad & 1);
+    const bool is_q = head < ep.n_q, is_v = head >= ep.n_q + ep.n_kv, live = head < ep.n_q + 2 * ep.n_kv;
+    const int kvh = is_v ? head - ep.n_q - ep.n_kv : head - ep.n_q;
+    __nv_bfloat16* layer = ep.kv_pool + kv_tile_base(ep.n_pages, ep.n_kv, D, ep.layer, 0, is_q ? 0 : kvh) + (is_v ? kv_tile_elems(D) : 0);
+    const size_t page_elems = kv_tile_base(ep.n_pages, ep.n_kv, D, 0, 1, 0);
 #pragma unroll 1
-    for (int hl = 0; hl < BN / D; ++hl) {        // heads in this tile
-      const int head = n0 / D + hl;
-      const bool is_q = head < ep.n_q, is_v = head >= ep.n_q + ep.n_kv;
-      __nv_bfloat16* kv_base = nullptr;
-      if (!is_q && slot >= 0) {
+    for (int c = c0; c < c1; ++c) {
+      float v[32];
+      load(c, v);
+      scale(c, v);
+      if (!is_v) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+          const float lo = v[i], hi = v[16 + i];
+          v[i] = lo * pre[2 * i] - hi * pre[2 * i + 1];
+          v[16 + i] = hi * pre[2 * i] + lo * pre[2 * i + 1];
+        }
+        if (c + 1 < c1) prefetch_chunk(ep, o, c + 1, pre);
+      }
+      stage_rows32(o, v);
+      unstage_rows32(o, o.nv - c * 32, [&](int t, int p, const uint4& w) {
+        if (!live) return;
+        const int dim = (p >> 1) * half + g * 16 + (p & 1) * 8;
+        if (is_q) {
+          *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(ep.out) + ((size_t)(o.t0 + c * 32 + t) * ep.n_q + head) * D + dim) = w;
+          return;
+        }
+        const int slot = o.slot[c * 32 + t];
+        if (slot < 0) return;
         const int64_t page = slot / kPageSize;
-        if (page < ep.n_pages) {
-          const int kvh = is_v ? head - ep.n_q - ep.n_kv : head - ep.n_q;
-          kv_base = ep.kv_pool + kv_tile_base(ep.n_pages, ep.n_kv, D, ep.layer, page, kvh) + (is_v ? kv_tile_elems(D) : 0);
-        } else {
+        if (page >= ep.n_pages) {
           set_status(ep.status, DEV_BAD_INDEX);
+          return;
         }
-      }
-      const int tok = slot >= 0 ? slot % kPageSize : 0;
-#pragma unroll 1
-      for (int c = 0; c < half / 32; ++c) {      // 32 low columns with their 32 partners half a head away
-        float lo[32], hi[32];
-        load(hl * D + c * 32, lo);
-        load(hl * D + half + c * 32, hi);
-#pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          lo[i] *= rstd;
-          hi[i] *= rstd;
-        }
-        if (row_ok && !is_v) {
-          const float2* cs = ep.rope_cs + (size_t)(c * 32) * ep.M + m;   // [frequency][token]
-#pragma unroll
-          for (int i = 0; i < 32; ++i) {
-            const float2 t = cs[(size_t)i * ep.M];
-            const float a = lo[i] * t.x - hi[i] * t.y, b = hi[i] * t.x + lo[i] * t.y;
-            lo[i] = a;
-            hi[i] = b;
-          }
-        }
-        if (is_q) {      // (the same for the whole warp): rows of the rotated queries [M, n_q * D] through the TMA unit
-          tma_store_rows_bf16(omap, os, lo, head * D + c * 32, m_base, active, lane);
-          tma_store_rows_bf16(omap, os, hi, head * D + half + c * 32, m_base, active, lane);
-        } else if (kv_base) {
-          // the pool tile is swizzled in 16-byte chunks: store chunk by chunk
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            uint4 a, b;
-            a.x = pack_bf16(lo[8 * j], lo[8 * j + 1]); a.y = pack_bf16(lo[8 * j + 2], lo[8 * j + 3]);
-            a.z = pack_bf16(lo[8 * j + 4], lo[8 * j + 5]); a.w = pack_bf16(lo[8 * j + 6], lo[8 * j + 7]);
-            b.x = pack_bf16(hi[8 * j], hi[8 * j + 1]); b.y = pack_bf16(hi[8 * j + 2], hi[8 * j + 3]);
-            b.z = pack_bf16(hi[8 * j + 4], hi[8 * j + 5]); b.w = pack_bf16(hi[8 * j + 6], hi[8 * j + 7]);
-            *reinterpret_cast<uint4*>(kv_base + kv_tile_offset(tok, c * 32 + j * 8, D)) = a;
-            *reinterpret_cast<uint4*>(kv_base + kv_tile_offset(tok, half + c * 32 + j * 8, D)) = b;
-          }
-        }
-      }
+        *reinterpret_cast<uint4*>(layer + page * page_elems + kv_tile_offset(slot % kPageSize, dim, D)) = w;
+      });
     }
-    tma_store_drain_reads(lane);
     return;
   }
 #pragma unroll 1
-  for (int c = 0; c < BN / 32; ++c) {
+  for (int c = c0; c < c1; ++c) {
+    const int nv = o.nv - c * 32;
     float v[32];
-    load(c * 32, v);
-    const int n = n0 + c * 32;
-    if (n >= ep.N) continue;
-    if (ep.ss_in) {
+    load(c, v);
+    scale(c, v);
+    if (ep.epi == EPI_PLAIN_BF16) {
+      stage_rows32(o, v);
+      __nv_bfloat16* out = static_cast<__nv_bfloat16*>(ep.out) + (size_t)(o.t0 + c * 32) * ep.N + f0;
+      unstage_rows32(o, nv, [&](int t, int p, const uint4& w) {
+        if (f0 + 8 * p < ep.N) *reinterpret_cast<uint4*>(out + (size_t)t * ep.N + 8 * p) = w;
+      });
+    } else {
+      float* out = static_cast<float*>(ep.out) + (size_t)(o.t0 + c * 32 + 2 * tq) * ep.N + f0 + rg;
 #pragma unroll
-      for (int i = 0; i < 32; ++i) v[i] *= rstd;
+      for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (2 * tq + 8 * k + e < nv && f0 + rg + 8 * q < ep.N) out[(size_t)(8 * k + e) * ep.N + 8 * q] = v[vidx(q, k, e)];
     }
-    // the box is clipped at the right edge (N is a multiple of 16 but not always of 32) and at the last row
-    if (ep.epi == EPI_PLAIN_BF16) tma_store_rows_bf16(omap, os, v, n, m_base, active, lane);
-    else tma_store_rows_f32(omap, os, v, n, m_base, ep.epi == EPI_RESIDUAL, active, lane);
   }
-  tma_store_drain_reads(lane);
 }
 
-template <int BN, bool PAIR, bool NORM>
+struct GemmLaunch {
+  int m_cap;                 // rows the maps cover
+  int n_cols;                // columns of tiles: feature tiles of 128, or of 256 for pairs
+  int K;
+  int tmax, gran, x_box;     // token tiles (token_tiles), rows of one x load
+  int dp_tiles;              // >= 0: the host's schedule; -1: whole tiles only; -2: stream-K, divided here from the device's row count
+  long long per;
+  int cl;                    // parts per tile that form a cluster (0: no clusters)
+  int w_step3, w_step4;      // what a 128-feature tile advances in dimensions 3 and 4 of w's tensor map
+  float* split_ws;
+  int* split_counters;
+  const int* m_dev;
+  int m_dev_wait;
+};
+
+template <bool PAIR>
 __global__ void __launch_bounds__(kTcThreads, 1)
-gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
-               const __grid_constant__ CUtensorMap map_out, const __grid_constant__ CUtensorMap map_xout, int M_cap, int n_tiles_n,
-               int K, int up_row_offset, int dp_tiles_in, long long per_in, int thin, int cl_parts, float* split_ws,
-               int* split_counters, const int* __restrict__ m_dev, int m_dev_wait, EpiParams ep_in) {
-  // Device-resident rounds: the row count comes from device memory; the tensor maps cover the capacity M_cap, and rows
+gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x, GemmLaunch G, EpiParams ep) {
+  // Device-resident rounds: the row count comes from device memory; the tensor maps cover the capacity, and rows
   // between the count and the capacity hold stale data and are computed but never used.  The count is written by the
   // first kernel of the step, and the small kernels between it and the first projection signal their dependents before
   // they wait themselves, so the FIRST projection of a step can be running before that one has finished: it has to wait
   // for its predecessors before it reads the count (m_dev_wait; it gives up the early weight requests).  The first
   // projection signals its own dependents only after that wait, so for every kernel behind it the count is settled.
-  if (m_dev && m_dev_wait) griddep_wait();
-  const int M = m_dev ? *reinterpret_cast<const volatile int*>(m_dev) : M_cap;
+  if (G.m_dev && G.m_dev_wait) griddep_wait();
+  const int M = G.m_dev ? *reinterpret_cast<const volatile int*>(G.m_dev) : G.m_cap;
   if (M <= 0) {                // an empty round (the same for every thread of the grid): nothing to do, nothing was set up yet
     griddep_wait();            // (this grid must not count as complete before the ones it follows are)
     return;
   }
-  EpiParams ep = ep_in;
-  ep.M = M;
-  using Cfg = TcCfg<BN, PAIR, NORM>;
-  constexpr int kRows = PAIR ? 2 * BM : BM;              // rows of a scheduling unit's tile
-  constexpr int kSlotMul = PAIR ? 2 : 1;                 // the CTAs of a pair use separate slots and counters
-  const uint32_t rank = PAIR ? cluster_ctarank() : 0u;
-  const int unit = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;      // scheduling unit: CTA or cluster
-  const int n_units = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x;
+  constexpr int kMul = PAIR ? 2 : 1;                     // CTAs of a scheduling unit; they use separate slots and counters
+  const uint32_t crank = (PAIR || G.cl) ? cluster_ctarank() : 0u;
+  const uint32_t rank = PAIR ? (crank & 1u) : 0u;        // within the pair
+  const uint32_t lead_rank = crank & ~1u;                // cluster rank of the pair's leader (PAIR)
+  const int cl = G.cl;
+  const uint32_t part_rank = cl ? crank / kMul : 0u;     // which part of the cluster's tile this unit computes
+  const int unit = (int)blockIdx.x / kMul;               // scheduling unit: CTA or pair
+  const int n_units = (int)gridDim.x / kMul;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  // Problems of one row tile (at most 128 rows) whose tiles are cut over K can run as CLUSTERS of cl CTAs per tile
-  // (cl_parts > 1; single CTAs only): rank r computes k-blocks [r KB / cl, (r + 1) KB / cl) and hands its partial tile
-  // (the rows in use, rounded up to 32) to the cluster's leader (rank 0) through distributed shared memory, into a
-  // reserve at the top of the leader's ring budget; the leader adds the parts in rank order and runs the epilogue.  No
-  // trip through global memory, no counter.
-  const int cl = (!PAIR && cl_parts > 1) ? cl_parts : 0;
-  const uint32_t crank = cl ? cluster_ctarank() : 0u;
-  const int cl_rows = ((M < BM ? M : BM) + 31) & ~31;            // rows of a handed-over part
-  const int cl_part_bytes = cl_rows * BN * 4;
-  const int cl_reserve = cl ? (cl - 1) * cl_part_bytes : 0;
-  const int a_bytes = thin ? Cfg::kThinABytes : Cfg::kABytes;
-  const int stage_bytes = a_bytes + Cfg::kBBytes;
-  const int cl_stages = (Cfg::kBudget - cl_reserve) / stage_bytes;
-  const int n_stages = cl ? (cl_stages > Cfg::kMaxStages ? Cfg::kMaxStages : cl_stages) : (thin ? Cfg::kThinStages : Cfg::kStages);
-  uint64_t* full_bar = reinterpret_cast<uint64_t*>(smem + Cfg::kBarOff);
-  uint64_t* empty_bar = full_bar + Cfg::kMaxStages;
-  uint64_t* tfull_bar = empty_bar + Cfg::kMaxStages;
+
+  int nt_tok, mt;              // tokens per tile, token tiles
+  token_tiles(M, G.tmax, G.gran, &nt_tok, &mt);
+  const int x_rows = nt_tok / kMul;                       // rows of x this CTA loads per k-block
+  const int stage_bytes = kABytes + x_rows * BK * 2;
+  const int part_f4 = (nt_tok + 31) / 32 * 8;             // a partial tile: float4 x 128 threads
+  const int part_bytes = part_f4 * FT * 16;
+  // Clusters: chunk c of the tile (32 tokens) is finished by member c % cl, into whose shared memory the others write their
+  // partial sums of it (16 KB each).  A tile of one chunk has a reserve for them at the top of the ring; else they go into the
+  // ring itself, once its owner says that its own products have read it.
+  const bool reserve = cl && nt_tok <= 32;
+  const int ring_bytes = kRingBytes - (reserve ? (cl - 1) * kChunkBytes : 0);
+  const int n_stages = ring_bytes / stage_bytes > kMaxStages ? kMaxStages : ring_bytes / stage_bytes;
+  uint64_t* full_bar = reinterpret_cast<uint64_t*>(smem + kOffBar);
+  uint64_t* empty_bar = full_bar + kMaxStages;
+  uint64_t* tfull_bar = empty_bar + kMaxStages;
   uint64_t* tempty_bar = tfull_bar + 2;
-  uint64_t* red_bar = tempty_bar + 2;      // completion of the partial tiles fetched into the idle ring (used once)
-  uint64_t* h_bar = red_bar + 1;           // [4 epilogue warps][2 slots]: old residual rows have landed (NORM only)
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(h_bar + 8);
+  uint64_t* red_bar = tempty_bar + 2;      // the parts of the others have landed (bulk copies, or the cluster's peers)
+  uint64_t* go_bar = red_bar + 1;          // clusters: the other members' rings may be written
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(go_bar + 1);
+  float* s_rstd = reinterpret_cast<float*>(smem + kOffRstd);
+  int* s_slot = reinterpret_cast<int*>(smem + kOffSlot);
+  float* s_ss = reinterpret_cast<float*>(smem + kOffSs);
 
   // Bounded waits.  The producer and the MMA issuer leave their loops when a wait runs out.  The four epilogue warps
   // must all keep meeting at the named barriers and must keep counting the arrivals of cut tiles (so that the counters
@@ -596,65 +632,63 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
   __shared__ volatile int s_abort;
   auto wait_bar = [&](uint64_t* bar, uint32_t parity) -> bool {
     for (uint32_t i = 0; i < kSpin; ++i) {
-      uint32_t ok;
-      if constexpr (PAIR)
-        asm volatile(
-            "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-            : "=r"(ok)
-            : "r"(smem_u32(bar)), "r"(parity)
-            : "memory");
-      else
-        ok = mbar_try_wait(bar, parity) ? 1u : 0u;
-      if (ok) return true;
+      if (PAIR ? mbar_try_wait_cluster(bar, parity) : mbar_try_wait(bar, parity)) return true;
       if (i > 64) __nanosleep(32);
     }
     return false;
   };
-  auto wait_or_abort = [&](uint64_t* bar, uint32_t parity, int code) {   // epilogue warps only
+  auto wait_or_abort = [&](uint64_t* bar, uint32_t parity, int code, bool cluster = false) {   // epilogue warps only
     if (s_abort) return;
-    if (!wait_bar(bar, parity)) {
+    bool ok = false;
+    if (cluster) {
+      for (uint32_t i = 0; i < kSpin && !ok; ++i) {
+        ok = mbar_try_wait_cluster(bar, parity);
+        if (!ok && i > 64) __nanosleep(32);
+      }
+    } else {
+      ok = wait_bar(bar, parity);
+    }
+    if (!ok) {
       set_status(ep.status, code);
       s_abort = 1;
     }
   };
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int n_tiles_m = (M + kRows - 1) / kRows;
-  const int n_tiles = n_tiles_m * n_tiles_n;
-  const int KB = K / BK;
-  // dp_tiles_in >= 0: the host's schedule; -1: whole tiles only; -2: stream-K, divided here from the device's row count
-  int dp_tiles = dp_tiles_in < 0 ? n_tiles : dp_tiles_in;
-  long long per = per_in;
-  if (dp_tiles_in == -2) {
-    if (n_tiles_m >= 1 && n_tiles_m <= n_units) {
+  const int n_tiles = mt * G.n_cols;
+  const int KB = G.K / BK;
+  int dp_tiles = G.dp_tiles < 0 ? n_tiles : G.dp_tiles;
+  long long per = G.per;
+  if (G.dp_tiles == -2) {
+    if (mt >= 1 && mt <= n_units) {
       int used;
-      stream_k_schedule(n_tiles, n_tiles_m, KB, n_units, &dp_tiles, &per, &used);
+      stream_k_schedule(n_tiles, mt, KB, n_units, &dp_tiles, &per, &used);
     } else {
       dp_tiles = n_tiles;
     }
   }
-  const bool swiglu = ep.epi == EPI_SWIGLU;
-  // schedule: the k-blocks of tiles [dp_tiles, n_tiles) as one line cut into equal ranges per CTA; then tiles
+  // schedule: the k-blocks of tiles [dp_tiles, n_tiles) as one line cut into equal ranges per unit; then tiles
   // [0, dp_tiles) whole, strided over the grid (CTAs that run together share a weight tile through L2)
-  const long long total = (long long)((n_tiles - dp_tiles) / n_tiles_m) * KB;
-  const long long lo_raw = (long long)(unit / n_tiles_m) * per;
+  const long long total = (long long)((n_tiles - dp_tiles) / mt) * KB;
+  const long long lo_raw = (long long)(unit / mt) * per;
+  const bool cl_live = cl && unit / cl < n_tiles;          // (the grid of a device-resident step is sized for the capacity)
   const long long range_lo = cl ? 0 : (lo_raw < total ? lo_raw : total);
-  const long long range_hi = cl ? 1 : (range_lo + per < total ? range_lo + per : total);
+  const long long range_hi = cl ? (cl_live ? 1 : 0) : (range_lo + per < total ? range_lo + per : total);
   const int dp_count = cl ? 0 : (unit < dp_tiles ? (dp_tiles - 1 - unit) / n_units + 1 : 0);
-  // the next piece of this CTA (a cluster member has exactly one)
+  // the next piece of this unit (a cluster member has exactly one)
   auto next_piece = [&](int& jd, long long& pos) -> Piece {
     if (cl) {
       Piece p;
-      p.tile = (int)blockIdx.x / cl;
-      p.kb0 = (int)((long long)crank * KB / cl);
-      p.kb1 = (int)((long long)(crank + 1) * KB / cl);
-      p.part = (int)crank;
+      p.tile = unit / cl;
+      p.kb0 = (int)((long long)part_rank * KB / cl);
+      p.kb1 = (int)((long long)(part_rank + 1) * KB / cl);
+      p.part = (int)part_rank;
       p.n_parts = cl;
       p.slot = p.slot0 = p.slot_next = 0;
       pos = range_hi;
       return p;
     }
-    return make_piece(jd, dp_tiles, pos, range_hi, KB, per, unit, n_units, n_tiles_m);
+    return make_piece(jd, dp_tiles, pos, range_hi, KB, per, unit, n_units, mt);
   };
 
   if (threadIdx.x == 0) {
@@ -667,25 +701,24 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
       mbar_init(&tfull_bar[a], 1);
       mbar_init(&tempty_bar[a], PAIR ? 8 : 4);
     }
-    mbar_init(red_bar, cl ? (cl - 1) * (cl_rows / 32) : 1);      // (cluster leader: one arrival per peer and 32 rows)
-    for (int i = 0; i < 8; ++i) mbar_init(&h_bar[i], 1);
+    mbar_init(red_bar, cl ? (cl - 1) * 4 : 1);             // (clusters: one arrival per other member and epilogue warp)
+    mbar_init(go_bar, cl > 1 ? cl - 1 : 1);
     fence_barrier_init();
     prefetch_tmap(&map_x);
     prefetch_tmap(&map_w);
   }
   if (warp == 1) {
     if constexpr (PAIR) {
-      tmem_alloc_pair(tmem_slot, Cfg::kTmemCols);
+      tmem_alloc_pair(tmem_slot, kTmemCols);
       tmem_relinquish_pair();
     } else {
-      tmem_alloc(tmem_slot, Cfg::kTmemCols);
+      tmem_alloc(tmem_slot, kTmemCols);
       tmem_relinquish();
     }
   }
   tc_fence_before();
   __syncthreads();
-  if constexpr (PAIR) cluster_sync_all();   // both CTAs' barriers are initialised before anyone signals across
-  else if (cl) cluster_sync_all();
+  if (PAIR || cl) cluster_sync_all();       // all CTAs' barriers are initialised before anyone signals across
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   // (each role waits for the kernels before this one where it first needs their results)
@@ -693,8 +726,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
   if (warp == 0) {
     // ------------------------------ TMA producer ------------------------------
     if (elect_one()) {
-      // of a pair, rank r loads rows [128 r, 128 r + 128) of the x tile and half r of the weight tile (SwiGLU: rank 0
-      // the gate rows, rank 1 the up rows); all four loads of the pair complete on the leader's barrier
+      // of a pair, rank r loads the weight rows of feature tile 2 c + r and half r of the token tile; all loads of the pair
+      // complete on the leader's barrier
       auto expect = [&](int s) {
         if constexpr (PAIR) {
           if (rank == 0) mbar_arrive_expect_tx(&full_bar[s], 2 * stage_bytes);
@@ -702,27 +735,23 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
           mbar_arrive_expect_tx(&full_bar[s], stage_bytes);
         }
       };
-      auto load_w = [&](int s, int kb, int tn) {
-        uint8_t* b_dst = smem + s * stage_bytes + a_bytes;
-        if constexpr (PAIR) {
-          const uint32_t full0 = mapa_rank(smem_u32(&full_bar[s]), 0);
-          const int w_row = swiglu ? (rank == 0 ? tn * (BN / 2) : up_row_offset + tn * (BN / 2)) : tn * BN + (int)rank * (BN / 2);
-          tma_load_2d_pair(smem_u32(b_dst), &map_w, kb * BK, w_row, full0);
-        } else if (swiglu) {
-          tma_load_2d(b_dst, &map_w, kb * BK, tn * (BN / 2), &full_bar[s]);
-          tma_load_2d(b_dst + Cfg::kBBytes / 2, &map_w, kb * BK, up_row_offset + tn * (BN / 2), &full_bar[s]);
-        } else {
-          tma_load_2d(b_dst, &map_w, kb * BK, tn * BN, &full_bar[s]);
-        }
+      auto load_w = [&](int s, int kb, int col) {
+        const uint32_t dst = smem_u32(smem + s * stage_bytes);
+        const int ft = col * kMul + (int)rank;
+        if constexpr (PAIR) tma_load_w_pair(dst, &map_w, kb * BK, ft * G.w_step3, ft * G.w_step4, mapa_rank(smem_u32(&full_bar[s]), lead_rank));
+        else tma_load_w(dst, &map_w, kb * BK, ft * G.w_step3, ft * G.w_step4, &full_bar[s]);
       };
       auto load_x = [&](int s, int kb, int tm) {
-        uint8_t* a_dst = smem + s * stage_bytes;
-        if constexpr (PAIR) tma_load_2d_pair(smem_u32(a_dst), &map_x, kb * BK, tm * kRows + (int)rank * BM, mapa_rank(smem_u32(&full_bar[s]), 0));
-        else tma_load_2d(a_dst, &map_x, kb * BK, tm * BM, &full_bar[s]);
+        uint8_t* dst = smem + s * stage_bytes + kABytes;
+        const int row = tm * nt_tok + (int)rank * x_rows;
+        for (int r = 0; r < x_rows; r += G.x_box) {
+          if constexpr (PAIR) tma_load_2d_pair(smem_u32(dst + r * BK * 2), &map_x, kb * BK, row + r, mapa_rank(smem_u32(&full_bar[s]), lead_rank));
+          else tma_load_2d(dst + r * BK * 2, &map_x, kb * BK, row + r, &full_bar[s]);
+        }
       };
       // The weights do not depend on the kernels before this one: the weight tiles of the first stages are requested
-      // BEFORE waiting for those kernels, so the ring fills while they drain (or while a short kernel such as the
-      // RMSNorm in front of this projection runs); the x tiles of those stages follow right after the wait.
+      // BEFORE waiting for those kernels, so the ring fills while they drain (or while a short kernel runs); the x tiles of
+      // those stages follow right after the wait.
       int n_pre = 0, pre_kb0 = 0, pre_tm = 0;
       if (dp_count > 0 || range_lo < range_hi) {
         long long p0 = range_lo;
@@ -730,10 +759,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
         const Piece pc = next_piece(j0, p0);
         n_pre = pc.kb1 - pc.kb0 < n_stages ? pc.kb1 - pc.kb0 : n_stages;
         pre_kb0 = pc.kb0;
-        pre_tm = pc.tile % n_tiles_m;
+        pre_tm = pc.tile % mt;
         for (int i = 0; i < n_pre; ++i) {
           expect(i);
-          load_w(i, pre_kb0 + i, pc.tile / n_tiles_m);
+          load_w(i, pre_kb0 + i, pc.tile / mt);
         }
       }
       griddep_wait();
@@ -744,7 +773,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
       long long pos = range_lo;
       for (int jd = 0; (jd < dp_count || pos < range_hi) && ok;) {
         const Piece pc = next_piece(jd, pos);
-        const int tm = pc.tile % n_tiles_m, tn = pc.tile / n_tiles_m;
+        const int tm = pc.tile % mt, col = pc.tile / mt;
         const int kb0 = pc.kb0, kb1 = pc.kb1;
         for (int kb = kb0; kb < kb1; ++kb) {
           const int s = st_idx;
@@ -761,7 +790,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
           }
           expect(s);
           load_x(s, kb, tm);
-          load_w(s, kb, tn);
+          load_w(s, kb, col);
         }
       }
       if (!ok) {  // let loads already issued land before the CTA may exit
@@ -775,8 +804,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
   } else if (warp == 1) {
     // ------------------------------ MMA issuer ------------------------------
     if (rank == 0 && elect_one()) {         // of a pair only the leader issues (it touches shared memory and TMEM only)
-      constexpr uint32_t idesc = make_idesc(BN, kRows);
+      const uint32_t idesc = make_idesc(nt_tok, FT * kMul);
       const uint64_t desc0 = make_smem_desc(smem_u32(smem));
+      const uint16_t pair_mask = (uint16_t)(3u << lead_rank);
       int st_idx = 0;
       uint32_t st_phase = 0, tcount = 0;
       bool ok = true;
@@ -790,7 +820,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
           break;
         }
         tc_fence_after();
-        const uint32_t d_tmem = tmem_base + acc * BN;
+        const uint32_t d_tmem = tmem_base + acc * kAccStride;
         for (int kb = kb0; kb < kb1; ++kb) {
           const int s = st_idx;
           const uint32_t ph = st_phase;
@@ -804,18 +834,18 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
           // descriptors are linear in the address (the ring lies inside the 14-bit address field without carry), so
           // the descriptor of a 16-column slice is the stage's descriptor plus 32 bytes >> 4
           const uint64_t da0 = desc0 + (uint64_t)((s * stage_bytes) >> 4);
-          const uint64_t db0 = da0 + (uint64_t)(a_bytes >> 4);
+          const uint64_t db0 = da0 + (uint64_t)(kABytes >> 4);
 #pragma unroll
           for (int k = 0; k < BK / 16; ++k) {
             if constexpr (PAIR) umma_bf16_pair(d_tmem, da0 + 2 * k, db0 + 2 * k, idesc, ((kb - kb0) | k) ? 1u : 0u);
             else umma_bf16(d_tmem, da0 + 2 * k, db0 + 2 * k, idesc, ((kb - kb0) | k) ? 1u : 0u);
           }
           // frees the stage (in both CTAs of a pair) when these MMAs have read it
-          if constexpr (PAIR) umma_commit_pair(&empty_bar[s]);
+          if constexpr (PAIR) umma_commit_pair(&empty_bar[s], pair_mask);
           else umma_commit(&empty_bar[s]);
         }
         if (ok) {                            // accumulator complete
-          if constexpr (PAIR) umma_commit_pair(&tfull_bar[acc]);
+          if constexpr (PAIR) umma_commit_pair(&tfull_bar[acc], pair_mask);
           else umma_commit(&tfull_bar[acc]);
         }
       }
@@ -823,108 +853,103 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
   } else {
     // ------------------------------ epilogue warps ------------------------------
     const int quad = warp & 3;             // TMEM lane quadrant this warp may read
-    float* stg = reinterpret_cast<float*>(smem + Cfg::kRingBytes) + (warp - 2) * 1024;
+    const int row = quad * 32 + lane;      // this thread among the 128 of the epilogue
     uint32_t tcount = 0;
+    int prep_tm = -1;
     __shared__ int s_last;
-    NormStage ns{smem + Cfg::kNormOff + (warp - 2) * 8192, reinterpret_cast<uint4*>(smem + Cfg::kNormOff + kNormHBytes) + (warp - 2) * 32,
-                 h_bar + (warp - 2) * 2, 0u};
     griddep_wait();                        // the epilogue reads and writes what earlier kernels produced
     long long pos = range_lo;
     for (int jd = 0; jd < dp_count || pos < range_hi; ++tcount) {
       const Piece pc = next_piece(jd, pos);
       const int tile = pc.tile, n_splits = pc.n_parts;
-      const int tm = tile % n_tiles_m, tn = tile / n_tiles_m;
+      const int tm = tile % mt, ft = (tile / mt) * kMul + (int)rank;
       const int acc = tcount & 1;
-      const int row_in_tile = quad * 32 + lane;
-      const int m = tm * kRows + (int)rank * BM + row_in_tile;
-      // the row's normalisation factor, fetched while the accumulator is still being computed: the partial sums of
-      // squares in slot order (the same bits in every tile of the row)
-      float rstd = 1.f;
-      if (ep.ss_in) {
-        float sq = 0.f;
-        if (m < ep.M)
-          for (int k = 0; k < ep.ss_slots; ++k) sq += __ldcg(ep.ss_in + (size_t)k * ep.ss_stride + m);
-        rstd = rsqrtf(sq * ep.norm_inv_n + ep.norm_eps);
+      TileOut o{ft, tm * nt_tok, 0, quad, lane, s_rstd, s_slot, s_ss, smem + kOffStage + quad * 2048};
+      o.nv = M - o.t0 < nt_tok ? M - o.t0 : nt_tok;
+      const int n_chunks = (o.nv + 31) / 32;
+      // What the epilogue needs per token, fetched while the accumulator is still being computed: the row factors of a
+      // normalised input (the partial sums of squares in slot order: the same bits in every tile of the row) and the slots.
+      if (tm != prep_tm && (ep.ss_in || ep.epi == EPI_QKV_ROPE)) {
+        if (prep_tm >= 0) asm volatile("bar.sync 1, 128;" ::: "memory");
+        for (int t = (int)threadIdx.x - 64; t < o.nv; t += 128) {
+          if (ep.ss_in) {
+            float sq = 0.f;
+            const float* p = ep.ss_in + o.t0 + t;
+#pragma unroll 8
+            for (int k = 0; k < ep.ss_slots; ++k) sq += __ldcg(p + (size_t)k * ep.ss_stride);
+            s_rstd[t] = rsqrtf(sq * ep.norm_inv_n + ep.norm_eps);
+          }
+          if (ep.epi == EPI_QKV_ROPE) s_slot[t] = ep.tok_slot[o.t0 + t];
+        }
+        asm volatile("bar.sync 1, 128;" ::: "memory");
+        prep_tm = tm;
       }
-      // (likewise, for a whole tile, the gains and the first old residual rows)
-      const bool prepared = NORM && n_splits == 1;
-      if constexpr (NORM) {
-        if (prepared) norm_prepare(ep, ns, &map_out, tn * BN, BN, m - lane, lane);
-      }
+      // (likewise, where this CTA is sure to finish the tile, what its first tokens need)
+      float pre[32];
+      if (n_splits == 1 || (cl && (int)part_rank < n_chunks)) prefetch_chunk(ep, o, (int)part_rank, pre);
       wait_or_abort(&tfull_bar[acc], (tcount >> 1) & 1, DEV_TIMEOUT_MMA);   // after a timeout: carry on without blocking
       tc_fence_after();
-      const uint32_t tacc = tmem_base + ((uint32_t)(quad * 32) << 16) + acc * BN;
+      const uint32_t tacc = tmem_base + ((uint32_t)(quad * 32) << 16) + acc * kAccStride;
       // hands the accumulator back to the MMA issuer (of a pair: the leader's barrier collects both CTAs' warps)
       auto release_acc = [&]() {
         tc_fence_before();
         __syncwarp();
         if (lane == 0) {
-          if constexpr (PAIR) mbar_arrive_cluster(mapa_rank(smem_u32(&tempty_bar[acc]), 0));
+          if constexpr (PAIR) mbar_arrive_cluster(mapa_rank(smem_u32(&tempty_bar[acc]), lead_rank));
           else mbar_arrive(&tempty_bar[acc]);
         }
       };
-      const int n0 = swiglu ? tn * (BN / 2) : tn * BN;
       if (n_splits == 1) {
-        row_epilogue<BN, NORM>(ep, TmemLoader{tacc}, m, n0, stg, &map_out, &map_xout, rstd, tn, ns, prepared);
+        tile_out(ep, TmemLoader{tacc}, o, 0, n_chunks, pre);
         release_acc();
       } else if (cl) {
-        uint8_t* reserve = smem + Cfg::kBudget - cl_reserve;       // the leader's: cl - 1 parts of [BN/4][cl_rows] float4
-        if (crank != 0) {
-          if (quad * 32 < cl_rows) {           // the warps that hold rows in use
-            const uint32_t dst = mapa_rank(smem_u32(reserve + (crank - 1) * cl_part_bytes), 0) + row_in_tile * 16;
-            const uint32_t col_stride = (uint32_t)cl_rows * 16u;
-#pragma unroll 1
-            for (int c = 0; c < BN / 32; ++c) {
-              float v[32];
-              tmem_ld32(tacc + c * 32, v);
-#pragma unroll
-              for (int i = 0; i < 8; ++i)
-                st_cluster_f4(dst + (uint32_t)(c * 8 + i) * col_stride, make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]));
-            }
-            __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(mapa_rank(smem_u32(red_bar), 0));   // release: the warp's stores are visible
-          }
-          release_acc();
-        } else {
-          if (!s_abort) {            // the peers' parts have landed (acquire at cluster scope)
-            bool ok = false;
-            for (uint32_t i = 0; i < kSpin && !ok; ++i) {
-              uint32_t got;
-              asm volatile(
-                  "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-                  : "=r"(got)
-                  : "r"(smem_u32(red_bar)), "r"(0u)
-                  : "memory");
-              ok = got != 0;
-              if (!ok && i > 64) __nanosleep(32);
-            }
-            if (!ok) {
-              set_status(ep.status, DEV_TIMEOUT_FULL);
-              s_abort = 1;
-            }
-          }
-          RingLoader ld{tacc, reinterpret_cast<const float4*>(reserve) + row_in_tile, BN, 0, n_splits, cl_rows};
-          row_epilogue<BN, NORM>(ep, ld, m, n0, stg, &map_out, &map_xout, rstd, tn, ns, false);
-          release_acc();
+        uint8_t* land = smem + (reserve ? ring_bytes : 0);
+        if (!reserve) {            // this CTA's products are complete and have read its ring (its accumulator is)
+          asm volatile("bar.sync 1, 128;" ::: "memory");
+          if (warp == 2 && lane < cl && lane != (int)part_rank) mbar_arrive_cluster(mapa_rank(smem_u32(go_bar), lane * kMul + rank));
+          wait_or_abort(go_bar, 0, DEV_TIMEOUT_EMPTY, true);
         }
+#pragma unroll 1
+        for (int c = 0; c < n_chunks; ++c) {
+          const int owner = c % cl;
+          if (owner == (int)part_rank) continue;
+          const int at = (c / cl) * (cl - 1) + ((int)part_rank < owner ? (int)part_rank : (int)part_rank - 1);
+          const uint32_t dst = mapa_rank(smem_u32(land + at * kChunkBytes), owner * kMul + rank) + row * 16;
+          float v[32];
+          tmem_ld_chunk(tacc + c * 32, v);
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+            st_cluster_f4(dst + (uint32_t)i * (FT * 16), make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]));
+        }
+        __syncwarp();
+        if (lane < cl && lane != (int)part_rank && lane < n_chunks)    // release: the warp's stores are visible
+          mbar_arrive_cluster(mapa_rank(smem_u32(red_bar), lane * kMul + rank));
+        if ((int)part_rank < n_chunks) {
+          wait_or_abort(red_bar, 0, DEV_TIMEOUT_FULL, true);           // the others' parts have landed (acquire at cluster scope)
+#pragma unroll 1
+          for (int c = (int)part_rank; c < n_chunks; c += cl) {
+            RingLoader ld{tacc, reinterpret_cast<const float4*>(land + (c / cl) * (cl - 1) * kChunkBytes) + row, 8, (int)part_rank, cl, c};
+            if (c != (int)part_rank) prefetch_chunk(ep, o, c, pre);
+            tile_out(ep, ld, o, c, c + 1, pre);
+          }
+        }
+        release_acc();
       } else {
         // park this split's partial tile and let the LAST split to arrive reduce all partials in split order
         // (deterministic) and run the fused epilogue
-        // (the two CTAs of a pair park and reduce their 128-row halves independently: slot and counter index are
+        // (the two CTAs of a pair park and reduce their 128 features independently: slot and counter index are
         // doubled and offset by the rank)
-        const int slot_mine = pc.slot * kSlotMul + (int)rank, slot0 = pc.slot0 * kSlotMul + (int)rank;
-        const int slot_next = pc.slot_next * kSlotMul + (int)rank, slot_stride = 2 * n_tiles_m * kSlotMul;
-        const int counter = tile * kSlotMul + (int)rank;
-        float4* mine = reinterpret_cast<float4*>(split_ws) + (size_t)slot_mine * (BN / 4) * BM + row_in_tile;
+        const int slot_mine = pc.slot * kMul + (int)rank, slot0 = pc.slot0 * kMul + (int)rank;
+        const int slot_next = pc.slot_next * kMul + (int)rank, slot_stride = 2 * mt * kMul;
+        const int counter = tile * kMul + (int)rank;
+        float4* mine = reinterpret_cast<float4*>(G.split_ws) + (size_t)slot_mine * part_f4 * FT + row;
 #pragma unroll 1
-        for (int c = 0; c < BN / 32; ++c) {
+        for (int c = 0; c < n_chunks; ++c) {
           float v[32];
-          tmem_ld32(tacc + c * 32, v);
-          if (m < ep.M) {
+          tmem_ld_chunk(tacc + c * 32, v);
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
-              __stcg(mine + (size_t)(c * 8 + i) * BM, make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]));
-          }
+          for (int i = 0; i < 8; ++i)
+            __stcg(mine + (size_t)(c * 8 + i) * FT, make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]));
         }
         // the accumulator may be handed back at once: the own part is read from TMEM again only when nothing follows
         // in this CTA, and then nobody overwrites it
@@ -932,39 +957,40 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
         asm volatile("bar.sync 1, 128;" ::: "memory");
         if (warp == 2 && lane == 0) {
           __threadfence();   // cumulative: orders the partial rows all 128 threads wrote before the barrier
-          const int old = atomicAdd(&split_counters[counter], 1);
+          const int old = atomicAdd(&G.split_counters[counter], 1);
           s_last = (old == n_splits - 1);
-          if (old == n_splits - 1) split_counters[counter] = 0;   // ready for the next launch
+          if (old == n_splits - 1) G.split_counters[counter] = 0;   // ready for the next launch
           __threadfence();
         }
         asm volatile("bar.sync 1, 128;" ::: "memory");
         if (s_last) {
+          prefetch_chunk(ep, o, 0, pre);
           // When nothing follows in this CTA the operand ring is idle (every load was consumed before the accumulator
           // completed): the other parts are fetched into it with bulk copies at full bandwidth and the own part is
           // taken from TMEM.  Otherwise the parts are read from global memory while the next piece's main loop runs.
-          constexpr int kPartBytes = BM * BN * 4;
           const bool final_piece = !(jd < dp_count || pos < range_hi);
-          if (final_piece && (n_splits - 1) * kPartBytes <= Cfg::kBudget) {
+          if (final_piece && (n_splits - 1) * part_bytes <= kRingBytes) {
             if (warp == 2 && lane == 0) {
               asm volatile("fence.proxy.async;" ::: "memory");   // the parts were written with ordinary stores
-              mbar_arrive_expect_tx(red_bar, (uint32_t)((n_splits - 1) * kPartBytes));
+              mbar_arrive_expect_tx(red_bar, (uint32_t)((n_splits - 1) * part_bytes));
               int k = 0;
               for (int p = 0; p < n_splits; ++p) {
                 if (p == pc.part) continue;
                 const int slot = p == 0 ? slot0 : slot_next + slot_stride * (p - 1);
-                const uint8_t* src = reinterpret_cast<const uint8_t*>(split_ws) + (size_t)slot * kPartBytes;
-                constexpr int kChunk = kPartBytes < 32768 ? kPartBytes : 32768;
-                for (int off = 0; off < kPartBytes; off += kChunk)
-                  bulk_g2s(smem + (size_t)k * kPartBytes + off, src + off, kChunk, red_bar);
+                const uint8_t* src = reinterpret_cast<const uint8_t*>(G.split_ws) + (size_t)slot * part_bytes;
+                for (int off = 0; off < part_bytes; off += 16384) {
+                  const int n = part_bytes - off < 16384 ? part_bytes - off : 16384;
+                  bulk_g2s(smem + (size_t)k * part_bytes + off, src + off, n, red_bar);
+                }
                 ++k;
               }
             }
             wait_or_abort(red_bar, 0, DEV_TIMEOUT_FULL);
-            RingLoader ld{tacc, reinterpret_cast<const float4*>(smem) + row_in_tile, BN, pc.part, n_splits, BM};
-            row_epilogue<BN, NORM>(ep, ld, m, n0, stg, &map_out, &map_xout, rstd, tn, ns, false);
+            RingLoader ld{tacc, reinterpret_cast<const float4*>(smem) + row, part_f4, pc.part, n_splits, 0};
+            tile_out(ep, ld, o, 0, n_chunks, pre);
           } else {
-            SplitLoader ld{split_ws, BN, row_in_tile, slot0, slot_next, slot_stride, n_splits, m < ep.M};
-            row_epilogue<BN, NORM>(ep, ld, m, n0, stg, &map_out, &map_xout, rstd, tn, ns, false);
+            SplitLoader ld{reinterpret_cast<const float4*>(G.split_ws) + row, part_f4, slot0, slot_next, slot_stride, n_splits};
+            tile_out(ep, ld, o, 0, n_chunks, pre);
           }
         }
         asm volatile("bar.sync 1, 128;" ::: "memory");       // s_last is reused by the next unit
@@ -972,20 +998,19 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     }
   }
 
-  if (warp >= 2) tma_store_drain_all(threadIdx.x & 31);   // the output boxes handed to the TMA unit have been written
   griddep_launch();   // this CTA's work is done: the next kernel's CTAs may be scheduled onto freed SMs
   tc_fence_before();
   __syncthreads();
-  if constexpr (PAIR) cluster_sync_all();   // the peer may read this CTA's operands and signal its barriers until here
-  // (a cluster of a thin problem needs no meeting here: only the leader's shared memory is written by others, and the
-  // leader has waited for those stores; the peers are free to leave)
+  // of a pair, the other CTA may read this CTA's operands and signal its barriers until here; in a cluster without a reserve
+  // every member signals and writes the others.  (With a reserve only the shared memory of member 0 is written by others, and
+  // it has waited for those stores: they are free to leave.)
+  if (PAIR || (cl && !reserve)) cluster_sync_all();
   if (warp == 1) {
     tc_fence_after();
-    if constexpr (PAIR) tmem_dealloc_pair(tmem_base, Cfg::kTmemCols);
-    else tmem_dealloc(tmem_base, Cfg::kTmemCols);
+    if constexpr (PAIR) tmem_dealloc_pair(tmem_base, kTmemCols);
+    else tmem_dealloc(tmem_base, kTmemCols);
   }
 }
-
 
 // ---- host side -------------------------------------------------------------------------------------
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -995,7 +1020,7 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
 struct MapKey {
   const void* ptr;
   uint64_t rows, cols;
-  uint32_t box_rows;
+  uint32_t box_rows;     // rows of the box (x), or 0x10000 + the order of w's rows (WeightOrder)
   bool operator==(const MapKey& o) const { return ptr == o.ptr && rows == o.rows && cols == o.cols && box_rows == o.box_rows; }
 };
 struct MapKeyHash {
@@ -1008,20 +1033,23 @@ constexpr size_t kSplitWsBytes = 96ull << 20;   // partial tiles of split-K laun
 constexpr int kSplitCounters = 1 << 16;
 constexpr size_t kMapCacheMax = 4096;           // entries; the keys include the row count, so a serving loop keeps adding
 
-// Cache of encoded tensor maps (cached_map below).  Maps are handed out BY VALUE: a launch needs three maps at once,
-// and a miss on the second or third lookup may empty the full cache, so nothing may point into it.
+// Cache of encoded tensor maps (cached_map below).  Maps are handed out BY VALUE: a launch needs several at once,
+// and a miss on a later lookup may empty the full cache, so nothing may point into it.
+struct Config {        // how a projection runs: single CTAs or CTA pairs, the widest token tile, whole tiles / stream-K / clusters of cl parts
+  bool pair, stream_k;
+  int tmax, cl;
+};
 struct TcState {
   int n_sm = 0;
-  int force_bn = 0, force_s = 0;
+  int force_tile = 0, force_s = 0;
   float* split_ws = nullptr;
   int* split_counters = nullptr;
   EncodeTiledFn encode = nullptr;
   std::unordered_map<MapKey, CUtensorMap, MapKeyHash> maps;
   size_t evictions = 0;
-  int last_tiles_n = 0;       // column tiles of the last launch
-  bool configured[10] = {false, false, false, false, false, false, false, false, false, false};
-  bool thin_clusters = true;  // problems of one row tile with cut tiles run as clusters that reduce through distributed shared memory
-  int max_clusters[10][5];    // cached occupancy answers per kernel and cluster size (-1: not asked yet)
+  bool configured[2] = {false, false};
+  bool clusters = true;       // tiles cut over K may be handed over inside clusters
+  int max_clusters[2][9];     // cached occupancy answers per kernel and cluster size in CTAs (-1: not asked yet)
   TcState() {
     for (auto& row : max_clusters)
       for (int& v : row) v = -1;
@@ -1046,8 +1074,8 @@ bool cached_map(TcState* st, const MapKey& key, CUtensorMap* out, Encode&& encod
   return true;
 }
 
-// [rows, cols] bf16 row-major, box = [box_rows, 64 columns], 128-byte swizzle, zero fill out of bounds
-bool get_map(TcState* st, const void* ptr, uint64_t rows, uint64_t cols, uint32_t box_rows, CUtensorMap* out) {
+// x [rows, cols] bf16 row-major, box = [box_rows, 64 columns], 128-byte swizzle, zero fill out of bounds
+bool get_x_map(TcState* st, const void* ptr, uint64_t rows, uint64_t cols, uint32_t box_rows, CUtensorMap* out) {
   return cached_map(st, MapKey{ptr, rows, cols, box_rows}, out, [&](CUtensorMap* m) {
     cuuint64_t dims[2] = {cols, rows};
     cuuint64_t strides[1] = {cols * 2};
@@ -1059,129 +1087,178 @@ bool get_map(TcState* st, const void* ptr, uint64_t rows, uint64_t cols, uint32_
   });
 }
 
-// Output [rows, cols] of 2- or 4-byte elements, row-major: box = 32 rows x 64 bytes, 64-byte swizzle
-bool get_out_map(TcState* st, const void* ptr, uint64_t rows, uint64_t cols, int elem_bytes, CUtensorMap* out) {
-  return cached_map(st, MapKey{ptr, rows, cols, (uint32_t)(0x10000 + elem_bytes)}, out, [&](CUtensorMap* m) {
-    cuuint64_t dims[2] = {cols, rows};
-    cuuint64_t strides[1] = {cols * (uint64_t)elem_bytes};
-    cuuint32_t box[2] = {(cuuint32_t)(64 / elem_bytes), 32};
-    cuuint32_t estr[2] = {1, 1};
-    return st->encode(m, elem_bytes == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2,
-                      const_cast<void*>(ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                      CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+// w [rows, K] as five dimensions (k, 16 rows, halves, groups, heads); one box is the 128 rows of a feature tile in the order
+// the epilogue wants them in the TMEM lanes:
+//   plain   rows as they are
+//   SwiGLU  16 gate rows, the 16 up rows that belong to them, the next 16 gate rows ... (rows = 2 F)
+//   rotary  per head: 16 low dims, their 16 partners half a head away, the next 16 low dims ...
+enum WeightOrder { kWPlain = 0, kWSwiglu = 1, kWRope128 = 2, kWRope64 = 3 };
+bool get_w_map(TcState* st, const void* ptr, uint64_t rows, uint64_t K, WeightOrder order, CUtensorMap* out, int* step3, int* step4) {
+  *step3 = order == kWPlain ? 8 : (order == kWSwiglu ? 4 : 0);
+  *step4 = order == kWRope128 ? 1 : (order == kWRope64 ? 2 : 0);
+  return cached_map(st, MapKey{ptr, rows, K, 0x10000u + (uint32_t)order}, out, [&](CUtensorMap* m) {
+    const cuuint64_t r = K * 2;      // bytes of a row
+    cuuint64_t dims[5] = {K, 16, 1, rows / 16, 1}, strides[4] = {r, 16 * r, 16 * r, 128 * r};
+    cuuint32_t box[5] = {BK, 16, 1, 8, 1}, estr[5] = {1, 1, 1, 1, 1};
+    if (order == kWSwiglu) {
+      dims[2] = 2; dims[3] = rows / 32;
+      strides[1] = rows / 2 * r;
+      box[2] = 2; box[3] = 4;
+    } else if (order == kWRope128 || order == kWRope64) {
+      const int D = order == kWRope128 ? 128 : 64;
+      dims[2] = 2; dims[3] = D / 32; dims[4] = rows / D;
+      strides[1] = D / 2 * r; strides[3] = D * r;
+      box[2] = 2; box[3] = D / 32; box[4] = 128 / D;
+    }
+    return st->encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(ptr), dims, strides, box, estr,
+                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
   });
 }
 
-template <int BN, bool PAIR, bool NORM>
-bool launch_bn_t(TcState* st, int idx, const GemmArgs& a, const EpiParams& ep, bool stream_k, cudaStream_t stream);
-
-template <int BN, bool PAIR>
-bool launch_bn(TcState* st, int idx, const GemmArgs& a, const EpiParams& ep, bool stream_k, cudaStream_t stream) {
-  return a.epi == EPI_RESIDUAL_NORM ? launch_bn_t<BN, PAIR, true>(st, idx + 5, a, ep, stream_k, stream)
-                                    : launch_bn_t<BN, PAIR, false>(st, idx, a, ep, stream_k, stream);
+bool configure(TcState* st, bool pair) {
+  if (st->configured[pair]) return true;
+  const void* k = pair ? reinterpret_cast<const void*>(gemm_tc_kernel<true>) : reinterpret_cast<const void*>(gemm_tc_kernel<false>);
+  if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) != cudaSuccess) return false;
+  return st->configured[pair] = true;
 }
 
-template <int BN, bool PAIR, bool NORM>
-int max_active_clusters(TcState* st, int idx, int n_tiles, int parts);
-
-// Problems of one row tile (at most 128 rows) whose tiles would be cut over K: how many CTAs form the cluster that shares
-// a tile (0: no clusters).  The whole grid has to be resident at once, which the occupancy query decides (cached).
-template <int BN, bool PAIR, bool NORM>
-int cluster_parts(TcState* st, int idx, int n_tiles, int KB, int rows) {
-  if (PAIR || !st->thin_clusters || n_tiles <= 0) return 0;
-  using Cfg = TcCfg<BN, PAIR, NORM>;
-  int parts = st->n_sm / n_tiles;
-  if (parts > 4) parts = 4;
-  if (parts > KB) parts = KB;
-  // the leader keeps the peers' parts at the top of its ring budget: at least four stages must remain
-  const int part_bytes = ((rows + 31) & ~31) * BN * 4;
-  const int stage_bytes = (rows <= 32 ? Cfg::kThinABytes : Cfg::kABytes) + Cfg::kBBytes;
-  while (parts >= 2 && (Cfg::kBudget - (parts - 1) * part_bytes) / stage_bytes < 4) --parts;
-  for (; parts >= 2; --parts) {
-    if (max_active_clusters<BN, PAIR, NORM>(st, idx, n_tiles, parts) >= n_tiles) return parts;
-  }
-  return 0;
-}
-
-template <int BN, bool PAIR, bool NORM>
-int max_active_clusters(TcState* st, int idx, int n_tiles, int parts) {
-  int& cached = st->max_clusters[idx][parts];
+// Whether n clusters of `size` CTAs are resident at once (the occupancy query's answer is kept).
+bool clusters_fit(TcState* st, bool pair, int size, int n) {
+  if (size > 8 || !configure(st, pair)) return false;
+  int& cached = st->max_clusters[pair][size];
   if (cached < 0) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(n_tiles * parts);
+    cfg.gridDim = dim3(size * n);
     cfg.blockDim = dim3(kTcThreads);
-    cfg.dynamicSmemBytes = TcCfg<BN, PAIR, NORM>::kSmemBytes;
+    cfg.dynamicSmemBytes = kSmemBytes;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = parts;
+    attr[0].val.clusterDim.x = size;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, gemm_tc_kernel<BN, PAIR, NORM>, &cfg) != cudaSuccess) {
+    int got = 0;
+    if ((pair ? cudaOccupancyMaxActiveClusters(&got, gemm_tc_kernel<true>, &cfg)
+              : cudaOccupancyMaxActiveClusters(&got, gemm_tc_kernel<false>, &cfg)) != cudaSuccess) {
       cudaGetLastError();
-      n = 0;
+      got = 0;
     }
-    cached = n;
+    cached = got;
   }
-  return cached;
+  return cached >= n;
 }
 
-template <int BN, bool PAIR, bool NORM>
-bool launch_bn_t(TcState* st, int idx, const GemmArgs& a, const EpiParams& ep, bool stream_k, cudaStream_t stream) {
-  st->last_tiles_n = (a.N + (a.epi == EPI_SWIGLU ? BN / 2 : BN) - 1) / (a.epi == EPI_SWIGLU ? BN / 2 : BN);
-  using Cfg = TcCfg<BN, PAIR, NORM>;
-  if (!st->configured[idx]) {
-    if (cudaFuncSetAttribute(gemm_tc_kernel<BN, PAIR, NORM>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes) !=
-        cudaSuccess)
-      return false;
-    st->configured[idx] = true;
+// Estimated time in microseconds, fitted to B200 measurements of the five 8B-class projections at 8 to 1864 rows (single calls
+// back to back, weights from HBM; within about 10 %).
+// A k-block of a tile costs (.075 + .001 x tokens) us alone and a third more when all SMs pull operands through L2; a CTA pair
+// .085 + .00085 x tokens and a quarter more.  Examples, all SMs busy: 128 features x 256 tokens .44 us, 256 x 256 .37, 256 x 128
+// .24.  Below .18 us a CTA is bound by the latency of its loads.
+// The weights come from HBM once: bytes / 6.7 TB/s.
+// On top come the ends (launch, first loads, last tile's epilogue): 4.5 us + .003 x tokens for whole tiles; 6 us when clusters
+// reduce tiles of one chunk, 6.5 us + 1 us per chunk that a member sends for wider ones; 11.5 us + .05 x tokens when cut tiles go
+// through the workspace (parking, counting, fetching, the epilogue in the last part to arrive).
+struct Shape {
+  int M, n_feat, K;       // n_feat: rows of w
+};
+double est_kblock(bool pair, int width, double busy) {
+  if (busy > 1.0) busy = 1.0;
+  const double t = pair ? (.085 + .00085 * width) * (.95 + .25 * busy) : (.075 + .001 * width) * (.92 + .40 * busy);
+  return fmax(t, .18);
+}
+
+Config choose_config(TcState* st, const Shape& s) {
+  const int KB = s.K / BK;
+  const double t_hbm = 2.0 * s.n_feat * s.K / 6.7e6;
+  Config best{false, false, kMaxTok, 0};
+  double best_t = 1e30;
+  for (int pair = 0; pair < 2; ++pair) {
+    const int gran = pair ? 32 : 16, units = pair ? st->n_sm / 2 : st->n_sm;
+    const int cols = (s.n_feat + FT * (pair + 1) - 1) / (FT * (pair + 1));
+    const int fewest = (s.M + kMaxTok - 1) / kMaxTok;
+    int last = 0;
+    for (int want = fewest; want <= fewest + 3 + fewest / 4; ++want) {
+      const int tmax = ((s.M + want - 1) / want + gran - 1) / gran * gran;    // the widest tile that gives `want` tiles
+      if (tmax == last || tmax < gran) continue;
+      last = tmax;
+      int width, mt;
+      token_tiles(s.M, tmax, gran, &width, &mt);
+      const long long tiles = (long long)mt * cols;
+      if (tiles * (pair + 1) > kSplitCounters || (want > fewest && width < 32)) continue;
+      auto consider = [&](double t, bool sk, int cl) {
+        if (t < best_t) {
+          best_t = t;
+          best = Config{pair != 0, sk, tmax, cl};
+        }
+      };
+      const long long full = tiles / units, rem = tiles % units;      // full waves, and a last one that has the machine to itself
+      const double t_whole = KB * (full * est_kblock(pair, width, 1.0) + (rem ? est_kblock(pair, width, (double)rem / units) : 0.0));
+      consider(fmax(t_whole, t_hbm) + 4.5 + .003 * width, false, 0);
+      // cut over K through the workspace; with two waves or more only the ragged end is cut (and done first)
+      if (mt <= units && (full < 2 || rem))
+        consider(fmax((double)tiles * KB / ((units / mt) * mt) * est_kblock(pair, width, 1.0), t_hbm) + 11.5 + .05 * width, true, 0);
+      // clusters of 2 to 4 parts per tile, all resident at once
+      const int chunks = (width + 31) / 32;
+      for (int cl = 2; cl <= 4 && st->clusters; ++cl) {
+        if (tiles * cl > units || cl * 4 > KB || !clusters_fit(st, pair, cl * (pair + 1), (int)tiles)) break;
+        const double ends = chunks == 1 ? 6.0 : 6.5 + (double)chunks * (cl - 1) / cl;
+        consider(fmax((KB + cl - 1) / cl * est_kblock(pair, width, (double)tiles * cl / units), t_hbm) + ends, true, cl);
+      }
+    }
   }
-  constexpr int kRows = PAIR ? 2 * BM : BM;
+  return best;
+}
+
+bool launch_config(TcState* st, const GemmArgs& a, const EpiParams& ep, const Config& c, cudaStream_t stream) {
+  if (!configure(st, c.pair)) return false;
   const bool swiglu = a.epi == EPI_SWIGLU;
+  const int mul = c.pair ? 2 : 1;
   const uint64_t w_rows = swiglu ? 2ull * a.N : (uint64_t)a.N;
-  const int thin = (!PAIR && a.M <= 32) ? 1 : 0;
-  CUtensorMap mx, mw, mo;     // copies: see cached_map
-  if (!get_map(st, a.x, a.M, a.K, thin ? 32 : BM, &mx)) return false;
-  if (!get_map(st, a.w, w_rows, a.K, (swiglu || PAIR) ? BN / 2 : BN, &mw)) return false;
-  // the epilogue stores through the TMA unit (of the rotary / KV-append epilogue: the rotated queries [M, n_q * d];
-  // K and V are scattered into the paged pool by hand)
-  const bool f32 = a.epi == EPI_PLAIN_F32 || a.epi == EPI_RESIDUAL || a.epi == EPI_RESIDUAL_NORM;
-  CUtensorMap mxo = mx;       // only read by EPI_RESIDUAL_NORM
-  if (a.epi == EPI_RESIDUAL_NORM && !get_out_map(st, a.x_out, a.M, (uint64_t)a.N, 2, &mxo)) return false;
-  if (!get_out_map(st, a.out, a.M, a.epi == EPI_QKV_ROPE ? (uint64_t)a.n_q * a.head_dim : (uint64_t)a.N, f32 ? 4 : 2, &mo))
-    return false;
-  const int out_per_tile = swiglu ? BN / 2 : BN;
-  const int n_tiles_n = (a.N + out_per_tile - 1) / out_per_tile;
-  const int mt = (a.M + kRows - 1) / kRows;
-  const int n_tiles = mt * n_tiles_n;
-  const long long KB = a.K / BK;
-  const int n_units = PAIR ? st->n_sm / 2 : st->n_sm;       // scheduling units: CTAs, or clusters of two
+  GemmLaunch g{};
+  g.m_cap = a.M;
+  g.K = a.K;
+  g.n_cols = (int)((w_rows + FT * mul - 1) / (FT * mul));
+  // (with the row count on the device the width of the token tiles is, too: x is then loaded in boxes of 32 or 16 rows)
+  g.gran = a.m_dev ? 32 : (c.pair ? 32 : 16);
+  g.tmax = (c.tmax + g.gran - 1) / g.gran * g.gran;
+  int width, mt;
+  token_tiles(a.M, g.tmax, g.gran, &width, &mt);
+  g.x_box = a.m_dev ? 32 / mul : width / mul;
+  CUtensorMap mw, mx;     // copies: see cached_map
+  const WeightOrder order = swiglu ? kWSwiglu : (a.epi == EPI_QKV_ROPE ? (a.head_dim == 128 ? kWRope128 : kWRope64) : kWPlain);
+  if (!get_w_map(st, a.w, w_rows, a.K, order, &mw, &g.w_step3, &g.w_step4)) return false;
+  if (!get_x_map(st, a.x, a.M, a.K, g.x_box, &mx)) return false;
+  const int n_tiles = mt * g.n_cols, KB = a.K / BK;
+  const int n_units = c.pair ? st->n_sm / 2 : st->n_sm;       // scheduling units: CTAs or pairs
   int units = n_tiles < n_units ? n_tiles : n_units;
-  int dp_tiles = n_tiles;       // whole tiles, strided
-  long long per = 1;
-  const int cl = (stream_k && mt == 1 && a.M <= BM) ? cluster_parts<BN, PAIR, NORM>(st, idx, n_tiles, (int)KB, a.M) : 0;
-  if (cl) {
-    units = n_tiles * cl;       // one cluster per tile; the kernel derives each member's k-blocks from its rank
+  g.dp_tiles = n_tiles;       // whole tiles, strided
+  g.per = 1;
+  g.cl = c.cl;
+  if (c.cl) {
+    units = n_tiles * c.cl;   // one cluster per tile; the kernel derives each member's k-blocks from its rank
   } else if (a.m_dev) {
     // the row count is on the device: the kernel counts the tiles and, for stream-K, divides the k-blocks itself; the
     // grid has every unit (units without work leave at once)
-    dp_tiles = stream_k ? -2 : -1;
+    g.dp_tiles = c.stream_k ? -2 : -1;
     units = n_units;
-  } else if (stream_k) {
-    stream_k_schedule(n_tiles, mt, (int)KB, n_units, &dp_tiles, &per, &units);     // the caller made sure that mt <= n_units
+  } else if (c.stream_k) {
+    stream_k_schedule(n_tiles, mt, KB, n_units, &g.dp_tiles, &g.per, &units);     // the caller made sure that mt <= n_units
   }
+  g.split_ws = st->split_ws;
+  g.split_counters = st->split_counters;
+  g.m_dev = a.m_dev;
+  g.m_dev_wait = a.m_dev_settled ? 0 : 1;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(PAIR ? 2 * units : units);
+  cfg.gridDim = dim3(mul * units);
   cfg.blockDim = dim3(kTcThreads);
-  cfg.dynamicSmemBytes = Cfg::kSmemBytes;
+  cfg.dynamicSmemBytes = kSmemBytes;
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
   int n_attr = 0;
-  if (PAIR || cl) {
+  if (c.pair || c.cl) {
     attr[n_attr].id = cudaLaunchAttributeClusterDimension;
-    attr[n_attr].val.clusterDim.x = PAIR ? 2 : cl;
+    attr[n_attr].val.clusterDim.x = mul * (c.cl ? c.cl : 1);
     attr[n_attr].val.clusterDim.y = 1;
     attr[n_attr].val.clusterDim.z = 1;
     ++n_attr;
@@ -1195,8 +1272,8 @@ bool launch_bn_t(TcState* st, int idx, const GemmArgs& a, const EpiParams& ep, b
   }
   cfg.attrs = attr;
   cfg.numAttrs = n_attr;
-  return cudaLaunchKernelEx(&cfg, gemm_tc_kernel<BN, PAIR, NORM>, mx, mw, mo, mxo, a.M, n_tiles_n, a.K, a.N, dp_tiles, per, thin, cl,
-                            st->split_ws, st->split_counters, a.m_dev, a.m_dev_settled ? 0 : 1, ep) == cudaSuccess;
+  return (c.pair ? cudaLaunchKernelEx(&cfg, gemm_tc_kernel<true>, mw, mx, g, ep)
+                 : cudaLaunchKernelEx(&cfg, gemm_tc_kernel<false>, mw, mx, g, ep)) == cudaSuccess;
 }
 
 }  // namespace
@@ -1223,12 +1300,12 @@ void* tc_state_create(int n_sm) {
   return st;
 }
 
-void tc_state_force(void* s, int bn, int stream_k) {
+void tc_state_force(void* s, int tile, int stream_k) {
   TcState* st = static_cast<TcState*>(s);
   if (!st) return;
-  st->force_bn = bn;
-  st->force_s = stream_k != 0;
-  st->thin_clusters = stream_k != 2;     // 2: cut tiles always go through the partial-tile workspace
+  st->force_tile = tile;
+  st->force_s = stream_k;
+  st->clusters = stream_k != 2;     // 2: cut tiles always go through the partial-tile workspace
 }
 
 void tc_state_reset(void* s, cudaStream_t stream) {
@@ -1279,23 +1356,17 @@ void tc_state_destroy(void* s) {
   delete st;
 }
 
-static bool launch_gemm_tc_impl(const GemmArgs& a, TcState* st, int* status, cudaStream_t stream);
-
 bool launch_gemm_tc(const GemmArgs& a, void* tc_state, int* status, cudaStream_t stream, int* ss_slots_out) {
   TcState* st = static_cast<TcState*>(tc_state);
-  if (!st || a.M <= 0) return false;
-  if (a.epi == EPI_RESIDUAL_NORM && (!a.x_out || !a.gain || !a.ss_out || a.N % 32)) return false;
-  const bool ok = launch_gemm_tc_impl(a, st, status, stream);
-  if (ok && ss_slots_out) *ss_slots_out = st->last_tiles_n;
-  return ok;
-}
-
-static bool launch_gemm_tc_impl(const GemmArgs& a, TcState* st, int* status, cudaStream_t stream) {
-  if (a.K % BK) return false;
+  if (!st || a.M <= 0 || a.K % BK || a.N % 16) return false;
   if ((reinterpret_cast<uintptr_t>(a.x) | reinterpret_cast<uintptr_t>(a.w)) & 15) return false;
+  if (a.epi == EPI_RESIDUAL_NORM && (!a.x_out || !a.gain || !a.ss_out)) return false;
+  if (a.epi == EPI_SWIGLU && a.N % 64) return false;
+  if (a.epi == EPI_QKV_ROPE && (a.N % 128 || (a.head_dim != 64 && a.head_dim != 128))) return false;
   EpiParams ep;
   ep.epi = a.epi;
   ep.out = a.out;
+  ep.x_out = static_cast<__nv_bfloat16*>(a.x_out);
   ep.M = a.M;
   ep.N = a.N;
   ep.tok_slot = a.tok_slot;
@@ -1314,91 +1385,28 @@ static bool launch_gemm_tc_impl(const GemmArgs& a, TcState* st, int* status, cud
   ep.norm_eps = a.norm_eps;
   ep.gain = static_cast<const __nv_bfloat16*>(a.gain);
   ep.ss_out = a.ss_out;
-  const bool swiglu = a.epi == EPI_SWIGLU;
-  // Choose the tile width and the decomposition with a small cost model in microseconds, calibrated on B200:
-  // whole tiles cost waves x k-blocks x (tensor time of one k-block at that width); the stream-K decomposition
-  // spreads all k-blocks evenly over the SMs and pays a fixed hand-over for the cut tiles (park the partial,
-  // fence, counter, reduction read).  Rotary tiles must hold whole heads.
+  const int n_feat = a.epi == EPI_SWIGLU ? 2 * a.N : a.N;
   // (device-resident rounds: the configuration is chosen for the caller's hint of the row count, the launch covers the capacity)
   const int Mc = (a.m_dev && a.m_hint > 0 && a.m_hint < a.M) ? a.m_hint : a.M;
-  const int mt = (Mc + BM - 1) / BM;
-  const int KB = a.K / BK;
-  int best_bn = 0;
-  bool best_sk = false, best_pair = false;
-  double best_t = 1e30;
-  // configurations: single CTAs with 128-row tiles of width 256 / 128 / 64, and CTA pairs with 256 x 256 or 256 x 128
-  // tiles (a k-block of a pair takes about 0.87 / 0.76 of the single CTA's, for twice the rows: the pair halves the
-  // weight bytes each SM's tensor core pulls out of its own shared memory)
-  constexpr int kConfigs = 5;
-  const int bns[kConfigs] = {256, 128, 64, 256, 128};
-  const double kb_tensor[kConfigs] = {0.44, 0.27, 0.22, 0.385, 0.205};
-  const bool pair_ok = Mc > BM && (swiglu ? a.N % 128 == 0 : a.N % 256 == 0) && !(a.epi == EPI_QKV_ROPE && 256 % a.head_dim);
-  const bool pair128_ok = Mc > BM && !swiglu && a.N % 128 == 0 && !(a.epi == EPI_QKV_ROPE && 128 % a.head_dim);
-  for (int bi = 0; bi < kConfigs; ++bi) {
-    const int bn = bns[bi];
-    const bool pair = bi >= 3;
-    if (bi == 3 && !pair_ok) continue;
-    if (bi == 4 && !pair128_ok) continue;
-    const int rows_tile = pair ? 2 * BM : BM;
-    const int units = pair ? st->n_sm / 2 : st->n_sm;            // CTAs or clusters
-    const int mtc = (Mc + rows_tile - 1) / rows_tile;
-    const int per = swiglu ? bn / 2 : bn;
-    if (a.epi == EPI_QKV_ROPE && (bn < a.head_dim || a.N % bn)) continue;
-    if (swiglu && (a.N % per)) continue;
-    const int tiles = mtc * ((a.N + per - 1) / per);
-    if (tiles * (pair ? 2 : 1) > kSplitCounters) continue;
-    const long long waves = (tiles + units - 1) / units;
-    // a k-block costs its tensor time, or the time one SM needs to stream its share of the weight bytes (the
-    // CTAs that work on one weight tile at the same time share them through L2)
-    const double kbt = fmax(kb_tensor[bi], (bn * 128.0 / mt) / 35e3);
-    const double rows = Mc < BM ? Mc : BM;
-    const double t_plain = (double)waves * KB * kbt;
-    const int sk_units = mtc <= units ? (units / mtc) * mtc : 1;     // teams of mtc units
-    const double t_sk = ((double)tiles * KB / sk_units + 1.0) * kbt + 3.0 + rows * bn * 4.0 * 2.5 / 16e3;
-    if (t_plain < best_t) { best_t = t_plain; best_bn = bn; best_sk = false; best_pair = pair; }
-    const bool ws_fits = (size_t)2 * st->n_sm * BM * bn * 4 <= kSplitWsBytes && mtc <= units;
-    const long long full = tiles / units, rem = tiles % units;
-    if (ws_fits && full >= 2) {
-      // a ragged last wave: the last (units + rem) tiles are cut evenly over the SMs and done FIRST, so that their
-      // hand-over (park the partial, counter, reduction by the last arriver) hides under the whole tiles after it.
-      // Measured: the cut tiles run a little slower than whole ones, so this only pays when the last wave would
-      // leave a good part of the machine idle.
-      const double idle = rem ? (double)(units - rem) / units / (double)(full + 1) : 0.0;
-      const double t_h = (double)tiles * KB / units * kbt + 2.0;
-      if (idle > 0.12 && t_h < best_t) { best_t = t_h; best_bn = bn; best_sk = true; best_pair = pair; }
-    } else if (ws_fits && t_sk < best_t) {
-      // no whole tiles to hide the hand-over under: it happens in every CTA at once at the end of the kernel and
-      // costs about 3 us + 0.6 us per KB of partial tile, which t_sk charges
-      best_t = t_sk; best_bn = bn; best_sk = true; best_pair = pair;
+  Config c = choose_config(st, Shape{Mc, n_feat, a.K});
+  if (st->force_tile || st->force_s == 1) {   // debugging aid: single CTAs (64, 128, 256 tokens) or pairs (384: 128, 512: 256 tokens)
+    const int f = st->force_tile;
+    if (f) {
+      const bool pair = f > 256;
+      const int tmax = f == 384 ? 128 : (f == 512 ? 256 : f);
+      if ((long long)((a.M + tmax - 1) / tmax) * ((n_feat + FT - 1) / FT + 1) * 2 <= kSplitCounters) c = Config{pair, false, tmax, 0};
     }
+    const int gran = c.pair ? 32 : 16, units = c.pair ? st->n_sm / 2 : st->n_sm;
+    int width, mt;
+    token_tiles(a.M, c.tmax, gran, &width, &mt);
+    c.stream_k = st->force_s != 0 && mt <= units;
+    c.cl = 0;
+    const int tiles = mt * ((n_feat + FT * (c.pair + 1) - 1) / (FT * (c.pair + 1)));
+    for (int cl = 4; cl >= 2 && c.stream_k && st->clusters && !c.cl; --cl)
+      if (tiles * cl <= units && cl * 4 <= a.K / BK && clusters_fit(st, c.pair, cl * (c.pair + 1), tiles)) c.cl = cl;
   }
-  if (st->force_bn == 384) {    // tuning aid: CTA pairs with 256 x 128 tiles, "384,<0 whole tiles | 1 stream-K>"
-    if (pair128_ok && (a.M + 255) / 256 <= st->n_sm / 2) return launch_bn<128, true>(st, 4, a, ep, st->force_s != 0, stream);
-  } else
-  if (st->force_bn == 512) {    // tuning aid: the 256 x 256 CTA-pair kernel, "512,<0 whole tiles | 1 stream-K>"
-    if (pair_ok && (a.M + 255) / 256 <= st->n_sm / 2) return launch_bn<256, true>(st, 3, a, ep, st->force_s != 0, stream);
-  } else
-  if (st->force_bn) {   // tuning aid (tc_state_force): tile width, 0 whole tiles | 1 stream-K; ignored where it does not fit
-    const int bn = st->force_bn;
-    const int per = swiglu ? bn / 2 : bn;
-    const bool shape_ok = (bn == 256 || bn == 128 || bn == 64) &&
-                          !(a.epi == EPI_QKV_ROPE && (bn < a.head_dim || a.N % bn)) && !(swiglu && (a.N % per)) &&
-                          mt * ((a.N + per - 1) / per) <= kSplitCounters;
-    if (shape_ok) {
-      best_bn = bn;
-      best_pair = false;
-      best_sk = st->force_s != 0 && mt <= st->n_sm && (size_t)2 * st->n_sm * BM * bn * 4 <= kSplitWsBytes;
-    }
-  }
-  if (!best_bn) return false;
-  if (swiglu && (a.N % 32)) return false;
-  if (best_pair && best_bn == 128) return launch_bn<128, true>(st, 4, a, ep, best_sk, stream);
-  if (best_pair) return launch_bn<256, true>(st, 3, a, ep, best_sk, stream);
-  switch (best_bn) {
-    case 256: return launch_bn<256, false>(st, 0, a, ep, best_sk, stream);
-    case 128: return launch_bn<128, false>(st, 1, a, ep, best_sk, stream);
-    default: return launch_bn<64, false>(st, 2, a, ep, best_sk, stream);
-  }
+  if (ss_slots_out) *ss_slots_out = (a.N + FT - 1) / FT;
+  return launch_config(st, a, ep, c, stream);
 }
 
 }  // namespace recg

@@ -69,7 +69,7 @@ void launch_guard_fill(void* base, const size_t* offs_dev, int n, cudaStream_t s
 void launch_guard_check(const void* base, const size_t* offs_dev, int n, int* status, cudaStream_t st);
 void launch_wait_timeout(uint32_t max_polls, int* status, cudaStream_t st);
 // S2: h[t] = embed[tok_id[t]] (fp32 residual stream), the rotary table (cos, sin) of pos * base^(-2i/d) as float2
-// [head_dim/2][T] (frequency-major), and the input of the first normalised projection: x[t] = rmsnorm(h[t]) * gain, or with
+// [T][head_dim/2], and the input of the first normalised projection: x[t] = rmsnorm(h[t]) * gain, or with
 // ss != null (folded RMSNorm) x[t] = bf16(h[t] * gain) and ss[t] = sum h[t]^2 (one slot).
 void launch_embed(const BatchLayout& bl, const Dims& dm, const void* embed, float* h, const void* gain, void* x, float* ss,
                   void* rope_cs, cudaStream_t st);
@@ -109,7 +109,7 @@ enum Epilogue : int {
   EPI_SWIGLU = 3,      // w is [2F,K]; out bf16 [M,F] = silu(x.wg) * (x.wu)
   EPI_QKV_ROPE = 4,    // rotate q and k heads, q -> bf16 [M, n_q*d], k/v -> paged pool at tok_slot
   EPI_RESIDUAL_NORM = 5  // h fp32 [M,N] += acc, and the input of the next RMSNorm-ed projection: x_out bf16 [M,N] =
-                         // h * gain, ss_out[column tile][row] = sum over the tile's columns of h^2 (tcgen05 path only)
+                         // h * gain, ss_out[128-feature tile][row] = sum over the tile's columns of h^2 (tcgen05 path only)
 };
 struct GemmArgs {
   const void* x;   // bf16 [M,K]
@@ -123,7 +123,7 @@ struct GemmArgs {
   void* kv_pool;
   int64_t n_pages;
   int layer, n_q, n_kv, head_dim;
-  const void* rope_cs;  // float2 [head_dim/2][M]: (cos, sin) of each token's rotary angles, frequency-major
+  const void* rope_cs;  // float2 [M][head_dim/2]: (cos, sin) of each token's rotary angles
   // device-resident rounds: the true row count (M is then the capacity the tensor maps cover), and the row count the
   // tile configuration is chosen for (0: M)
   const int* m_dev;
@@ -135,7 +135,7 @@ struct GemmArgs {
   float norm_eps;       // the mean is over K (the width of x)
   void* x_out;          // EPI_RESIDUAL_NORM: bf16 [M,N]
   const void* gain;     // EPI_RESIDUAL_NORM: bf16 [N]
-  float* ss_out;        // EPI_RESIDUAL_NORM: [column tiles][ss_stride]; *ss_slots_out receives the tile count
+  float* ss_out;        // EPI_RESIDUAL_NORM: [128-feature tiles][ss_stride]; *ss_slots_out receives the tile count
 };
 // legacy tensor path (mma.sync), any M; N multiple of 64 (EPI_SWIGLU: F multiple of 32), K multiple of 32
 void launch_gemm_simt(const GemmArgs& a, int* status, cudaStream_t st);
@@ -145,10 +145,10 @@ struct TcGemmPlan;  // opaque: cached tensor maps
 bool launch_gemm_tc(const GemmArgs& a, void* tc_state, int* status, cudaStream_t st, int* ss_slots_out = nullptr);
 void* tc_state_create(int n_sm);
 void tc_state_destroy(void* s);
-// debugging aid: force the tile configuration of the following launches (bn 64 / 128 / 256 single CTAs, 384 = CTA pairs
-// with 256 x 128 tiles, 512 = CTA pairs with 256 x 256 tiles; 0 = back to the cost model) and the decomposition
-// (0 whole tiles, 1 tiles cut over K, 2 the same without the cluster hand-over of thin problems)
-void tc_state_force(void* s, int bn, int stream_k);
+// debugging aid: force the tile configuration of the following launches (tile 64 / 128 / 256: single CTAs with token tiles of
+// at most that width, 384 / 512: CTA pairs with token tiles of at most 128 / 256; 0 = back to the cost model) and the
+// decomposition (0 whole tiles, 1 tiles cut over K, 2 the same without the hand-over inside clusters)
+void tc_state_force(void* s, int tile, int stream_k);
 // zero the arrival counters of cut tiles (after a launch that ended with an error status)
 void tc_state_reset(void* s, cudaStream_t st);
 // host-only self-test of the tensor-map cache; returns the number of wrong maps handed out

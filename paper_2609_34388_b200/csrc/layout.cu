@@ -362,11 +362,11 @@ __global__ void __launch_bounds__(256) embed_kernel(const int* __restrict__ tok_
       sq += f.x * f.x + f.y * f.y + f.z * f.z + f.w * f.w;
     }
   }
-  // rotary factors, frequency-major [half][n_tok]: the projection epilogue has one token per thread, so a warp reads 32
-  // consecutive tokens of one frequency in one 256-byte request.  Angles in double.
+  // rotary factors [token][half]: in the projection epilogue a lane has one frequency, so a warp reads a token's 16
+  // consecutive frequencies in one 128-byte request.  Angles in double.
   for (int i = threadIdx.x; i < half; i += 256) {
     const double ang = (double)pos * exp(-log_base * (double)i / (double)half);  // pos * base^(-2i/d)
-    cs[(size_t)i * n_tok + t] = make_float2((float)cos(ang), (float)sin(ang));
+    cs[(size_t)t * half + i] = make_float2((float)cos(ang), (float)sin(ang));
   }
   const float tot = row_sum(sq);
   const float rstd = ss ? 1.f : rsqrtf(tot / hidden + eps);

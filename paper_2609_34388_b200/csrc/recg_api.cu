@@ -528,15 +528,15 @@ static recg_status run_forward(recg_ctx* ctx, void* kv_pool, int64_t kv_pool_pag
   const BatchLayout& bl = ctx->bl;
   const int T = bl.n_tok;
   cudaStream_t st = ctx->stream;
-  // RMSNorm runs as a kernel of its own, or (RECG_FLAG_FOLD_NORM, tcgen05 path only) folded into the projections:
-  // whoever writes the residual stream also writes x = bf16(h * gain of the next norm) and partial sums of squares per
-  // row, and the projection that reads x scales its accumulator rows by the row's rstd.
+  // RMSNorm is folded into the projections of the tcgen05 path: whoever writes the residual stream also writes x =
+  // bf16(h * gain of the next norm) and partial sums of squares per row, and the projection that reads x scales its
+  // accumulator rows by the row's rstd.  (The mma.sync projections of RECG_FLAG_SIMT_GEMM run it as a kernel of its own.)
   // (RECG_FLAG_CHAIN: steps of at most 128 rows run the projections between two attention calls as one persistent kernel)
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   const bool chain = ctx->chain_state && !bl.dyn && T <= 128 && d.n_layers > 0 && (d.n_q * d.head_dim) % 64 == 0 &&
                      d.hidden % 128 == 0 && d.ffn % 64 == 0 &&
                      cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
-  const bool fold = ((ctx->cfg.flags & RECG_FLAG_FOLD_NORM) || chain) && !(ctx->cfg.flags & RECG_FLAG_SIMT_GEMM);
+  const bool fold = ctx->tc_state && !(ctx->cfg.flags & RECG_FLAG_SIMT_GEMM);
   const int Tm = ctx->cfg.max_tokens;
   const void* first_gain = d.n_layers > 0 ? ctx->attn_norm[0] : ctx->final_norm;
   launch_embed(bl, d, ctx->embed, ctx->h, first_gain, ctx->x, fold ? ctx->ss : nullptr, ctx->rope_cs, st);
