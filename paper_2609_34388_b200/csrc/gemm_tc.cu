@@ -14,7 +14,10 @@
 //            then the fused epilogue straight from registers (residual add with the next norm's input, SwiGLU, rotary +
 //            paged KV append, or plain store) while the MMA warp already fills the other accumulator.  One warp per
 //            scheduler runs it, so what counts is its instructions: the 16x256b form of tcgen05.ld hands out 8 x 8 fragments,
-//            stmatrix.trans turns them into rows of tokens, and stores are whole 32-byte sectors.
+//            stmatrix.trans turns them into rows of tokens, and stores are whole 32-byte sectors.  32 tokens take .6 us to
+//            1 us, and 3.5 us more when the code is not in the SM's instruction cache, which is so for the projections
+//            behind an attention kernel: all ways of finishing a tile share one instance of it, and the warps run it once
+//            without effect while they wait for the kernels in front of this one.
 // Operands of an epilogue that belong together sit in the same thread: the tensor map over w lists its rows 16 by 16 in the
 // order the tile wants them (16 gate rows, their 16 up rows, ...; 16 low dims of a head, their 16 rotation partners, ...), and
 // a thread holds the same row of both halves of a 32-row quadrant.
@@ -174,54 +177,30 @@ __device__ __forceinline__ void tmem_ld_chunk(uint32_t taddr, float (&v)[32]) { 
 #pragma unroll
   for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
+__device__ __forceinline__ float4 ld_volatile_f4(const float4* p) {   // generic address: shared or global memory
+  float4 t;
+  asm volatile("ld.volatile.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(t.x), "=f"(t.y), "=f"(t.z), "=f"(t.w) : "l"(p) : "memory");
+  return t;
+}
 // Partial tiles hold the values as the threads hold them, [chunk][8][128 threads][4] fp32: a warp's access is 512 contiguous
 // bytes.  Parts are added in part order starting from zero, so the result does not depend on who arrived last.
-struct TmemLoader {
-  uint32_t tacc;   // TMEM address of (lane quadrant, column 0)
-  __device__ __forceinline__ void operator()(int c, float (&v)[32]) const { tmem_ld_chunk(tacc + c * 32, v); }
-};
-struct SplitLoader {
-  const float4* ws;       // partial-tile workspace + this thread
-  int part_f4;            // float4 x 128 threads per part (8 per chunk)
-  int slot0;              // slot of part 0
-  int slot_next;          // slot of part 1; part p >= 1 is in slot_next + slot_stride (p - 1)
-  int slot_stride;
-  int n_parts;
-  __device__ __forceinline__ void operator()(int c, float (&v)[32]) const {
-#pragma unroll
-    for (int i = 0; i < 32; ++i) v[i] = 0.f;
-    // the loads of two parts are issued together so that their latencies overlap
-    for (int p = 0; p < n_parts; p += 2) {
-      const int sa = p == 0 ? slot0 : slot_next + slot_stride * (p - 1);
-      const bool two = p + 1 < n_parts;
-      const int sb = slot_next + slot_stride * p;   // slot of part p + 1 (>= 1)
-      float4 a[8], b[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        a[i] = __ldcg(ws + ((size_t)sa * part_f4 + c * 8 + i) * FT);
-        b[i] = two ? __ldcg(ws + ((size_t)sb * part_f4 + c * 8 + i) * FT) : make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        v[4 * i] += a[i].x; v[4 * i + 1] += a[i].y; v[4 * i + 2] += a[i].z; v[4 * i + 3] += a[i].w;
-        v[4 * i] += b[i].x; v[4 * i + 1] += b[i].y; v[4 * i + 2] += b[i].z; v[4 * i + 3] += b[i].w;
-      }
+struct Source {
+  uint32_t tacc;          // TMEM address of (lane quadrant, column 0): the only part, or part `own`
+  int n_parts, own;
+  bool cluster;           // the copies are of this member's chunks only, the parts of a chunk one after the other
+  const float4* first;    // part 0 where it lies apart from the others (workspace), else null
+  const float4* rest;     // the other parts (+ this thread): from part 1 on if `first`, else without part `own`
+  size_t stride;          // from one part to the next
+  // chunk c, the nth one that this CTA finishes
+  __device__ __forceinline__ void load(int c, int nth, float (&v)[32]) const {
+    if (n_parts == 1) {
+      tmem_ld_chunk(tacc + c * 32, v);
+      return;
     }
-  }
-};
-// The finishing CTA's own part comes from its TMEM accumulator, the other parts from copies in shared memory (the idle operand
-// ring or a reserve at its top), one part after the other in part order without the own one.  Every lane takes part (the TMEM
-// load is a warp-wide instruction).
-struct RingLoader {
-  uint32_t tacc;
-  const float4* ring;     // + this thread
-  int part_f4;            // float4 x 128 threads per part
-  int own, n_parts;
-  int c_off;              // token chunk the copies begin with
-  __device__ __forceinline__ void operator()(int c, float (&v)[32]) const {
 #pragma unroll
     for (int i = 0; i < 32; ++i) v[i] = 0.f;
-    int k = 0;
+    const size_t at = (size_t)(cluster ? nth * (n_parts - 1) : c) * (kChunkBytes / 16);
+#pragma unroll 1
     for (int p = 0; p < n_parts; ++p) {
       if (p == own) {
         float t[32];
@@ -229,12 +208,13 @@ struct RingLoader {
 #pragma unroll
         for (int i = 0; i < 32; ++i) v[i] += t[i];
       } else {
-        const float4* src = ring + ((size_t)k * part_f4 + (c - c_off) * 8) * FT;
-        ++k;
+        const float4* q = (first && p == 0 ? first : rest + (size_t)(p - ((first || p > own) ? 1 : 0)) * stride) + at;
+        float4 t[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) t[i] = ld_volatile_f4(q + (size_t)i * FT);
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-          const float4 a = src[(size_t)i * FT];
-          v[4 * i] += a.x; v[4 * i + 1] += a.y; v[4 * i + 2] += a.z; v[4 * i + 3] += a.w;
+          v[4 * i] += t[i].x; v[4 * i + 1] += t[i].y; v[4 * i + 2] += t[i].z; v[4 * i + 3] += t[i].w;
         }
       }
     }
@@ -259,18 +239,17 @@ __host__ __device__ inline void token_tiles(int M, int tmax, int gran, int* widt
 // slot, 2 * unit + (first piece ? 0 : 1).
 // All but the last one-to-two waves stay whole tiles (dp_tiles of them, done after the cut ones).  Computed on the host, or in
 // the kernel when the row count (hence mt) is only known on the device.  Needs mt <= n_units.
-__host__ __device__ inline void stream_k_schedule(int n_tiles, int mt, int KB, int n_units, int* dp_tiles, long long* per,
-                                                  int* used_units) {
+__host__ __device__ inline void stream_k_schedule(int n_tiles, int mt, int KB, int n_units, int* dp_tiles, int* per, int* used_units) {
   const int n_teams = n_units / mt;
   const int full = n_tiles / n_units;
   *dp_tiles = full >= 2 ? ((full - 1) * n_units / mt) * mt : 0;
-  const long long total = (long long)((n_tiles - *dp_tiles) / mt) * KB;
-  const long long teams = total < n_teams ? total : n_teams;
-  long long p = teams > 0 ? (total + teams - 1) / teams : 1;
+  const int total = (n_tiles - *dp_tiles) / mt * KB;       // (launch_gemm_tc keeps the line within int)
+  const int teams = total < n_teams ? total : n_teams;
+  int p = teams > 0 ? (total + teams - 1) / teams : 1;
   if (p < 4 && total >= 4) p = 4;                     // keep pieces long enough to amortise their hand-over
   if (p < 1) p = 1;
   *per = p;
-  const int used = (int)((total + p - 1) / p);        // teams that get a range
+  const int used = (total + p - 1) / p;               // teams that get a range
   *used_units = *dp_tiles ? n_units : used * mt;      // (with whole tiles behind, the grid stays at full size)
 }
 
@@ -283,8 +262,8 @@ struct Piece {
 // Next piece of this unit: first its range of the stream-K line (pos advances by reference), then its whole tiles
 // (jd counts them).  The cut tiles come first so that parking and reducing their partials overlaps the main loop
 // of the whole tiles that follow, instead of happening in every CTA at once at the end of the kernel.
-__device__ __forceinline__ Piece make_piece(int& jd, int dp_tiles, long long& pos, long long hi, int KB,
-                                            long long per, int unit, int n_units, int mt) {
+__device__ __forceinline__ Piece make_piece(int& jd, int dp_tiles, int& pos, int hi, int KB, int per, int unit, int n_units,
+                                            int mt) {
   Piece p;
   if (pos >= hi) {
     p.tile = unit + jd * n_units;
@@ -297,17 +276,17 @@ __device__ __forceinline__ Piece make_piece(int& jd, int dp_tiles, long long& po
     return p;
   }
   const int team = unit / mt, member = unit % mt;
-  const int col = (int)(pos / KB);
-  p.kb0 = (int)(pos - (long long)col * KB);
-  const long long room = hi - pos;
-  p.kb1 = (int)(room < KB - p.kb0 ? p.kb0 + room : KB);
-  const long long t0 = (long long)col * KB, t1 = t0 + KB;
-  const int c_first = (int)(t0 / per), c_last = (int)((t1 - 1) / per);    // first and last team on this column
+  const int col = pos / KB;
+  p.kb0 = pos - col * KB;
+  const int room = hi - pos;
+  p.kb1 = room < KB - p.kb0 ? p.kb0 + room : KB;
+  const int t0 = col * KB, t1 = t0 + KB;
+  const int c_first = t0 / per, c_last = (t1 - 1) / per;    // first and last team on this column
   p.n_parts = c_last - c_first + 1;
   p.part = team - c_first;
-  const bool first_piece = pos == (long long)team * per;
+  const bool first_piece = pos == team * per;
   p.slot = 2 * unit + (first_piece ? 0 : 1);
-  p.slot0 = 2 * (c_first * mt + member) + (((long long)c_first * per >= t0) ? 0 : 1);
+  p.slot0 = 2 * (c_first * mt + member) + (c_first * per >= t0 ? 0 : 1);
   p.slot_next = 2 * ((c_first + 1) * mt + member);
   p.tile = dp_tiles + col * mt + member;
   pos += p.kb1 - p.kb0;
@@ -326,7 +305,14 @@ struct TileOut {
 };
 // What the epilogue of a chunk reads besides the accumulator: the old residual values (index as the accumulator's), or the
 // rotary factors: (cos, sin) of (q = 0 / 1, k, e) at 2 vidx(q, k, e).  Fetched ahead: for the first chunk while the accumulator is
-// still being computed.
+// still being computed, like the next norm's gains of the thread's four features.
+__device__ __forceinline__ void load_gain(const EpiParams& ep, int tile, int quad, int lane, float (&gain)[4]) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int f = tile * FT + quad * 32 + (lane >> 2) + 8 * q;
+    gain[q] = ep.epi == EPI_RESIDUAL_NORM && f < ep.N ? __bfloat162float(ep.gain[f]) : 0.f;
+  }
+}
 __device__ __forceinline__ void prefetch_chunk(const EpiParams& ep, const TileOut& o, int c, float (&pre)[32]) {
   const int rg = o.lane >> 2, tok = c * 32 + 2 * (o.lane & 3), nv = o.nv;
   if (ep.epi == EPI_RESIDUAL || ep.epi == EPI_RESIDUAL_NORM) {
@@ -383,10 +369,10 @@ __device__ __forceinline__ void unstage_rows32(const TileOut& o, int nv, const P
     if (t < nv) put(t, p, w);
   }
 }
-// Epilogue of token chunks [c0, c1) (32 tokens each) of an accumulator tile; all 32 lanes of the warp call together.
-// pre: what prefetch_chunk brings for chunk c0.
-template <typename Loader>
-__device__ __forceinline__ void tile_out(const EpiParams& ep, const Loader& load, const TileOut& o, int c0, int c1, float (&pre)[32]) {
+// Epilogue of the token chunks c0, c0 + step, ... < c1 (32 tokens each) of an accumulator tile; the four epilogue warps call
+// together.  pre: what prefetch_chunk brings for chunk c0.
+__device__ __forceinline__ void tile_out(const EpiParams& ep, const Source& src, const TileOut& o, int c0, int c1, int step,
+                                         float (&pre)[32], const float (&gain)[4]) {
   const int lane = o.lane, rg = lane >> 2, tq = lane & 3;
   const int f0 = o.tile * FT + o.quad * 32;    // first feature of the warp (not of SwiGLU and the rotary epilogue)
   auto scale = [&](int c, float (&v)[32]) {    // the row factors of a normalised input
@@ -405,18 +391,12 @@ __device__ __forceinline__ void tile_out(const EpiParams& ep, const Loader& load
     // every element has one writer, so the residual add is a load (ahead of the accumulator) and a store; the new value also
     // gives the next norm's input x = bf16(h * gain) and the row's sum of squares over this tile's features
     const bool norm = ep.epi == EPI_RESIDUAL_NORM;
-    float gain[4] = {0.f, 0.f, 0.f, 0.f};
-    if (norm) {
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-        if (f0 + rg + 8 * q < ep.N) gain[q] = __bfloat162float(ep.gain[f0 + rg + 8 * q]);
-    }
 #pragma unroll 1
-    for (int c = c0; c < c1; ++c) {
+    for (int c = c0, nth = 0; c < c1; c += step, ++nth) {
       const int nv = o.nv - c * 32;
       float* h = static_cast<float*>(ep.out) + (size_t)(o.t0 + c * 32 + 2 * tq) * ep.N + f0 + rg;
       float v[32], sq[8];
-      load(c, v);
+      src.load(c, nth, v);
 #pragma unroll
       for (int k = 0; k < 4; ++k)
 #pragma unroll
@@ -433,7 +413,7 @@ __device__ __forceinline__ void tile_out(const EpiParams& ep, const Loader& load
           }
           sq[2 * k + e] = s;
         }
-      if (c + 1 < c1) prefetch_chunk(ep, o, c + 1, pre);
+      if (c + step < c1) prefetch_chunk(ep, o, c + step, pre);
       if (!norm) continue;
       stage_rows32(o, v);
       __nv_bfloat16* xp = ep.x_out + (size_t)(o.t0 + c * 32) * ep.N + f0;
@@ -455,7 +435,7 @@ __device__ __forceinline__ void tile_out(const EpiParams& ep, const Loader& load
     }
     if (norm) {
       asm volatile("bar.sync 1, 128;" ::: "memory");
-      for (int t = c0 * 32 + o.quad * 32 + lane; t < o.nv && t < c1 * 32; t += 128)
+      for (int t = (c0 + o.quad * step) * 32 + lane; t < o.nv; t += 128 * step)       // warp w sums the chunks c0 + w step, ...
         ep.ss_out[(size_t)o.tile * ep.ss_stride + o.t0 + t] =
             (o.ss[t] + o.ss[kMaxTok + t]) + (o.ss[2 * kMaxTok + t] + o.ss[3 * kMaxTok + t]);
       asm volatile("bar.sync 1, 128;" ::: "memory");      // (the sums may be overwritten)
@@ -467,9 +447,9 @@ __device__ __forceinline__ void tile_out(const EpiParams& ep, const Loader& load
     const int fo = o.tile * (FT / 2) + o.quad * 16;
     __nv_bfloat16* out = static_cast<__nv_bfloat16*>(ep.out) + (size_t)o.t0 * ep.N + fo;
 #pragma unroll 1
-    for (int c = c0; c < c1; ++c) {
+    for (int c = c0, nth = 0; c < c1; c += step, ++nth) {
       float v[32];
-      load(c, v);
+      src.load(c, nth, v);
       scale(c, v);
 #pragma unroll
       for (int i = 0; i < 16; ++i) v[i] = silu_f(v[i]) * v[16 + i];
@@ -501,9 +481,9 @@ __device__ __forceinline__ void tile_out(const EpiParams& ep, const Loader& load
     __nv_bfloat16* layer = ep.kv_pool + kv_tile_base(ep.n_pages, ep.n_kv, D, ep.layer, 0, is_q ? 0 : kvh) + (is_v ? kv_tile_elems(D) : 0);
     const size_t page_elems = kv_tile_base(ep.n_pages, ep.n_kv, D, 0, 1, 0);
 #pragma unroll 1
-    for (int c = c0; c < c1; ++c) {
+    for (int c = c0, nth = 0; c < c1; c += step, ++nth) {
       float v[32];
-      load(c, v);
+      src.load(c, nth, v);
       scale(c, v);
       if (!is_v) {
 #pragma unroll
@@ -512,7 +492,7 @@ __device__ __forceinline__ void tile_out(const EpiParams& ep, const Loader& load
           v[i] = lo * pre[2 * i] - hi * pre[2 * i + 1];
           v[16 + i] = hi * pre[2 * i] + lo * pre[2 * i + 1];
         }
-        if (c + 1 < c1) prefetch_chunk(ep, o, c + 1, pre);
+        if (c + step < c1) prefetch_chunk(ep, o, c + step, pre);
       }
       stage_rows32(o, v);
       unstage_rows32(o, o.nv - c * 32, [&](int t, int p, const uint4& w) {
@@ -535,10 +515,10 @@ __device__ __forceinline__ void tile_out(const EpiParams& ep, const Loader& load
     return;
   }
 #pragma unroll 1
-  for (int c = c0; c < c1; ++c) {
+  for (int c = c0, nth = 0; c < c1; c += step, ++nth) {
     const int nv = o.nv - c * 32;
     float v[32];
-    load(c, v);
+    src.load(c, nth, v);
     scale(c, v);
     if (ep.epi == EPI_PLAIN_BF16) {
       stage_rows32(o, v);
@@ -564,8 +544,9 @@ struct GemmLaunch {
   int n_cols;                // columns of tiles: feature tiles of 128, or of 256 for pairs
   int K;
   int tmax, gran, x_box;     // token tiles (token_tiles), rows of one x load
+  int width, mt;             // ... their width and number, where the row count is known
   int dp_tiles;              // >= 0: the host's schedule; -1: whole tiles only; -2: stream-K, divided here from the device's row count
-  long long per;
+  int per;
   int cl;                    // parts per tile that form a cluster (0: no clusters)
   int w_step3, w_step4;      // what a 128-feature tile advances in dimensions 3 and 4 of w's tensor map
   float* split_ws;
@@ -600,12 +581,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
 
-  int nt_tok, mt;              // tokens per tile, token tiles
-  token_tiles(M, G.tmax, G.gran, &nt_tok, &mt);
+  int nt_tok = G.width, mt = G.mt;                        // tokens per tile, token tiles
+  if (G.m_dev) token_tiles(M, G.tmax, G.gran, &nt_tok, &mt);
   const int x_rows = nt_tok / kMul;                       // rows of x this CTA loads per k-block
   const int stage_bytes = kABytes + x_rows * BK * 2;
-  const int part_f4 = (nt_tok + 31) / 32 * 8;             // a partial tile: float4 x 128 threads
-  const int part_bytes = part_f4 * FT * 16;
+  const int part_bytes = (nt_tok + 31) / 32 * kChunkBytes;   // a partial tile
   // Clusters: chunk c of the tile (32 tokens) is finished by member c % cl, into whose shared memory the others write their
   // partial sums of it (16 KB each).  A tile of one chunk has a reserve for them at the top of the ring; else they go into the
   // ring itself, once its owner says that its own products have read it.
@@ -658,7 +638,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
   const int n_tiles = mt * G.n_cols;
   const int KB = G.K / BK;
   int dp_tiles = G.dp_tiles < 0 ? n_tiles : G.dp_tiles;
-  long long per = G.per;
+  int per = G.per;
   if (G.dp_tiles == -2) {
     if (mt >= 1 && mt <= n_units) {
       int used;
@@ -669,19 +649,19 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
   }
   // schedule: the k-blocks of tiles [dp_tiles, n_tiles) as one line cut into equal ranges per unit; then tiles
   // [0, dp_tiles) whole, strided over the grid (CTAs that run together share a weight tile through L2)
-  const long long total = (long long)((n_tiles - dp_tiles) / mt) * KB;
-  const long long lo_raw = (long long)(unit / mt) * per;
+  const int total = (n_tiles - dp_tiles) / mt * KB;
+  const int lo_raw = unit / mt * per;
   const bool cl_live = cl && unit / cl < n_tiles;          // (the grid of a device-resident step is sized for the capacity)
-  const long long range_lo = cl ? 0 : (lo_raw < total ? lo_raw : total);
-  const long long range_hi = cl ? (cl_live ? 1 : 0) : (range_lo + per < total ? range_lo + per : total);
+  const int range_lo = cl ? 0 : (lo_raw < total ? lo_raw : total);
+  const int range_hi = cl ? (cl_live ? 1 : 0) : (range_lo + per < total ? range_lo + per : total);
   const int dp_count = cl ? 0 : (unit < dp_tiles ? (dp_tiles - 1 - unit) / n_units + 1 : 0);
   // the next piece of this unit (a cluster member has exactly one)
-  auto next_piece = [&](int& jd, long long& pos) -> Piece {
+  auto next_piece = [&](int& jd, int& pos) -> Piece {
     if (cl) {
       Piece p;
       p.tile = unit / cl;
-      p.kb0 = (int)((long long)part_rank * KB / cl);
-      p.kb1 = (int)((long long)(part_rank + 1) * KB / cl);
+      p.kb0 = (int)part_rank * KB / cl;
+      p.kb1 = ((int)part_rank + 1) * KB / cl;
       p.part = (int)part_rank;
       p.n_parts = cl;
       p.slot = p.slot0 = p.slot_next = 0;
@@ -754,7 +734,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
       // those stages follow right after the wait.
       int n_pre = 0, pre_kb0 = 0, pre_tm = 0;
       if (dp_count > 0 || range_lo < range_hi) {
-        long long p0 = range_lo;
+        int p0 = range_lo;
         int j0 = 0;
         const Piece pc = next_piece(j0, p0);
         n_pre = pc.kb1 - pc.kb0 < n_stages ? pc.kb1 - pc.kb0 : n_stages;
@@ -770,7 +750,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
       int st_idx = 0, issued = 0;
       uint32_t st_phase = 0;
       bool ok = true;
-      long long pos = range_lo;
+      int pos = range_lo;
       for (int jd = 0; (jd < dp_count || pos < range_hi) && ok;) {
         const Piece pc = next_piece(jd, pos);
         const int tm = pc.tile % mt, col = pc.tile / mt;
@@ -810,7 +790,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
       int st_idx = 0;
       uint32_t st_phase = 0, tcount = 0;
       bool ok = true;
-      long long pos = range_lo;
+      int pos = range_lo;
       for (int jd = 0; (jd < dp_count || pos < range_hi) && ok; ++tcount) {
         const Piece pc = next_piece(jd, pos);
         const int kb0 = pc.kb0, kb1 = pc.kb1;
@@ -854,42 +834,18 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
     // ------------------------------ epilogue warps ------------------------------
     const int quad = warp & 3;             // TMEM lane quadrant this warp may read
     const int row = quad * 32 + lane;      // this thread among the 128 of the epilogue
+    const uint32_t tmem_quad = tmem_base + ((uint32_t)(quad * 32) << 16);
     uint32_t tcount = 0;
     int prep_tm = -1;
     __shared__ int s_last;
-    griddep_wait();                        // the epilogue reads and writes what earlier kernels produced
-    long long pos = range_lo;
-    for (int jd = 0; jd < dp_count || pos < range_hi; ++tcount) {
-      const Piece pc = next_piece(jd, pos);
-      const int tile = pc.tile, n_splits = pc.n_parts;
-      const int tm = tile % mt, ft = (tile / mt) * kMul + (int)rank;
-      const int acc = tcount & 1;
-      TileOut o{ft, tm * nt_tok, 0, quad, lane, s_rstd, s_slot, s_ss, smem + kOffStage + quad * 2048};
-      o.nv = M - o.t0 < nt_tok ? M - o.t0 : nt_tok;
-      const int n_chunks = (o.nv + 31) / 32;
-      // What the epilogue needs per token, fetched while the accumulator is still being computed: the row factors of a
-      // normalised input (the partial sums of squares in slot order: the same bits in every tile of the row) and the slots.
-      if (tm != prep_tm && (ep.ss_in || ep.epi == EPI_QKV_ROPE)) {
-        if (prep_tm >= 0) asm volatile("bar.sync 1, 128;" ::: "memory");
-        for (int t = (int)threadIdx.x - 64; t < o.nv; t += 128) {
-          if (ep.ss_in) {
-            float sq = 0.f;
-            const float* p = ep.ss_in + o.t0 + t;
-#pragma unroll 8
-            for (int k = 0; k < ep.ss_slots; ++k) sq += __ldcg(p + (size_t)k * ep.ss_stride);
-            s_rstd[t] = rsqrtf(sq * ep.norm_inv_n + ep.norm_eps);
-          }
-          if (ep.epi == EPI_QKV_ROPE) s_slot[t] = ep.tok_slot[o.t0 + t];
-        }
-        asm volatile("bar.sync 1, 128;" ::: "memory");
-        prep_tm = tm;
-      }
-      // (likewise, where this CTA is sure to finish the tile, what its first tokens need)
-      float pre[32];
-      if (n_splits == 1 || (cl && (int)part_rank < n_chunks)) prefetch_chunk(ep, o, (int)part_rank, pre);
-      wait_or_abort(&tfull_bar[acc], (tcount >> 1) & 1, DEV_TIMEOUT_MMA);   // after a timeout: carry on without blocking
-      tc_fence_after();
-      const uint32_t tacc = tmem_base + ((uint32_t)(quad * 32) << 16) + acc * kAccStride;
+    TileOut o{0, 0, 0, quad, lane, s_rstd, s_slot, s_ss, smem + kOffStage + quad * 2048};
+    float pre[32], gain[4] = {0.f, 0.f, 0.f, 0.f};
+    int pos = range_lo;
+    bool dry = true;                       // first pass: the epilogue's code without effect (no token exists, values are arbitrary)
+    for (int jd = 0; jd < dp_count || pos < range_hi;) {
+      Source src{tmem_quad + kAccStride, 1, 0, false, nullptr, nullptr, 0};
+      int c_begin = 0, c_end = 1, c_step = 1;     // the chunks that are finished here
+      int acc = 0;
       // hands the accumulator back to the MMA issuer (of a pair: the leader's barrier collects both CTAs' warps)
       auto release_acc = [&]() {
         tc_fence_before();
@@ -899,102 +855,155 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
           else mbar_arrive(&tempty_bar[acc]);
         }
       };
-      if (n_splits == 1) {
-        tile_out(ep, TmemLoader{tacc}, o, 0, n_chunks, pre);
-        release_acc();
-      } else if (cl) {
-        uint8_t* land = smem + (reserve ? ring_bytes : 0);
-        if (!reserve) {            // this CTA's products are complete and have read its ring (its accumulator is)
-          asm volatile("bar.sync 1, 128;" ::: "memory");
-          if (warp == 2 && lane < cl && lane != (int)part_rank) mbar_arrive_cluster(mapa_rank(smem_u32(go_bar), lane * kMul + rank));
-          wait_or_abort(go_bar, 0, DEV_TIMEOUT_EMPTY, true);
+      bool release = false, last_sync = false;
+      if (dry) {
+        if (cl) {
+          src.n_parts = cl;
+          src.own = (int)part_rank;
+          src.rest = reinterpret_cast<const float4*>(smem) + row;
+          src.stride = kChunkBytes / 16;
         }
-#pragma unroll 1
-        for (int c = 0; c < n_chunks; ++c) {
-          const int owner = c % cl;
-          if (owner == (int)part_rank) continue;
-          const int at = (c / cl) * (cl - 1) + ((int)part_rank < owner ? (int)part_rank : (int)part_rank - 1);
-          const uint32_t dst = mapa_rank(smem_u32(land + at * kChunkBytes), owner * kMul + rank) + row * 16;
-          float v[32];
-          tmem_ld_chunk(tacc + c * 32, v);
-#pragma unroll
-          for (int i = 0; i < 8; ++i)
-            st_cluster_f4(dst + (uint32_t)i * (FT * 16), make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]));
-        }
-        __syncwarp();
-        if (lane < cl && lane != (int)part_rank && lane < n_chunks)    // release: the warp's stores are visible
-          mbar_arrive_cluster(mapa_rank(smem_u32(red_bar), lane * kMul + rank));
-        if ((int)part_rank < n_chunks) {
-          wait_or_abort(red_bar, 0, DEV_TIMEOUT_FULL, true);           // the others' parts have landed (acquire at cluster scope)
-#pragma unroll 1
-          for (int c = (int)part_rank; c < n_chunks; c += cl) {
-            RingLoader ld{tacc, reinterpret_cast<const float4*>(land + (c / cl) * (cl - 1) * kChunkBytes) + row, 8, (int)part_rank, cl, c};
-            if (c != (int)part_rank) prefetch_chunk(ep, o, c, pre);
-            tile_out(ep, ld, o, c, c + 1, pre);
-          }
-        }
-        release_acc();
       } else {
-        // park this split's partial tile and let the LAST split to arrive reduce all partials in split order
-        // (deterministic) and run the fused epilogue
-        // (the two CTAs of a pair park and reduce their 128 features independently: slot and counter index are
-        // doubled and offset by the rank)
-        const int slot_mine = pc.slot * kMul + (int)rank, slot0 = pc.slot0 * kMul + (int)rank;
-        const int slot_next = pc.slot_next * kMul + (int)rank, slot_stride = 2 * mt * kMul;
-        const int counter = tile * kMul + (int)rank;
-        float4* mine = reinterpret_cast<float4*>(G.split_ws) + (size_t)slot_mine * part_f4 * FT + row;
-#pragma unroll 1
-        for (int c = 0; c < n_chunks; ++c) {
-          float v[32];
-          tmem_ld_chunk(tacc + c * 32, v);
-#pragma unroll
-          for (int i = 0; i < 8; ++i)
-            __stcg(mine + (size_t)(c * 8 + i) * FT, make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]));
-        }
-        // the accumulator may be handed back at once: the own part is read from TMEM again only when nothing follows
-        // in this CTA, and then nobody overwrites it
-        release_acc();
-        asm volatile("bar.sync 1, 128;" ::: "memory");
-        if (warp == 2 && lane == 0) {
-          __threadfence();   // cumulative: orders the partial rows all 128 threads wrote before the barrier
-          const int old = atomicAdd(&G.split_counters[counter], 1);
-          s_last = (old == n_splits - 1);
-          if (old == n_splits - 1) G.split_counters[counter] = 0;   // ready for the next launch
-          __threadfence();
-        }
-        asm volatile("bar.sync 1, 128;" ::: "memory");
-        if (s_last) {
-          prefetch_chunk(ep, o, 0, pre);
-          // When nothing follows in this CTA the operand ring is idle (every load was consumed before the accumulator
-          // completed): the other parts are fetched into it with bulk copies at full bandwidth and the own part is
-          // taken from TMEM.  Otherwise the parts are read from global memory while the next piece's main loop runs.
-          const bool final_piece = !(jd < dp_count || pos < range_hi);
-          if (final_piece && (n_splits - 1) * part_bytes <= kRingBytes) {
-            if (warp == 2 && lane == 0) {
-              asm volatile("fence.proxy.async;" ::: "memory");   // the parts were written with ordinary stores
-              mbar_arrive_expect_tx(red_bar, (uint32_t)((n_splits - 1) * part_bytes));
-              int k = 0;
-              for (int p = 0; p < n_splits; ++p) {
-                if (p == pc.part) continue;
-                const int slot = p == 0 ? slot0 : slot_next + slot_stride * (p - 1);
-                const uint8_t* src = reinterpret_cast<const uint8_t*>(G.split_ws) + (size_t)slot * part_bytes;
-                for (int off = 0; off < part_bytes; off += 16384) {
-                  const int n = part_bytes - off < 16384 ? part_bytes - off : 16384;
-                  bulk_g2s(smem + (size_t)k * part_bytes + off, src + off, n, red_bar);
-                }
-                ++k;
-              }
+        const Piece pc = next_piece(jd, pos);
+        const int tile = pc.tile, n_splits = pc.n_parts;
+        const int tm = tile % mt;
+        o.tile = (tile / mt) * kMul + (int)rank;
+        o.t0 = tm * nt_tok;
+        o.nv = M - o.t0 < nt_tok ? M - o.t0 : nt_tok;
+        acc = tcount & 1;
+        src.tacc = tmem_quad + acc * kAccStride;
+        const int n_chunks = (o.nv + 31) / 32;
+        // What the epilogue needs per token, fetched while the accumulator is still being computed: the row factors of a
+        // normalised input (the partial sums of squares in slot order: the same bits in every tile of the row) and the slots.
+        if (tm != prep_tm && (ep.ss_in || ep.epi == EPI_QKV_ROPE)) {
+          if (prep_tm >= 0) asm volatile("bar.sync 1, 128;" ::: "memory");
+          for (int t = (int)threadIdx.x - 64; t < o.nv; t += 128) {
+            if (ep.ss_in) {
+              float sq = 0.f;
+              const float* p = ep.ss_in + o.t0 + t;
+#pragma unroll 8
+              for (int k = 0; k < ep.ss_slots; ++k) sq += __ldcg(p + (size_t)k * ep.ss_stride);
+              s_rstd[t] = rsqrtf(sq * ep.norm_inv_n + ep.norm_eps);
             }
-            wait_or_abort(red_bar, 0, DEV_TIMEOUT_FULL);
-            RingLoader ld{tacc, reinterpret_cast<const float4*>(smem) + row, part_f4, pc.part, n_splits, 0};
-            tile_out(ep, ld, o, 0, n_chunks, pre);
+            if (ep.epi == EPI_QKV_ROPE) s_slot[t] = ep.tok_slot[o.t0 + t];
+          }
+          asm volatile("bar.sync 1, 128;" ::: "memory");
+          prep_tm = tm;
+        }
+        c_end = n_chunks;
+        if (cl) {
+          c_begin = (int)part_rank;
+          c_step = cl;
+        }
+        // (likewise, where this CTA is sure to finish the tile, what its first tokens need)
+        load_gain(ep, o.tile, quad, lane, gain);
+        if ((n_splits == 1 || cl) && c_begin < c_end) prefetch_chunk(ep, o, c_begin, pre);
+        wait_or_abort(&tfull_bar[acc], (tcount >> 1) & 1, DEV_TIMEOUT_MMA);   // after a timeout: carry on without blocking
+        tc_fence_after();
+        ++tcount;
+        if (n_splits == 1) {
+          release = true;
+        } else if (cl) {
+          uint8_t* land = smem + (reserve ? ring_bytes : 0);
+          if (!reserve) {            // this CTA's products are complete and have read its ring (its accumulator is)
+            asm volatile("bar.sync 1, 128;" ::: "memory");
+            if (warp == 2 && lane < cl && lane != (int)part_rank) mbar_arrive_cluster(mapa_rank(smem_u32(go_bar), lane * kMul + rank));
+            wait_or_abort(go_bar, 0, DEV_TIMEOUT_EMPTY, true);
+          }
+#pragma unroll 1
+          for (int c = 0; c < n_chunks; ++c) {
+            const int owner = c % cl;
+            if (owner == (int)part_rank) continue;
+            const int at = (c / cl) * (cl - 1) + ((int)part_rank < owner ? (int)part_rank : (int)part_rank - 1);
+            const uint32_t dst = mapa_rank(smem_u32(land + at * kChunkBytes), owner * kMul + rank) + row * 16;
+            float v[32];
+            tmem_ld_chunk(src.tacc + c * 32, v);
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+              st_cluster_f4(dst + (uint32_t)i * (FT * 16), make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]));
+          }
+          __syncwarp();
+          if (lane < cl && lane != (int)part_rank && lane < n_chunks)    // release: the warp's stores are visible
+            mbar_arrive_cluster(mapa_rank(smem_u32(red_bar), lane * kMul + rank));
+          if (c_begin < c_end) wait_or_abort(red_bar, 0, DEV_TIMEOUT_FULL, true);  // the others' parts have landed (acquire at cluster scope)
+          src.n_parts = cl;
+          src.own = (int)part_rank;
+          src.cluster = true;
+          src.rest = reinterpret_cast<const float4*>(land) + row;
+          src.stride = kChunkBytes / 16;
+          release = true;
+        } else {
+          // park this split's partial tile and let the LAST split to arrive reduce all partials in split order
+          // (deterministic) and run the fused epilogue
+          // (the two CTAs of a pair park and reduce their 128 features independently: slot and counter index are
+          // doubled and offset by the rank)
+          const int slot_mine = pc.slot * kMul + (int)rank, slot0 = pc.slot0 * kMul + (int)rank;
+          const int slot_next = pc.slot_next * kMul + (int)rank, slot_stride = 2 * mt * kMul;
+          const int counter = tile * kMul + (int)rank;
+          const size_t part_f4 = part_bytes / 16;
+          float4* mine = reinterpret_cast<float4*>(G.split_ws) + slot_mine * part_f4 + row;
+#pragma unroll 1
+          for (int c = 0; c < n_chunks; ++c) {
+            float v[32];
+            tmem_ld_chunk(src.tacc + c * 32, v);
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+              __stcg(mine + (size_t)(c * 8 + i) * FT, make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]));
+          }
+          // the accumulator may be handed back at once: the own part is read from TMEM again only when nothing follows
+          // in this CTA, and then nobody overwrites it
+          release_acc();
+          asm volatile("bar.sync 1, 128;" ::: "memory");
+          if (warp == 2 && lane == 0) {
+            __threadfence();   // cumulative: orders the partial rows all 128 threads wrote before the barrier
+            const int old = atomicAdd(&G.split_counters[counter], 1);
+            s_last = (old == n_splits - 1);
+            if (old == n_splits - 1) G.split_counters[counter] = 0;   // ready for the next launch
+            __threadfence();
+          }
+          asm volatile("bar.sync 1, 128;" ::: "memory");
+          last_sync = true;
+          if (!s_last) {
+            c_end = 0;
           } else {
-            SplitLoader ld{reinterpret_cast<const float4*>(G.split_ws) + row, part_f4, slot0, slot_next, slot_stride, n_splits};
-            tile_out(ep, ld, o, 0, n_chunks, pre);
+            prefetch_chunk(ep, o, 0, pre);
+            src.n_parts = n_splits;
+            // When nothing follows in this CTA the operand ring is idle (every load was consumed before the accumulator
+            // completed): the other parts are fetched into it with bulk copies at full bandwidth and the own part is
+            // taken from TMEM.  Otherwise the parts are read from global memory while the next piece's main loop runs.
+            const bool final_piece = !(jd < dp_count || pos < range_hi);
+            if (final_piece && (n_splits - 1) * part_bytes <= kRingBytes) {
+              if (warp == 2 && lane == 0) {
+                asm volatile("fence.proxy.async;" ::: "memory");   // the parts were written with ordinary stores
+                mbar_arrive_expect_tx(red_bar, (uint32_t)((n_splits - 1) * part_bytes));
+                int k = 0;
+                for (int p = 0; p < n_splits; ++p) {
+                  if (p == pc.part) continue;
+                  const int slot = p == 0 ? slot0 : slot_next + slot_stride * (p - 1);
+                  const uint8_t* from = reinterpret_cast<const uint8_t*>(G.split_ws) + (size_t)slot * part_bytes;
+                  for (int off = 0; off < part_bytes; off += kChunkBytes)
+                    bulk_g2s(smem + (size_t)k * part_bytes + off, from + off, kChunkBytes, red_bar);
+                  ++k;
+                }
+              }
+              wait_or_abort(red_bar, 0, DEV_TIMEOUT_FULL);
+              src.own = pc.part;
+              src.rest = reinterpret_cast<const float4*>(smem) + row;
+              src.stride = part_f4;
+            } else {
+              src.own = -1;
+              src.first = reinterpret_cast<const float4*>(G.split_ws) + slot0 * part_f4 + row;
+              src.rest = reinterpret_cast<const float4*>(G.split_ws) + slot_next * part_f4 + row;
+              src.stride = slot_stride * part_f4;
+            }
           }
         }
-        asm volatile("bar.sync 1, 128;" ::: "memory");       // s_last is reused by the next unit
       }
+      if (c_begin < c_end) tile_out(ep, src, o, c_begin, c_end, c_step, pre, gain);
+      if (release) release_acc();
+      if (last_sync) asm volatile("bar.sync 1, 128;" ::: "memory");       // s_last is reused by the next unit
+      if (dry) griddep_wait();             // from here on the epilogue reads and writes what earlier kernels produced
+      dry = false;
     }
   }
 
@@ -1222,8 +1231,8 @@ bool launch_config(TcState* st, const GemmArgs& a, const EpiParams& ep, const Co
   // (with the row count on the device the width of the token tiles is, too: x is then loaded in boxes of 32 or 16 rows)
   g.gran = a.m_dev ? 32 : (c.pair ? 32 : 16);
   g.tmax = (c.tmax + g.gran - 1) / g.gran * g.gran;
-  int width, mt;
-  token_tiles(a.M, g.tmax, g.gran, &width, &mt);
+  token_tiles(a.M, g.tmax, g.gran, &g.width, &g.mt);
+  const int width = g.width, mt = g.mt;
   g.x_box = a.m_dev ? 32 / mul : width / mul;
   CUtensorMap mw, mx;     // copies: see cached_map
   const WeightOrder order = swiglu ? kWSwiglu : (a.epi == EPI_QKV_ROPE ? (a.head_dim == 128 ? kWRope128 : kWRope64) : kWPlain);
@@ -1362,6 +1371,7 @@ bool launch_gemm_tc(const GemmArgs& a, void* tc_state, int* status, cudaStream_t
   if ((reinterpret_cast<uintptr_t>(a.x) | reinterpret_cast<uintptr_t>(a.w)) & 15) return false;
   if (a.epi == EPI_RESIDUAL_NORM && (!a.x_out || !a.gain || !a.ss_out)) return false;
   if (a.epi == EPI_SWIGLU && a.N % 64) return false;
+  if (((int64_t)a.N * 2 / FT + 2) * (a.K / BK) > (1 << 30)) return false;      // the line of k-blocks is counted in int
   if (a.epi == EPI_QKV_ROPE && (a.N % 128 || (a.head_dim != 64 && a.head_dim != 128))) return false;
   EpiParams ep;
   ep.epi = a.epi;
