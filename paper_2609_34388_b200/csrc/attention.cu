@@ -449,7 +449,7 @@ __global__ void __launch_bounds__(512, 2) attention_combine_kernel(const AttnTil
 template <int D>
 void launch_attention_t(const BatchLayout& bl, const Dims& dm, int layer, const void* q, void* o, const void* kv_pool,
                         int64_t n_pages, float* part_o, float* part_ml, int tok_per_tile, int n_sm, int* status,
-                        cudaStream_t st) {
+                        cudaStream_t st, bool whole) {
   static bool configured[kMaxDevices] = {false};
   if (first_use_on_device(configured))
     cudaFuncSetAttribute(attention_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnSmem<D>::kTotal);
@@ -475,6 +475,7 @@ void launch_attention_t(const BatchLayout& bl, const Dims& dm, int layer, const 
   P.part_ml = part_ml;
   P.status = status;
   launch_pdl(attention_kernel<D>, dim3(n_sm), dim3(kAttnThreads), AttnSmem<D>::kTotal, st, P);
+  if (whole) return;
   launch_pdl(attention_combine_kernel<D>, dim3(4 * n_sm), dim3(512), 0, st, (const AttnTile*)bl.tiles, (const int*)bl.counts,
              dm.n_q, P.group, (const float*)part_o, (const float*)part_ml, static_cast<__nv_bfloat16*>(o), 0);
 }
@@ -487,18 +488,19 @@ size_t attention_smem_bytes(int head_dim) {
 
 void launch_attention(const BatchLayout& bl, const Dims& dm, int layer, const void* q, void* o, const void* kv_pool,
                       int64_t n_pages, float* part_o, float* part_ml, int tok_per_tile, int n_sm, int* status,
-                      cudaStream_t st, bool use_tc, bool layout_settled) {
+                      cudaStream_t st, bool use_tc, bool layout_settled, bool whole) {
   if (use_tc && dm.head_dim == 128) {
     launch_attention_tc_main(bl, dm, layer, q, o, kv_pool, n_pages, part_o, part_ml, n_sm, status, st, layout_settled);
+    if (whole) return;
     launch_pdl(attention_combine_kernel<128>, dim3(4 * n_sm), dim3(512), 0, st, (const AttnTile*)bl.tiles,
                (const int*)bl.counts, dm.n_q, dm.n_q / dm.n_kv, (const float*)part_o, (const float*)part_ml,
                static_cast<__nv_bfloat16*>(o), 1);    // (the kernel in front signals its dependents after its own wait)
     return;
   }
   if (dm.head_dim == 64)
-    launch_attention_t<64>(bl, dm, layer, q, o, kv_pool, n_pages, part_o, part_ml, tok_per_tile, n_sm, status, st);
+    launch_attention_t<64>(bl, dm, layer, q, o, kv_pool, n_pages, part_o, part_ml, tok_per_tile, n_sm, status, st, whole);
   else
-    launch_attention_t<128>(bl, dm, layer, q, o, kv_pool, n_pages, part_o, part_ml, tok_per_tile, n_sm, status, st);
+    launch_attention_t<128>(bl, dm, layer, q, o, kv_pool, n_pages, part_o, part_ml, tok_per_tile, n_sm, status, st, whole);
 }
 
 }  // namespace recg

@@ -59,8 +59,11 @@ struct BatchLayout {
 };
 
 // S1: per-token arrays and the attention work list (batches with a page table: a verify-only batch needs neither).
-void launch_layout(const BatchLayout& bl, const Dims& dm, int tok_per_tile, int n_ctas, int64_t n_pages,
+// whole: no tile is cut (attention_whole_tiles), and no combine kernel has to follow the attention kernel.
+void launch_layout(const BatchLayout& bl, const Dims& dm, int tok_per_tile, int n_ctas, bool whole, int64_t n_pages,
                    int* status, cudaStream_t st);
+// HOST arrays [n_req]; rows: rows per request
+bool attention_whole_tiles(int n_req, const int* ctx_len, const int* rows, int n_kv, int tok_per_tile, int n_ctas);
 // the layout kernel keeps six ints per request in shared memory: requests per step are bounded by this
 constexpr int kMaxLayoutRequests = 4096;
 size_t layout_smem_bytes(int n_req, int n_ctas);
@@ -189,9 +192,10 @@ bool launch_gemm_chain(void* s, const ChainOp* ops, int n_ops, int M, const Chai
 // use_tc: run the tcgen05 kernel (head_dim 128 only); otherwise the mma.sync kernel
 // layout_settled: the work list was written by a kernel that is known to have finished when this one starts (anything but
 // the launch right before it): the tcgen05 kernel then reads its work range before it waits for its predecessor
+// whole: the work list was laid out with whole tiles
 void launch_attention(const BatchLayout& bl, const Dims& dm, int layer, const void* q, void* o, const void* kv_pool,
                       int64_t n_pages, float* part_o, float* part_ml, int tok_per_tile, int n_sm, int* status,
-                      cudaStream_t st, bool use_tc, bool layout_settled = false);
+                      cudaStream_t st, bool use_tc, bool layout_settled, bool whole);
 void launch_attention_tc_main(const BatchLayout& bl, const Dims& dm, int layer, const void* q, void* o,
                               const void* kv_pool, int64_t n_pages, float* part_o, float* part_ml, int n_sm, int* status,
                               cudaStream_t st, bool layout_settled);

@@ -31,6 +31,8 @@ __device__ __forceinline__ int upper_request(const int* cu, int n_req, int t) {
 // The CTAs are divided between the two lines in proportion to their work (line A: the first 2 n_pairs_a CTAs), so
 // that every CTA walks ONE range and all carry about the same load.  Each piece that holds real blocks is an item;
 // a tile whose blocks are cut by range boundaries gets one partial slot per piece.
+// Small work lists are not cut at all (`whole`, decided on the host from the same lengths): every tile is one item of a CTA of
+// its own, and no combine kernel follows.
 // Items: [line A, first siblings | line A, second siblings (same order) | line B]; cta_off holds, per CTA, two
 // index ranges it walks one after the other (the second one is empty in this division).
 //
@@ -40,6 +42,7 @@ __device__ __forceinline__ int upper_request(const int* cu, int n_req, int t) {
 // 58 us for 8448 rows of 256 requests.
 constexpr int kItemCost = 4;
 constexpr int kLayoutThreads = 1024;
+constexpr int kWholeBlocks = 5;
 
 // exclusive prefix sums over the threads of the CTA, and the totals; `carry` scratch: 3 x 33 ints of shared memory
 struct Scan3 { int a, b, c; };
@@ -107,7 +110,7 @@ __device__ __forceinline__ void layout_tokens(const BatchLayout& bl, const int* 
 }
 
 __global__ void __launch_bounds__(kLayoutThreads) layout_kernel(BatchLayout bl, int n_kv, int mask_id, int tok_per_tile,
-                                                                int n_ctas, int64_t n_pages, int* status) {
+                                                                int n_ctas, int whole, int64_t n_pages, int* status) {
   extern __shared__ int sm[];
   const int C = bl.n_req;
   const int max_pairs = n_ctas / 2;
@@ -198,6 +201,7 @@ __global__ void __launch_bounds__(kLayoutThreads) layout_kernel(BatchLayout bl, 
   if (pairs_a > max_pairs) pairs_a = max_pairs;
   if (wb > 0 && n_ctas - 2 * pairs_a < 1) pairs_a = (n_ctas - 1) / 2;
   if (wa == 0) pairs_a = 0;
+  if (whole) pairs_a = n_seg_a;            // (2 n_seg_a + n_seg_b <= n_ctas)
   const int n_ctas_b = n_ctas - 2 * pairs_a;
   const int per_a = pairs_a > 0 && wa > 0 ? (int)((wa + pairs_a - 1) / pairs_a) : 0x3fffffff;
   const int per_b = n_ctas_b > 0 && wb > 0 ? (int)((wb + n_ctas_b - 1) / n_ctas_b) : 0x3fffffff;
@@ -221,7 +225,7 @@ __global__ void __launch_bounds__(kLayoutThreads) layout_kernel(BatchLayout bl, 
       const Scan3 e1 = block_scan(Scan3{s < n_seg ? g.nb + kItemCost : 0, 0, 0}, &tot, scratch);
       const int g0 = off + e1.a + kItemCost;              // cost range of the real blocks: [g0, g0 + nb)
       off += tot.a;
-      const int c_first = g0 / per, c_last = (g0 + g.nb - 1) / per;
+      const int c_first = whole ? s : g0 / per, c_last = whole ? s : (g0 + g.nb - 1) / per;
       const int np = s < n_seg ? c_last - c_first + 1 : 0;
       const Scan3 e2 = block_scan(Scan3{np, np > 1 ? (pair ? 2 * np : np) : 0, 0}, &tot, scratch);
       const int item0 = pieces + e2.a;
@@ -230,7 +234,7 @@ __global__ void __launch_bounds__(kLayoutThreads) layout_kernel(BatchLayout bl, 
       if (pass > 0) parts += tot.b;
       if (pass == 0 || s >= n_seg) continue;
       // first piece of every owner: an owner without pieces starts where the next one does
-      const int c_prev = s == 0 ? -1 : (g0 - kItemCost - 1) / per;     // owner of the last block of the segment before
+      const int c_prev = s == 0 || whole ? s - 1 : (g0 - kItemCost - 1) / per;     // owner of the last block of the segment before
       for (int c = c_prev + 1; c <= c_last && c <= n_owners; ++c) owner_off[c] = c <= c_first ? item0 : item0 + (c - c_first);
       if (s == n_seg - 1)
         for (int c = c_last + 1; c <= n_owners; ++c) owner_off[c] = item0 + np;
@@ -250,8 +254,8 @@ __global__ void __launch_bounds__(kLayoutThreads) layout_kernel(BatchLayout bl, 
           a.kv_head = g.kvh;
           a.tok0 = tl.tok0;
           a.ntok = tl.ntok;
-          a.blk_begin = max(g0, c * per) - g0;
-          a.blk_end = min(g0 + g.nb, (c + 1) * per) - g0;
+          a.blk_begin = whole ? 0 : max(g0, c * per) - g0;
+          a.blk_end = whole ? g.nb : min(g0 + g.nb, (c + 1) * per) - g0;
           a.part = np > 1 ? part++ : -1;
           a.kv_len = kv_len;
           if (at + (c - c_first) < bl.max_items && a.part < bl.max_parts) bl.items[at + (c - c_first)] = a;
@@ -481,13 +485,29 @@ size_t layout_smem_bytes(int n_req, int n_ctas) {
   return (6 * (size_t)(n_req + 1) + (size_t)(n_ctas / 2 + 1) + (size_t)(n_ctas + 1)) * sizeof(int);
 }
 
-void launch_layout(const BatchLayout& bl, const Dims& dm, int tok_per_tile, int n_ctas, int64_t n_pages,
+// Whole tiles against work cut evenly.  A tile's 64-token block takes about .5 us of its CTA; cutting costs the write of the
+// partial results, the combine kernel and its boundary, about 2.5 us.  Measured (one request, 16 rows, a layer's attention): 64
+// tokens of context 6.3 us whole, 8.8 cut; 256 tokens 8.7 and 9.1; 512 tokens 10.8 and 10.3; with head_dim 64 4.3 and 5.8, 5.8
+// and 6.0, 7.8 and 6.4.
+bool attention_whole_tiles(int n_req, const int* ctx_len, const int* rows, int n_kv, int tok_per_tile, int n_ctas) {
+  long long tiles = 0, cost = 0;
+  int longest = 0;
+  for (int r = 0; r < n_req; ++r) {
+    const int rt = (rows[r] + tok_per_tile - 1) / tok_per_tile, nb = (ctx_len[r] + rows[r] + 63) / 64;
+    tiles += (long long)n_kv * rt;
+    cost += (long long)n_kv * rt * (nb + kItemCost);
+    if (nb > longest) longest = nb;
+  }
+  return tiles <= n_ctas && longest - (cost + n_ctas - 1) / n_ctas <= kWholeBlocks;
+}
+
+void launch_layout(const BatchLayout& bl, const Dims& dm, int tok_per_tile, int n_ctas, bool whole, int64_t n_pages,
                    int* status, cudaStream_t st) {
   const size_t smem = layout_smem_bytes(bl.n_req, n_ctas);
   static bool configured[kMaxDevices] = {false};
   if (first_use_on_device(configured))    // room for kMaxLayoutRequests requests (the default limit is 48 KB)
     cudaFuncSetAttribute(layout_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)layout_smem_bytes(kMaxLayoutRequests, 1024));
-  launch_pdl(layout_kernel, dim3(1 + (bl.n_tok + kLayoutThreads - 1) / kLayoutThreads), dim3(kLayoutThreads), smem, st, bl, dm.n_kv, dm.mask_id, tok_per_tile, n_ctas, n_pages, status);
+  launch_pdl(layout_kernel, dim3(1 + (bl.n_tok + kLayoutThreads - 1) / kLayoutThreads), dim3(kLayoutThreads), smem, st, bl, dm.n_kv, dm.mask_id, tok_per_tile, n_ctas, whole ? 1 : 0, n_pages, status);
 }
 
 void launch_embed(const BatchLayout& bl, const Dims& dm, const void* embed, float* h, const void* gain, void* x, float* ss,

@@ -55,6 +55,7 @@ struct recg_ctx {
   BatchLayout bl{};
   bool layout_valid = false;
   bool layout_has_pages = false;
+  bool layout_whole = false;     // no attention tile was cut: no combine kernel
   int64_t last_pool_pages = 0;
   void* last_pool = nullptr;
   // activations
@@ -83,6 +84,7 @@ struct recg_ctx {
   void* tc_state = nullptr;
   void* chain_state = nullptr;   // RECG_FLAG_CHAIN
   std::vector<int> h_desc;
+  std::vector<int> h_rows;
   std::vector<int> h_page_owner;   // debug checks: which request names a page
   // optional per-class timing
   bool timing = false;
@@ -325,7 +327,10 @@ recg_status upload_and_layout(recg_ctx* ctx, const recg_batch* b, bool need_page
                      ctx->stream));
   if (b->page_table) {       // (a verify-only batch without pages has neither slots nor attention work)
     const int64_t n_pages = b->kv_pool ? b->kv_pool_pages : (int64_t)1 << 40;
-    launch_layout(ctx->bl, ctx->dm, ctx->tok_per_tile, ctx->target_items, n_pages, ctx->d_status, ctx->stream);
+    ctx->h_rows.resize(b->n_req);
+    for (int r = 0; r < b->n_req; ++r) ctx->h_rows[r] = request_rows(b, r);
+    ctx->layout_whole = attention_whole_tiles(b->n_req, b->ctx_len, ctx->h_rows.data(), ctx->dm.n_kv, ctx->tok_per_tile, ctx->target_items);
+    launch_layout(ctx->bl, ctx->dm, ctx->tok_per_tile, ctx->target_items, ctx->layout_whole, n_pages, ctx->d_status, ctx->stream);
   }
   CU(cudaGetLastError());
   ctx->layout_valid = true;
@@ -581,9 +586,9 @@ static recg_status run_forward(recg_ctx* ctx, void* kv_pool, int64_t kv_pool_pag
     ctx->mark(2, 1);
     }
     launch_attention(bl, d, l, ctx->q, ctx->o, kv_pool, kv_pool_pages, ctx->part_o, ctx->part_ml,
-                     ctx->tok_per_tile, ctx->n_sm, ctx->d_status, st, !(ctx->cfg.flags & RECG_FLAG_SIMT_ATTENTION), true);
+                     ctx->tok_per_tile, ctx->n_sm, ctx->d_status, st, !(ctx->cfg.flags & RECG_FLAG_SIMT_ATTENTION), true, ctx->layout_whole);
     CU(cudaGetLastError());
-    ctx->mark(3, 2);
+    ctx->mark(3, ctx->layout_whole ? 1 : 2);
     if (chain) {
       const bool last = l + 1 == d.n_layers;
       const int slots_h = d.hidden / 128;      // sum-of-squares slots a residual op of the chain fills
@@ -717,7 +722,8 @@ recg_status recg_step_device(recg_ctx* ctx, const recg_device_batch* b, recg_log
   bl.page_table = b->page_table;
   bl.risk_delta = 0.5f;
   launch_pack_device(device_round(ctx, b), ctx->d_desc, ctx->d_dyn, ctx->d_status, ctx->stream);
-  launch_layout(bl, ctx->dm, ctx->tok_per_tile, ctx->target_items, b->kv_pool_pages, ctx->d_status, ctx->stream);
+  ctx->layout_whole = false;           // (the lengths are on the device)
+  launch_layout(bl, ctx->dm, ctx->tok_per_tile, ctx->target_items, false, b->kv_pool_pages, ctx->d_status, ctx->stream);
   CU(cudaGetLastError());
   ctx->layout_valid = true;
   ctx->layout_has_pages = true;
@@ -876,7 +882,7 @@ recg_status recg_attention(recg_ctx* ctx, const recg_batch* batch, int32_t layer
   }
   launch_attention(ctx->bl, ctx->dm, layer, q, o, ctx->last_pool, ctx->last_pool_pages, ctx->part_o, ctx->part_ml,
                    ctx->tok_per_tile, ctx->n_sm, ctx->d_status, ctx->stream, !(ctx->cfg.flags & RECG_FLAG_SIMT_ATTENTION),
-                   batch == nullptr);      // (a batch given with the call was laid out by the launch right before this one)
+                   batch == nullptr, ctx->layout_whole);      // (a batch given with the call was laid out by the launch right before this one)
   CU(cudaGetLastError());
   return RECG_OK;
 }

@@ -20,3 +20,11 @@ def test_more_requests_than_threads():
     shape = synth.ModelShape(n_layers=1, hidden=64, n_q_heads=4, n_kv_heads=2, head_dim=128, ffn=64, vocab=64)
     reqs = [(i % 19, 1 + i % 3, i % 2) for i in range(1100)] + [(40, 70, 0), (500, 33, 0)]
     assert run_attention_case(shape, reqs, seed=3) < ATTN_TOL
+
+
+@pytest.mark.parametrize("reqs", [[(0, 1, 0)], [(200, 8, 8)], [(300, 16, 16)], [(340, 16, 16)], [(100, 40, 0), (250, 33, 10)],
+                                  [(64, 100, 0)], [(400, 60, 4)] * 3, [(300, 8, 8)] * 18, [(300, 8, 8)] * 19])
+def test_whole_tiles_of_short_contexts(reqs):
+    """On both sides of the rule that leaves tiles uncut: about six blocks of context, and as many tiles as CTAs."""
+    for shape in (synth.llama8b_shape(1), synth.tiny_shape()):
+        assert run_attention_case(shape, reqs, seed=len(reqs) + reqs[0][0]) < ATTN_TOL
