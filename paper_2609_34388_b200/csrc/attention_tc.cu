@@ -211,8 +211,11 @@ __global__ void __launch_bounds__(kThreads, 1) attention_tc_kernel(const __grid_
   };
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // Warp 0 waits for the kernels before this one and fetches the CTA's item range and first item while the other
-  // warps set up barriers, the zeroed ring and TMEM: two dependent round trips off everybody's critical path.
+  // Warp 0 fetches the CTA's item range and first item while the other warps set up barriers, the zeroed ring and TMEM: two
+  // dependent round trips off everybody's critical path.  Where the work list is settled all that happens before the wait for
+  // the kernels in front of this one, and so do the first page ids and a pass of the softmax warps through their code without
+  // effect: behind a projection that code is not in the SM's instruction cache, and the first scores took 2.3 us instead of .9,
+  // the end of the item 2.2 instead of 1.7.
   int* s_range = reinterpret_cast<int*>(tmem_slot + 2);
   AttnItem* s_first = reinterpret_cast<AttnItem*>(tmem_slot + 6);
   // the CTA walks two ranges of the item list one after the other (see the layout kernel): logical item i is
@@ -224,8 +227,8 @@ __global__ void __launch_bounds__(kThreads, 1) attention_tc_kernel(const __grid_
   AttnItem w_next = {};
   if (warp == 0) {
     // (inside a step the work list was written many launches ago and the kernel in front of this one, the QKV
-    // projection, only signals its dependents when its own work is done: the two dependent reads below then overlap
-    // that kernel's tail instead of following it)
+    // projection, only signals its dependents after its own wait: the reads below then overlap that kernel instead of
+    // following it)
     if (!P.early_desc) griddep_wait();
     const int4 r4 = *reinterpret_cast<const int4*>(P.cta_off + 4 * blockIdx.x);
     range_b0 = r4.x;
@@ -240,7 +243,6 @@ __global__ void __launch_bounds__(kThreads, 1) attention_tc_kernel(const __grid_
       s_range[3] = item_end;
       *s_first = w_next;
     }
-    if (P.early_desc) griddep_wait();
   }
   if (threadIdx.x == 32) {
     *abort_flag = 0;
@@ -275,14 +277,16 @@ __global__ void __launch_bounds__(kThreads, 1) attention_tc_kernel(const __grid_
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   if (warp != 0) {
-    griddep_wait();   // these warps touched only shared memory and TMEM so far
     range_b0 = s_range[0];
     range_n0 = s_range[1];
     range_b1 = s_range[2];
     item_end = s_range[3];
     w_next = *s_first;
   }
+  // (the kernels in front are waited for below: by the producers when they have the first page ids, by the softmax warps after
+  // their pass without effect)
   const uint32_t smem_base = smem_u32(smem);
+  if (warp == 3) griddep_wait();   // (this warp is the first to signal the kernel's dependents)
 
   if (warp < 4) {
     if (warp == 0 || warp == 2) {
@@ -307,6 +311,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_tc_kernel(const __grid_
           return pg;
         };
         int pg_next = fetch_page(0);
+        if (item == item_begin) griddep_wait();
         if (part == 0) {
           // Q rows of the item: (64 dims) x (the kv head's query heads) x (128 / group tokens from tok0); rows past the
           // tile's own tokens belong to other tokens or are zero-filled, and nobody reads their S / O rows
@@ -379,6 +384,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_tc_kernel(const __grid_
       }
     } else if (warp == 1) {
       // ------------------------------------ MMA issuer ------------------------------------
+      griddep_wait();
       if (elect_one()) {
         uint32_t blk = 0, item_cnt = 0;      // running stage (128-token KV block) and item counters
         // Group g works on tokens [64 g, 64 g + 64) of EVERY stage.  S of stage b = Q K^T goes to S buffer b & 1 (one
@@ -457,24 +463,29 @@ __global__ void __launch_bounds__(kThreads, 1) attention_tc_kernel(const __grid_
       }
     };
     int nx_cl = -1, nx_lo = 0, nx_hi = 0;
-    if (item_begin < item_end) row_vis(w_next, nx_cl, nx_lo, nx_hi);
-    for (int item = item_begin; item < item_end; ++item) {
-      const AttnItem w = w_next;
-      if (item + 1 < item_end) w_next = P.items[item_at(item + 1)];
+    // The first turn of the loop is the one without effect: no row exists, nothing is waited for, signalled or stored but this
+    // group's own O accumulator, which the first product overwrites.
+    for (int item = item_begin - 1; item < item_end; ++item) {
+      const bool dry = item < item_begin;
+      AttnItem w = {};
+      if (!dry) {
+        w = w_next;
+        if (item + 1 < item_end) w_next = P.items[item_at(item + 1)];
+      }
       const int R = w.ntok * P.group;
       const int tok_begin = w.blk_begin * 64;
       const int tok_end = min(w.blk_end * 64, w.kv_len);
-      const int nblk = (tok_end - tok_begin + kBT - 1) / kBT;
+      const int nblk = dry ? 1 : (tok_end - tok_begin + kBT - 1) / kBT;
       const bool rvalid = row < R;
-      const bool warp_valid = quad * 32 < R;
+      const bool warp_valid = dry || quad * 32 < R;
       const int climit = nx_cl, vlo = nx_lo, vhi = nx_hi;
       float m_ref = -1e30f, l_run = 0.f;
       bool first = true;
 
       for (int n = 0; n < nblk; ++n, ++cs) {
         // this group's 64 tokens of stage n: S buffer cs & 1 (cs = running stage count, the same in every role)
-        const uint32_t s_buf = s_addr + (cs & 1) * kBT;
-        bwait(&s_full[cs & 1], (cs >> 1) & 1, DEV_TIMEOUT_MMA);
+        const uint32_t s_buf = dry ? o_addr : s_addr + (cs & 1) * kBT;
+        if (!dry) bwait(&s_full[cs & 1], (cs >> 1) & 1, DEV_TIMEOUT_MMA);
         tc_fence_after();
         const int pos0 = tok_begin + n * kBT + g * 64;
         uint32_t sr[2][32];   // the S row of this thread: 64 scores
@@ -554,6 +565,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_tc_kernel(const __grid_
         }
         tc_fence_before();
         __syncwarp();
+        if (dry) break;
         if (lane == 0) mbar_arrive(&p_full[2 * g + (cs & 1)]);
         if (first) {      // the next item's descriptor has arrived by now: fetch its rows' visibility for later
           first = false;
@@ -564,7 +576,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_tc_kernel(const __grid_
       // ---- merge the two groups' partial attentions and write out: this group finishes dims [64 g, 64 g + 64) ----
       const bool two = true;                      // both groups take part in every stage
       const int buf = item_cnt & 1;
-      bwait(o_full, item_cnt & 1, DEV_TIMEOUT_MMA);
+      if (!dry) bwait(o_full, item_cnt & 1, DEV_TIMEOUT_MMA);
       tc_fence_after();
       ml_smem[g * 128 + row] = make_float2(m_ref, l_run);
       softmax_bar();
@@ -616,7 +628,8 @@ __global__ void __launch_bounds__(kThreads, 1) attention_tc_kernel(const __grid_
             float4* s4 = reinterpret_cast<float4*>(stg);
 #pragma unroll
             for (int q = 0; q < 8; ++q)
-              s4[lane * 8 + (q ^ (lane & 7))] = make_float4(__uint_as_float(r[4 * q]), __uint_as_float(r[4 * q + 1]),
+              if (!dry)                // (the Q buffer may be on its way in)
+                s4[lane * 8 + (q ^ (lane & 7))] = make_float4(__uint_as_float(r[4 * q]), __uint_as_float(r[4 * q + 1]),
                                                             __uint_as_float(r[4 * q + 2]), __uint_as_float(r[4 * q + 3]));
             __syncwarp();
             const int rq = lane >> 3, q = lane & 7;
@@ -638,18 +651,23 @@ __global__ void __launch_bounds__(kThreads, 1) attention_tc_kernel(const __grid_
       tc_fence_before();
       fence_proxy_async();    // the Q buffer goes back to the TMA unit
       __syncwarp();
-      if (lane == 0) {
-        mbar_arrive(o_empty);
-        mbar_arrive(&q_empty[buf]);
+      if (!dry) {
+        if (lane == 0) {
+          mbar_arrive(o_empty);
+          mbar_arrive(&q_empty[buf]);
+        }
+        ++item_cnt;
       }
-      ++item_cnt;
       softmax_bar();          // the (max, sum) exchange area may be rewritten
+      if (dry) {
+        griddep_wait();
+        if (item_begin < item_end) row_vis(w_next, nx_cl, nx_lo, nx_hi);
+      }
     }
   }
 
-  // this CTA's work is done: let the next kernel's CTAs be scheduled (they run their prologue and then wait for
-  // this whole grid).  Signalling earlier would park their warps on the SMs while the softmax warps still need
-  // every issue slot.
+  // The next kernel's CTAs may be scheduled (they run their prologue and then wait for this whole grid).  The idle warp comes
+  // here as soon as the kernels in front are done.
   griddep_launch();
   tc_fence_before();
   __syncthreads();
