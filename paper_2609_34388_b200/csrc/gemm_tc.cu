@@ -230,65 +230,71 @@ __host__ __device__ inline void token_tiles(int M, int tmax, int gran, int* widt
   *count = (M + *width - 1) / *width;
 }
 
-// "Stream-K", done per COLUMN of output tiles (the mt token tiles that share one weight tile): the k-blocks of the columns
-// form one line of n_cols * KB units, column after column; a TEAM of mt units (unit team * mt + i works on token tile i) owns
-// the contiguous range [team * per, (team + 1) * per) and walks it in step, so that the members read the same weight k-blocks
-// at the same time and share them through L2, exactly like the CTAs of a wave of whole tiles.  A column may be cut by team
-// boundaries; each owner computes its K range of its token tile ("part").  Part p >= 1 of a tile is always the FIRST piece of
-// its unit, part 0 the last piece (or the first, when the range starts exactly at the column): that decides the workspace
-// slot, 2 * unit + (first piece ? 0 : 1).
-// All but the last one-to-two waves stay whole tiles (dp_tiles of them, done after the cut ones).  Computed on the host, or in
-// the kernel when the row count (hence mt) is only known on the device.  Needs mt <= n_units.
-__host__ __device__ inline void stream_k_schedule(int n_tiles, int mt, int KB, int n_units, int* dp_tiles, int* per, int* used_units) {
-  const int n_teams = n_units / mt;
-  const int full = n_tiles / n_units;
-  *dp_tiles = full >= 2 ? ((full - 1) * n_units / mt) * mt : 0;
-  const int total = (n_tiles - *dp_tiles) / mt * KB;       // (launch_gemm_tc keeps the line within int)
-  const int teams = total < n_teams ? total : n_teams;
-  int p = teams > 0 ? (total + teams - 1) / teams : 1;
-  if (p < 4 && total >= 4) p = 4;                     // keep pieces long enough to amortise their hand-over
-  if (p < 1) p = 1;
-  *per = p;
-  const int used = (total + p - 1) / p;               // teams that get a range
-  *used_units = *dp_tiles ? n_units : used * mt;      // (with whole tiles behind, the grid stays at full size)
+// Whole tiles, token-fastest, strided over the units; and "stream-K" for the last columns (all of them, or the ragged end of the
+// whole tiles), done per COLUMN of output tiles (the mt token tiles that share one weight tile; the cut columns may have
+// narrower token tiles of their own): the k-blocks of the columns form one line of cut_cols * KB units, column after column; a
+// TEAM of mt units (unit team * mt + i works on token tile i) owns the contiguous range [team * per, (team + 1) * per) and walks
+// it in step, so that the members read the same weight k-blocks at the same time and share them through L2, exactly like the
+// CTAs of a wave of whole tiles.  A column may be cut by team boundaries; each owner computes its K range of its token tile
+// ("part").  Part p >= 1 of a tile is always the FIRST piece of its unit, part 0 the last piece (or the first, when the range
+// starts exactly at the column): that decides the workspace slot, 2 * unit + (first piece ? 0 : 1).
+// K-blocks per team for a line of `cols` columns.
+__host__ __device__ inline int cut_range(int cols, int mt, int KB, int n_units) {
+  const int total = cols * KB, n_teams = n_units / mt;       // (launch_gemm_tc keeps the line within int; mt <= n_units)
+  const int per = (total + n_teams - 1) / n_teams;
+  return per < 4 && total >= 4 ? 4 : per;                    // pieces long enough to amortise their hand-over
 }
 
 struct Piece {
-  int tile, kb0, kb1;     // k-block range [kb0, kb1) of the tile
+  int col, tm;            // column of tiles and token tile
+  int kb0, kb1;           // k-block range
+  bool cut;               // of the stream-K line: token tiles of the cut columns
   int part, n_parts;      // which part of the tile this is
   int slot;               // workspace slot if n_parts > 1
   int slot0, slot_next;   // slots of part 0 and part 1 (for the reducing CTA)
+  int counter;            // arrival counter of the tile
+};
+struct Schedule {
+  int KB, n_units;
+  int whole, mt;          // whole tiles, token tiles of their columns
+  int cut_col0, cut_mt;   // first cut column, token tiles of the cut columns
+  int per;                // k-blocks of a team's range
 };
 // Next piece of this unit: first its range of the stream-K line (pos advances by reference), then its whole tiles
 // (jd counts them).  The cut tiles come first so that parking and reducing their partials overlaps the main loop
 // of the whole tiles that follow, instead of happening in every CTA at once at the end of the kernel.
-__device__ __forceinline__ Piece make_piece(int& jd, int dp_tiles, int& pos, int hi, int KB, int per, int unit, int n_units,
-                                            int mt) {
+__device__ __forceinline__ Piece make_piece(const Schedule& S, int& jd, int& pos, int hi, int unit) {
   Piece p;
   if (pos >= hi) {
-    p.tile = unit + jd * n_units;
+    const int tile = unit + jd * S.n_units;
     ++jd;
+    p.col = tile / S.mt;
+    p.tm = tile - p.col * S.mt;
     p.kb0 = 0;
-    p.kb1 = KB;
+    p.kb1 = S.KB;
+    p.cut = false;
     p.part = 0;
     p.n_parts = 1;
-    p.slot = p.slot0 = p.slot_next = 0;
+    p.slot = p.slot0 = p.slot_next = p.counter = 0;
     return p;
   }
-  const int team = unit / mt, member = unit % mt;
-  const int col = pos / KB;
-  p.kb0 = pos - col * KB;
+  const int team = unit / S.cut_mt, member = unit - team * S.cut_mt;
+  const int col = pos / S.KB;
+  p.kb0 = pos - col * S.KB;
   const int room = hi - pos;
-  p.kb1 = room < KB - p.kb0 ? p.kb0 + room : KB;
-  const int t0 = col * KB, t1 = t0 + KB;
-  const int c_first = t0 / per, c_last = (t1 - 1) / per;    // first and last team on this column
+  p.kb1 = room < S.KB - p.kb0 ? p.kb0 + room : S.KB;
+  const int t0 = col * S.KB, t1 = t0 + S.KB;
+  const int c_first = t0 / S.per, c_last = (t1 - 1) / S.per;    // first and last team on this column
+  p.cut = true;
   p.n_parts = c_last - c_first + 1;
   p.part = team - c_first;
-  const bool first_piece = pos == team * per;
+  const bool first_piece = pos == team * S.per;
   p.slot = 2 * unit + (first_piece ? 0 : 1);
-  p.slot0 = 2 * (c_first * mt + member) + (c_first * per >= t0 ? 0 : 1);
-  p.slot_next = 2 * ((c_first + 1) * mt + member);
-  p.tile = dp_tiles + col * mt + member;
+  p.slot0 = 2 * (c_first * S.cut_mt + member) + (c_first * S.per >= t0 ? 0 : 1);
+  p.slot_next = 2 * ((c_first + 1) * S.cut_mt + member);
+  p.counter = col * S.cut_mt + member;
+  p.col = S.cut_col0 + col;
+  p.tm = member;
   pos += p.kb1 - p.kb0;
   return p;
 }
@@ -545,8 +551,8 @@ struct GemmLaunch {
   int K;
   int tmax, gran, x_box;     // token tiles (token_tiles), rows of one x load
   int width, mt;             // ... their width and number, where the row count is known
-  int dp_tiles;              // >= 0: the host's schedule; -1: whole tiles only; -2: stream-K, divided here from the device's row count
-  int per;
+  int cut_cols;              // last columns whose tiles are cut over K; -1 (row count on the device): all of them
+  int cut_width, cut_mt, cut_box, per;   // their token tiles, rows of one x load, k-blocks of a team's range
   int cl;                    // parts per tile that form a cluster (0: no clusters)
   int w_step3, w_step4;      // what a 128-feature tile advances in dimensions 3 and 4 of w's tensor map
   float* split_ws;
@@ -557,7 +563,8 @@ struct GemmLaunch {
 
 template <bool PAIR>
 __global__ void __launch_bounds__(kTcThreads, 1)
-gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x, GemmLaunch G, EpiParams ep) {
+gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x,
+               const __grid_constant__ CUtensorMap map_xc, GemmLaunch G, EpiParams ep) {
   // Device-resident rounds: the row count comes from device memory; the tensor maps cover the capacity, and rows
   // between the count and the capacity hold stale data and are computed but never used.  The count is written by the
   // first kernel of the step, and the small kernels between it and the first projection signal their dependents before
@@ -581,11 +588,19 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
 
+  const int KB = G.K / BK;
   int nt_tok = G.width, mt = G.mt;                        // tokens per tile, token tiles
   if (G.m_dev) token_tiles(M, G.tmax, G.gran, &nt_tok, &mt);
-  const int x_rows = nt_tok / kMul;                       // rows of x this CTA loads per k-block
-  const int stage_bytes = kABytes + x_rows * BK * 2;
-  const int part_bytes = (nt_tok + 31) / 32 * kChunkBytes;   // a partial tile
+  int cut_cols = G.cut_cols, cut_tok = G.cut_width, cut_mt = G.cut_mt, per = G.per;      // the same for the cut columns
+  if (cut_cols < 0) {
+    cut_cols = mt <= n_units ? G.n_cols : 0;
+    cut_tok = nt_tok;
+    cut_mt = mt;
+    per = cut_cols ? cut_range(cut_cols, mt, KB, n_units) : 1;
+  }
+  // (the cut columns' token tiles are never wider than the others: one stage layout serves both)
+  const int stage_bytes = kABytes + nt_tok / kMul * BK * 2;
+  const int part_bytes = (cut_tok + 31) / 32 * kChunkBytes;   // a partial tile in the workspace
   // Clusters: chunk c of the tile (32 tokens) is finished by member c % cl, into whose shared memory the others write their
   // partial sums of it (16 KB each).  A tile of one chunk has a reserve for them at the top of the ring; else they go into the
   // ring itself, once its owner says that its own products have read it.
@@ -636,39 +651,31 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n_tiles = mt * G.n_cols;
-  const int KB = G.K / BK;
-  int dp_tiles = G.dp_tiles < 0 ? n_tiles : G.dp_tiles;
-  int per = G.per;
-  if (G.dp_tiles == -2) {
-    if (mt >= 1 && mt <= n_units) {
-      int used;
-      stream_k_schedule(n_tiles, mt, KB, n_units, &dp_tiles, &per, &used);
-    } else {
-      dp_tiles = n_tiles;
-    }
-  }
-  // schedule: the k-blocks of tiles [dp_tiles, n_tiles) as one line cut into equal ranges per unit; then tiles
-  // [0, dp_tiles) whole, strided over the grid (CTAs that run together share a weight tile through L2)
-  const int total = (n_tiles - dp_tiles) / mt * KB;
-  const int lo_raw = unit / mt * per;
+  const Schedule S{KB, n_units, (G.n_cols - cut_cols) * mt, mt, G.n_cols - cut_cols, cut_mt, per};
+  // the unit's range of the stream-K line, and its whole tiles
+  const int total = cut_cols * KB;
+  const int lo_raw = cut_cols ? unit / cut_mt * per : 0;
   const bool cl_live = cl && unit / cl < n_tiles;          // (the grid of a device-resident step is sized for the capacity)
   const int range_lo = cl ? 0 : (lo_raw < total ? lo_raw : total);
   const int range_hi = cl ? (cl_live ? 1 : 0) : (range_lo + per < total ? range_lo + per : total);
-  const int dp_count = cl ? 0 : (unit < dp_tiles ? (dp_tiles - 1 - unit) / n_units + 1 : 0);
+  const int dp_count = cl ? 0 : (unit < S.whole ? (S.whole - 1 - unit) / n_units + 1 : 0);
   // the next piece of this unit (a cluster member has exactly one)
   auto next_piece = [&](int& jd, int& pos) -> Piece {
     if (cl) {
       Piece p;
-      p.tile = unit / cl;
+      const int tile = unit / cl;
+      p.col = tile / mt;
+      p.tm = tile - p.col * mt;
+      p.cut = false;
       p.kb0 = (int)part_rank * KB / cl;
       p.kb1 = ((int)part_rank + 1) * KB / cl;
       p.part = (int)part_rank;
       p.n_parts = cl;
-      p.slot = p.slot0 = p.slot_next = 0;
+      p.slot = p.slot0 = p.slot_next = p.counter = 0;
       pos = range_hi;
       return p;
     }
-    return make_piece(jd, dp_tiles, pos, range_hi, KB, per, unit, n_units, mt);
+    return make_piece(S, jd, pos, range_hi, unit);
   };
 
   if (threadIdx.x == 0) {
@@ -708,12 +715,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
     if (elect_one()) {
       // of a pair, rank r loads the weight rows of feature tile 2 c + r and half r of the token tile; all loads of the pair
       // complete on the leader's barrier
-      auto expect = [&](int s) {
-        if constexpr (PAIR) {
-          if (rank == 0) mbar_arrive_expect_tx(&full_bar[s], 2 * stage_bytes);
-        } else {
-          mbar_arrive_expect_tx(&full_bar[s], stage_bytes);
-        }
+      auto expect = [&](int s, bool cut) {
+        const int bytes = kMul * kABytes + (cut ? cut_tok : nt_tok) * BK * 2;
+        if (rank == 0) mbar_arrive_expect_tx(&full_bar[s], bytes);
       };
       auto load_w = [&](int s, int kb, int col) {
         const uint32_t dst = smem_u32(smem + s * stage_bytes);
@@ -721,39 +725,42 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
         if constexpr (PAIR) tma_load_w_pair(dst, &map_w, kb * BK, ft * G.w_step3, ft * G.w_step4, mapa_rank(smem_u32(&full_bar[s]), lead_rank));
         else tma_load_w(dst, &map_w, kb * BK, ft * G.w_step3, ft * G.w_step4, &full_bar[s]);
       };
-      auto load_x = [&](int s, int kb, int tm) {
+      auto load_x = [&](int s, int kb, int tm, bool cut) {
         uint8_t* dst = smem + s * stage_bytes + kABytes;
-        const int row = tm * nt_tok + (int)rank * x_rows;
-        for (int r = 0; r < x_rows; r += G.x_box) {
-          if constexpr (PAIR) tma_load_2d_pair(smem_u32(dst + r * BK * 2), &map_x, kb * BK, row + r, mapa_rank(smem_u32(&full_bar[s]), lead_rank));
-          else tma_load_2d(dst + r * BK * 2, &map_x, kb * BK, row + r, &full_bar[s]);
+        const int rows = (cut ? cut_tok : nt_tok) / kMul, box = cut ? G.cut_box : G.x_box;
+        const int row = tm * rows * kMul + (int)rank * rows;
+        const CUtensorMap* map = cut ? &map_xc : &map_x;
+        for (int r = 0; r < rows; r += box) {
+          if constexpr (PAIR) tma_load_2d_pair(smem_u32(dst + r * BK * 2), map, kb * BK, row + r, mapa_rank(smem_u32(&full_bar[s]), lead_rank));
+          else tma_load_2d(dst + r * BK * 2, map, kb * BK, row + r, &full_bar[s]);
         }
       };
       // The weights do not depend on the kernels before this one: the weight tiles of the first stages are requested
       // BEFORE waiting for those kernels, so the ring fills while they drain (or while a short kernel runs); the x tiles of
       // those stages follow right after the wait.
       int n_pre = 0, pre_kb0 = 0, pre_tm = 0;
+      bool pre_cut = false;
       if (dp_count > 0 || range_lo < range_hi) {
         int p0 = range_lo;
         int j0 = 0;
         const Piece pc = next_piece(j0, p0);
         n_pre = pc.kb1 - pc.kb0 < n_stages ? pc.kb1 - pc.kb0 : n_stages;
         pre_kb0 = pc.kb0;
-        pre_tm = pc.tile % mt;
+        pre_tm = pc.tm;
+        pre_cut = pc.cut;
         for (int i = 0; i < n_pre; ++i) {
-          expect(i);
-          load_w(i, pre_kb0 + i, pc.tile / mt);
+          expect(i, pre_cut);
+          load_w(i, pre_kb0 + i, pc.col);
         }
       }
       griddep_wait();
-      for (int i = 0; i < n_pre; ++i) load_x(i, pre_kb0 + i, pre_tm);
+      for (int i = 0; i < n_pre; ++i) load_x(i, pre_kb0 + i, pre_tm, pre_cut);
       int st_idx = 0, issued = 0;
       uint32_t st_phase = 0;
       bool ok = true;
       int pos = range_lo;
       for (int jd = 0; (jd < dp_count || pos < range_hi) && ok;) {
         const Piece pc = next_piece(jd, pos);
-        const int tm = pc.tile % mt, col = pc.tile / mt;
         const int kb0 = pc.kb0, kb1 = pc.kb1;
         for (int kb = kb0; kb < kb1; ++kb) {
           const int s = st_idx;
@@ -768,9 +775,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
             ok = false;
             break;
           }
-          expect(s);
-          load_x(s, kb, tm);
-          load_w(s, kb, col);
+          expect(s, pc.cut);
+          load_x(s, kb, pc.tm, pc.cut);
+          load_w(s, kb, pc.col);
         }
       }
       if (!ok) {  // let loads already issued land before the CTA may exit
@@ -784,7 +791,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
   } else if (warp == 1) {
     // ------------------------------ MMA issuer ------------------------------
     if (rank == 0 && elect_one()) {         // of a pair only the leader issues (it touches shared memory and TMEM only)
-      const uint32_t idesc = make_idesc(nt_tok, FT * kMul);
+      const uint32_t idesc_whole = make_idesc(nt_tok, FT * kMul), idesc_cut = make_idesc(cut_cols ? cut_tok : nt_tok, FT * kMul);
       const uint64_t desc0 = make_smem_desc(smem_u32(smem));
       const uint16_t pair_mask = (uint16_t)(3u << lead_rank);
       int st_idx = 0;
@@ -800,7 +807,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
           break;
         }
         tc_fence_after();
-        const uint32_t d_tmem = tmem_base + acc * kAccStride;
+        const uint32_t d_tmem = tmem_base + acc * kAccStride, idesc = pc.cut ? idesc_cut : idesc_whole;
         for (int kb = kb0; kb < kb1; ++kb) {
           const int s = st_idx;
           const uint32_t ph = st_phase;
@@ -836,7 +843,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
     const int row = quad * 32 + lane;      // this thread among the 128 of the epilogue
     const uint32_t tmem_quad = tmem_base + ((uint32_t)(quad * 32) << 16);
     uint32_t tcount = 0;
-    int prep_tm = -1;
+    int prep_tm = -1;                      // the token tile whose row factors and slots are in shared memory
     __shared__ int s_last;
     TileOut o{0, 0, 0, quad, lane, s_rstd, s_slot, s_ss, smem + kOffStage + quad * 2048};
     float pre[32], gain[4] = {0.f, 0.f, 0.f, 0.f};
@@ -865,17 +872,17 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
         }
       } else {
         const Piece pc = next_piece(jd, pos);
-        const int tile = pc.tile, n_splits = pc.n_parts;
-        const int tm = tile % mt;
-        o.tile = (tile / mt) * kMul + (int)rank;
-        o.t0 = tm * nt_tok;
-        o.nv = M - o.t0 < nt_tok ? M - o.t0 : nt_tok;
+        const int n_splits = pc.n_parts, width = pc.cut ? cut_tok : nt_tok;
+        o.tile = pc.col * kMul + (int)rank;
+        o.t0 = pc.tm * width;
+        o.nv = M - o.t0 < width ? M - o.t0 : width;
         acc = tcount & 1;
         src.tacc = tmem_quad + acc * kAccStride;
         const int n_chunks = (o.nv + 31) / 32;
         // What the epilogue needs per token, fetched while the accumulator is still being computed: the row factors of a
         // normalised input (the partial sums of squares in slot order: the same bits in every tile of the row) and the slots.
-        if (tm != prep_tm && (ep.ss_in || ep.epi == EPI_QKV_ROPE)) {
+        const int prep = 2 * pc.tm + (pc.cut ? 1 : 0);
+        if (prep != prep_tm && (ep.ss_in || ep.epi == EPI_QKV_ROPE)) {
           if (prep_tm >= 0) asm volatile("bar.sync 1, 128;" ::: "memory");
           for (int t = (int)threadIdx.x - 64; t < o.nv; t += 128) {
             if (ep.ss_in) {
@@ -888,7 +895,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
             if (ep.epi == EPI_QKV_ROPE) s_slot[t] = ep.tok_slot[o.t0 + t];
           }
           asm volatile("bar.sync 1, 128;" ::: "memory");
-          prep_tm = tm;
+          prep_tm = prep;
         }
         c_end = n_chunks;
         if (cl) {
@@ -938,8 +945,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
           // (the two CTAs of a pair park and reduce their 128 features independently: slot and counter index are
           // doubled and offset by the rank)
           const int slot_mine = pc.slot * kMul + (int)rank, slot0 = pc.slot0 * kMul + (int)rank;
-          const int slot_next = pc.slot_next * kMul + (int)rank, slot_stride = 2 * mt * kMul;
-          const int counter = tile * kMul + (int)rank;
+          const int slot_next = pc.slot_next * kMul + (int)rank, slot_stride = 2 * cut_mt * kMul;
+          const int counter = pc.counter * kMul + (int)rank;
           const size_t part_f4 = part_bytes / 16;
           float4* mine = reinterpret_cast<float4*>(G.split_ws) + slot_mine * part_f4 + row;
 #pragma unroll 1
@@ -1042,11 +1049,18 @@ constexpr size_t kSplitWsBytes = 96ull << 20;   // partial tiles of split-K laun
 constexpr int kSplitCounters = 1 << 16;
 constexpr size_t kMapCacheMax = 4096;           // entries; the keys include the row count, so a serving loop keeps adding
 
-// Cache of encoded tensor maps (cached_map below).  Maps are handed out BY VALUE: a launch needs several at once,
-// and a miss on a later lookup may empty the full cache, so nothing may point into it.
-struct Config {        // how a projection runs: single CTAs or CTA pairs, the widest token tile, whole tiles / stream-K / clusters of cl parts
-  bool pair, stream_k;
-  int tmax, cl;
+// How a projection runs: single CTAs or CTA pairs, the widest token tile, clusters of cl parts per tile or the last cut_cols
+// columns cut over K in token tiles of at most cut_tmax.
+struct Config {
+  bool pair;
+  int tmax, cl, cut_cols, cut_tmax;
+};
+struct Shape {
+  int M, n_feat, K;       // n_feat: rows of w
+  bool operator==(const Shape& o) const { return M == o.M && n_feat == o.n_feat && K == o.K; }
+};
+struct ShapeHash {
+  size_t operator()(const Shape& s) const { return (size_t)s.M * 1000003u ^ (size_t)s.n_feat * 7919u ^ (size_t)s.K << 32; }
 };
 struct TcState {
   int n_sm = 0;
@@ -1056,6 +1070,7 @@ struct TcState {
   EncodeTiledFn encode = nullptr;
   std::unordered_map<MapKey, CUtensorMap, MapKeyHash> maps;
   size_t evictions = 0;
+  std::unordered_map<Shape, Config, ShapeHash> configs;    // choose_config's answers (emptied when there are kMapCacheMax)
   bool configured[2] = {false, false};
   bool clusters = true;       // tiles cut over K may be handed over inside clusters
   int max_clusters[2][9];     // cached occupancy answers per kernel and cluster size in CTAs (-1: not asked yet)
@@ -1065,6 +1080,8 @@ struct TcState {
   }
 };
 
+// Cache of encoded tensor maps (TcState::maps).  Maps are handed out BY VALUE: a launch needs several at once,
+// and a miss on a later lookup may empty the full cache, so nothing may point into it.
 template <typename Encode>
 bool cached_map(TcState* st, const MapKey& key, CUtensorMap* out, Encode&& encode) {
   auto it = st->maps.find(key);
@@ -1166,11 +1183,12 @@ bool clusters_fit(TcState* st, bool pair, int size, int n) {
 // .24.  Below .18 us a CTA is bound by the latency of its loads.
 // The weights come from HBM once: bytes / 6.7 TB/s.
 // On top come the ends (launch, first loads, last tile's epilogue): 4.5 us + .003 x tokens for whole tiles; 6 us when clusters
-// reduce tiles of one chunk, 6.5 us + 1 us per chunk that a member sends for wider ones; 11.5 us + .05 x tokens when cut tiles go
-// through the workspace (parking, counting, fetching, the epilogue in the last part to arrive).
-struct Shape {
-  int M, n_feat, K;       // n_feat: rows of w
-};
+// reduce tiles of one chunk, 6.5 us + 1 us per chunk that a member sends for wider ones; 11.5 us + .05 x tokens when all tiles are
+// cut and go through the workspace (parking, counting, fetching, the epilogue in the last part to arrive).
+// A ragged last wave of whole tiles: its columns can be cut over all units and done first, in narrower token tiles so that a tile
+// has few parts; their hand-over hides under the whole tiles behind them.  28672 x 4096
+// weights at 320, 376, 416 and 1024 rows: 65.5, 72.6, 79.9 and 161.9 us, all tiles whole 69.8, 77.6, 85.1 and 167.3; 4096 x 14336
+// at 1331 rows 111.4 instead of 118.9 with the cut tiles as wide as the others.
 double est_kblock(bool pair, int width, double busy) {
   if (busy > 1.0) busy = 1.0;
   const double t = pair ? (.085 + .00085 * width) * (.95 + .25 * busy) : (.075 + .001 * width) * (.92 + .40 * busy);
@@ -1178,9 +1196,11 @@ double est_kblock(bool pair, int width, double busy) {
 }
 
 Config choose_config(TcState* st, const Shape& s) {
+  const auto known = st->configs.find(s);
+  if (known != st->configs.end()) return known->second;
   const int KB = s.K / BK;
   const double t_hbm = 2.0 * s.n_feat * s.K / 6.7e6;
-  Config best{false, false, kMaxTok, 0};
+  Config best{false, kMaxTok, 0, 0, 0};
   double best_t = 1e30;
   for (int pair = 0; pair < 2; ++pair) {
     const int gran = pair ? 32 : 16, units = pair ? st->n_sm / 2 : st->n_sm;
@@ -1194,28 +1214,51 @@ Config choose_config(TcState* st, const Shape& s) {
       int width, mt;
       token_tiles(s.M, tmax, gran, &width, &mt);
       const long long tiles = (long long)mt * cols;
-      if (tiles * (pair + 1) > kSplitCounters || (want > fewest && width < 32)) continue;
-      auto consider = [&](double t, bool sk, int cl) {
+      if (want > fewest && width < 32) continue;
+      auto consider = [&](double t, int cl, int cut_cols, int cut_tmax) {
         if (t < best_t) {
           best_t = t;
-          best = Config{pair != 0, sk, tmax, cl};
+          best = Config{pair != 0, tmax, cl, cut_cols, cut_tmax};
         }
       };
       const long long full = tiles / units, rem = tiles % units;      // full waves, and a last one that has the machine to itself
-      const double t_whole = KB * (full * est_kblock(pair, width, 1.0) + (rem ? est_kblock(pair, width, (double)rem / units) : 0.0));
-      consider(fmax(t_whole, t_hbm) + 4.5 + .003 * width, false, 0);
-      // cut over K through the workspace; with two waves or more only the ragged end is cut (and done first)
-      if (mt <= units && (full < 2 || rem))
-        consider(fmax((double)tiles * KB / ((units / mt) * mt) * est_kblock(pair, width, 1.0), t_hbm) + 11.5 + .05 * width, true, 0);
+      const double ends = 4.5 + .003 * width, t_full = full * KB * est_kblock(pair, width, 1.0);
+      consider(fmax(t_full + (rem ? KB * est_kblock(pair, width, (double)rem / units) : 0.0), t_hbm) + ends, 0, 0, 0);
+      if (full == 0) {
+        // all tiles cut over K through the workspace
+        if (mt <= units)
+          consider(fmax((double)tiles * KB / ((units / mt) * mt) * est_kblock(pair, width, 1.0), t_hbm) + 11.5 + .05 * width, 0, cols, tmax);
+      } else if (rem) {
+        const int cut = cols - (int)(full * units / mt);
+        int cut_last = 0;
+        for (int cw = fewest; cw <= s.M / 16 && cw <= units; ++cw) {     // token tiles of the cut columns
+          const int ctmax = ((s.M + cw - 1) / cw + gran - 1) / gran * gran;
+          if (ctmax == cut_last || ctmax > width) continue;
+          cut_last = ctmax;
+          int c_width, c_mt;
+          token_tiles(s.M, ctmax, gran, &c_width, &c_mt);
+          if (c_mt > units || c_mt * cut * (pair + 1) > kSplitCounters) continue;
+          const int per = cut_range(cut, c_mt, KB, units), parts = (KB + per - 1) / per + 1;
+          // (6 %: below that the cut lost as often as it won; under the power limit a ragged wave's idle time is given back as
+          // clock.  28672 features, 256 tokens: 60 us cut, 56 whole; the LM head at 480: 384 and 375.)
+          // reducing (the parts of a chunk fetched one after the other) holds the reducing unit's epilogue; what exceeds the main
+          // loop of its next tile holds its products, too
+          const double hand = (c_width + 31) / 32 * (.6 + 1.3 * parts);
+          const double t = t_full + per * est_kblock(pair, c_width, 1.0) + 3.0 + fmax(0.0, hand - KB * est_kblock(pair, width, 1.0));
+          consider(1.06 * (fmax(t, t_hbm) + ends), 0, cut, ctmax);
+        }
+      }
       // clusters of 2 to 4 parts per tile, all resident at once
       const int chunks = (width + 31) / 32;
       for (int cl = 2; cl <= 4 && st->clusters; ++cl) {
         if (tiles * cl > units || cl * 4 > KB || !clusters_fit(st, pair, cl * (pair + 1), (int)tiles)) break;
-        const double ends = chunks == 1 ? 6.0 : 6.5 + (double)chunks * (cl - 1) / cl;
-        consider(fmax((KB + cl - 1) / cl * est_kblock(pair, width, (double)tiles * cl / units), t_hbm) + ends, true, cl);
+        const double cl_ends = chunks == 1 ? 6.0 : 6.5 + (double)chunks * (cl - 1) / cl;
+        consider(fmax((KB + cl - 1) / cl * est_kblock(pair, width, (double)tiles * cl / units), t_hbm) + cl_ends, cl, 0, 0);
       }
     }
   }
+  if (st->configs.size() >= kMapCacheMax) st->configs.clear();
+  st->configs.emplace(s, best);
   return best;
 }
 
@@ -1234,26 +1277,32 @@ bool launch_config(TcState* st, const GemmArgs& a, const EpiParams& ep, const Co
   token_tiles(a.M, g.tmax, g.gran, &g.width, &g.mt);
   const int width = g.width, mt = g.mt;
   g.x_box = a.m_dev ? 32 / mul : width / mul;
-  CUtensorMap mw, mx;     // copies: see cached_map
-  const WeightOrder order = swiglu ? kWSwiglu : (a.epi == EPI_QKV_ROPE ? (a.head_dim == 128 ? kWRope128 : kWRope64) : kWPlain);
-  if (!get_w_map(st, a.w, w_rows, a.K, order, &mw, &g.w_step3, &g.w_step4)) return false;
-  if (!get_x_map(st, a.x, a.M, a.K, g.x_box, &mx)) return false;
-  const int n_tiles = mt * g.n_cols, KB = a.K / BK;
   const int n_units = c.pair ? st->n_sm / 2 : st->n_sm;       // scheduling units: CTAs or pairs
+  const int n_tiles = mt * g.n_cols, KB = a.K / BK;
   int units = n_tiles < n_units ? n_tiles : n_units;
-  g.dp_tiles = n_tiles;       // whole tiles, strided
-  g.per = 1;
   g.cl = c.cl;
+  g.cut_box = g.x_box;
   if (c.cl) {
     units = n_tiles * c.cl;   // one cluster per tile; the kernel derives each member's k-blocks from its rank
   } else if (a.m_dev) {
-    // the row count is on the device: the kernel counts the tiles and, for stream-K, divides the k-blocks itself; the
-    // grid has every unit (units without work leave at once)
-    g.dp_tiles = c.stream_k ? -2 : -1;
+    // the row count is on the device: the kernel counts the tiles and divides the cut ones itself; the grid has every unit
+    // (units without work leave at once)
+    g.cut_cols = c.cut_cols && (long long)n_tiles * mul <= kSplitCounters ? -1 : 0;
     units = n_units;
-  } else if (c.stream_k) {
-    stream_k_schedule(n_tiles, mt, KB, n_units, &g.dp_tiles, &g.per, &units);     // the caller made sure that mt <= n_units
+  } else if (c.cut_cols) {
+    const int cut_tmax = (c.cut_tmax + g.gran - 1) / g.gran * g.gran;
+    g.cut_cols = c.cut_cols;
+    token_tiles(a.M, cut_tmax < width ? cut_tmax : width, g.gran, &g.cut_width, &g.cut_mt);
+    g.cut_box = g.cut_width / mul;
+    if (g.cut_mt > n_units || g.cut_mt * g.cut_cols * mul > kSplitCounters) return false;
+    g.per = cut_range(g.cut_cols, g.cut_mt, KB, n_units);
+    const int whole = (g.n_cols - g.cut_cols) * mt, used = (g.cut_cols * KB + g.per - 1) / g.per * g.cut_mt;
+    units = whole > used ? (whole < n_units ? whole : n_units) : used;
   }
+  CUtensorMap mw, mx, mxc;     // copies: see cached_map
+  const WeightOrder order = swiglu ? kWSwiglu : (a.epi == EPI_QKV_ROPE ? (a.head_dim == 128 ? kWRope128 : kWRope64) : kWPlain);
+  if (!get_w_map(st, a.w, w_rows, a.K, order, &mw, &g.w_step3, &g.w_step4)) return false;
+  if (!get_x_map(st, a.x, a.M, a.K, g.x_box, &mx) || !get_x_map(st, a.x, a.M, a.K, g.cut_box, &mxc)) return false;
   g.split_ws = st->split_ws;
   g.split_counters = st->split_counters;
   g.m_dev = a.m_dev;
@@ -1281,8 +1330,8 @@ bool launch_config(TcState* st, const GemmArgs& a, const EpiParams& ep, const Co
   }
   cfg.attrs = attr;
   cfg.numAttrs = n_attr;
-  return (c.pair ? cudaLaunchKernelEx(&cfg, gemm_tc_kernel<true>, mw, mx, g, ep)
-                 : cudaLaunchKernelEx(&cfg, gemm_tc_kernel<false>, mw, mx, g, ep)) == cudaSuccess;
+  return (c.pair ? cudaLaunchKernelEx(&cfg, gemm_tc_kernel<true>, mw, mx, mxc, g, ep)
+                 : cudaLaunchKernelEx(&cfg, gemm_tc_kernel<false>, mw, mx, mxc, g, ep)) == cudaSuccess;
 }
 
 }  // namespace
@@ -1315,6 +1364,7 @@ void tc_state_force(void* s, int tile, int stream_k) {
   st->force_tile = tile;
   st->force_s = stream_k;
   st->clusters = stream_k != 2;     // 2: cut tiles always go through the partial-tile workspace
+  st->configs.clear();
 }
 
 void tc_state_reset(void* s, cudaStream_t stream) {
@@ -1401,19 +1451,21 @@ bool launch_gemm_tc(const GemmArgs& a, void* tc_state, int* status, cudaStream_t
   Config c = choose_config(st, Shape{Mc, n_feat, a.K});
   if (st->force_tile || st->force_s == 1) {   // debugging aid: single CTAs (64, 128, 256 tokens) or pairs (384: 128, 512: 256 tokens)
     const int f = st->force_tile;
-    if (f) {
-      const bool pair = f > 256;
-      const int tmax = f == 384 ? 128 : (f == 512 ? 256 : f);
-      if ((long long)((a.M + tmax - 1) / tmax) * ((n_feat + FT - 1) / FT + 1) * 2 <= kSplitCounters) c = Config{pair, false, tmax, 0};
-    }
+    if (f) c = Config{f > 256, f == 384 ? 128 : (f == 512 ? 256 : f), 0, 0, 0};
     const int gran = c.pair ? 32 : 16, units = c.pair ? st->n_sm / 2 : st->n_sm;
     int width, mt;
     token_tiles(a.M, c.tmax, gran, &width, &mt);
-    c.stream_k = st->force_s != 0 && mt <= units;
+    const int cols = (n_feat + FT * (c.pair + 1) - 1) / (FT * (c.pair + 1)), tiles = mt * cols;
     c.cl = 0;
-    const int tiles = mt * ((n_feat + FT * (c.pair + 1) - 1) / (FT * (c.pair + 1)));
-    for (int cl = 4; cl >= 2 && c.stream_k && st->clusters && !c.cl; --cl)
-      if (tiles * cl <= units && cl * 4 <= a.K / BK && clusters_fit(st, c.pair, cl * (c.pair + 1), tiles)) c.cl = cl;
+    c.cut_cols = 0;
+    c.cut_tmax = c.tmax;
+    if (st->force_s) {
+      for (int cl = 4; cl >= 2 && st->clusters && !c.cl; --cl)
+        if (tiles * cl <= units && cl * 4 <= a.K / BK && clusters_fit(st, c.pair, cl * (c.pair + 1), tiles)) c.cl = cl;
+      // else all columns of less than two waves, or the last one-to-two waves of more
+      const int cut = tiles < 2 * units ? cols : cols - (tiles / units - 1) * units / mt;
+      if (!c.cl && mt <= units && mt * cut * (c.pair + 1) <= kSplitCounters) c.cut_cols = cut;
+    }
   }
   if (ss_slots_out) *ss_slots_out = (a.N + FT - 1) / FT;
   return launch_config(st, a, ep, c, stream);

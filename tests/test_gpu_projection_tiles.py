@@ -83,3 +83,38 @@ def test_step_of_a_model_that_fills_no_tile(head_dim, n_q, n_kv, force):
                 assert np.max(np.abs(f64(vg) - V[L[r]:])) <= HID_TOL * np.max(np.abs(V[L[r]:])), (specs, r, l)
             t0 += n
         ctx.recg_free()
+
+
+@pytest.mark.parametrize("M,N,K", [(333, 19088, 2048), (376, 9600, 4096), (700, 14336, 4096), (701, 19088, 2048)])
+def test_ragged_end_cut_in_narrower_tiles(M, N, K):
+    """Sizes at which the columns of the last wave are cut over K, in token tiles narrower than the others' (one to seven such
+    columns, two to eight parts per tile, the last feature tile half empty)."""
+    ctx = binding.Context(binding.make_config(synth.tiny_shape(), 1, 8, 1))
+    g = torch.Generator().manual_seed(M)
+    w = (torch.randn((N, K), generator=g) * 0.05).to(torch.bfloat16).cuda()
+    x = torch.randn((M, K), generator=g).to(torch.bfloat16).cuda()
+    ref = f64(x.double() @ w.double().T)
+    for rep in range(2):
+        got = f64(ctx.recg_linear(x, w))
+        # fp32 sums of 4096 exact bf16 products: sqrt(K) 2^-24 = 4e-6 of the largest
+        assert np.max(np.abs(got - ref)) <= 1e-5 * np.max(np.abs(ref)), rep
+    ctx.recg_free()
+
+
+@pytest.mark.parametrize("n", [333, 376])
+def test_ragged_end_cut_of_a_whole_step(n):
+    """The same division inside a step: 28672 gate and up rows of 2048 at these row counts (SwiGLU epilogue, RMSNorm folded)."""
+    shape = synth.ModelShape(n_layers=1, hidden=2048, n_q_heads=4, n_kv_heads=1, head_dim=128, ffn=14336, vocab=2064)
+    W = synth.model_weights(shape, seed=0, dtype=torch.bfloat16)
+    ctx = binding.Context(binding.make_config(shape, 1, n, 64), to_dev(W))
+    desc = synth.fixed_descriptor([0], [n], [0], seed=9)
+    pool = binding.alloc_kv_pool(ctx, desc.n_pages, fill=None)
+    pool.fill_(float("nan"))
+    y = synth.token_ids(n, shape.vocab, seed=1).tolist()
+    batch = binding.Batch(desc.ctx_len, desc.verify_len, desc.block_size, y, desc.page_table, pool, desc.n_pages)
+    logits = f64(ctx.logits_tensor(ctx.recg_step(batch)))
+    ctx.recg_sync()
+    none = (np.zeros((0, 1, 128)), np.zeros((0, 1, 128)))
+    ref, _, _ = orc.fused_round_cached(oracle_cfg(shape), oracle_weights(W), [none], 0, y, 0)
+    assert np.max(np.abs(logits - ref)) <= HID_TOL * np.max(np.abs(ref))
+    ctx.recg_free()
