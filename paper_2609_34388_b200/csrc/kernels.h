@@ -54,14 +54,35 @@ struct BatchLayout {
   AttnTile* tiles;
   int* tile_off;    // [C+1] first tile entry of each request
   int* cta_off;     // [4 n_ctas] per CTA of the persistent attention grid: the two item index ranges [b0, e0), [b1, e1) it walks
+#ifdef __CUDACC__
+  // the descriptor arrays at another address: what lies `from` .. now lies `to` ..
+  __host__ __device__ void rebase(const int* from, const int* to) {
+    ctx_len = to + (ctx_len - from);
+    verify_len = to + (verify_len - from);
+    block_size = to + (block_size - from);
+    corr = to + (corr - from);
+    cu_tok = to + (cu_tok - from);
+    cu_ver = to + (cu_ver - from);
+    verify_tokens = to + (verify_tokens - from);
+    if (page_table) page_table = to + (page_table - from);
+  }
+#endif
   int* counts;      // [0] number of items, [1] number of tiles, [2], [3] cost units per CTA / per CTA pair
   int max_items, max_parts;
 };
 
+// A small batch descriptor as a kernel parameter (n = 0: none): the kernels that need it first read it from there and leave it in
+// device memory for the others; no copy has to go ahead of them.
+constexpr int kSmallDesc = 255;
+struct SmallDesc {
+  int n;
+  int v[kSmallDesc];
+};
 // S1: per-token arrays and the attention work list (batches with a page table: a verify-only batch needs neither).
 // whole: no tile is cut (attention_whole_tiles), and no combine kernel has to follow the attention kernel.
+// desc (may be null): the descriptor to be written to desc_dev, where bl points.
 void launch_layout(const BatchLayout& bl, const Dims& dm, int tok_per_tile, int n_ctas, bool whole, int64_t n_pages,
-                   int* status, cudaStream_t st);
+                   int* status, int* desc_dev, const SmallDesc* desc, cudaStream_t st);
 // HOST arrays [n_req]; rows: rows per request
 bool attention_whole_tiles(int n_req, const int* ctx_len, const int* rows, int n_kv, int tok_per_tile, int n_ctas);
 // the layout kernel keeps six ints per request in shared memory: requests per step are bounded by this
@@ -209,6 +230,7 @@ struct VerifyBuffers {   // DEVICE outputs (library workspace or caller buffers)
   int *corr_hit, *risky_n, *risky_index, *risky_token;
   int *freed_page_ids;
 };
+// desc: as in launch_layout; null: bl is settled in device memory before these kernels start, or comes from the device (bl.dyn).
 // mirror: byte distance from every output array to its copy in mapped host memory (0: no copy is wanted)
 struct RowPartial {      // per (row, vocab chunk)
   float m1, m2;          // largest and second-largest logit of the chunk
@@ -216,8 +238,8 @@ struct RowPartial {      // per (row, vocab chunk)
   float s, t;            // sum exp(x - m1), sum x exp(x - m1)
 };
 void launch_verify(const BatchLayout& bl, const void* logits, int logits_dtype, int vocab, RowPartial* partials,
-                   int max_chunks_total, const VerifyBuffers& vb, int n_sm, cudaStream_t st,
-                   ptrdiff_t mirror = 0);   // (bl.dyn: rows from the device)
+                   int max_chunks_total, const VerifyBuffers& vb, int* desc_dev, const SmallDesc* desc, int n_sm,
+                   cudaStream_t st, ptrdiff_t mirror = 0);   // (bl.dyn: rows from the device)
 int verify_chunks_per_row(int rows, int vocab, int n_sm);
 
 // Block-size rule (Eq. 2-3): table = [blocks (int) x8 | cost x8 | edges x64 | value n_blocks*n_bins*n_blocks*2]

@@ -110,7 +110,8 @@ __device__ __forceinline__ void layout_tokens(const BatchLayout& bl, const int* 
 }
 
 __global__ void __launch_bounds__(kLayoutThreads) layout_kernel(BatchLayout bl, int n_kv, int mask_id, int tok_per_tile,
-                                                                int n_ctas, int whole, int64_t n_pages, int* status) {
+                                                                int n_ctas, int whole, int64_t n_pages, int* status, int* desc_dev,
+                                                                const __grid_constant__ SmallDesc desc) {
   extern __shared__ int sm[];
   const int C = bl.n_req;
   const int max_pairs = n_ctas / 2;
@@ -127,6 +128,11 @@ __global__ void __launch_bounds__(kLayoutThreads) layout_kernel(BatchLayout bl, 
   const int tid = threadIdx.x;
   griddep_launch();
   griddep_wait();   // the previous step's kernels may still be reading the arrays this kernel rewrites
+  if (desc.n) {     // (no copy went ahead of this kernel: it reads the descriptor from its parameters and leaves it for the others)
+    bl.rebase(desc_dev, desc.v);
+    if (blockIdx.x == 0)
+      for (int i = tid; i < desc.n; i += kLayoutThreads) desc_dev[i] = desc.v[i];
+  }
   for (int r = tid; r <= C; r += kLayoutThreads) cu_tok[r] = bl.cu_tok[r];
 
   // ---- per-token arrays ----
@@ -502,12 +508,14 @@ bool attention_whole_tiles(int n_req, const int* ctx_len, const int* rows, int n
 }
 
 void launch_layout(const BatchLayout& bl, const Dims& dm, int tok_per_tile, int n_ctas, bool whole, int64_t n_pages,
-                   int* status, cudaStream_t st) {
+                   int* status, int* desc_dev, const SmallDesc* desc, cudaStream_t st) {
+  static const SmallDesc none{};
   const size_t smem = layout_smem_bytes(bl.n_req, n_ctas);
   static bool configured[kMaxDevices] = {false};
   if (first_use_on_device(configured))    // room for kMaxLayoutRequests requests (the default limit is 48 KB)
     cudaFuncSetAttribute(layout_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)layout_smem_bytes(kMaxLayoutRequests, 1024));
-  launch_pdl(layout_kernel, dim3(1 + (bl.n_tok + kLayoutThreads - 1) / kLayoutThreads), dim3(kLayoutThreads), smem, st, bl, dm.n_kv, dm.mask_id, tok_per_tile, n_ctas, whole ? 1 : 0, n_pages, status);
+  launch_pdl(layout_kernel, dim3(1 + (bl.n_tok + kLayoutThreads - 1) / kLayoutThreads), dim3(kLayoutThreads), smem, st, bl, dm.n_kv, dm.mask_id, tok_per_tile, n_ctas, whole ? 1 : 0, n_pages, status,
+             desc_dev, desc ? *desc : none);
 }
 
 void launch_embed(const BatchLayout& bl, const Dims& dm, const void* embed, float* h, const void* gain, void* x, float* ss,

@@ -324,12 +324,14 @@ __host__ __device__ inline int stat_lanes(int chunks) {
 constexpr int kFinalThreads = 256, kFinalRows = 256;
 __global__ void __launch_bounds__(kFinalThreads) verify_finalize_kernel(BatchLayout bl, const RowPartial* __restrict__ partials,
                                                                         int chunks_per_row, VerifyBuffers vb, int desc_settled,
-                                                                        ptrdiff_t mirror) {
+                                                                        ptrdiff_t mirror, int* desc_dev,
+                                                                        const __grid_constant__ SmallDesc desc) {
   __shared__ int s_top1[kFinalRows], s_top2[kFinalRows], s_vt[kFinalRows];
   __shared__ float s_p1[kFinalRows], s_p2[kFinalRows], s_ent[kFinalRows];
   __shared__ int s_a, s_first_free, s_last;
   griddep_launch();
   if (!desc_settled) griddep_wait();
+  if (desc.n) bl.rebase(desc_dev, desc.v);
   const int r = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int t0 = bl.cu_tok[r], tv0 = bl.cu_ver[r];
   const int n = bl.cu_tok[r + 1] - t0;          // v + b + n_corr * span; 0 in a round that broke a capacity on the device
@@ -340,6 +342,8 @@ __global__ void __launch_bounds__(kFinalThreads) verify_finalize_kernel(BatchLay
   if (small)
     for (int j = tid; j < v; j += kFinalThreads) s_vt[j] = bl.verify_tokens[tv0 + j];
   if (desc_settled) griddep_wait();
+  if (desc.n && r == 0 && !bl.page_table)      // for the kernels that may follow (the layout kernel has not written it)
+    for (int i = tid; i < desc.n; i += kFinalThreads) desc_dev[i] = desc.v[i];
   auto put = [&](auto* p, auto x) {
     *p = x;
     if (mirror) *reinterpret_cast<decltype(p)>(reinterpret_cast<char*>(p) + mirror) = x;
@@ -457,7 +461,9 @@ int verify_chunks_per_row(int rows, int vocab, int n_sm) {
 }
 
 void launch_verify(const BatchLayout& bl, const void* logits, int logits_dtype, int vocab, RowPartial* partials,
-                   int max_chunks_total, const VerifyBuffers& vb, int n_sm, cudaStream_t st, ptrdiff_t mirror) {
+                   int max_chunks_total, const VerifyBuffers& vb, int* desc_dev, const SmallDesc* desc, int n_sm, cudaStream_t st,
+                   ptrdiff_t mirror) {
+  static const SmallDesc none{};
   const int rows = bl.n_tok;
   if (rows <= 0) return;
   int chunks = verify_chunks_per_row(rows, vocab, n_sm);
@@ -472,10 +478,10 @@ void launch_verify(const BatchLayout& bl, const void* logits, int logits_dtype, 
   else
     launch_pdl(verify_partial_kernel<float>, grid, dim3(kVerifyThreads), 0, st, static_cast<const float*>(logits), vocab,
                chunk_len, chunks, partials, bl.dyn);
-  // (a descriptor that the host uploaded was in place before the vocabulary scan could start; one that a kernel of this
-  // round packs on the device is not)
+  // (a descriptor that the host uploaded was in place before the vocabulary scan could start, and a small one comes with this
+  // launch; one that a kernel of this round packs on the device is not settled before the wait)
   launch_pdl(verify_finalize_kernel, dim3(bl.n_req), dim3(kFinalThreads), 0, st, bl, (const RowPartial*)partials, chunks, vb,
-             bl.dyn ? 0 : 1, mirror);
+             bl.dyn ? 0 : 1, mirror, desc_dev, desc ? *desc : none);
 }
 
 }  // namespace recg
