@@ -160,7 +160,10 @@ def _ptr(a) -> Optional[int]:
         return None
     if isinstance(a, torch.Tensor):
         return a.data_ptr()
-    return a.ctypes.data
+    try:      # a.ctypes.data takes 2.2 us, this .3: more than the launch it precedes (writable, contiguous, not empty)
+        return C.addressof(C.c_char.from_buffer(a))
+    except (TypeError, ValueError, BufferError):
+        return a.ctypes.data
 
 
 class Batch:
@@ -245,9 +248,10 @@ class VerifyOut:
             else:
                 self.bufs[name] = torch.zeros(max(n, 1), dtype=torch.float32 if isf else torch.int32, device="cuda")
             setattr(self.c, name, _ptr(self.bufs[name]))
+        self._views = {k: v[:self.sizes[k]] for k, v in self.bufs.items()}    # (19 slices per call: 4 us of numpy, 45 of torch)
 
     def views(self):
-        return {k: v[:self.sizes[k]] for k, v in self.bufs.items()}
+        return dict(self._views)
 
     def nbytes(self) -> int:
         return 4 * sum(self.sizes.values())
