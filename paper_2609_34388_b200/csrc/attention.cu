@@ -360,8 +360,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attention_kernel(AttnParams P
   }
 }
 
-// Merges the KV-range partials of the tiles that were split.  Tiles with a single part were written by the
-// attention kernel itself and are skipped.  Work unit = 16 rows of a tile, one warp per query row, each lane D/32
+// Merges the KV-range partials of the tiles that were split (`tiles` lists no others: tiles with a single part were written by
+// the attention kernel itself).  Work unit = 16 rows of a tile, one warp per query row, each lane D/32
 // consecutive dims.  Bound by latency, not by its bytes (a tile entry, the (max, sum) pairs and the partial rows are
 // dependent reads): the tile entry is read ahead of the wait where the work list is settled, lane p fetches the pair of part
 // p, so that one read and a few shuffles give all weights of up to 32 parts, and the rows of the first kRows parts are on
@@ -384,7 +384,6 @@ __global__ void __launch_bounds__(512, 2) attention_combine_kernel(const AttnTil
   if (list_settled) griddep_wait();
   for (int wu = blockIdx.x; wu < n_tiles * 8; wu += gridDim.x) {
     if (wu != (int)blockIdx.x) tl = tiles[wu >> 3];
-    if (tl.n_parts <= 1) continue;
     const int rho = (wu & 7) * 16 + warp;
     if (rho >= tl.ntok * group) continue;
     const float* rows = part_o + ((size_t)tl.part_begin * 128 + rho) * D + lane * E;

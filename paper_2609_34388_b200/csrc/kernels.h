@@ -20,7 +20,7 @@ struct AttnItem {
   int part;              // index into the partial buffers, or -1 when the item covers the whole KV range
   int kv_len;            // L + n of the request
 };
-struct AttnTile {        // per (request, kv head, row tile): where its partials are, and which rows it covers
+struct AttnTile {        // a (request, kv head, row tile) that was cut: where its partials are, and which rows it covers
   int part_begin, n_parts;
   int tok0, ntok, kv_head;
 };
@@ -52,7 +52,6 @@ struct BatchLayout {
   // attention work list
   AttnItem* items;
   AttnTile* tiles;
-  int* tile_off;    // [C+1] first tile entry of each request
   int* cta_off;     // [4 n_ctas] per CTA of the persistent attention grid: the two item index ranges [b0, e0), [b1, e1) it walks
 #ifdef __CUDACC__
   // the descriptor arrays at another address: what lies `from` .. now lies `to` ..
@@ -67,7 +66,7 @@ struct BatchLayout {
     if (page_table) page_table = to + (page_table - from);
   }
 #endif
-  int* counts;      // [0] number of items, [1] number of tiles, [2], [3] cost units per CTA / per CTA pair
+  int* counts;      // [0] number of items, [1] number of entries in tiles, [2], [3] cost units per CTA / per CTA pair
   int max_items, max_parts;
 };
 

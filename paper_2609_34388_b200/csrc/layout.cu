@@ -118,10 +118,9 @@ __global__ void __launch_bounds__(kLayoutThreads) layout_kernel(BatchLayout bl, 
   int* cu_tok = sm;                      // [C + 1] rows of the batch in front of request r
   int* seg_a = sm + (C + 1);             // [C + 1] line-A segments in front of request r
   int* seg_b = sm + 2 * (C + 1);         // [C + 1] line-B segments
-  int* tile_off = sm + 3 * (C + 1);      // [C + 1] first tile entry
-  int* ctx = sm + 4 * (C + 1);           // [C]
-  int* vis = sm + 5 * (C + 1);           // [C] verify rows (causal) of request r
-  int* a_off = sm + 6 * (C + 1);         // [max_pairs + 1] first line-A piece of every CTA pair
+  int* ctx = sm + 3 * (C + 1);           // [C]
+  int* vis = sm + 4 * (C + 1);           // [C] verify rows (causal) of request r
+  int* a_off = sm + 5 * (C + 1);         // [max_pairs + 1] first line-A piece of every CTA pair
   int* b_off = a_off + (max_pairs + 1);  // [n_ctas + 1]  first line-B piece of every line-B CTA
   __shared__ int scratch[3][33];
   __shared__ long long s_cost[2];
@@ -155,23 +154,18 @@ __global__ void __launch_bounds__(kLayoutThreads) layout_kernel(BatchLayout bl, 
     const int r = r0 + tid;
     const int rt = r < C ? (cu_tok[r + 1] - cu_tok[r] + tok_per_tile - 1) / tok_per_tile : 0;
     Scan3 tot;
-    const Scan3 e = block_scan(Scan3{n_kv * (rt / 2), n_kv * (rt & 1), n_kv * rt}, &tot, scratch);
+    const Scan3 e = block_scan(Scan3{n_kv * (rt / 2), n_kv * (rt & 1), 0}, &tot, scratch);
     if (r < C) {
       seg_a[r] = carry.a + e.a;
       seg_b[r] = carry.b + e.b;
-      tile_off[r] = carry.c + e.c;
-      bl.tile_off[r] = carry.c + e.c;
     }
     carry.a += tot.a;
     carry.b += tot.b;
-    carry.c += tot.c;
   }
-  const int n_seg_a = carry.a, n_seg_b = carry.b, n_tiles = carry.c;
+  const int n_seg_a = carry.a, n_seg_b = carry.b;
   if (tid == 0) {
     seg_a[C] = n_seg_a;
     seg_b[C] = n_seg_b;
-    tile_off[C] = n_tiles;
-    bl.tile_off[C] = n_tiles;
   }
   __syncthreads();
   // segment s of a line: its request, kv head, (first) tile and KV blocks
@@ -213,7 +207,9 @@ __global__ void __launch_bounds__(kLayoutThreads) layout_kernel(BatchLayout bl, 
   const int per_b = n_ctas_b > 0 && wb > 0 ? (int)((wb + n_ctas_b - 1) / n_ctas_b) : 0x3fffffff;
 
   // Lines A, then B: offsets by scans over the segments, then every thread emits the pieces of its segment.
-  int n_pieces_a = 0, n_pieces_b = 0, parts = 0;
+  // The tiles that are cut are listed one behind the other for the combine kernel: with all tiles in the list it took 23 us per
+  // layer of 128 requests, 27 dependent reads of entries of which one in ten was cut.
+  int n_pieces_a = 0, n_pieces_b = 0, parts = 0, n_cut = 0;
   bool overflow = too_long;
   // pass 0 counts line A's pieces (the second siblings' items lie behind all first ones), passes 1 and 2 emit
   for (int pass = too_long ? 3 : 0; pass < 3; ++pass) {
@@ -233,26 +229,30 @@ __global__ void __launch_bounds__(kLayoutThreads) layout_kernel(BatchLayout bl, 
       off += tot.a;
       const int c_first = whole ? s : g0 / per, c_last = whole ? s : (g0 + g.nb - 1) / per;
       const int np = s < n_seg ? c_last - c_first + 1 : 0;
-      const Scan3 e2 = block_scan(Scan3{np, np > 1 ? (pair ? 2 * np : np) : 0, 0}, &tot, scratch);
-      const int item0 = pieces + e2.a;
+      const int cut_tiles = np > 1 ? (pair ? 2 : 1) : 0;
+      const Scan3 e2 = block_scan(Scan3{np, cut_tiles * np, cut_tiles}, &tot, scratch);
+      const int item0 = pieces + e2.a, cut0 = n_cut + e2.c;
       int part = parts + e2.b;
       pieces += tot.a;
-      if (pass > 0) parts += tot.b;
+      if (pass > 0) {
+        parts += tot.b;
+        n_cut += tot.c;
+      }
       if (pass == 0 || s >= n_seg) continue;
       // first piece of every owner: an owner without pieces starts where the next one does
       const int c_prev = s == 0 || whole ? s - 1 : (g0 - kItemCost - 1) / per;     // owner of the last block of the segment before
       for (int c = c_prev + 1; c <= c_last && c <= n_owners; ++c) owner_off[c] = c <= c_first ? item0 : item0 + (c - c_first);
       if (s == n_seg - 1)
         for (int c = c_last + 1; c <= n_owners; ++c) owner_off[c] = item0 + np;
-      const int n = cu_tok[g.r + 1] - cu_tok[g.r], kv_len = ctx[g.r] + n, rt = (n + tok_per_tile - 1) / tok_per_tile;
+      const int n = cu_tok[g.r + 1] - cu_tok[g.r], kv_len = ctx[g.r] + n;
       for (int sib = 0; sib < (pair ? 2 : 1); ++sib) {
         AttnTile tl;
-        tl.part_begin = np > 1 ? part : -1;
+        tl.part_begin = part;
         tl.n_parts = np;
         tl.tok0 = cu_tok[g.r] + (g.tile + sib) * tok_per_tile;
         tl.ntok = min(tok_per_tile, n - (g.tile + sib) * tok_per_tile);
         tl.kv_head = g.kvh;
-        bl.tiles[tile_off[g.r] + g.kvh * rt + g.tile + sib] = tl;
+        if (np > 1) bl.tiles[cut0 + sib] = tl;
         const int at = pair ? (sib ? n_pieces_a : 0) + item0 : 2 * n_pieces_a + item0;
         for (int c = c_first; c <= c_last; ++c) {
           AttnItem a;
@@ -277,7 +277,7 @@ __global__ void __launch_bounds__(kLayoutThreads) layout_kernel(BatchLayout bl, 
   if (tid == 0) {
     if (overflow) set_status(status, DEV_BAD_INDEX);
     bl.counts[0] = overflow ? 0 : 2 * n_pieces_a + n_pieces_b;
-    bl.counts[1] = n_tiles;
+    bl.counts[1] = overflow ? 0 : n_cut;
     bl.counts[2] = per_b;
     bl.counts[3] = per_a;
   }
@@ -488,7 +488,7 @@ __global__ void __launch_bounds__(kKvIoThreads) kv_io_kernel(__nv_bfloat16* pool
 }  // namespace
 
 size_t layout_smem_bytes(int n_req, int n_ctas) {
-  return (6 * (size_t)(n_req + 1) + (size_t)(n_ctas / 2 + 1) + (size_t)(n_ctas + 1)) * sizeof(int);
+  return (5 * (size_t)(n_req + 1) + (size_t)(n_ctas / 2 + 1) + (size_t)(n_ctas + 1)) * sizeof(int);
 }
 
 // Whole tiles against work cut evenly.  A tile's 64-token block takes about .5 us of its CTA; cutting costs the write of the

@@ -141,7 +141,6 @@ size_t carve(recg_ctx* c, DeviceArena& A) {
   bl.max_items = (int)(4 * c->target_items + max_tiles);
   bl.items = A.take<AttnItem>(bl.max_items);
   bl.tiles = A.take<AttnTile>(max_tiles);
-  bl.tile_off = A.take<int>(Cm + 1);
   bl.cta_off = A.take<int>(4 * (c->target_items + 1));
   bl.counts = A.take<int>(4);
   c->d_status = A.take<int>(1);
