@@ -226,9 +226,8 @@ __global__ void __launch_bounds__(kThreads, 1) attention_tc_kernel(const __grid_
   auto item_at = [&](int i) { return i < range_n0 ? range_b0 + i : range_b1 + (i - range_n0); };
   AttnItem w_next = {};
   if (warp == 0) {
-    // (inside a step the work list was written many launches ago and the kernel in front of this one, the QKV
-    // projection, only signals its dependents after its own wait: the reads below then overlap that kernel instead of
-    // following it)
+    // (behind the first layer of a step the work list was written a whole layer of kernels ago, each of which fills the SMs:
+    // the reads below then overlap the kernel in front of this one instead of following it)
     if (!P.early_desc) griddep_wait();
     const int4 r4 = *reinterpret_cast<const int4*>(P.cta_off + 4 * blockIdx.x);
     range_b0 = r4.x;

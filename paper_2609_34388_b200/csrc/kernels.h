@@ -79,23 +79,24 @@ struct SmallDesc {
 };
 // S1: per-token arrays and the attention work list (batches with a page table: a verify-only batch needs neither).
 // whole: no tile is cut (attention_whole_tiles), and no combine kernel has to follow the attention kernel.
+// tokens: the per-token arrays as well (else launch_embed follows, which fills them).
 // desc (may be null): the descriptor to be written to desc_dev, where bl points.
 void launch_layout(const BatchLayout& bl, const Dims& dm, int tok_per_tile, int n_ctas, bool whole, int64_t n_pages,
-                   int* status, int* desc_dev, const SmallDesc* desc, cudaStream_t st);
+                   int* status, bool tokens, int* desc_dev, const SmallDesc* desc, cudaStream_t st);
 // HOST arrays [n_req]; rows: rows per request
 bool attention_whole_tiles(int n_req, const int* ctx_len, const int* rows, int n_kv, int tok_per_tile, int n_ctas);
-// the layout kernel keeps six ints per request in shared memory: requests per step are bounded by this
+// the layout kernel keeps five ints per request in shared memory: requests per step are bounded by this
 constexpr int kMaxLayoutRequests = 4096;
 size_t layout_smem_bytes(int n_req, int n_ctas);
 // debug checks
 void launch_guard_fill(void* base, const size_t* offs_dev, int n, cudaStream_t st);
 void launch_guard_check(const void* base, const size_t* offs_dev, int n, int* status, cudaStream_t st);
 void launch_wait_timeout(uint32_t max_polls, int* status, cudaStream_t st);
-// S2: h[t] = embed[tok_id[t]] (fp32 residual stream), the rotary table (cos, sin) of pos * base^(-2i/d) as float2
+// S2, right behind launch_layout: the per-token arrays, h[t] = embed[tok_id[t]] (fp32 residual stream), the rotary table (cos, sin) of pos * base^(-2i/d) as float2
 // [T][head_dim/2], and the input of the first normalised projection: x[t] = rmsnorm(h[t]) * gain, or with
 // ss != null (folded RMSNorm) x[t] = bf16(h[t] * gain) and ss[t] = sum h[t]^2 (one slot).
 void launch_embed(const BatchLayout& bl, const Dims& dm, const void* embed, float* h, const void* gain, void* x, float* ss,
-                  void* rope_cs, cudaStream_t st);
+                  void* rope_cs, int64_t n_pages, int* status, const int* desc_dev, const SmallDesc* desc, cudaStream_t st);
 // x = rmsnorm(h) * g, bf16 out.  rows_dev (may be null): the true row count on the device (rows is then the capacity).
 void launch_rmsnorm(const float* h, const void* gain, void* x, int rows, int hidden, float eps, cudaStream_t st,
                     const int* rows_dev = nullptr);

@@ -318,7 +318,19 @@ recg_status pack_batch(recg_ctx* ctx, const recg_batch* b, bool need_pages, bool
   return RECG_OK;
 }
 
-recg_status upload_and_layout(recg_ctx* ctx, const recg_batch* b, bool need_pages, bool need_tokens = true) {
+// The embedding kernel of a forward pass, right behind its layout kernel (on the tcgen05 path RMSNorm is folded into the
+// projections: whoever writes the residual stream also writes x = bf16(h * gain of the next norm) and partial sums of squares
+// per row, and the projection that reads x scales its accumulator rows by the row's rstd; the mma.sync projections of
+// RECG_FLAG_SIMT_GEMM run it as a kernel of its own).
+bool folds_norm(const recg_ctx* ctx) { return ctx->tc_state && !(ctx->cfg.flags & RECG_FLAG_SIMT_GEMM); }
+void embed_tokens(recg_ctx* ctx, int64_t n_pages) {
+  const Dims& d = ctx->dm;
+  launch_embed(ctx->bl, d, ctx->embed, ctx->h, d.n_layers > 0 ? ctx->attn_norm[0] : ctx->final_norm, ctx->x,
+               folds_norm(ctx) ? ctx->ss : nullptr, ctx->rope_cs, n_pages, ctx->d_status, ctx->d_desc,
+               ctx->small_desc.n ? &ctx->small_desc : nullptr, ctx->stream);
+}
+
+recg_status upload_and_layout(recg_ctx* ctx, const recg_batch* b, bool need_pages, bool need_tokens = true, bool forward = false) {
   int T = 0, Tv = 0;
   ctx->layout_valid = false;
   recg_status s = pack_batch(ctx, b, need_pages, need_tokens, &T, &Tv);
@@ -340,7 +352,8 @@ recg_status upload_and_layout(recg_ctx* ctx, const recg_batch* b, bool need_page
     for (int r = 0; r < b->n_req; ++r) ctx->h_rows[r] = request_rows(b, r);
     ctx->layout_whole = attention_whole_tiles(b->n_req, b->ctx_len, ctx->h_rows.data(), ctx->dm.n_kv, ctx->tok_per_tile, ctx->target_items);
     launch_layout(ctx->bl, ctx->dm, ctx->tok_per_tile, ctx->target_items, ctx->layout_whole, n_pages, ctx->d_status,
-                  ctx->d_desc, small ? &ctx->small_desc : nullptr, ctx->stream);
+                  !forward, ctx->d_desc, small ? &ctx->small_desc : nullptr, ctx->stream);
+    if (forward) embed_tokens(ctx, n_pages);
   }
   CU(cudaGetLastError());
   ctx->layout_valid = true;
@@ -535,7 +548,7 @@ recg_status recg_sync(recg_ctx* ctx) {
   return RECG_OK;
 }
 
-// The forward over the batch laid out last (ctx->bl): embedding, the layers, final norm and LM head.  m_hint: device-
+// The forward over the batch laid out and embedded last (ctx->bl): the layers, final norm and LM head.  m_hint: device-
 // resident rounds only, the row count the projections' tile configurations are chosen for.
 static recg_status run_forward(recg_ctx* ctx, void* kv_pool, int64_t kv_pool_pages, int m_hint, recg_logits* logits) {
   recg_status s = RECG_OK;
@@ -543,20 +556,14 @@ static recg_status run_forward(recg_ctx* ctx, void* kv_pool, int64_t kv_pool_pag
   const BatchLayout& bl = ctx->bl;
   const int T = bl.n_tok;
   cudaStream_t st = ctx->stream;
-  // RMSNorm is folded into the projections of the tcgen05 path: whoever writes the residual stream also writes x =
-  // bf16(h * gain of the next norm) and partial sums of squares per row, and the projection that reads x scales its
-  // accumulator rows by the row's rstd.  (The mma.sync projections of RECG_FLAG_SIMT_GEMM run it as a kernel of its own.)
   // (RECG_FLAG_CHAIN: steps of at most 128 rows run the projections between two attention calls as one persistent kernel)
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   const bool chain = ctx->chain_state && !bl.dyn && T <= 128 && d.n_layers > 0 && (d.n_q * d.head_dim) % 64 == 0 &&
                      d.hidden % 128 == 0 && d.ffn % 64 == 0 &&
                      cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
-  const bool fold = ctx->tc_state && !(ctx->cfg.flags & RECG_FLAG_SIMT_GEMM);
+  const bool fold = folds_norm(ctx);
   const int Tm = ctx->cfg.max_tokens;
-  const void* first_gain = d.n_layers > 0 ? ctx->attn_norm[0] : ctx->final_norm;
-  launch_embed(bl, d, ctx->embed, ctx->h, first_gain, ctx->x, fold ? ctx->ss : nullptr, ctx->rope_cs, st);
-  int slots = 1;
-  CU(cudaGetLastError());
+  int slots = 1;                         // (the embedding kernel's sums of squares)
   ctx->mark(0, 2);
   const int qdim = d.n_q * d.head_dim;
   int n_proj = 0;                        // projections enqueued so far in this step
@@ -595,8 +602,11 @@ static recg_status run_forward(recg_ctx* ctx, void* kv_pool, int64_t kv_pool_pag
     if ((s = run_gemm(ctx, a)) != RECG_OK) return s;
     ctx->mark(2, 1);
     }
+    // (The first layer's attention kernel may be resident while the work list is still being built: idle lanes of a projection
+    // signal its dependents before the projection has waited.  It waits before it reads the list; behind a whole layer of
+    // kernels that fill every SM the list is settled.)
     launch_attention(bl, d, l, ctx->q, ctx->o, kv_pool, kv_pool_pages, ctx->part_o, ctx->part_ml,
-                     ctx->tok_per_tile, ctx->n_sm, ctx->d_status, st, !(ctx->cfg.flags & RECG_FLAG_SIMT_ATTENTION), fold, ctx->layout_whole);
+                     ctx->tok_per_tile, ctx->n_sm, ctx->d_status, st, !(ctx->cfg.flags & RECG_FLAG_SIMT_ATTENTION), fold && l > 0, ctx->layout_whole);
     CU(cudaGetLastError());
     ctx->mark(3, ctx->layout_whole ? 1 : 2);
     if (chain) {
@@ -673,7 +683,7 @@ recg_status recg_step(recg_ctx* ctx, const recg_batch* batch, recg_logits* logit
   if (!ctx->has_weights) return fail(ctx, RECG_ERR_INVALID_ARG, "recg_step: the context was created without weights");
   ctx->logits_valid = false;
   ctx->mark(-1);
-  recg_status s = upload_and_layout(ctx, batch, true);
+  recg_status s = upload_and_layout(ctx, batch, true, true, true);
   if (s != RECG_OK) return s;
   return run_forward(ctx, batch->kv_pool, batch->kv_pool_pages, 0, logits);
 }
@@ -733,8 +743,9 @@ recg_status recg_step_device(recg_ctx* ctx, const recg_device_batch* b, recg_log
   bl.risk_delta = 0.5f;
   launch_pack_device(device_round(ctx, b), ctx->d_desc, ctx->d_dyn, ctx->d_status, ctx->stream);
   ctx->layout_whole = false;           // (the lengths are on the device)
-  launch_layout(bl, ctx->dm, ctx->tok_per_tile, ctx->target_items, false, b->kv_pool_pages, ctx->d_status, ctx->d_desc, nullptr, ctx->stream);
+  launch_layout(bl, ctx->dm, ctx->tok_per_tile, ctx->target_items, false, b->kv_pool_pages, ctx->d_status, false, ctx->d_desc, nullptr, ctx->stream);
   ctx->small_desc.n = 0;
+  embed_tokens(ctx, b->kv_pool_pages);
   CU(cudaGetLastError());
   ctx->layout_valid = true;
   ctx->layout_has_pages = true;

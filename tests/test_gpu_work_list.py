@@ -1,10 +1,15 @@
 """The attention work list where its segments change: causal chunks around the 32-token tiles, their pairs and the 64-token
 KV blocks (early tiles of a chunk read fewer blocks than late ones), and more requests and segments than the list's CTA has
 threads."""
+import numpy as np
 import pytest
+import torch
 
-from paper_2609_34388_b200 import synth
+from oracle import recg_oracle as orc
+from paper_2609_34388_b200 import binding, synth
+from tests._util import f64, oracle_cfg, oracle_weights
 from tests.test_gpu_ops import ATTN_TOL, run_attention_case
+from tests.test_gpu_step import HID_TOL, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -28,3 +33,36 @@ def test_whole_tiles_of_short_contexts(reqs):
     """On both sides of the rule that leaves tiles uncut: about six blocks of context, and as many tiles as CTAs."""
     for shape in (synth.llama8b_shape(1), synth.tiny_shape()):
         assert run_attention_case(shape, reqs, seed=len(reqs) + reqs[0][0]) < ATTN_TOL
+
+
+@pytest.mark.parametrize("n_req", [2, 257, 300, 513])
+def test_tokens_of_many_requests(n_req):
+    """A whole step finds every row's request among more requests than the embedding kernel's CTA has threads (256), some of
+    one row, some that only draft: the rows of the first and last request and of those around the 256th and 512th."""
+    shape = synth.ModelShape(n_layers=1, hidden=128, n_q_heads=2, n_kv_heads=1, head_dim=64, ffn=256, vocab=512)
+    W = synth.model_weights(shape, seed=0, dtype=torch.bfloat16)
+    v = [0 if r % 7 == 3 else 1 + r % 2 for r in range(n_req)]
+    b = [2 if v[r] == 0 or r % 3 == 0 else 0 for r in range(n_req)]
+    L = [r % 5 for r in range(n_req)]
+    desc = synth.fixed_descriptor(L, v, b, seed=9)
+    ctx = binding.Context(binding.make_config(shape, n_req, desc.n_tokens, desc.page_table.shape[1]), to_dev(W))
+    pool = binding.alloc_kv_pool(ctx, desc.n_pages, fill=None)
+    pool.fill_(float("nan"))
+    checked = [r for r in (0, 1, 254, 255, 256, 257, 258, 511, 512, n_req - 1) if r < n_req]
+    kvs, ys = {}, []
+    for r in range(n_req):
+        ys.append(synth.token_ids(v[r], shape.vocab, seed=r + 1).tolist() if v[r] else [])
+        K, V = synth.kv_values(max(L[r], 1), 1, 64, seed=r)
+        kvs[r] = (K[:L[r]], V[:L[r]])
+        if L[r]:
+            ctx.recg_kv_write(pool, desc.n_pages, 0, desc.page_table[r], 0, kvs[r][0].cuda(), kvs[r][1].cuda())
+    batch = binding.Batch(desc.ctx_len, desc.verify_len, desc.block_size, [t for y in ys for t in y], desc.page_table, pool, desc.n_pages)
+    logits = f64(ctx.logits_tensor(ctx.recg_step(batch)))
+    ctx.recg_sync()
+    first = np.concatenate([[0], np.cumsum(np.array(v) + np.array(b))])
+    for r in checked:
+        K, V = kvs[r]
+        ref, _, _ = orc.fused_round_cached(oracle_cfg(shape), oracle_weights(W), [(K.double().numpy(), V.double().numpy())], L[r], ys[r], b[r])
+        got = logits[first[r]:first[r + 1]]
+        assert np.max(np.abs(got - ref)) <= HID_TOL * np.max(np.abs(ref)), r
+    ctx.recg_free()
