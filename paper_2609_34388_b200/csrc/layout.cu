@@ -24,8 +24,10 @@ __device__ __forceinline__ int upper_request(const int* cu, int n_req, int t) {
 // 2 j and 2 j + 1 of a kv head are "siblings": they read the same K/V.  A tile reads the 64-token KV blocks up to the last
 // position that one of its rows may see (verify rows are causal, so the early tiles of a long chunk of prompt need fewer
 // blocks than the late ones; siblings share the range of the later one).  Two lines of KV blocks are built, every tile
-// preceded by kItemCost virtual blocks that stand for the fixed cost of starting an item (fetching Q, refilling and draining
-// the pipeline):
+// preceded by virtual blocks that stand for the fixed cost of starting an item (fetching Q, refilling and draining the
+// pipeline; kItemCostPair, kItemCostSingle, in blocks: the blocks of a pair take less time, every second one comes from L2.
+// Attention of a layer with 4 for both / 6 and 4 / 8 and 4: two chunks of 1000 prompt tokens 158 / 143 / 143 us, eight requests
+// with two branches each 79.9 / 73.9 / 72.6, sixteen requests 66.7 / 66.7 / 68.0; 6 for both: the last one 67.5):
 //   line A holds one segment per sibling PAIR and is cut into equal contiguous ranges, one per pair of CTAs
 //          (2 p, 2 p + 1): the even CTA works on the first sibling and the odd CTA on the second sibling of the SAME
 //          block ranges, at the same time, so that the second reader of a K/V block finds it in L2;
@@ -42,7 +44,7 @@ __device__ __forceinline__ int upper_request(const int* cu, int n_req, int t) {
 // per-request sums are block-wide scans), and descriptors are read into shared memory once.  Measured before, with one
 // thread per request and sums over the requests in one thread: 5.6 us for one request, 13 us with its attention work list,
 // 58 us for 8448 rows of 256 requests.
-constexpr int kItemCost = 4;
+constexpr int kItemCostPair = 6, kItemCostSingle = 4;
 constexpr int kLayoutThreads = 1024;
 constexpr int kWholeBlocks = 5;
 
@@ -192,7 +194,7 @@ __global__ void __launch_bounds__(kLayoutThreads) layout_kernel(BatchLayout bl, 
     for (int s0 = 0; s0 < n_seg; s0 += kLayoutThreads) {
       const int s = s0 + tid;
       int cost = 0;
-      if (s < n_seg) cost = (line ? segment(seg_b, s, false) : segment(seg_a, s, true)).nb + kItemCost;
+      if (s < n_seg) cost = line ? segment(seg_b, s, false).nb + kItemCostSingle : segment(seg_a, s, true).nb + kItemCostPair;
       cost = __reduce_add_sync(0xffffffffu, cost);
       if ((tid & 31) == 0 && cost) atomicAdd(reinterpret_cast<unsigned long long*>(&s_cost[line]), (unsigned long long)cost);
     }
@@ -219,6 +221,7 @@ __global__ void __launch_bounds__(kLayoutThreads) layout_kernel(BatchLayout bl, 
   // pass 0 counts line A's pieces (the second siblings' items lie behind all first ones), passes 1 and 2 emit
   for (int pass = too_long ? 3 : 0; pass < 3; ++pass) {
     const bool pair = pass < 2;
+    const int item_cost = pair ? kItemCostPair : kItemCostSingle;
     const int n_seg = pair ? n_seg_a : n_seg_b, per = pair ? per_a : per_b;
     const int* first = pair ? seg_a : seg_b;
     int* owner_off = pair ? a_off : b_off;
@@ -229,8 +232,8 @@ __global__ void __launch_bounds__(kLayoutThreads) layout_kernel(BatchLayout bl, 
       Seg g{0, 0, 0, 0};
       if (s < n_seg) g = segment(first, s, pair);
       Scan3 tot;
-      const Scan3 e1 = block_scan(Scan3{s < n_seg ? g.nb + kItemCost : 0, 0, 0}, &tot, scratch);
-      const int g0 = off + e1.a + kItemCost;              // cost range of the real blocks: [g0, g0 + nb)
+      const Scan3 e1 = block_scan(Scan3{s < n_seg ? g.nb + item_cost : 0, 0, 0}, &tot, scratch);
+      const int g0 = off + e1.a + item_cost;              // cost range of the real blocks: [g0, g0 + nb)
       off += tot.a;
       const int c_first = whole ? s : g0 / per, c_last = whole ? s : (g0 + g.nb - 1) / per;
       const int np = s < n_seg ? c_last - c_first + 1 : 0;
@@ -245,7 +248,7 @@ __global__ void __launch_bounds__(kLayoutThreads) layout_kernel(BatchLayout bl, 
       }
       if (pass == 0 || s >= n_seg) continue;
       // first piece of every owner: an owner without pieces starts where the next one does
-      const int c_prev = s == 0 || whole ? s - 1 : (g0 - kItemCost - 1) / per;     // owner of the last block of the segment before
+      const int c_prev = s == 0 || whole ? s - 1 : (g0 - item_cost - 1) / per;     // owner of the last block of the segment before
       for (int c = c_prev + 1; c <= c_last && c <= n_owners; ++c) owner_off[c] = c <= c_first ? item0 : item0 + (c - c_first);
       if (s == n_seg - 1)
         for (int c = c_last + 1; c <= n_owners; ++c) owner_off[c] = item0 + np;
@@ -516,7 +519,7 @@ bool attention_whole_tiles(int n_req, const int* ctx_len, const int* rows, int n
   for (int r = 0; r < n_req; ++r) {
     const int rt = (rows[r] + tok_per_tile - 1) / tok_per_tile, nb = (ctx_len[r] + rows[r] + 63) / 64;
     tiles += (long long)n_kv * rt;
-    cost += (long long)n_kv * rt * (nb + kItemCost);
+    cost += (long long)n_kv * (rt * nb + (rt & ~1) * kItemCostPair + (rt & 1) * kItemCostSingle);
     if (nb > longest) longest = nb;
   }
   return tiles <= n_ctas && longest - (cost + n_ctas - 1) / n_ctas <= kWholeBlocks;
