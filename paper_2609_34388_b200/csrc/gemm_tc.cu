@@ -1057,10 +1057,11 @@ struct Config {
 };
 struct Shape {
   int M, n_feat, K;       // n_feat: rows of w
-  bool operator==(const Shape& o) const { return M == o.M && n_feat == o.n_feat && K == o.K; }
+  int cap;                // 0, or (row count on the device) the rows that the launch has to cover
+  bool operator==(const Shape& o) const { return M == o.M && n_feat == o.n_feat && K == o.K && cap == o.cap; }
 };
 struct ShapeHash {
-  size_t operator()(const Shape& s) const { return (size_t)s.M * 1000003u ^ (size_t)s.n_feat * 7919u ^ (size_t)s.K << 32; }
+  size_t operator()(const Shape& s) const { return (size_t)s.M * 1000003u ^ (size_t)s.n_feat * 7919u ^ (size_t)s.K << 32 ^ (size_t)s.cap << 20; }
 };
 struct TcState {
   int n_sm = 0;
@@ -1181,10 +1182,14 @@ bool clusters_fit(TcState* st, bool pair, int size, int n) {
 // A k-block of a tile costs (.075 + .001 x tokens) us alone and a third more when all SMs pull operands through L2; a CTA pair
 // .085 + .00085 x tokens and a quarter more.  Examples, all SMs busy: 128 features x 256 tokens .44 us, 256 x 256 .37, 256 x 128
 // .24.  Below .18 us a CTA is bound by the latency of its loads.
-// The weights come from HBM once: bytes / 6.7 TB/s.
-// On top come the ends (launch, first loads, last tile's epilogue): 4.5 us + .003 x tokens for whole tiles; 6 us when clusters
-// reduce tiles of one chunk, 6.5 us + 1 us per chunk that a member sends for wider ones; 11.5 us + .05 x tokens when all tiles are
-// cut and go through the workspace (parking, counting, fetching, the epilogue in the last part to arrive).
+// The weights come from HBM once, at 6.7 TB/s when 105 CTAs or more stream them, .093 TB/s per CTA for a few, 2.2 TB/s + .043 per
+// CTA in between (so four parts per tile and not two: 5120 x 17408 weights at 80 rows 39.7 us on 80 CTAs, 34.9 on 120).  The
+// shorter of the two, products and stream, shows through by a tenth (128256 x 4096 at 128 rows 180 us on single CTAs, 174 on
+// pairs, with 121 and 104 us of products under 157 us of stream).
+// On top come the ends (launch, first loads, last tile's epilogue; more for pairs): 4.5 us + .003 x tokens for whole tiles; 5.6 us when
+// clusters reduce tiles of one chunk, 6 us + 1 us per chunk that a member sends for wider ones, .4 us per further token tile;
+// 11.5 us + .05 x tokens when all tiles are cut and go through the workspace (parking, counting, fetching, the epilogue in the
+// last part to arrive).
 // A ragged last wave of whole tiles: its columns can be cut over all units and done first, in narrower token tiles so that a tile
 // has few parts; their hand-over hides under the whole tiles behind them.  28672 x 4096
 // weights at 320, 376, 416 and 1024 rows: 65.5, 72.6, 79.9 and 161.9 us, all tiles whole 69.8, 77.6, 85.1 and 167.3; 4096 x 14336
@@ -1199,13 +1204,17 @@ Config choose_config(TcState* st, const Shape& s) {
   const auto known = st->configs.find(s);
   if (known != st->configs.end()) return known->second;
   const int KB = s.K / BK;
-  const double t_hbm = 2.0 * s.n_feat * s.K / 6.7e6;
+  const auto with_stream = [&](double products, double ctas) {
+    const double t = 2.0 * s.n_feat * s.K / fmin(6.7e6, fmin(93e3 * ctas, 2.2e6 + 43e3 * ctas));
+    return fmax(products, t) + .1 * fmin(products, t);
+  };
   Config best{false, kMaxTok, 0, 0, 0};
   double best_t = 1e30;
   for (int pair = 0; pair < 2; ++pair) {
     const int gran = pair ? 32 : 16, units = pair ? st->n_sm / 2 : st->n_sm;
     const int cols = (s.n_feat + FT * (pair + 1) - 1) / (FT * (pair + 1));
     const int fewest = (s.M + kMaxTok - 1) / kMaxTok;
+    const double pair_end = pair ? (s.cap ? 2.0 : .3) : 0.0;      // (with the row count on the device x comes in boxes of 16 rows)
     int last = 0;
     for (int want = fewest; want <= fewest + 3 + fewest / 4; ++want) {
       const int tmax = ((s.M + want - 1) / want + gran - 1) / gran * gran;    // the widest tile that gives `want` tiles
@@ -1215,19 +1224,24 @@ Config choose_config(TcState* st, const Shape& s) {
       token_tiles(s.M, tmax, gran, &width, &mt);
       const long long tiles = (long long)mt * cols;
       if (want > fewest && width < 32) continue;
+      // With the row count on the device one token tile takes any of them, so it is as wide as the capacity allows: there are no
+      // clusters for tiles that turn out not to exist, which take SMs from the others.
+      const int launch_tmax = s.cap && mt == 1 ? (s.cap < kMaxTok ? (s.cap + 31) / 32 * 32 : kMaxTok) : tmax;
       auto consider = [&](double t, int cl, int cut_cols, int cut_tmax) {
         if (t < best_t) {
           best_t = t;
-          best = Config{pair != 0, tmax, cl, cut_cols, cut_tmax};
+          best = Config{pair != 0, launch_tmax, cl, cut_cols, cut_tmax};
         }
       };
       const long long full = tiles / units, rem = tiles % units;      // full waves, and a last one that has the machine to itself
-      const double ends = 4.5 + .003 * width, t_full = full * KB * est_kblock(pair, width, 1.0);
-      consider(fmax(t_full + (rem ? KB * est_kblock(pair, width, (double)rem / units) : 0.0), t_hbm) + ends, 0, 0, 0);
+      const double ends = 4.5 + .003 * width + pair_end, t_full = full * KB * est_kblock(pair, width, 1.0);
+      consider(with_stream(t_full + (rem ? KB * est_kblock(pair, width, (double)rem / units) : 0.0), (full ? units : rem) * (pair + 1.0)) + ends,
+               0, 0, 0);
       if (full == 0) {
         // all tiles cut over K through the workspace
         if (mt <= units)
-          consider(fmax((double)tiles * KB / ((units / mt) * mt) * est_kblock(pair, width, 1.0), t_hbm) + 11.5 + .05 * width, 0, cols, tmax);
+          consider(with_stream((double)tiles * KB / ((units / mt) * mt) * est_kblock(pair, width, 1.0), st->n_sm) + 11.5 + .05 * width, 0,
+                   cols, tmax);
       } else if (rem) {
         const int cut = cols - (int)(full * units / mt);
         int cut_last = 0;
@@ -1245,15 +1259,16 @@ Config choose_config(TcState* st, const Shape& s) {
           // loop of its next tile holds its products, too
           const double hand = (c_width + 31) / 32 * (.6 + 1.3 * parts);
           const double t = t_full + per * est_kblock(pair, c_width, 1.0) + 3.0 + fmax(0.0, hand - KB * est_kblock(pair, width, 1.0));
-          consider(1.06 * (fmax(t, t_hbm) + ends), 0, cut, ctmax);
+          consider(1.06 * (with_stream(t, st->n_sm) + ends), 0, cut, ctmax);
         }
       }
       // clusters of 2 to 4 parts per tile, all resident at once
       const int chunks = (width + 31) / 32;
       for (int cl = 2; cl <= 4 && st->clusters; ++cl) {
         if (tiles * cl > units || cl * 4 > KB || !clusters_fit(st, pair, cl * (pair + 1), (int)tiles)) break;
-        const double cl_ends = chunks == 1 ? 6.0 : 6.5 + (double)chunks * (cl - 1) / cl;
-        consider(fmax((KB + cl - 1) / cl * est_kblock(pair, width, (double)tiles * cl / units), t_hbm) + cl_ends, cl, 0, 0);
+        const double cl_ends = (chunks == 1 ? 5.6 : 6.0 + (double)chunks * (cl - 1) / cl) + .4 * (mt - 1) + pair_end;
+        consider(with_stream((KB + cl - 1) / cl * est_kblock(pair, width, (double)tiles * cl / units), tiles * cl * (pair + 1.0)) + cl_ends,
+                 cl, 0, 0);
       }
     }
   }
@@ -1448,7 +1463,7 @@ bool launch_gemm_tc(const GemmArgs& a, void* tc_state, int* status, cudaStream_t
   const int n_feat = a.epi == EPI_SWIGLU ? 2 * a.N : a.N;
   // (device-resident rounds: the configuration is chosen for the caller's hint of the row count, the launch covers the capacity)
   const int Mc = (a.m_dev && a.m_hint > 0 && a.m_hint < a.M) ? a.m_hint : a.M;
-  Config c = choose_config(st, Shape{Mc, n_feat, a.K});
+  Config c = choose_config(st, Shape{Mc, n_feat, a.K, a.m_dev ? a.M : 0});
   if (st->force_tile || st->force_s == 1) {   // debugging aid: single CTAs (64, 128, 256 tokens) or pairs (384: 128, 512: 256 tokens)
     const int f = st->force_tile;
     if (f) c = Config{f > 256, f == 384 ? 128 : (f == 512 ? 256 : f), 0, 0, 0};
