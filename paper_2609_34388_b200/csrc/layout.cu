@@ -456,20 +456,24 @@ __global__ void __launch_bounds__(256) rmsnorm_kernel(const float* __restrict__ 
 // kKvIoUnroll 16-byte chunks of K and the same of V, all loads in flight before the first store; consecutive threads take
 // consecutive chunks, so the logical side is one contiguous stream and the pool side whole 128-byte rows of the swizzled
 // tiles.  The page ids come with the launch (constant bank: a warp covers few positions), so no upload goes ahead of it.
-// 4001 positions of 8 heads x 128 (33 MB in and out): 22.5 us a call with one 16-thread CTA per (position, head) and a page
-// row copied ahead of it, 9.2 us with this kernel.
+// Calls for one layer after the other follow on each other's heels: the addresses are ready before the wait for the kernel in
+// front, and two chunks a thread (32 registers: eight CTAs per SM) let more of the next kernel's CTAs move in early than four (48).
+// 8000 positions of 8 heads x 128 (66 MB in and out), write / read of a layer: four chunks, addresses behind the wait 13.0 /
+// 12.5 us, ahead of it 12.5 / 11.8, two chunks 11.5 / 11.6, eight 12.7 / 12.7.  Up to 4001 positions the host's calls bound it
+// (8.1 us; 22.5 with one 16-thread CTA per (position, head) and a page row copied ahead of it).
 constexpr int kKvIoPages = 896;       // page ids per launch: 3.5 of the 4 KB of kernel parameters
-constexpr int kKvIoThreads = 256, kKvIoUnroll = 4;
+constexpr int kKvIoPagesFew = 256;    // up to 4081 positions: fewer parameters for the host to copy, 8.5 -> 8.1 us a call (16 positions)
+constexpr int kKvIoThreads = 256, kKvIoUnroll = 2;
+template <int N>
 struct KvIoPages {
   int first;                          // logical page of ids[0]
-  int ids[kKvIoPages];
+  int ids[N];
 };
-template <bool WRITE>
+template <bool WRITE, int N>
 __global__ void __launch_bounds__(kKvIoThreads) kv_io_kernel(__nv_bfloat16* pool, int64_t n_pages, int layer, int n_kv, int log2_cpr,
-                                                             const __grid_constant__ KvIoPages pages, int pos0, int n_pos,
+                                                             const __grid_constant__ KvIoPages<N> pages, int pos0, int n_pos,
                                                              uint4* __restrict__ k, uint4* __restrict__ v) {
   griddep_launch();
-  griddep_wait();
   const int cpr = 1 << log2_cpr, head_dim = cpr * 8;          // 16-byte chunks per row
   const int total = (n_pos * n_kv) << log2_cpr;
   const int base = blockIdx.x * (kKvIoThreads * kKvIoUnroll) + threadIdx.x;
@@ -486,6 +490,12 @@ __global__ void __launch_bounds__(kKvIoThreads) kv_io_kernel(__nv_bfloat16* pool
     const int page = pages.ids[pos / kPageSize - pages.first];
     at[u] = reinterpret_cast<uint4*>(pool + kv_tile_base(n_pages, n_kv, head_dim, layer, page, hk) +
                                      kv_tile_offset(pos % kPageSize, c * 8, head_dim));
+  }
+  griddep_wait();
+#pragma unroll
+  for (int u = 0; u < kKvIoUnroll; ++u) {
+    if (!at[u]) continue;
+    const int i = base + u * kKvIoThreads;
     a[u] = WRITE ? k[i] : at[u][0];
     b[u] = WRITE ? v[i] : at[u][v_off];
   }
@@ -501,6 +511,21 @@ __global__ void __launch_bounds__(kKvIoThreads) kv_io_kernel(__nv_bfloat16* pool
       v[i] = b[u];
     }
   }
+}
+
+// one launch: positions [pos0, pos0 + n), whose pages are page_row[first], ... (at most N)
+template <int N>
+void kv_io_part(bool write, __nv_bfloat16* pool, int64_t n_pages, int layer, const Dims& dm, const int* page_row, int pos0, int n,
+                uint4* k, uint4* v, cudaStream_t st) {
+  const int log2_cpr = dm.head_dim == 128 ? 4 : 3;
+  KvIoPages<N> pg;
+  pg.first = pos0 / kPageSize;
+  const int last = (pos0 + n - 1) / kPageSize;
+  for (int i = pg.first; i <= last; ++i) pg.ids[i - pg.first] = page_row[i];
+  constexpr size_t kPer = (size_t)kKvIoThreads * kKvIoUnroll;
+  const dim3 grid((unsigned)((((size_t)n * dm.n_kv << log2_cpr) + kPer - 1) / kPer));
+  launch_pdl(write ? kv_io_kernel<true, N> : kv_io_kernel<false, N>, grid, dim3(kKvIoThreads), 0, st, pool, n_pages, layer, dm.n_kv,
+             log2_cpr, pg, pos0, n, k, v);
 }
 
 }  // namespace
@@ -553,23 +578,21 @@ void launch_rmsnorm(const float* h, const void* gain, void* x, int rows, int hid
 
 void launch_kv_io(bool write, void* pool, int64_t n_pages, int layer, const Dims& dm, const int* page_row, int pos0, int n_pos,
                   void* k, void* v, cudaStream_t st) {
-  const int log2_cpr = dm.head_dim == 128 ? 4 : 3;
-  const size_t row = (size_t)dm.n_kv << log2_cpr;             // chunks per position
+  const size_t row = (size_t)dm.n_kv * (dm.head_dim / 8);     // chunks per position
+  __nv_bfloat16* to = static_cast<__nv_bfloat16*>(pool);
   while (n_pos > 0) {
-    KvIoPages pg;
-    pg.first = pos0 / kPageSize;
-    int n = (pg.first + kKvIoPages) * kPageSize - pos0;       // positions this launch's page ids cover
+    const int first = pos0 / kPageSize;
+    int n = (first + kKvIoPages) * kPageSize - pos0;          // positions that a launch's page ids cover
     if (n > n_pos) n = n_pos;
-    const int last = (pos0 + n - 1) / kPageSize;
-    for (int i = pg.first; i <= last; ++i) pg.ids[i - pg.first] = page_row[i];
-    constexpr size_t kPer = (size_t)kKvIoThreads * kKvIoUnroll;
-    const dim3 grid((unsigned)((n * row + kPer - 1) / kPer));
-    launch_pdl(write ? kv_io_kernel<true> : kv_io_kernel<false>, grid, dim3(kKvIoThreads), 0, st, static_cast<__nv_bfloat16*>(pool),
-               n_pages, layer, dm.n_kv, log2_cpr, pg, pos0, n, static_cast<uint4*>(k), static_cast<uint4*>(v));
+    uint4 *kp = static_cast<uint4*>(k), *vp = static_cast<uint4*>(v);
+    if ((pos0 + n - 1) / kPageSize - first < kKvIoPagesFew)
+      kv_io_part<kKvIoPagesFew>(write, to, n_pages, layer, dm, page_row, pos0, n, kp, vp, st);
+    else
+      kv_io_part<kKvIoPages>(write, to, n_pages, layer, dm, page_row, pos0, n, kp, vp, st);
     pos0 += n;
     n_pos -= n;
-    k = static_cast<uint4*>(k) + n * row;
-    v = static_cast<uint4*>(v) + n * row;
+    k = kp + n * row;
+    v = vp + n * row;
   }
 }
 

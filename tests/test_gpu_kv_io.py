@@ -9,7 +9,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("head_dim,n_kv", [(64, 2), (128, 1), (128, 8), (128, 5)])
-@pytest.mark.parametrize("pos0,n_pos", [(0, 1), (5, 16), (15, 2), (37, 403), (3, 14333), (3, 14334), (9, 14400)])
+@pytest.mark.parametrize("pos0,n_pos", [(0, 1), (5, 16), (15, 2), (37, 403), (3, 4093), (3, 4094), (3, 14333), (3, 14334), (9, 14400)])
 def test_kv_round_trip_touches_its_positions_only(head_dim, n_kv, pos0, n_pos):
     shape = synth.ModelShape(n_layers=2, hidden=64, n_q_heads=n_kv, n_kv_heads=n_kv, head_dim=head_dim, ffn=64, vocab=64)
     if (n_kv * 3 * head_dim) % 128:
