@@ -334,10 +334,11 @@ __global__ void __launch_bounds__(kFinalThreads) verify_finalize_kernel(BatchLay
   if (desc.n) bl.rebase(desc_dev, desc.v);
   const int r = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int t0 = bl.cu_tok[r], tv0 = bl.cu_ver[r];
-  const int n = bl.cu_tok[r + 1] - t0;          // v + b + n_corr * span; 0 in a round that broke a capacity on the device
-  const int v = min(bl.verify_len[r], n), b = min(bl.block_size[r], n - v), L = bl.ctx_len[r];
+  const int n = bl.cu_tok[r + 1] - t0;          // v + b + n_corr * span; 0 in a round that broke a capacity on the device,
+  // whose lengths come as they were given: v and b must name rows of the request in any case
+  const int v = max(0, min(bl.verify_len[r], n)), b = max(0, min(bl.block_size[r], n - v)), L = bl.ctx_len[r];
   const int* cr = bl.corr + 6 * r;              // correction branches: count, mask tokens per branch, indices, tokens
-  const int n_corr = cr[0], span = 1 + cr[1];
+  const int n_corr = n > 0 ? cr[0] : 0, span = 1 + cr[1];
   const bool small = n <= kFinalRows;
   if (small)
     for (int j = tid; j < v; j += kFinalThreads) s_vt[j] = bl.verify_tokens[tv0 + j];

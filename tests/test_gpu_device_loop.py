@@ -154,6 +154,35 @@ def test_device_round_that_breaks_a_capacity_is_refused_on_the_device():
     ctx.recg_free()
 
 
+@pytest.mark.parametrize("verify,block", [([-1, 1], [4, 4]), ([1, -3], [4, 9]), ([1, 1], [4, -2]), ([0, 1], [0, 4])])
+def test_device_round_with_broken_lengths_is_an_empty_round(verify, block):
+    """Negative lengths, and a request without rows: the verification of the empty round looks at no row of any request (no
+    accepted draft, no risky draft, nothing freed), the status word says what happened, and the context stays usable."""
+    shape, Wd, ocfg, W64 = tiny()
+    pt, n_pages = synth.page_tables([10, 10], [40, 40], 16, seed=7)
+    ctx = binding.Context(binding.make_config(shape, 2, 32, pt.shape[1]), Wd)
+    pool = binding.alloc_kv_pool(ctx, n_pages, fill="normal")
+    db = binding.DeviceBatch([10, 10], verify, block, [[1], [2]], 8, pt, pool, n_pages)
+    out = binding.VerifyOut(2, 32, 32, host=False)
+    log = binding.RoundLog(2, 1, 16)
+    ctx.recg_step_device(db)
+    ctx.recg_verify(None, None, host=False, out=out)
+    ctx.recg_next_round(db, 0, log=log)
+    with pytest.raises(binding.RecgError) as e:
+        ctx.recg_sync()
+    assert e.value.status == 6
+    got = {k: t.cpu().numpy() for k, t in out.views().items()}
+    for k in ("accept_len", "n_emitted", "cont_hit", "corr_hit", "freed_pages", "risky_n"):
+        assert (got[k] == 0).all(), k
+    assert (got["risky_index"] == -1).all() and (got["risky_token"] == -1).all() and (got["entropy_mean"] == 0).all()
+    assert db.verify_len.cpu().tolist() == verify and db.block_size.cpu().tolist() == block and log.n_tokens.cpu().tolist() == [0, 0]
+    db2 = binding.DeviceBatch([10, 10], [1, 1], [4, 4], [[1], [2]], 8, pt, pool, n_pages)
+    ctx.recg_step_device(db2)
+    ctx.recg_verify_device()
+    ctx.recg_sync()
+    ctx.recg_free()
+
+
 @pytest.mark.parametrize("n_req,capacity,blocks", [(12, 512, [4, 8, 16, 32]), (3, 128, [4, 8, 16]), (1, 64, [16]), (1, 32, [8])])
 def test_device_round_on_8b_shaped_layers_equals_the_host_round(n_req, capacity, blocks):
     """The same ragged batch through two 8B-shaped layers (tcgen05 projections and attention) once with host descriptor
