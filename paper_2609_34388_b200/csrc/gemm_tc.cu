@@ -1434,6 +1434,8 @@ bool launch_gemm_tc(const GemmArgs& a, void* tc_state, int* status, cudaStream_t
   TcState* st = static_cast<TcState*>(tc_state);
   if (!st || a.M <= 0 || a.K % BK || a.N % 16) return false;
   if ((reinterpret_cast<uintptr_t>(a.x) | reinterpret_cast<uintptr_t>(a.w)) & 15) return false;
+  // (bf16 rows leave in pieces of 16 bytes, fp32 ones element by element)
+  if (reinterpret_cast<uintptr_t>(a.out) & (a.epi == EPI_PLAIN_F32 || a.epi == EPI_RESIDUAL || a.epi == EPI_RESIDUAL_NORM ? 3 : 15)) return false;
   if (a.epi == EPI_RESIDUAL_NORM && (!a.x_out || !a.gain || !a.ss_out)) return false;
   if (a.epi == EPI_SWIGLU && a.N % 64) return false;
   if (((int64_t)a.N * 2 / FT + 2) * (a.K / BK) > (1 << 30)) return false;      // the line of k-blocks is counted in int

@@ -372,6 +372,10 @@ recg_status run_gemm(recg_ctx* ctx, const GemmArgs& a, int* ss_slots_out = nullp
       cudaGetLastError();
       return fail(ctx, RECG_ERR_INTERNAL, "projection: the tcgen05 kernel refused a shape of the step");
     }
+    // the mma.sync kernel loads 16 bytes and stores four elements at a time
+    const bool f32 = a.epi == EPI_PLAIN_F32 || a.epi == EPI_RESIDUAL;
+    if (((reinterpret_cast<uintptr_t>(a.x) | reinterpret_cast<uintptr_t>(a.w)) & 15) || (reinterpret_cast<uintptr_t>(a.out) & (f32 ? 15 : 7)))
+      return fail(ctx, RECG_ERR_INVALID_ARG, "projection: an operand or the result is not aligned as its kernel needs it");
     launch_gemm_simt(a, ctx->d_status, ctx->stream);
   }
   CU(cudaGetLastError());

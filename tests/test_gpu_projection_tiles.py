@@ -39,6 +39,41 @@ def test_rows_around_the_tiles(tile, sk, N, K):
     ctx.recg_free()
 
 
+@pytest.mark.parametrize("flags", [0, binding.FLAG_SIMT_GEMM])
+@pytest.mark.parametrize("dt", [torch.float32, torch.bfloat16])
+def test_results_of_any_alignment(dt, flags):
+    """A result that starts 0 to 16 bytes behind a 16-byte boundary: computed where a kernel can store it (bf16: multiples of 8
+    bytes; fp32: any element, multiples of 16 bytes with the mma.sync kernel), an error anywhere else; x and w likewise."""
+    M, N, K = 37, 144, 320
+    ctx = binding.Context(binding.make_config(synth.tiny_shape(), 1, 8, 1, flags))
+    g = torch.Generator().manual_seed(1)
+    w = (torch.randn((N, K), generator=g) * 0.05).to(torch.bfloat16)
+    x = torch.randn((M, K), generator=g).to(torch.bfloat16)
+    ref = x.double().numpy() @ w.double().numpy().T
+    wd, xd = w.cuda(), x.cuda()
+    size = 4 if dt == torch.float32 else 2
+    need = 8 if dt == torch.bfloat16 else (16 if flags else 4)
+    call = lambda xp, wp, yp: binding.lib().recg_linear(ctx.h, xp, wp, yp, M, N, K, binding.DTYPE_F32 if size == 4 else binding.DTYPE_BF16)
+    for off in range(0, 17, size):
+        buf = torch.full((M * N + 32,), float("nan"), dtype=dt, device="cuda")
+        i = off // size
+        assert buf.data_ptr() % 16 == 0
+        status = call(xd.data_ptr(), wd.data_ptr(), buf.data_ptr() + off)
+        assert status == (0 if off % need == 0 else 1), off
+        ctx.recg_sync()
+        got = f64(buf)
+        assert np.isnan(got[:i]).all() and np.isnan(got[i + M * N:]).all(), off
+        if status:
+            assert np.isnan(got).all()
+        else:          # the bounds of the test above
+            tol = 1e-5 if size == 4 else 2.0 ** -8
+            assert np.max(np.abs(got[i:i + M * N].reshape(M, N) - ref)) <= tol * np.max(np.abs(ref)), off
+    y = torch.empty((M, N), dtype=dt, device="cuda")
+    assert call(xd.data_ptr() + 8, wd.data_ptr(), y.data_ptr()) == 1 and call(xd.data_ptr(), wd.data_ptr() + 2, y.data_ptr()) == 1
+    ctx.recg_sync()
+    ctx.recg_free()
+
+
 @pytest.mark.parametrize("force", [(0, 0), (64, 1), (256, 2), (384, 0), (512, 1)])
 @pytest.mark.parametrize("head_dim,n_q,n_kv", [(64, 2, 1), (128, 1, 1), (64, 6, 2)])
 def test_step_of_a_model_that_fills_no_tile(head_dim, n_q, n_kv, force):
