@@ -493,7 +493,7 @@ void launch_attention(const BatchLayout& bl, const Dims& dm, int layer, const vo
     if (whole) return;
     launch_pdl(attention_combine_kernel<128>, dim3(4 * n_sm), dim3(512), 0, st, (const AttnTile*)bl.tiles,
                (const int*)bl.counts, dm.n_q, dm.n_q / dm.n_kv, (const float*)part_o, (const float*)part_ml,
-               static_cast<__nv_bfloat16*>(o), 1);    // (the kernel in front signals its dependents after its own wait)
+               static_cast<__nv_bfloat16*>(o), 1);    // (the kernel in front signals its dependents when the list is settled)
     return;
   }
   if (dm.head_dim == 64)

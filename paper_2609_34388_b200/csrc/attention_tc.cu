@@ -226,8 +226,8 @@ __global__ void __launch_bounds__(kThreads, 1) attention_tc_kernel(const __grid_
   auto item_at = [&](int i) { return i < range_n0 ? range_b0 + i : range_b1 + (i - range_n0); };
   AttnItem w_next = {};
   if (warp == 0) {
-    // (behind the first layer of a step the work list was written a whole layer of kernels ago, each of which fills the SMs:
-    // the reads below then overlap the kernel in front of this one instead of following it)
+    // (early_desc: an attention kernel has run since the work list was written, so the reads below overlap the kernel in front
+    // of this one instead of following it.  Otherwise all warps meet behind this wait before any of them signals the dependents)
     if (!P.early_desc) griddep_wait();
     const int4 r4 = *reinterpret_cast<const int4*>(P.cta_off + 4 * blockIdx.x);
     range_b0 = r4.x;

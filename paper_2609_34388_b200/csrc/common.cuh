@@ -25,11 +25,17 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
 }
 
 // ---- programmatic dependent launch ------------------------------------------------------------------
-// Every kernel of a step is launched with programmatic stream serialisation: it signals at once that its
-// dependent may be scheduled (launch_dependents), runs its own prologue (barrier init, TMEM allocation, shared
-// memory clearing), and only then waits for the kernels before it to complete and flush (griddep_wait).  No
-// kernel reads or writes global memory before its wait, so the launch latency and prologue of kernel n+1 overlap
-// the tail of kernel n and nothing else changes.  Without the launch attribute both instructions do nothing.
+// Every kernel of a step is launched with programmatic stream serialisation: it signals that its dependent may be scheduled
+// (launch_dependents), runs its own prologue (barrier init, TMEM allocation, shared memory clearing), and waits for the
+// kernels before it to complete and flush (griddep_wait), so that the launch latency and prologue of kernel n+1 overlap the
+// tail of kernel n.  What a kernel does ahead of its wait:
+//   reads of what no kernel in flight writes: weights (projections), the work list and page ids when an attention kernel has
+//     run since they were written (attention, combine), the descriptor where it was in place before the kernel in front could
+//     start (finalize, embedding);
+//   writes in the embedding kernel only: the layout kernel in front of it signals BEHIND its own wait, so everything older
+//     is complete; one CTA waits at the end, since a grid must not count as complete before its predecessors are (the next
+//     kernel's wait looks no further back).
+// Everything else follows the wait.  Without the launch attribute both instructions do nothing.
 __device__ __forceinline__ void griddep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

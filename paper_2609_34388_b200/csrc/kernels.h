@@ -211,8 +211,8 @@ bool launch_gemm_chain(void* s, const ChainOp* ops, int n_ops, int M, const Chai
 
 // S5
 // use_tc: run the tcgen05 kernel (head_dim 128 only); otherwise the mma.sync kernel
-// layout_settled: the work list was written by a kernel that is known to have finished when this one starts (anything but
-// the launch right before it): the tcgen05 kernel then reads its work range before it waits for its predecessor
+// layout_settled: an attention kernel has been enqueued behind the kernel that wrote the work list (and has waited for it):
+// the tcgen05 kernel then reads its work range before it waits for its predecessor
 // whole: the work list was laid out with whole tiles
 void launch_attention(const BatchLayout& bl, const Dims& dm, int layer, const void* q, void* o, const void* kv_pool,
                       int64_t n_pages, float* part_o, float* part_ml, int tok_per_tile, int n_sm, int* status,

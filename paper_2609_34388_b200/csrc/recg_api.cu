@@ -56,6 +56,10 @@ struct recg_ctx {
   bool layout_valid = false;
   bool layout_has_pages = false;
   bool layout_whole = false;     // no attention tile was cut: no combine kernel
+  // An attention kernel has been enqueued behind the last layout kernel.  The first one waits for its predecessors before it
+  // reads the work list, and no thread of it signals its dependents before that wait: whatever runs behind it finds the list
+  // settled and may read it ahead of its own wait.
+  bool list_settled = false;
   int64_t last_pool_pages = 0;
   void* last_pool = nullptr;
   // activations
@@ -353,6 +357,7 @@ recg_status upload_and_layout(recg_ctx* ctx, const recg_batch* b, bool need_page
     ctx->layout_whole = attention_whole_tiles(b->n_req, b->ctx_len, ctx->h_rows.data(), ctx->dm.n_kv, ctx->tok_per_tile, ctx->target_items);
     launch_layout(ctx->bl, ctx->dm, ctx->tok_per_tile, ctx->target_items, ctx->layout_whole, n_pages, ctx->d_status,
                   !forward, ctx->d_desc, small ? &ctx->small_desc : nullptr, ctx->stream);
+    ctx->list_settled = false;
     if (forward) embed_tokens(ctx, n_pages);
   }
   CU(cudaGetLastError());
@@ -606,12 +611,12 @@ static recg_status run_forward(recg_ctx* ctx, void* kv_pool, int64_t kv_pool_pag
     if ((s = run_gemm(ctx, a)) != RECG_OK) return s;
     ctx->mark(2, 1);
     }
-    // (The first layer's attention kernel may be resident while the work list is still being built: idle lanes of a projection
-    // signal its dependents before the projection has waited.  It waits before it reads the list; behind a whole layer of
-    // kernels that fill every SM the list is settled.)
-    launch_attention(bl, d, l, ctx->q, ctx->o, kv_pool, kv_pool_pages, ctx->part_o, ctx->part_ml,
-                     ctx->tok_per_tile, ctx->n_sm, ctx->d_status, st, !(ctx->cfg.flags & RECG_FLAG_SIMT_ATTENTION), fold && l > 0, ctx->layout_whole);
+    // (the first layer's attention kernel may be resident while the work list is still being built: idle lanes of a projection
+    // signal its dependents before the projection has waited)
+    launch_attention(bl, d, l, ctx->q, ctx->o, kv_pool, kv_pool_pages, ctx->part_o, ctx->part_ml, ctx->tok_per_tile, ctx->n_sm,
+                     ctx->d_status, st, !(ctx->cfg.flags & RECG_FLAG_SIMT_ATTENTION), ctx->list_settled, ctx->layout_whole);
     CU(cudaGetLastError());
+    ctx->list_settled = true;
     ctx->mark(3, ctx->layout_whole ? 1 : 2);
     if (chain) {
       const bool last = l + 1 == d.n_layers;
@@ -748,6 +753,7 @@ recg_status recg_step_device(recg_ctx* ctx, const recg_device_batch* b, recg_log
   launch_pack_device(device_round(ctx, b), ctx->d_desc, ctx->d_dyn, ctx->d_status, ctx->stream);
   ctx->layout_whole = false;           // (the lengths are on the device)
   launch_layout(bl, ctx->dm, ctx->tok_per_tile, ctx->target_items, false, b->kv_pool_pages, ctx->d_status, false, ctx->d_desc, nullptr, ctx->stream);
+  ctx->list_settled = false;
   ctx->small_desc.n = 0;
   embed_tokens(ctx, b->kv_pool_pages);
   CU(cudaGetLastError());
@@ -909,8 +915,9 @@ recg_status recg_attention(recg_ctx* ctx, const recg_batch* batch, int32_t layer
   }
   launch_attention(ctx->bl, ctx->dm, layer, q, o, ctx->last_pool, ctx->last_pool_pages, ctx->part_o, ctx->part_ml,
                    ctx->tok_per_tile, ctx->n_sm, ctx->d_status, ctx->stream, !(ctx->cfg.flags & RECG_FLAG_SIMT_ATTENTION),
-                   batch == nullptr, ctx->layout_whole);      // (a batch given with the call was laid out by the launch right before this one)
+                   ctx->list_settled, ctx->layout_whole);
   CU(cudaGetLastError());
+  ctx->list_settled = true;
   return RECG_OK;
 }
 

@@ -66,3 +66,40 @@ def test_tokens_of_many_requests(n_req):
         got = logits[first[r]:first[r + 1]]
         assert np.max(np.abs(got - ref)) <= HID_TOL * np.max(np.abs(ref)), r
     ctx.recg_free()
+
+
+@pytest.mark.parametrize("n_layers", [1, 3])
+def test_attention_right_behind_a_verification_with_pages(n_layers):
+    """A verification of given logits lays its batch out, and the attention calls that follow name no batch: they work on that
+    layout, also the first one, in front of which no kernel of any size has run (device results: nothing waits for the host).
+    Batches of few and many requests take turns, so that a list of the batch before would show."""
+    shape = synth.ModelShape(n_layers=n_layers, hidden=512, n_q_heads=4, n_kv_heads=2, head_dim=128, ffn=64, vocab=64)
+    sets = [[(300, 3, 2)], [(40, 1, 3), (700, 2, 0), (5, 4, 4)], [(20 * i % 333, 1 + i % 3, i % 2) for i in range(40)]]
+    descs = [synth.fixed_descriptor([r[0] for r in s], [r[1] for r in s], [r[2] for r in s], seed=9 + i) for i, s in enumerate(sets)]
+    n_pages = max(d.n_pages for d in descs)
+    ctx = binding.Context(binding.make_config(shape, 40, max(d.n_tokens for d in descs), max(d.page_table.shape[1] for d in descs)))
+    pool = binding.alloc_kv_pool(ctx, n_pages, fill="normal")
+    work = []
+    for i, d in enumerate(descs):
+        y = synth.token_ids(int(d.verify_len.sum()), shape.vocab, seed=i)
+        batch = binding.Batch(d.ctx_len, d.verify_len, d.block_size, y, d.page_table, pool, n_pages)
+        logits = synth.logits_normal(d.n_tokens, shape.vocab, seed=i, device="cuda")
+        q = synth.queries(d.n_tokens * n_layers, 4, 128, seed=i).cuda().view(n_layers, d.n_tokens, 4, 128)
+        want = torch.empty_like(q)
+        for l in range(n_layers):
+            ctx.recg_attention(batch, l, q[l], want[l])
+        ctx.recg_sync()
+        work.append((batch, logits, q, want, binding.VerifyOut(d.n_req, d.n_tokens, len(y), host=False)))
+    got = []
+    for rep in range(60):
+        batch, logits, q, want, out = work[rep % 3]
+        o = torch.full_like(q, float("nan"))
+        torch.cuda.synchronize()
+        ctx.recg_verify(batch, logits, out=out)
+        for l in range(n_layers):
+            ctx.recg_attention(None, l, q[l], o[l])
+        got.append(o)
+    ctx.recg_sync()
+    for rep, o in enumerate(got):
+        assert torch.equal(o, work[rep % 3][3]), rep
+    ctx.recg_free()
