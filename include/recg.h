@@ -266,6 +266,11 @@ recg_status recg_debug_buffer(recg_ctx *ctx, int32_t which, const void **ptr, in
  *   K range of the tiles over the SMs, stream_k = 2 does the same and also (with any tile value, 0 included) keeps
  *   partial tiles from being handed over inside thread-block clusters: they go through the partial-tile workspace;
  *   stream_k = 0: whole tiles.  A configuration that does not fit a shape is ignored for that launch.
+ * recg_debug_gemm_plan(): how a projection of `rows` rows and n_features x K weights (gate|up: both matrices) is divided on
+ *   this context.  capacity = 0: row count known to the host; else the launch of a device-resident step with that capacity
+ *   (max_tokens) and rows_hint expected rows, when it finds `rows`.  out (HOST) [8]: 1 for CTA pairs, tokens per tile,
+ *   token tiles, parts per tile that form a cluster (0: none), columns of feature tiles, last columns whose tiles are cut over
+ *   K, tokens per tile of those, k-blocks in a team's range of them.
  * recg_debug_wait_timeout(): enqueue a one-thread kernel that waits on a barrier nobody arrives on, bounded by
  *   max_polls polls (1 .. 1048576) exactly like the waits inside the kernels; it gives up, records the timeout in the
  *   device status word and returns.  The next recg_sync() then reports RECG_ERR_TIMEOUT and clears the word; the
@@ -275,6 +280,8 @@ recg_status recg_debug_buffer(recg_ctx *ctx, int32_t which, const void **ptr, in
  *   *evictions receives how often the full cache was emptied on the way.
  */
 recg_status recg_debug_gemm_config(recg_ctx *ctx, int32_t tile, int32_t stream_k);
+recg_status recg_debug_gemm_plan(recg_ctx *ctx, int32_t rows, int32_t n_features, int32_t K, int32_t rows_hint, int32_t capacity,
+                                 int32_t *out);
 recg_status recg_debug_wait_timeout(recg_ctx *ctx, int32_t max_polls);
 int32_t recg_debug_map_cache_selftest(int32_t n_keys, int32_t *evictions);
 
@@ -348,8 +355,8 @@ recg_status recg_policy_step(recg_ctx *ctx, const recg_policy_state *state, cons
  *   rows_hint                                 the expected number of rows per round, used to choose the projections'
  *                                             tile configurations (0: the context's max_tokens)
  * Correction branches are not available in this mode.  Because the row count of a round is only known on the device,
- * every launch is sized for the context's max_tokens and max_requests, projections use whole tiles only, and
- * recg_logits.n_rows reports max_tokens; the true counts are in the device arrays.  Lengths that break a capacity
+ * every launch is sized for the context's max_tokens and max_requests (the projections take the division of their tiles
+ * from a table by the row count), and recg_logits.n_rows reports max_tokens; the true counts are in the device arrays.  Lengths that break a capacity
  * (negative, a request without rows, verify_len > max_verify, rows beyond the page-table row, more than max_tokens rows
  * in total) set the device status word and turn the round into an empty one: recg_sync() then returns
  * RECG_ERR_INTERNAL.  Not available with RECG_FLAG_SIMT_GEMM or RECG_FLAG_FOLD_NORM.

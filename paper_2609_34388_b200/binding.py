@@ -123,12 +123,13 @@ def lib() -> C.CDLL:
         L.recg_next_round.argtypes = [C.c_void_p, C.POINTER(recg_device_batch), C.c_void_p, C.c_void_p, C.POINTER(recg_round_log),
                                       C.c_int32]
         L.recg_debug_gemm_config.argtypes = [C.c_void_p, C.c_int32, C.c_int32]
+        L.recg_debug_gemm_plan.argtypes = [C.c_void_p, C.c_int32, C.c_int32, C.c_int32, C.c_int32, C.c_int32, C.POINTER(C.c_int32)]
         L.recg_debug_wait_timeout.argtypes = [C.c_void_p, C.c_int32]
         L.recg_debug_map_cache_selftest.argtypes = [C.c_int32, C.POINTER(C.c_int32)]
         L.recg_debug_map_cache_selftest.restype = C.c_int32
         for f in ("recg_init", "recg_step", "recg_verify", "recg_attention", "recg_kv_write", "recg_kv_read",
                   "recg_linear", "recg_debug_buffer", "recg_sync", "recg_free", "recg_timing_enable", "recg_timing_read",
-                  "recg_policy_load", "recg_policy_step", "recg_debug_gemm_config", "recg_debug_wait_timeout",
+                  "recg_policy_load", "recg_policy_step", "recg_debug_gemm_config", "recg_debug_gemm_plan", "recg_debug_wait_timeout",
                   "recg_step_device", "recg_next_round"):
             getattr(L, f).restype = C.c_int32
         _lib = L
@@ -138,7 +139,7 @@ def lib() -> C.CDLL:
 EXPORTS = ("recg_kv_pool_bytes", "recg_init", "recg_step", "recg_verify", "recg_attention", "recg_kv_write",
            "recg_kv_read", "recg_linear", "recg_debug_buffer", "recg_sync", "recg_free", "recg_last_error",
            "recg_timing_enable", "recg_timing_read", "recg_row_stats_static", "recg_row_stats_static_error",
-           "recg_policy_load", "recg_policy_step", "recg_debug_gemm_config", "recg_debug_wait_timeout",
+           "recg_policy_load", "recg_policy_step", "recg_debug_gemm_config", "recg_debug_gemm_plan", "recg_debug_wait_timeout",
            "recg_debug_map_cache_selftest", "recg_step_device", "recg_next_round")
 TIMING_CLASSES = ("layout", "rmsnorm", "gemm_qkv", "attention", "gemm_o", "gemm_gate_up", "gemm_down", "lm_head", "verify")
 
@@ -389,6 +390,11 @@ class Context:
 
     def recg_debug_gemm_config(self, tile: int, stream_k: int):
         self._check(lib().recg_debug_gemm_config(self.h, int(tile), int(stream_k)))
+
+    def recg_debug_gemm_plan(self, rows: int, n_features: int, K: int, rows_hint: int = 0, capacity: int = 0) -> Dict[str, int]:
+        out = (C.c_int32 * 8)()
+        self._check(lib().recg_debug_gemm_plan(self.h, rows, n_features, K, rows_hint, capacity, out))
+        return dict(zip(("pair", "width", "tiles", "cluster", "columns", "cut_columns", "cut_width", "cut_range"), out))
 
     def recg_debug_wait_timeout(self, max_polls: int):
         self._check(lib().recg_debug_wait_timeout(self.h, int(max_polls)))

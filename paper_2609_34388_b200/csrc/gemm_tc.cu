@@ -36,6 +36,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <cmath>
+#include <functional>
 #include <mutex>
 #include <unordered_map>
 
@@ -243,6 +244,39 @@ __host__ __device__ inline int cut_range(int cols, int mt, int KB, int n_units) 
   const int total = cols * KB, n_teams = n_units / mt;       // (launch_gemm_tc keeps the line within int; mt <= n_units)
   const int per = (total + n_teams - 1) / n_teams;
   return per < 4 && total >= 4 ? 4 : per;                    // pieces long enough to amortise their hand-over
+}
+
+// Row count on the device: the token tiles and the columns that are cut over K for every 32 rows up to kPlanRows * 32, as the
+// host's estimate chooses them (device_plan); more rows come in whole tiles of the widest kind.  Widths in units of 32 tokens.
+// (28672 x 4096 weights at 320, 512, 848 and 1024 rows: 67.7, 99, 158 and 179 us; when any choice of cut columns cut all of
+// them, 94, 131, 238 and 243.)
+constexpr int kPlanRows = 64;
+struct DevPlan {
+  uint8_t tmax[kPlanRows], cut_tmax[kPlanRows];
+  uint16_t cut_cols[kPlanRows];
+};
+struct Tiling {
+  int width, mt;                       // tokens per tile, token tiles
+  int cut_cols, cut_width, cut_mt;     // last columns whose tiles are cut, their token tiles (never wider than the others)
+  int per;                             // k-blocks of a team's range
+};
+__host__ __device__ inline Tiling tiling(int M, int tmax, int gran, int cut_cols, int cut_tmax, int KB, int n_units) {
+  Tiling t;
+  token_tiles(M, tmax, gran, &t.width, &t.mt);
+  t.cut_cols = cut_cols;
+  t.cut_width = t.width;
+  t.cut_mt = t.mt;
+  t.per = 1;
+  if (cut_cols) {
+    token_tiles(M, cut_tmax < t.width ? cut_tmax : t.width, gran, &t.cut_width, &t.cut_mt);
+    if (t.cut_mt <= n_units) t.per = cut_range(cut_cols, t.cut_mt, KB, n_units);      // (else refused by the host)
+  }
+  return t;
+}
+__host__ __device__ inline Tiling planned(const DevPlan& p, int M, int KB, int n_units) {
+  const int i = (M - 1) / 32;
+  return i < kPlanRows ? tiling(M, 32 * p.tmax[i], 32, p.cut_cols[i], 32 * p.cut_tmax[i], KB, n_units)
+                       : tiling(M, kMaxTok, 32, 0, 0, KB, n_units);
 }
 
 struct Piece {
@@ -549,10 +583,8 @@ struct GemmLaunch {
   int m_cap;                 // rows the maps cover
   int n_cols;                // columns of tiles: feature tiles of 128, or of 256 for pairs
   int K;
-  int tmax, gran, x_box;     // token tiles (token_tiles), rows of one x load
-  int width, mt;             // ... their width and number, where the row count is known
-  int cut_cols;              // last columns whose tiles are cut over K; -1 (row count on the device): all of them
-  int cut_width, cut_mt, cut_box, per;   // their token tiles, rows of one x load, k-blocks of a team's range
+  Tiling tiles;              // (row count on the device: of the capacity; the kernel takes its own from the plan)
+  int tmax;                  // widest token tile
   int cl;                    // parts per tile that form a cluster (0: no clusters)
   int w_step3, w_step4;      // what a 128-feature tile advances in dimensions 3 and 4 of w's tensor map
   float* split_ws;
@@ -561,18 +593,29 @@ struct GemmLaunch {
   int m_dev_wait;
 };
 
-template <bool PAIR>
+// x: one load per k-block whatever the width of the token tile.  With the row count on the device that is any multiple of 32, and
+// there is a map for each: 4096 x 4096 weights at 376, 848 and 1024 rows 34.1, 54.6 and 59.9 us, with loads of 32 rows (a pair's
+// CTAs 16) 37.4, 63.2 and 65.6.
+template <bool DEV> struct XMaps;
+template <> struct XMaps<false> {
+  CUtensorMap whole, cut;              // boxes of a token tile's rows (of a pair's CTA: half of them)
+};
+template <> struct XMaps<true> {
+  CUtensorMap wide[kMaxTok / 32];      // likewise, by width / 32 - 1
+  DevPlan plan;
+};
+
+template <bool PAIR, bool DEV>
 __global__ void __launch_bounds__(kTcThreads, 1)
-gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x,
-               const __grid_constant__ CUtensorMap map_xc, GemmLaunch G, EpiParams ep) {
+gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ XMaps<DEV> X, GemmLaunch G, EpiParams ep) {
   // Device-resident rounds: the row count comes from device memory; the tensor maps cover the capacity, and rows
   // between the count and the capacity hold stale data and are computed but never used.  The count is written by the
   // first kernel of the step, and the small kernels between it and the first projection signal their dependents before
   // they wait themselves, so the FIRST projection of a step can be running before that one has finished: it has to wait
   // for its predecessors before it reads the count (m_dev_wait; it gives up the early weight requests).  The first
   // projection signals its own dependents only after that wait, so for every kernel behind it the count is settled.
-  if (G.m_dev && G.m_dev_wait) griddep_wait();
-  const int M = G.m_dev ? *reinterpret_cast<const volatile int*>(G.m_dev) : G.m_cap;
+  if (DEV && G.m_dev_wait) griddep_wait();
+  const int M = DEV ? *reinterpret_cast<const volatile int*>(G.m_dev) : G.m_cap;
   if (M <= 0) {                // an empty round (the same for every thread of the grid): nothing to do, nothing was set up yet
     griddep_wait();            // (this grid must not count as complete before the ones it follows are)
     return;
@@ -589,15 +632,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
 
   const int KB = G.K / BK;
-  int nt_tok = G.width, mt = G.mt;                        // tokens per tile, token tiles
-  if (G.m_dev) token_tiles(M, G.tmax, G.gran, &nt_tok, &mt);
-  int cut_cols = G.cut_cols, cut_tok = G.cut_width, cut_mt = G.cut_mt, per = G.per;      // the same for the cut columns
-  if (cut_cols < 0) {
-    cut_cols = mt <= n_units ? G.n_cols : 0;
-    cut_tok = nt_tok;
-    cut_mt = mt;
-    per = cut_cols ? cut_range(cut_cols, mt, KB, n_units) : 1;
-  }
+  Tiling tl = G.tiles;
+  if constexpr (DEV) tl = cl ? tiling(M, G.tmax, 32, 0, 0, KB, n_units) : planned(X.plan, M, KB, n_units);
+  const int nt_tok = tl.width, mt = tl.mt, cut_cols = tl.cut_cols, cut_tok = tl.cut_width, cut_mt = tl.cut_mt, per = tl.per;
   // (the cut columns' token tiles are never wider than the others: one stage layout serves both)
   const int stage_bytes = kABytes + nt_tok / kMul * BK * 2;
   const int part_bytes = (cut_tok + 31) / 32 * kChunkBytes;   // a partial tile in the workspace
@@ -691,7 +728,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
     mbar_init(red_bar, cl ? (cl - 1) * 4 : 1);             // (clusters: one arrival per other member and epilogue warp)
     mbar_init(go_bar, cl > 1 ? cl - 1 : 1);
     fence_barrier_init();
-    prefetch_tmap(&map_x);
+    if constexpr (DEV) prefetch_tmap(&X.wide[nt_tok / 32 - 1]);
+    else prefetch_tmap(&X.whole);
     prefetch_tmap(&map_w);
   }
   if (warp == 1) {
@@ -727,13 +765,12 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
       };
       auto load_x = [&](int s, int kb, int tm, bool cut) {
         uint8_t* dst = smem + s * stage_bytes + kABytes;
-        const int rows = (cut ? cut_tok : nt_tok) / kMul, box = cut ? G.cut_box : G.x_box;
-        const int row = tm * rows * kMul + (int)rank * rows;
-        const CUtensorMap* map = cut ? &map_xc : &map_x;
-        for (int r = 0; r < rows; r += box) {
-          if constexpr (PAIR) tma_load_2d_pair(smem_u32(dst + r * BK * 2), map, kb * BK, row + r, mapa_rank(smem_u32(&full_bar[s]), lead_rank));
-          else tma_load_2d(dst + r * BK * 2, map, kb * BK, row + r, &full_bar[s]);
-        }
+        const int tok = cut ? cut_tok : nt_tok, row = tm * tok + (int)rank * (tok / kMul);
+        const CUtensorMap* map;
+        if constexpr (DEV) map = &X.wide[tok / 32 - 1];
+        else map = cut ? &X.cut : &X.whole;
+        if constexpr (PAIR) tma_load_2d_pair(smem_u32(dst), map, kb * BK, row, mapa_rank(smem_u32(&full_bar[s]), lead_rank));
+        else tma_load_2d(dst, map, kb * BK, row, &full_bar[s]);
       };
       // The weights do not depend on the kernels before this one: the weight tiles of the first stages are requested
       // BEFORE waiting for those kernels, so the ring fills while they drain (or while a short kernel runs); the x tiles of
@@ -1072,9 +1109,10 @@ struct TcState {
   std::unordered_map<MapKey, CUtensorMap, MapKeyHash> maps;
   size_t evictions = 0;
   std::unordered_map<Shape, Config, ShapeHash> configs;    // choose_config's answers (emptied when there are kMapCacheMax)
-  bool configured[2] = {false, false};
+  std::unordered_map<Shape, DevPlan, ShapeHash> plans;     // device_plan's, with `pair` in the place of the rows
+  bool configured[2][2] = {{false, false}, {false, false}};
   bool clusters = true;       // tiles cut over K may be handed over inside clusters
-  int max_clusters[2][9];     // cached occupancy answers per kernel and cluster size in CTAs (-1: not asked yet)
+  int max_clusters[2][9];     // cached occupancy answers, single CTAs / pairs and cluster size in CTAs (-1: not asked yet)
   TcState() {
     for (auto& row : max_clusters)
       for (int& v : row) v = -1;
@@ -1143,16 +1181,21 @@ bool get_w_map(TcState* st, const void* ptr, uint64_t rows, uint64_t K, WeightOr
   });
 }
 
-bool configure(TcState* st, bool pair) {
-  if (st->configured[pair]) return true;
-  const void* k = pair ? reinterpret_cast<const void*>(gemm_tc_kernel<true>) : reinterpret_cast<const void*>(gemm_tc_kernel<false>);
+typedef void (*KernelHost)(CUtensorMap, XMaps<false>, GemmLaunch, EpiParams);
+typedef void (*KernelDev)(CUtensorMap, XMaps<true>, GemmLaunch, EpiParams);
+KernelHost kernel_host(bool pair) { return pair ? gemm_tc_kernel<true, false> : gemm_tc_kernel<false, false>; }
+KernelDev kernel_dev(bool pair) { return pair ? gemm_tc_kernel<true, true> : gemm_tc_kernel<false, true>; }
+
+bool configure(TcState* st, bool pair, bool dev) {
+  if (st->configured[pair][dev]) return true;
+  const void* k = dev ? reinterpret_cast<const void*>(kernel_dev(pair)) : reinterpret_cast<const void*>(kernel_host(pair));
   if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) != cudaSuccess) return false;
-  return st->configured[pair] = true;
+  return st->configured[pair][dev] = true;
 }
 
 // Whether n clusters of `size` CTAs are resident at once (the occupancy query's answer is kept).
 bool clusters_fit(TcState* st, bool pair, int size, int n) {
-  if (size > 8 || !configure(st, pair)) return false;
+  if (size > 8 || !configure(st, pair, false)) return false;
   int& cached = st->max_clusters[pair][size];
   if (cached < 0) {
     cudaLaunchConfig_t cfg = {};
@@ -1167,8 +1210,7 @@ bool clusters_fit(TcState* st, bool pair, int size, int n) {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int got = 0;
-    if ((pair ? cudaOccupancyMaxActiveClusters(&got, gemm_tc_kernel<true>, &cfg)
-              : cudaOccupancyMaxActiveClusters(&got, gemm_tc_kernel<false>, &cfg)) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&got, kernel_host(pair), &cfg) != cudaSuccess) {
       cudaGetLastError();
       got = 0;
     }
@@ -1200,9 +1242,8 @@ double est_kblock(bool pair, int width, double busy) {
   return fmax(t, .18);
 }
 
-Config choose_config(TcState* st, const Shape& s) {
-  const auto known = st->configs.find(s);
-  if (known != st->configs.end()) return known->second;
+// kinds: which of single CTAs (1) and pairs (2) to look at, and whether clusters may be chosen (4)
+Config estimate(TcState* st, const Shape& s, int kinds) {
   const int KB = s.K / BK;
   const auto with_stream = [&](double products, double ctas) {
     const double t = 2.0 * s.n_feat * s.K / fmin(6.7e6, fmin(93e3 * ctas, 2.2e6 + 43e3 * ctas));
@@ -1211,10 +1252,11 @@ Config choose_config(TcState* st, const Shape& s) {
   Config best{false, kMaxTok, 0, 0, 0};
   double best_t = 1e30;
   for (int pair = 0; pair < 2; ++pair) {
-    const int gran = pair ? 32 : 16, units = pair ? st->n_sm / 2 : st->n_sm;
+    if (!(kinds & (pair + 1))) continue;
+    const int gran = pair || s.cap ? 32 : 16, units = pair ? st->n_sm / 2 : st->n_sm;
     const int cols = (s.n_feat + FT * (pair + 1) - 1) / (FT * (pair + 1));
     const int fewest = (s.M + kMaxTok - 1) / kMaxTok;
-    const double pair_end = pair ? (s.cap ? 2.0 : .3) : 0.0;      // (with the row count on the device x comes in boxes of 16 rows)
+    const double pair_end = pair ? .3 : 0.0;
     int last = 0;
     for (int want = fewest; want <= fewest + 3 + fewest / 4; ++want) {
       const int tmax = ((s.M + want - 1) / want + gran - 1) / gran * gran;    // the widest tile that gives `want` tiles
@@ -1224,13 +1266,10 @@ Config choose_config(TcState* st, const Shape& s) {
       token_tiles(s.M, tmax, gran, &width, &mt);
       const long long tiles = (long long)mt * cols;
       if (want > fewest && width < 32) continue;
-      // With the row count on the device one token tile takes any of them, so it is as wide as the capacity allows: there are no
-      // clusters for tiles that turn out not to exist, which take SMs from the others.
-      const int launch_tmax = s.cap && mt == 1 ? (s.cap < kMaxTok ? (s.cap + 31) / 32 * 32 : kMaxTok) : tmax;
       auto consider = [&](double t, int cl, int cut_cols, int cut_tmax) {
         if (t < best_t) {
           best_t = t;
-          best = Config{pair != 0, launch_tmax, cl, cut_cols, cut_tmax};
+          best = Config{pair != 0, tmax, cl, cut_cols, cut_tmax};
         }
       };
       const long long full = tiles / units, rem = tiles % units;      // full waves, and a last one that has the machine to itself
@@ -1264,7 +1303,7 @@ Config choose_config(TcState* st, const Shape& s) {
       }
       // clusters of 2 to 4 parts per tile, all resident at once
       const int chunks = (width + 31) / 32;
-      for (int cl = 2; cl <= 4 && st->clusters; ++cl) {
+      for (int cl = 2; cl <= 4 && st->clusters && (kinds & 4); ++cl) {
         if (tiles * cl > units || cl * 4 > KB || !clusters_fit(st, pair, cl * (pair + 1), (int)tiles)) break;
         const double cl_ends = (chunks == 1 ? 5.6 : 6.0 + (double)chunks * (cl - 1) / cl) + .4 * (mt - 1) + pair_end;
         consider(with_stream((KB + cl - 1) / cl * est_kblock(pair, width, (double)tiles * cl / units), tiles * cl * (pair + 1.0)) + cl_ends,
@@ -1272,13 +1311,98 @@ Config choose_config(TcState* st, const Shape& s) {
       }
     }
   }
-  if (st->configs.size() >= kMapCacheMax) st->configs.clear();
-  st->configs.emplace(s, best);
   return best;
 }
 
-bool launch_config(TcState* st, const GemmArgs& a, const EpiParams& ep, const Config& c, cudaStream_t stream) {
-  if (!configure(st, c.pair)) return false;
+Config choose_config(TcState* st, const Shape& s) {
+  const auto known = st->configs.find(s);
+  if (known != st->configs.end()) return known->second;
+  Config c = estimate(st, s, 7);
+  // With the row count on the device one token tile takes any of them, so that of a cluster is as wide as the capacity allows:
+  // there are no clusters for tiles that turn out not to exist, which take SMs from the others.
+  if (s.cap && c.cl && s.M <= c.tmax) c.tmax = s.cap < kMaxTok ? (s.cap + 31) / 32 * 32 : kMaxTok;
+  if (st->configs.size() >= kMapCacheMax) st->configs.clear();
+  st->configs.emplace(s, c);
+  return c;
+}
+
+// The division for every row count that a launch may find on the device: the caller's hint decides between single CTAs, pairs and
+// clusters, everything else is chosen as if the row count were known.  All rows of an entry have the same token tiles (tile
+// widths and entries are multiples of 32 rows).
+DevPlan make_plan(const std::function<Config(int)>& config_of, int cap, int n_feat, int K, bool pair, int n_sm) {
+  const int mul = pair ? 2 : 1, n_units = n_sm / mul, n_cols = (n_feat + FT * mul - 1) / (FT * mul);
+  DevPlan p;
+  for (int i = 0; i < kPlanRows; ++i) {
+    const int rows = 32 * (i + 1) < cap ? 32 * (i + 1) : cap;      // (entries behind the capacity are not read)
+    if (i > 0 && 32 * i >= cap) {
+      p.tmax[i] = p.tmax[i - 1];
+      p.cut_tmax[i] = p.cut_tmax[i - 1];
+      p.cut_cols[i] = p.cut_cols[i - 1];
+      continue;
+    }
+    const Config c = config_of(rows);
+    p.tmax[i] = (uint8_t)((c.tmax + 31) / 32);
+    p.cut_tmax[i] = (uint8_t)((c.cut_tmax + 31) / 32);
+    const Tiling t = tiling(rows, 32 * p.tmax[i], 32, c.cut_cols, 32 * p.cut_tmax[i], K / BK, n_units);
+    const bool fits = c.cut_cols <= n_cols && c.cut_cols < 65536 && t.cut_mt <= n_units && (long long)t.cut_mt * c.cut_cols * mul <= kSplitCounters;
+    p.cut_cols[i] = (uint16_t)(fits ? c.cut_cols : 0);
+  }
+  return p;
+}
+DevPlan device_plan(TcState* st, const Shape& s, bool pair) {
+  const Shape key{pair ? 2 : 1, s.n_feat, s.K, s.cap};
+  const auto known = st->plans.find(key);
+  if (known != st->plans.end()) return known->second;
+  const DevPlan p = make_plan([&](int rows) { return estimate(st, Shape{rows, s.n_feat, s.K, s.cap}, pair ? 2 : 1); }, s.cap, s.n_feat,
+                              s.K, pair, st->n_sm);
+  if (st->plans.size() >= kMapCacheMax) st->plans.clear();
+  st->plans.emplace(key, p);
+  return p;
+}
+
+// What a launch of M rows (row count on the device, cap > 0: of any number up to cap, M of them expected) runs: the estimate's
+// choice, or what the debugging aid forces: single CTAs (64, 128, 256 tokens) or pairs (384: 128, 512: 256 tokens), tiles whole
+// or cut over K.  *plan: with the row count on the device and no clusters, the division for every row count.
+Config configuration(TcState* st, int M, int n_feat, int K, int cap, DevPlan* plan) {
+  const Shape s{M, n_feat, K, cap};
+  const Config chosen = choose_config(st, s);
+  const int f = st->force_tile;
+  if (!f && st->force_s != 1) {
+    if (cap && !chosen.cl) *plan = device_plan(st, s, chosen.pair);
+    return chosen;
+  }
+  auto forced = [&](int rows) {
+    Config c = f ? Config{f > 256, f == 384 ? 128 : (f == 512 ? 256 : f), 0, 0, 0} : chosen;
+    const int gran = c.pair || cap ? 32 : 16, units = c.pair ? st->n_sm / 2 : st->n_sm, mul = c.pair ? 2 : 1;
+    const int cols = (n_feat + FT * mul - 1) / (FT * mul);
+    int width, mt;
+    token_tiles(rows, c.tmax, gran, &width, &mt);
+    const int tiles = mt * cols;
+    c.cl = 0;
+    c.cut_cols = 0;
+    c.cut_tmax = c.tmax;
+    if (!st->force_s) return c;
+    for (int cl = 4; cl >= 2 && st->clusters && !c.cl; --cl)
+      if (tiles * cl <= units && cl * 4 <= K / BK && clusters_fit(st, c.pair, cl * mul, tiles)) c.cl = cl;
+    // else all columns of less than two waves, or the last one-to-two waves of more
+    const int cut = tiles < 2 * units ? cols : cols - (tiles / units - 1) * units / mt;
+    if (!c.cl && mt <= units && mt * cut * mul <= kSplitCounters) c.cut_cols = cut;
+    return c;
+  };
+  const Config c = forced(cap ? cap : M);
+  const int mul = c.pair ? 2 : 1;
+  if (cap && !c.cl)
+    *plan = make_plan([&](int rows) {
+      Config r = forced(rows);
+      if (r.cl) r.cut_cols = (n_feat + FT * mul - 1) / (FT * mul);       // (no clusters in this launch)
+      return r;
+    }, cap, n_feat, K, c.pair, st->n_sm);
+  return c;
+}
+
+bool launch_config(TcState* st, const GemmArgs& a, const EpiParams& ep, const Config& c, const DevPlan* plan, cudaStream_t stream) {
+  const bool dev = a.m_dev != nullptr;
+  if (!configure(st, c.pair, dev)) return false;
   const bool swiglu = a.epi == EPI_SWIGLU;
   const int mul = c.pair ? 2 : 1;
   const uint64_t w_rows = swiglu ? 2ull * a.N : (uint64_t)a.N;
@@ -1286,38 +1410,35 @@ bool launch_config(TcState* st, const GemmArgs& a, const EpiParams& ep, const Co
   g.m_cap = a.M;
   g.K = a.K;
   g.n_cols = (int)((w_rows + FT * mul - 1) / (FT * mul));
-  // (with the row count on the device the width of the token tiles is, too: x is then loaded in boxes of 32 or 16 rows)
-  g.gran = a.m_dev ? 32 : (c.pair ? 32 : 16);
-  g.tmax = (c.tmax + g.gran - 1) / g.gran * g.gran;
-  token_tiles(a.M, g.tmax, g.gran, &g.width, &g.mt);
-  const int width = g.width, mt = g.mt;
-  g.x_box = a.m_dev ? 32 / mul : width / mul;
-  const int n_units = c.pair ? st->n_sm / 2 : st->n_sm;       // scheduling units: CTAs or pairs
-  const int n_tiles = mt * g.n_cols, KB = a.K / BK;
+  const int gran = c.pair || dev ? 32 : 16, n_units = c.pair ? st->n_sm / 2 : st->n_sm;       // scheduling units: CTAs or pairs
+  const int KB = a.K / BK;
+  g.tmax = (c.tmax + gran - 1) / gran * gran;
+  g.tiles = tiling(a.M, g.tmax, gran, dev ? 0 : c.cut_cols, (c.cut_tmax + gran - 1) / gran * gran, KB, n_units);
+  const Tiling& t = g.tiles;
+  const int n_tiles = t.mt * g.n_cols;
   int units = n_tiles < n_units ? n_tiles : n_units;
   g.cl = c.cl;
-  g.cut_box = g.x_box;
   if (c.cl) {
     units = n_tiles * c.cl;   // one cluster per tile; the kernel derives each member's k-blocks from its rank
-  } else if (a.m_dev) {
-    // the row count is on the device: the kernel counts the tiles and divides the cut ones itself; the grid has every unit
-    // (units without work leave at once)
-    g.cut_cols = c.cut_cols && (long long)n_tiles * mul <= kSplitCounters ? -1 : 0;
-    units = n_units;
-  } else if (c.cut_cols) {
-    const int cut_tmax = (c.cut_tmax + g.gran - 1) / g.gran * g.gran;
-    g.cut_cols = c.cut_cols;
-    token_tiles(a.M, cut_tmax < width ? cut_tmax : width, g.gran, &g.cut_width, &g.cut_mt);
-    g.cut_box = g.cut_width / mul;
-    if (g.cut_mt > n_units || g.cut_mt * g.cut_cols * mul > kSplitCounters) return false;
-    g.per = cut_range(g.cut_cols, g.cut_mt, KB, n_units);
-    const int whole = (g.n_cols - g.cut_cols) * mt, used = (g.cut_cols * KB + g.per - 1) / g.per * g.cut_mt;
+  } else if (dev) {
+    units = n_units;          // (units without work leave at once)
+  } else if (t.cut_cols) {
+    if (t.cut_mt > n_units || t.cut_mt * t.cut_cols * mul > kSplitCounters) return false;
+    const int whole = (g.n_cols - t.cut_cols) * t.mt, used = (t.cut_cols * KB + t.per - 1) / t.per * t.cut_mt;
     units = whole > used ? (whole < n_units ? whole : n_units) : used;
   }
-  CUtensorMap mw, mx, mxc;     // copies: see cached_map
+  CUtensorMap mw;              // copies: see cached_map
+  XMaps<false> xh;
+  XMaps<true> xd;
   const WeightOrder order = swiglu ? kWSwiglu : (a.epi == EPI_QKV_ROPE ? (a.head_dim == 128 ? kWRope128 : kWRope64) : kWPlain);
   if (!get_w_map(st, a.w, w_rows, a.K, order, &mw, &g.w_step3, &g.w_step4)) return false;
-  if (!get_x_map(st, a.x, a.M, a.K, g.x_box, &mx) || !get_x_map(st, a.x, a.M, a.K, g.cut_box, &mxc)) return false;
+  if (dev) {
+    for (int i = 0; i < kMaxTok / 32; ++i)
+      if (!get_x_map(st, a.x, a.M, a.K, 32 * (i + 1) / mul, &xd.wide[i])) return false;
+    if (plan) xd.plan = *plan;
+  } else if (!get_x_map(st, a.x, a.M, a.K, t.width / mul, &xh.whole) || !get_x_map(st, a.x, a.M, a.K, t.cut_width / mul, &xh.cut)) {
+    return false;
+  }
   g.split_ws = st->split_ws;
   g.split_counters = st->split_counters;
   g.m_dev = a.m_dev;
@@ -1345,8 +1466,8 @@ bool launch_config(TcState* st, const GemmArgs& a, const EpiParams& ep, const Co
   }
   cfg.attrs = attr;
   cfg.numAttrs = n_attr;
-  return (c.pair ? cudaLaunchKernelEx(&cfg, gemm_tc_kernel<true>, mw, mx, mxc, g, ep)
-                 : cudaLaunchKernelEx(&cfg, gemm_tc_kernel<false>, mw, mx, mxc, g, ep)) == cudaSuccess;
+  return (dev ? cudaLaunchKernelEx(&cfg, kernel_dev(c.pair), mw, xd, g, ep)
+              : cudaLaunchKernelEx(&cfg, kernel_host(c.pair), mw, xh, g, ep)) == cudaSuccess;
 }
 
 }  // namespace
@@ -1380,6 +1501,21 @@ void tc_state_force(void* s, int tile, int stream_k) {
   st->force_s = stream_k;
   st->clusters = stream_k != 2;     // 2: cut tiles always go through the partial-tile workspace
   st->configs.clear();
+  st->plans.clear();
+}
+
+// debugging aid: what a launch of `rows` rows runs (cap > 0: row count on the device, `hint` rows expected and at most cap)
+bool tc_state_plan(void* s, int rows, int n_feat, int K, int hint, int cap, int (&out)[8]) {
+  TcState* st = static_cast<TcState*>(s);
+  if (!st || rows <= 0 || n_feat <= 0 || n_feat % 16 || K <= 0 || K % BK || (cap && (rows > cap || hint <= 0 || hint > cap))) return false;
+  DevPlan plan;
+  const Config c = configuration(st, cap ? hint : rows, n_feat, K, cap, &plan);
+  const int mul = c.pair ? 2 : 1, gran = c.pair || cap ? 32 : 16, n_units = st->n_sm / mul;
+  const Tiling t = cap && !c.cl ? planned(plan, rows, K / BK, n_units)
+                                : tiling(rows, (c.tmax + gran - 1) / gran * gran, gran, cap ? 0 : c.cut_cols, (c.cut_tmax + gran - 1) / gran * gran, K / BK, n_units);
+  const int got[8] = {c.pair, t.width, t.mt, c.cl, (n_feat + FT * mul - 1) / (FT * mul), t.cut_cols, t.cut_width, t.per};
+  memcpy(out, got, sizeof(got));
+  return true;
 }
 
 void tc_state_reset(void* s, cudaStream_t stream) {
@@ -1465,27 +1601,10 @@ bool launch_gemm_tc(const GemmArgs& a, void* tc_state, int* status, cudaStream_t
   const int n_feat = a.epi == EPI_SWIGLU ? 2 * a.N : a.N;
   // (device-resident rounds: the configuration is chosen for the caller's hint of the row count, the launch covers the capacity)
   const int Mc = (a.m_dev && a.m_hint > 0 && a.m_hint < a.M) ? a.m_hint : a.M;
-  Config c = choose_config(st, Shape{Mc, n_feat, a.K, a.m_dev ? a.M : 0});
-  if (st->force_tile || st->force_s == 1) {   // debugging aid: single CTAs (64, 128, 256 tokens) or pairs (384: 128, 512: 256 tokens)
-    const int f = st->force_tile;
-    if (f) c = Config{f > 256, f == 384 ? 128 : (f == 512 ? 256 : f), 0, 0, 0};
-    const int gran = c.pair ? 32 : 16, units = c.pair ? st->n_sm / 2 : st->n_sm;
-    int width, mt;
-    token_tiles(a.M, c.tmax, gran, &width, &mt);
-    const int cols = (n_feat + FT * (c.pair + 1) - 1) / (FT * (c.pair + 1)), tiles = mt * cols;
-    c.cl = 0;
-    c.cut_cols = 0;
-    c.cut_tmax = c.tmax;
-    if (st->force_s) {
-      for (int cl = 4; cl >= 2 && st->clusters && !c.cl; --cl)
-        if (tiles * cl <= units && cl * 4 <= a.K / BK && clusters_fit(st, c.pair, cl * (c.pair + 1), tiles)) c.cl = cl;
-      // else all columns of less than two waves, or the last one-to-two waves of more
-      const int cut = tiles < 2 * units ? cols : cols - (tiles / units - 1) * units / mt;
-      if (!c.cl && mt <= units && mt * cut * (c.pair + 1) <= kSplitCounters) c.cut_cols = cut;
-    }
-  }
+  DevPlan plan;
+  const Config c = configuration(st, Mc, n_feat, a.K, a.m_dev ? a.M : 0, &plan);
   if (ss_slots_out) *ss_slots_out = (a.N + FT - 1) / FT;
-  return launch_config(st, a, ep, c, stream);
+  return launch_config(st, a, ep, c, a.m_dev && !c.cl ? &plan : nullptr, stream);
 }
 
 }  // namespace recg

@@ -173,6 +173,7 @@ void tc_state_destroy(void* s);
 // at most that width, 384 / 512: CTA pairs with token tiles of at most 128 / 256; 0 = back to the cost model) and the
 // decomposition (0 whole tiles, 1 tiles cut over K, 2 the same without the hand-over inside clusters)
 void tc_state_force(void* s, int tile, int stream_k);
+bool tc_state_plan(void* s, int rows, int n_feat, int K, int hint, int cap, int (&out)[8]);
 // zero the arrival counters of cut tiles (after a launch that ended with an error status)
 void tc_state_reset(void* s, cudaStream_t st);
 // host-only self-test of the tensor-map cache; returns the number of wrong maps handed out

@@ -967,6 +967,16 @@ recg_status recg_debug_gemm_config(recg_ctx* ctx, int32_t tile, int32_t stream_k
   return RECG_OK;
 }
 
+recg_status recg_debug_gemm_plan(recg_ctx* ctx, int32_t rows, int32_t n_features, int32_t K, int32_t rows_hint, int32_t capacity,
+                                 int32_t* out) {
+  if (!ctx || !out) return RECG_ERR_INVALID_ARG;
+  int got[8];
+  if (capacity < 0 || !tc_state_plan(ctx->tc_state, rows, n_features, K, rows_hint, capacity, got))
+    return fail(ctx, RECG_ERR_INVALID_ARG, "recg_debug_gemm_plan: no such launch");
+  memcpy(out, got, sizeof(got));
+  return RECG_OK;
+}
+
 recg_status recg_debug_wait_timeout(recg_ctx* ctx, int32_t max_polls) {
   if (!ctx) return RECG_ERR_INVALID_ARG;
   if (max_polls < 1 || max_polls > (1 << 20)) return fail(ctx, RECG_ERR_INVALID_ARG, "recg_debug_wait_timeout: max_polls must be 1 .. 1048576");

@@ -154,6 +154,49 @@ def test_device_round_that_breaks_a_capacity_is_refused_on_the_device():
     ctx.recg_free()
 
 
+@pytest.mark.parametrize("rows,hint,capacity", [(300, 300, 1000), (376, 376, 1024), (376, 1024, 1024), (512, 512, 512), (700, 700, 1024),
+                                                (1000, 1000, 1000), (1000, 300, 1000), (257, 700, 704), (290, 64, 320), (2100, 2100, 2112)])
+def test_device_round_of_several_token_tiles(rows, hint, capacity):
+    """Rows in two and more token tiles: whole tiles, tiles cut over K in the last columns or in all of them, as many rows as
+    expected, fewer and more.  The division is the one a launch with the rows known to the host has (where it uses CTA pairs,
+    too, and no clusters), and the logits are those of the host's step within the batch-invariance tolerance."""
+    shape = synth.llama8b_shape(1)
+    shape.vocab = 8192
+    W = synth.model_weights(shape, seed=0, dtype=torch.bfloat16)
+    Wd = {k: ([t.cuda() for t in v] if isinstance(v, list) else v.cuda()) for k, v in W.items()}
+    n = 12
+    tot = np.array([rows // n] * n)
+    tot[:rows - tot.sum()] += 1
+    v = np.arange(n) * 7 % np.minimum(tot, 64)
+    desc = synth.fixed_descriptor(np.arange(n) * 37, v, tot - v, seed=31)
+    ctx = binding.Context(binding.make_config(shape, n, capacity, desc.page_table.shape[1]), Wd)
+    compared = 0
+    for n_feat, K in ((6144, 4096), (4096, 4096), (28672, 4096), (4096, 14336), (8192, 4096)):
+        host, dev = ctx.recg_debug_gemm_plan(rows, n_feat, K), ctx.recg_debug_gemm_plan(rows, n_feat, K, hint, capacity)
+        assert dev["width"] % 32 == 0 and (dev["tiles"] - 1) * dev["width"] < rows <= dev["tiles"] * dev["width"]
+        assert 0 <= dev["cut_columns"] <= dev["columns"] and dev["cut_width"] % 32 == 0 and dev["cut_width"] <= dev["width"]
+        if rows <= 2048 and host["pair"] and dev["pair"] and not host["cluster"] and not dev["cluster"]:
+            assert host == dev, (n_feat, K)
+            compared += 1
+        if n_feat == 28672 and hint > 256 and rows not in (700, 2100):
+            assert 0 < dev["cut_columns"] < dev["columns"] and dev["cut_width"] < dev["width"]       # a ragged end
+    assert compared >= (3 if hint > 256 and rows <= 2048 else 0)
+    pool = binding.alloc_kv_pool(ctx, desc.n_pages, fill="normal")
+    ys = synth.token_ids(int(desc.verify_len.sum()), shape.vocab, seed=1)
+    batch = binding.Batch(desc.ctx_len, desc.verify_len, desc.block_size, ys, desc.page_table, pool, desc.n_pages)
+    ref = ctx.logits_tensor(ctx.recg_step(batch))
+    cuv = np.concatenate([[0], np.cumsum(desc.verify_len)])
+    pt = np.where(desc.page_table >= 0, desc.page_table, 0)
+    db = binding.DeviceBatch(desc.ctx_len, desc.verify_len, desc.block_size, [ys[cuv[i]:cuv[i + 1]].tolist() for i in range(n)], 64, pt,
+                             pool, desc.n_pages, rows_hint=hint)
+    for _ in range(2):                       # (the arrival counters of cut tiles are clean again behind the first one)
+        lg = ctx.recg_step_device(db)
+        got = binding.device_view(lg.data, (lg.n_rows, lg.vocab), torch.float32)[:rows].clone()
+        ctx.recg_sync()
+        assert float((got - ref).abs().max()) <= 1e-2 * float(ref.abs().max())
+    ctx.recg_free()
+
+
 @pytest.mark.parametrize("verify,block", [([-1, 1], [4, 4]), ([1, -3], [4, 9]), ([1, 1], [4, -2]), ([0, 1], [0, 4])])
 def test_device_round_with_broken_lengths_is_an_empty_round(verify, block):
     """Negative lengths, and a request without rows: the verification of the empty round looks at no row of any request (no

@@ -136,6 +136,17 @@ def test_ragged_end_cut_in_narrower_tiles(M, N, K):
     ctx.recg_free()
 
 
+@pytest.mark.parametrize("M,N,K", [(333, 19088, 2048), (376, 9600, 4096), (700, 14336, 4096), (701, 19088, 2048), (333, 28672, 2048),
+                                   (376, 28672, 2048)])
+def test_sizes_of_the_ragged_end_tests_are_cut(M, N, K):
+    """The sizes of the tests above and below are divided as those say: some of the columns cut, in narrower token tiles."""
+    ctx = binding.Context(binding.make_config(synth.tiny_shape(), 1, 8, 1))
+    p = ctx.recg_debug_gemm_plan(M, N, K)
+    assert 0 < p["cut_columns"] < p["columns"] and p["cut_width"] < p["width"] and not p["cluster"], p
+    assert p["cut_range"] < p["cut_columns"] * K // 64           # several teams, so tiles in several parts
+    ctx.recg_free()
+
+
 @pytest.mark.parametrize("n", [333, 376])
 def test_ragged_end_cut_of_a_whole_step(n):
     """The same division inside a step: 28672 gate and up rows of 2048 at these row counts (SwiGLU epilogue, RMSNorm folded)."""
