@@ -53,7 +53,7 @@ enum {
   RECG_FLAG_FOLD_NORM = 16,  /* fold every RMSNorm into the projections around it: the projection that updates the residual
                                 stream also writes x = bf16(h * gain) and per-row partial sums of squares, the projection
                                 that reads x scales its rows by the row's rstd.  This is what the tcgen05 projections do
-                                in any case; the flag is kept for callers that set it                         */
+                                in any case: the flag is kept for callers that set it and changes nothing     */
   RECG_FLAG_CHAIN = 32,      /* steps of at most 128 rows (low concurrency): run the projections between two attention
                                 calls (output projection, gate|up, down, the next layer's QKV projection or the LM head)
                                 as ONE persistent kernel with grid-wide barriers, so that the weight stream does not stop
@@ -359,7 +359,7 @@ recg_status recg_policy_step(recg_ctx *ctx, const recg_policy_state *state, cons
  * from a table by the row count), and recg_logits.n_rows reports max_tokens; the true counts are in the device arrays.  Lengths that break a capacity
  * (negative, a request without rows, verify_len > max_verify, rows beyond the page-table row, more than max_tokens rows
  * in total) set the device status word and turn the round into an empty one: recg_sync() then returns
- * RECG_ERR_INTERNAL.  Not available with RECG_FLAG_SIMT_GEMM or RECG_FLAG_FOLD_NORM.
+ * RECG_ERR_INTERNAL.  Not available with RECG_FLAG_SIMT_GEMM.
  *
  * recg_next_round() turns the finished round (the library's own verification buffers: call recg_verify with NULL
  * output pointers or leave them out) into the next one, per request:

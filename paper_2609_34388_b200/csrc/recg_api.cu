@@ -726,8 +726,8 @@ static DeviceRound device_round(const recg_ctx* ctx, const recg_device_batch* b)
 recg_status recg_step_device(recg_ctx* ctx, const recg_device_batch* b, recg_logits* logits) {
   if (!ctx) return RECG_ERR_INVALID_ARG;
   if (!ctx->has_weights) return fail(ctx, RECG_ERR_INVALID_ARG, "recg_step_device: the context was created without weights");
-  if (ctx->cfg.flags & (RECG_FLAG_SIMT_GEMM | RECG_FLAG_FOLD_NORM))
-    return fail(ctx, RECG_ERR_INVALID_ARG, "recg_step_device: not available with RECG_FLAG_SIMT_GEMM or RECG_FLAG_FOLD_NORM");
+  if (ctx->cfg.flags & RECG_FLAG_SIMT_GEMM)
+    return fail(ctx, RECG_ERR_INVALID_ARG, "recg_step_device: not available with RECG_FLAG_SIMT_GEMM");
   recg_status s = check_device_batch(ctx, b, "recg_step_device");
   if (s != RECG_OK) return s;
   ctx->logits_valid = false;

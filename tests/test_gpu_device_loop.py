@@ -154,6 +154,28 @@ def test_device_round_that_breaks_a_capacity_is_refused_on_the_device():
     ctx.recg_free()
 
 
+def test_device_round_with_the_folded_norm_flag():
+    """RECG_FLAG_FOLD_NORM names what the projections do in any case: a device round of a context that has it is the round of one
+    that has not, bit for bit."""
+    shape, Wd, ocfg, W64 = tiny()
+    pt, n_pages = synth.page_tables([10, 30], [40, 40], 16, seed=7)
+    got = []
+    for flags in (0, binding.FLAG_FOLD_NORM):
+        ctx = binding.Context(binding.make_config(shape, 2, 64, pt.shape[1], flags), Wd)
+        pool = torch.empty(ctx.kv_pool_bytes(n_pages) // 2, dtype=torch.bfloat16, device="cuda")
+        pool.normal_(generator=torch.Generator(device="cuda").manual_seed(3))
+        db = binding.DeviceBatch([10, 30], [3, 1], [8, 16], [[1, 2, 3], [4]], 8, pt, pool, n_pages)
+        lg = ctx.recg_step_device(db)
+        logits = binding.device_view(lg.data, (lg.n_rows, lg.vocab), torch.float32)[:28].clone()
+        out = binding.VerifyOut(2, 28, 4, host=False)
+        ctx.recg_verify(None, None, host=False, out=out)
+        ctx.recg_sync()
+        got.append((logits, {k: t.clone() for k, t in out.views().items()}))
+        ctx.recg_free()
+    assert torch.equal(got[0][0], got[1][0])
+    assert all(torch.equal(t, got[1][1][k]) for k, t in got[0][1].items())
+
+
 @pytest.mark.parametrize("rows,hint,capacity", [(300, 300, 1000), (376, 376, 1024), (376, 1024, 1024), (512, 512, 512), (700, 700, 1024),
                                                 (1000, 1000, 1000), (1000, 300, 1000), (257, 700, 704), (290, 64, 320), (2100, 2100, 2112)])
 def test_device_round_of_several_token_tiles(rows, hint, capacity):
