@@ -203,12 +203,19 @@ __global__ void __launch_bounds__(kVerifyThreads, 4) verify_partial_kernel(const
     ms.s = s2.x + s2.y;
     ms.t = t2.x + t2.y;
   }
-  // elements outside whole vectors (unaligned rows: all of them)
-  for (int i = c0 + nvec * N + tid; i < c1; i += kVerifyThreads) {
-    const float x = Vec<T>::one(base + i);
-    mass_rebase(ms, x);
-    mass_add(ms, x, ms.m > -INFINITY ? -ms.m * kLog2e : 0.f);
-    if (x >= tp.m2) top2_insert(tp, x, i);
+  // elements outside whole vectors (unaligned rows: all of them), four loads in flight per thread: 5000 x 50257 fp32 379 us, one
+  // by one 743
+  for (int i = c0 + nvec * N + tid; i < c1; i += 4 * kVerifyThreads) {
+    float x[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) x[u] = i + u * kVerifyThreads < c1 ? Vec<T>::one(base + i + u * kVerifyThreads) : -INFINITY;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      if (i + u * kVerifyThreads >= c1) break;
+      mass_rebase(ms, x[u]);
+      mass_add(ms, x[u], ms.m > -INFINITY ? -ms.m * kLog2e : 0.f);
+      if (x[u] >= tp.m2) top2_insert(tp, x[u], i + u * kVerifyThreads);
+    }
   }
   const float e1 = tp.m1, e2 = tp.m2;
   // the CTA's largest and second-largest of the groups' maxima and the single elements

@@ -70,3 +70,20 @@ def test_rows_of_a_request(reqs, vocab, host):
         tv0 += v[r]
         tb0 += b[r]
     ctx.recg_free()
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("vocab", [3, 255, 257, 1023, 1025, 1279, 2049, 5001, 50257])
+def test_rows_of_any_alignment(vocab, dtype):
+    """Rows of an odd vocabulary begin on every element boundary: most have no 16-byte vectors, and the elements of a thread end in
+    every remainder of four.  Every second row has many equal values: the lowest index wins."""
+    logits = synth.logits_normal(9, vocab, seed=vocab, device="cuda", dtype=dtype)
+    logits[::2] = logits[::2].round()
+    got = binding.recg_row_stats_static(logits)
+    torch.cuda.synchronize()
+    host = logits.double().cpu().numpy()
+    for r in range(9):
+        want = orc.row_stats(host[r])
+        assert int(got["top1"][r]) == want["top1"] and int(got["top2"][r]) == want["top2"], r
+        for k in ("p1", "p2", "entropy"):          # as above: fp32 sums, 2^x of the hardware
+            assert abs(float(got[k][r]) - want[k]) <= 1e-5 * max(want[k], 1e-3 if k == "entropy" else 0.0), (k, r)
