@@ -1258,7 +1258,11 @@ Config estimate(TcState* st, const Shape& s, int kinds) {
     const int fewest = (s.M + kMaxTok - 1) / kMaxTok;
     const double pair_end = pair ? .3 : 0.0;
     int last = 0;
-    for (int want = fewest; want <= fewest + 3 + fewest / 4; ++want) {
+    // (few k-blocks: the epilogue is what takes time, so as many and narrow tiles as one wave holds.  256 x 256 weights at 1024
+    // rows, fp32 results, 3.7 us, 4.9 with a few more tiles than the fewest; 16 x 64 at 4000 rows 4.7 and 5.2; a prefill of the
+    // 2-layer model of width 256 at 1024 rows 103 and 118)
+    const int most = fewest + 3 + fewest / 4, wave = KB <= 4 ? units / cols : 0;
+    for (int want = fewest; want <= (wave > most ? wave : most); ++want) {
       const int tmax = ((s.M + want - 1) / want + gran - 1) / gran * gran;    // the widest tile that gives `want` tiles
       if (tmax == last || tmax < gran) continue;
       last = tmax;
