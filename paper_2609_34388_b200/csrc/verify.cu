@@ -34,6 +34,10 @@ struct Mass {
   float m, s, t;
 };
 constexpr float kLog2e = 1.4426950408889634f;
+// The moving maximum starts no lower than this: masked logits (-inf, the type's lowest value, -1e30) then underflow to zero while
+// a thread or a chunk has seen nothing else, where x log2(e) - m log2(e) would overflow or cancel to anything.  (Below it the
+// product's rounding error reaches the exponent's range; no logit that counts lies there.)
+constexpr float kMassFloor = -1.0e9f;
 __device__ __forceinline__ void mass_rebase(Mass& a, float m_new) {
   if (m_new > a.m) {
     const float f = a.s > 0.f ? exp2f((a.m - m_new) * kLog2e) : 0.f;   // a.m may be -inf with s = t = 0
@@ -176,9 +180,9 @@ __global__ void __launch_bounds__(kVerifyThreads, 4) verify_partial_kernel(const
       fetch(i + 4 * kVerifyThreads, nxt);
       const float gm = Vec<T>::max_of(cur);
       if (gm > ms.m) {
-        const float f = exp2f((ms.m - gm) * kLog2e);      // 0 the first time
+        const float m = fmaxf(gm, kMassFloor), f = exp2f((ms.m - m) * kLog2e);      // 0 the first time
         s2.x *= f; s2.y *= f; t2.x *= f; t2.y *= f;
-        ms.m = gm;
+        ms.m = m;
       }
       const bool b1 = gm > g1, b2 = gm > g2;
       i2 = b1 ? i1 : (b2 ? i : i2);
@@ -212,7 +216,7 @@ __global__ void __launch_bounds__(kVerifyThreads, 4) verify_partial_kernel(const
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       if (i + u * kVerifyThreads >= c1) break;
-      mass_rebase(ms, x[u]);
+      mass_rebase(ms, fmaxf(x[u], kMassFloor));
       mass_add(ms, x[u], ms.m > -INFINITY ? -ms.m * kLog2e : 0.f);
       if (x[u] >= tp.m2) top2_insert(tp, x[u], i + u * kVerifyThreads);
     }
@@ -255,7 +259,7 @@ __global__ void __launch_bounds__(kVerifyThreads, 4) verify_partial_kernel(const
           if (x[k] >= tp.m2) top2_insert(tp, x[k], c0 + (i + u * kVerifyThreads) * N + k);
     }
   }
-  const float f = ms.m > -INFINITY ? exp2f((ms.m - h1) * kLog2e) : 0.f;
+  const float f = ms.m > -INFINITY ? exp2f((ms.m - fmaxf(h1, kMassFloor)) * kLog2e) : 0.f;
   ms.s *= f;
   ms.t *= f;
   const bool any = __any_sync(0xffffffffu, tp.i1 != 0x7fffffff);

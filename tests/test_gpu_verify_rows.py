@@ -1,5 +1,7 @@
 """The per-request end of verification where its paths change: requests on both sides of the rows it keeps in shared memory
 (256), accept scans that cross a warp's 32 rows, few and many vocabulary chunks per row, results on the host and on the device."""
+import math
+
 import numpy as np
 import pytest
 import torch
@@ -86,4 +88,29 @@ def test_rows_of_any_alignment(vocab, dtype):
         want = orc.row_stats(host[r])
         assert int(got["top1"][r]) == want["top1"] and int(got["top2"][r]) == want["top2"], r
         for k in ("p1", "p2", "entropy"):          # as above: fp32 sums, 2^x of the hardware
+            assert abs(float(got[k][r]) - want[k]) <= 1e-5 * max(want[k], 1e-3 if k == "entropy" else 0.0), (k, r)
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("mask", ["lowest", -1e30, -2e9, -1e9, -math.inf])
+@pytest.mark.parametrize("vocab", [2048, 50257, 128256])
+def test_masked_logits(vocab, mask, dtype):
+    """Masked entries carry no probability whatever value stands for them, also where a thread or a whole chunk of the vocabulary
+    sees nothing else: a masked tail (a padded vocabulary), a masked head, all but every 97th and all but three entries."""
+    value = torch.finfo(dtype).min if mask == "lowest" else mask
+    logits = synth.logits_normal(4, vocab, seed=vocab, device="cuda", dtype=dtype)
+    keep = torch.zeros((4, vocab), dtype=torch.bool, device="cuda")
+    keep[0, :vocab - vocab // 3] = True
+    keep[1, vocab // 2:] = True
+    keep[2, ::97] = True
+    keep[3, [5, vocab // 2, vocab - 1]] = True
+    logits = logits.masked_fill(~keep, value)
+    got = binding.recg_row_stats_static(logits)
+    torch.cuda.synchronize()
+    host, kept = logits.double().cpu().numpy(), keep.cpu().numpy()
+    for r in range(4):
+        ids = np.nonzero(kept[r])[0]
+        want = orc.row_stats(host[r][ids])       # the entries that are not masked are all there is
+        assert int(got["top1"][r]) == ids[want["top1"]] and int(got["top2"][r]) == ids[want["top2"]], r
+        for k in ("p1", "p2", "entropy"):
             assert abs(float(got[k][r]) - want[k]) <= 1e-5 * max(want[k], 1e-3 if k == "entropy" else 0.0), (k, r)
