@@ -355,7 +355,7 @@ __device__ __forceinline__ void load_gain(const EpiParams& ep, int tile, int qua
 }
 __device__ __forceinline__ void prefetch_chunk(const EpiParams& ep, const TileOut& o, int c, float (&pre)[32]) {
   const int rg = o.lane >> 2, tok = c * 32 + 2 * (o.lane & 3), nv = o.nv;
-  if (ep.epi == EPI_RESIDUAL || ep.epi == EPI_RESIDUAL_NORM) {
+  if (ep.epi == EPI_RESIDUAL_NORM) {
     const int f = o.tile * FT + o.quad * 32 + rg;
     const float* h = static_cast<const float*>(ep.out) + (size_t)(o.t0 + tok) * ep.N + f;
 #pragma unroll
@@ -427,10 +427,9 @@ __device__ __forceinline__ void tile_out(const EpiParams& ep, const Source& src,
       }
     }
   };
-  if (ep.epi == EPI_RESIDUAL || ep.epi == EPI_RESIDUAL_NORM) {
+  if (ep.epi == EPI_RESIDUAL_NORM) {
     // every element has one writer, so the residual add is a load (ahead of the accumulator) and a store; the new value also
     // gives the next norm's input x = bf16(h * gain) and the row's sum of squares over this tile's features
-    const bool norm = ep.epi == EPI_RESIDUAL_NORM;
 #pragma unroll 1
     for (int c = c0, nth = 0; c < c1; c += step, ++nth) {
       const int nv = o.nv - c * 32;
@@ -454,7 +453,6 @@ __device__ __forceinline__ void tile_out(const EpiParams& ep, const Source& src,
           sq[2 * k + e] = s;
         }
       if (c + step < c1) prefetch_chunk(ep, o, c + step, pre);
-      if (!norm) continue;
       stage_rows32(o, v);
       __nv_bfloat16* xp = ep.x_out + (size_t)(o.t0 + c * 32) * ep.N + f0;
       unstage_rows32(o, nv, [&](int t, int p, const uint4& w) {
@@ -473,13 +471,11 @@ __device__ __forceinline__ void tile_out(const EpiParams& ep, const Source& src,
       // thread holds index rg = 2 k + e
       o.ss[o.quad * kMaxTok + c * 32 + 8 * (rg >> 1) + 2 * tq + (rg & 1)] = sq[0];
     }
-    if (norm) {
-      asm volatile("bar.sync 1, 128;" ::: "memory");
-      for (int t = (c0 + o.quad * step) * 32 + lane; t < o.nv; t += 128 * step)       // warp w sums the chunks c0 + w step, ...
-        ep.ss_out[(size_t)o.tile * ep.ss_stride + o.t0 + t] =
-            (o.ss[t] + o.ss[kMaxTok + t]) + (o.ss[2 * kMaxTok + t] + o.ss[3 * kMaxTok + t]);
-      asm volatile("bar.sync 1, 128;" ::: "memory");      // (the sums may be overwritten)
-    }
+    asm volatile("bar.sync 1, 128;" ::: "memory");
+    for (int t = (c0 + o.quad * step) * 32 + lane; t < o.nv; t += 128 * step)       // warp w sums the chunks c0 + w step, ...
+      ep.ss_out[(size_t)o.tile * ep.ss_stride + o.t0 + t] =
+          (o.ss[t] + o.ss[kMaxTok + t]) + (o.ss[2 * kMaxTok + t] + o.ss[3 * kMaxTok + t]);
+    asm volatile("bar.sync 1, 128;" ::: "memory");      // (the sums may be overwritten)
     return;
   }
   if (ep.epi == EPI_SWIGLU) {
@@ -1575,8 +1571,8 @@ bool launch_gemm_tc(const GemmArgs& a, void* tc_state, int* status, cudaStream_t
   if (!st || a.M <= 0 || a.K % BK || a.N % 16) return false;
   if ((reinterpret_cast<uintptr_t>(a.x) | reinterpret_cast<uintptr_t>(a.w)) & 15) return false;
   // (bf16 rows leave in pieces of 16 bytes, fp32 ones element by element)
-  if (reinterpret_cast<uintptr_t>(a.out) & (a.epi == EPI_PLAIN_F32 || a.epi == EPI_RESIDUAL || a.epi == EPI_RESIDUAL_NORM ? 3 : 15)) return false;
-  if (a.epi == EPI_RESIDUAL_NORM && (!a.x_out || !a.gain || !a.ss_out)) return false;
+  if (reinterpret_cast<uintptr_t>(a.out) & (a.epi == EPI_PLAIN_F32 || a.epi == EPI_RESIDUAL_NORM ? 3 : 15)) return false;
+  if (a.epi == EPI_RESIDUAL || (a.epi == EPI_RESIDUAL_NORM && (!a.x_out || !a.gain || !a.ss_out))) return false;
   if (a.epi == EPI_SWIGLU && a.N % 64) return false;
   if (((int64_t)a.N * 2 / FT + 2) * (a.K / BK) > (1 << 30)) return false;      // the line of k-blocks is counted in int
   if (a.epi == EPI_QKV_ROPE && (a.N % 128 || (a.head_dim != 64 && a.head_dim != 128))) return false;

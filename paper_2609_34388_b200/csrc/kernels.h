@@ -129,7 +129,7 @@ void launch_next_round(const DeviceRound& dr, const BatchLayout& bl, const Verif
 enum Epilogue : int {
   EPI_PLAIN_BF16 = 0,  // C bf16 [M,N]
   EPI_PLAIN_F32 = 1,   // C fp32 [M,N]
-  EPI_RESIDUAL = 2,    // h fp32 [M,N] += acc
+  EPI_RESIDUAL = 2,    // h fp32 [M,N] += acc (mma.sync path only)
   EPI_SWIGLU = 3,      // w is [2F,K]; out bf16 [M,F] = silu(x.wg) * (x.wu)
   EPI_QKV_ROPE = 4,    // rotate q and k heads, q -> bf16 [M, n_q*d], k/v -> paged pool at tok_slot
   EPI_RESIDUAL_NORM = 5  // h fp32 [M,N] += acc, and the input of the next RMSNorm-ed projection: x_out bf16 [M,N] =

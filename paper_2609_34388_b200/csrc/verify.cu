@@ -134,12 +134,13 @@ __device__ __forceinline__ float2 add2(const float2& a, const float2& b) {
 
 // One-dimensional grid of rows x chunks_per_row CTAs, chunk-fastest (consecutive CTAs read consecutive memory; the
 // row count is not bound by the 65535 limit of the other grid dimensions).  Each CTA scans [c0, c1) of one row.
-// Bound by HBM for bf16 logits only if little else is done per element (6.4 TB/s is 22 elements per SM and clock, the 2^x
-// unit gives 16 of them, the issue slots 128): vectors stay packed (maxima and the clamp of -inf on two bf16 at a time), sums
-// use two-element instructions, the next four vectors of a thread are on their way while it works on four, and the search
-// for the two largest elements remembers only the two best GROUPS of four vectors per thread, of which the CTA afterwards
-// re-reads those that reach its second-largest group maximum (two, as a rule).  8448 rows x 128256 bf16, the kernel: 435 us
-// with unpacked arithmetic, loads behind the arithmetic and a search per thread, 358 us (6.05 TB/s) like this.
+// Bound by HBM for bf16 logits only if little else is done per element (6.4 TB/s is 11 elements per SM and clock: two thirds of
+// what the 2^x unit gives, and the issue slots leave 11 instructions for each): vectors stay packed (maxima and the clamp of
+// -inf on two bf16 at a time), sums use two-element instructions, the next four vectors of a thread are on their way while it
+// works on four, and the search for the two largest elements remembers only the two best GROUPS of four vectors per thread, of
+// which the CTA afterwards re-reads those that reach its second-largest group maximum (two, as a rule).  8448 rows x 128256
+// bf16, the kernel: 435 us with unpacked arithmetic, loads behind the arithmetic and a search per thread, 358 us (6.05 TB/s)
+// like this.
 template <typename T>
 __global__ void __launch_bounds__(kVerifyThreads, 4) verify_partial_kernel(const T* __restrict__ logits, int vocab,
                                                                            int chunk_len, int chunks_per_row,
