@@ -246,8 +246,8 @@ def test_tiny_prefill_through_the_step():
 
 @pytest.mark.parametrize("flags", [0, binding.FLAG_FOLD_NORM])
 def test_llama8b_shape_one_layer_round(flags):
-    """One 8B-shaped layer + LM head on a ragged batch (spans several GEMM tiles and a ragged tail); also with RMSNorm
-    folded into the projections."""
+    """One 8B-shaped layer + LM head on a ragged batch (spans several GEMM tiles and a ragged tail); also with
+    RECG_FLAG_FOLD_NORM, which names what the projections do in any case: the same round."""
     shape = synth.llama8b_shape(1)
     shape.vocab = 16384            # keeps the oracle's LM head quick; every other dimension is the 8B one
     W = synth.model_weights(shape, seed=0, dtype=torch.bfloat16)
