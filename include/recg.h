@@ -244,7 +244,8 @@ recg_status recg_kv_read(recg_ctx *ctx, const void *kv_pool, int64_t kv_pool_pag
  * y[M, N] = x[M, K] . w[N, K]^T, the projection kernel without an epilogue (for checking it alone).
  * x, w: DEVICE bf16, 16-byte aligned, K a multiple of 64 and N a multiple of 16; y: DEVICE, out_dtype, 8-byte aligned for
  * bf16 (16-byte: the tcgen05 kernel, else the mma.sync one), 4-byte for fp32 (16-byte with RECG_FLAG_SIMT_GEMM).  Pointers
- * that are not aligned like that return RECG_ERR_INVALID_ARG.
+ * that are not aligned like that return RECG_ERR_INVALID_ARG.  Like all weights, w is read ahead of the library's kernels that
+ * are still running on the stream: it must not be the result of a library call right before this one.
  */
 recg_status recg_linear(recg_ctx *ctx, const void *x, const void *w, void *y, int32_t M, int32_t N, int32_t K,
                         int32_t out_dtype);
