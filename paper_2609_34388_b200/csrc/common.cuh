@@ -110,6 +110,21 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 }
 __device__ __forceinline__ float bf16_bits_to_float(uint16_t b) { return __uint_as_float(static_cast<uint32_t>(b) << 16); }
 
+// two fp32 operations per instruction
+__device__ __forceinline__ float2 fma2(const float2& a, const float2& b, const float2& c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;"
+      : "=l"(d)
+      : "l"(reinterpret_cast<const uint64_t&>(a)), "l"(reinterpret_cast<const uint64_t&>(b)), "l"(reinterpret_cast<const uint64_t&>(c)));
+  return reinterpret_cast<float2&>(d);
+}
+__device__ __forceinline__ float2 add2(const float2& a, const float2& b) {
+  uint64_t d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(reinterpret_cast<const uint64_t&>(a)), "l"(reinterpret_cast<const uint64_t&>(b)));
+  return reinterpret_cast<float2&>(d);
+}
+
+
 // ---- KV pool addressing ------------------------------------------------------------------------
 // Pool = [layer][page][kv_head][K tile | V tile]; a tile holds 16 tokens x head_dim bf16 as 8-row atoms
 // [token group g = tok / 8][dim half h = dim / 64][8 tokens][64 elements = 128 bytes], the eight 16-byte chunks

@@ -118,20 +118,6 @@ __device__ __forceinline__ uint4 ld_stream(const void* p) {
   asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(u.x), "=r"(u.y), "=r"(u.z), "=r"(u.w) : "l"(p));
   return u;
 }
-// two fp32 operations per instruction
-__device__ __forceinline__ float2 fma2(const float2& a, const float2& b, const float2& c) {
-  uint64_t d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;"
-      : "=l"(d)
-      : "l"(reinterpret_cast<const uint64_t&>(a)), "l"(reinterpret_cast<const uint64_t&>(b)), "l"(reinterpret_cast<const uint64_t&>(c)));
-  return reinterpret_cast<float2&>(d);
-}
-__device__ __forceinline__ float2 add2(const float2& a, const float2& b) {
-  uint64_t d;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(reinterpret_cast<const uint64_t&>(a)), "l"(reinterpret_cast<const uint64_t&>(b)));
-  return reinterpret_cast<float2&>(d);
-}
-
 // One-dimensional grid of rows x chunks_per_row CTAs, chunk-fastest (consecutive CTAs read consecutive memory; the
 // row count is not bound by the 65535 limit of the other grid dimensions).  Each CTA scans [c0, c1) of one row.
 // Bound by HBM for bf16 logits only if little else is done per element (6.4 TB/s is 11 elements per SM and clock: two thirds of

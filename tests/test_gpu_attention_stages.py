@@ -1,0 +1,38 @@
+"""The attention kernel's reference maximum where its paths change: scores that outgrow it in every stage or never, and rows that
+see nothing of their first stages."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import recg_oracle as orc
+from paper_2609_34388_b200 import binding, synth
+from tests._util import f64
+from tests.test_gpu_ops import ATTN_TOL, ops_ctx
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("kind", ["rising", "falling", "steps", "large"])
+@pytest.mark.parametrize("L,v,b", [(0, 200, 0), (130, 3, 60), (1000, 16, 16), (2500, 40, 5)])
+def test_scores_against_the_standing_reference(kind, L, v, b):
+    shape = synth.ModelShape(n_layers=1, hidden=64, n_q_heads=4, n_kv_heads=1, head_dim=128, ffn=64, vocab=64)
+    n = L + v + b
+    desc = synth.fixed_descriptor([L], [v], [b], seed=L)
+    ctx = ops_ctx(shape, 1, desc.n_tokens, desc.page_table.shape[1])
+    pool = binding.alloc_kv_pool(ctx, desc.n_pages, fill=None)
+    pool.fill_(float("nan"))
+    q = synth.queries(v + b, 4, 128, seed=5)
+    k, vals = synth.kv_values(n, 1, 128, seed=7)
+    pos = torch.arange(n, dtype=torch.float32)
+    scale = {"rising": 1 + 40 * pos / n, "falling": 41 - 40 * pos / n, "steps": 1 + 12 * (pos // 100 % 4), "large": torch.full((n,), 60.0)}[kind]
+    k = (k.float() * scale[:, None, None]).to(torch.bfloat16)
+    ctx.recg_kv_write(pool, desc.n_pages, 0, desc.page_table[0], 0, k.cuda(), vals.cuda())
+    batch = binding.Batch(desc.ctx_len, desc.verify_len, desc.block_size, None, desc.page_table, pool, desc.n_pages)
+    o = torch.full((v + b, 4, 128), float("nan"), dtype=torch.bfloat16, device="cuda")
+    ctx.recg_attention(batch, 0, q.cuda(), o)
+    ctx.recg_sync()
+    ref = orc.hybrid_attention(f64(q), f64(k), f64(vals), L, v, b)
+    # (the scores reach 300; fp32 sums of 128 exact products of that size are off by less than 300 x 128 x 2^-24 = 2e-3 at worst,
+    # 2e-3 of a probability; P and the result are rounded to bf16, 2^-9 each)
+    assert np.max(np.abs(f64(o) - ref)) <= ATTN_TOL * np.max(np.abs(ref))
+    ctx.recg_free()
