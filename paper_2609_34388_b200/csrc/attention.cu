@@ -365,34 +365,41 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attention_kernel(AttnParams P
 // consecutive dims.  Bound by latency, not by its bytes (a tile entry, the (max, sum) pairs and the partial rows are
 // dependent reads): the tile entry is read ahead of the wait where the work list is settled, lane p fetches the pair of part
 // p, so that one read and a few shuffles give all weights of up to 32 parts, and the rows of the first kRows parts are on
-// their way at the same time.  Measured for one request (18 parts per row), attention and combine kernel of a layer together:
+// their way at the same time.  With few tiles (combine_split) the parts of a row are dealt out over 2^log_s warps, which merge
+// their sums through shared memory.  Measured for one request (18 parts per row), attention and combine kernel of a layer together:
 // 19.5 us with four parts fetched at a time, each with its own pair, 16.1 us like this.
-template <int D>
+template <int D, bool SPLIT>
 __global__ void __launch_bounds__(512, 2) attention_combine_kernel(const AttnTile* __restrict__ tiles,
                                                                 const int* __restrict__ counts, int n_q, int group,
                                                                 const float* __restrict__ part_o,
                                                                 const float* __restrict__ part_ml,
-                                                                __nv_bfloat16* __restrict__ o, int list_settled) {
+                                                                __nv_bfloat16* __restrict__ o, int list_settled, int log_split) {
   constexpr int E = D / 32;
   constexpr int kRows = 6;     // partial rows in flight
+  // (without a split no shared memory: the next projection's CTA has room beside this one's)
+  __shared__ float s_acc[SPLIT ? 16 : 1][D + 2];
   griddep_launch();
   if (!list_settled) griddep_wait();
   const int n_tiles = counts[1];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int log_s = SPLIT ? log_split : 0, S = 1 << log_s;
+  const int n_units = n_tiles << (3 + log_s), my = warp & (S - 1);
   AttnTile tl = {};
-  if ((int)blockIdx.x < n_tiles * 8) tl = tiles[blockIdx.x >> 3];
+  if ((int)blockIdx.x < n_units) tl = tiles[blockIdx.x >> (3 + log_s)];
   if (list_settled) griddep_wait();
-  for (int wu = blockIdx.x; wu < n_tiles * 8; wu += gridDim.x) {
-    if (wu != (int)blockIdx.x) tl = tiles[wu >> 3];
-    const int rho = (wu & 7) * 16 + warp;
-    if (rho >= tl.ntok * group) continue;
-    const float* rows = part_o + ((size_t)tl.part_begin * 128 + rho) * D + lane * E;
+  for (int wu = blockIdx.x; wu < n_units; wu += gridDim.x) {
+    if (wu != (int)blockIdx.x) tl = tiles[wu >> (3 + log_s)];
+    const int rho = (((wu & ((8 << log_s) - 1)) << 4) + warp) >> log_s;
+    const bool live = rho < tl.ntok * group;
+    const int n_mine = live ? (tl.n_parts - my + S - 1) >> log_s : 0;       // parts my, my + S, ...
+    const size_t first = tl.part_begin + my;
+    const float* rows = part_o + (first * 128 + rho) * D + lane * E;
     auto fetch = [&](int p, float (&v)[E]) {
       if constexpr (E == 4) {
-        const float4 t = __ldcg(reinterpret_cast<const float4*>(rows + (size_t)p * 128 * D));
+        const float4 t = __ldcg(reinterpret_cast<const float4*>(rows + (size_t)(p << log_s) * 128 * D));
         v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
       } else {
-        const float2 t = __ldcg(reinterpret_cast<const float2*>(rows + (size_t)p * 128 * D));
+        const float2 t = __ldcg(reinterpret_cast<const float2*>(rows + (size_t)(p << log_s) * 128 * D));
         v[0] = t.x; v[1] = t.y;
       }
     };
@@ -400,10 +407,10 @@ __global__ void __launch_bounds__(512, 2) attention_combine_kernel(const AttnTil
 #pragma unroll
     for (int e = 0; e < E; ++e) acc[e] = 0.f;
     float m = -1e30f, l = 0.f;
-    for (int p0 = 0; p0 < tl.n_parts; p0 += 32) {
-      const int np = min(32, tl.n_parts - p0);
+    for (int p0 = 0; p0 < n_mine; p0 += 32) {
+      const int np = min(32, n_mine - p0);
       float2 ml = make_float2(-1e30f, 0.f);
-      if (lane < np) ml = __ldcg(reinterpret_cast<const float2*>(part_ml) + (size_t)(tl.part_begin + p0 + lane) * 128 + rho);
+      if (lane < np) ml = __ldcg(reinterpret_cast<const float2*>(part_ml) + (first + ((p0 + lane) << log_s)) * 128 + rho);
       float v[kRows][E];
 #pragma unroll
       for (int k = 0; k < kRows; ++k)
@@ -431,24 +438,56 @@ __global__ void __launch_bounds__(512, 2) attention_combine_kernel(const AttnTil
         }
       }
     }
-    const float inv = l > 0.f ? 1.f / l : 0.f;
-    const int j = rho / group, hg = rho % group;
-    __nv_bfloat16* dst = o + ((size_t)(tl.tok0 + j) * n_q + tl.kv_head * group + hg) * D + lane * E;
-    if constexpr (E == 4) {
-      uint2 pk;
-      pk.x = pack_bf16(acc[0] * inv, acc[1] * inv);
-      pk.y = pack_bf16(acc[2] * inv, acc[3] * inv);
-      *reinterpret_cast<uint2*>(dst) = pk;
-    } else {
-      *reinterpret_cast<uint32_t*>(dst) = pack_bf16(acc[0] * inv, acc[1] * inv);
+    if constexpr (SPLIT) {
+      if (my) {
+#pragma unroll
+        for (int e = 0; e < E; ++e) s_acc[warp][lane * E + e] = acc[e];
+        if (lane == 0) {
+          s_acc[warp][D] = m;
+          s_acc[warp][D + 1] = l;
+        }
+      }
+      __syncthreads();
+      for (int k = 1; my == 0 && k < S; ++k) {
+        const float* other = s_acc[warp + k];
+        const float m_k = other[D], m_new = fmaxf(m, m_k), f = exp2f(m - m_new), g = exp2f(m_k - m_new);
+        m = m_new;
+        l = l * f + other[D + 1] * g;
+#pragma unroll
+        for (int e = 0; e < E; ++e) acc[e] = acc[e] * f + other[lane * E + e] * g;
+      }
+      __syncthreads();
+    }
+    if (live && my == 0) {
+      const float inv = l > 0.f ? 1.f / l : 0.f;
+      const int j = rho / group, hg = rho % group;
+      __nv_bfloat16* dst = o + ((size_t)(tl.tok0 + j) * n_q + tl.kv_head * group + hg) * D + lane * E;
+      if constexpr (E == 4) {
+        uint2 pk;
+        pk.x = pack_bf16(acc[0] * inv, acc[1] * inv);
+        pk.y = pack_bf16(acc[2] * inv, acc[3] * inv);
+        *reinterpret_cast<uint2*>(dst) = pk;
+      } else {
+        *reinterpret_cast<uint32_t*>(dst) = pack_bf16(acc[0] * inv, acc[1] * inv);
+      }
     }
   }
 }
 
+// Few row tiles (at most `tiles`, 0: not known, or not wanted) are merged by few warps, each with many parts: a chain of dependent
+// reads while most SMs are idle.  Two or four warps share a row where the CTAs for it are resident at once, two per SM.  One
+// request over 4096 tokens (8 tiles of 18 parts), 32 layers: 479 us with one warp per row, 446 with four.  Inside a step the
+// idle SMs are worth more to the next projection, whose CTAs come in early and request weights: a round of that request 3548 us
+// with one warp per row, 3600 with four.
+int combine_split(int tiles, int n_sm) {
+  return tiles <= 0 ? 0 : (tiles * 32 <= 2 * n_sm ? 2 : (tiles * 16 <= 2 * n_sm ? 1 : 0));
+}
+unsigned combine_ctas(int tiles, int log_s, int n_sm) { return log_s ? (unsigned)tiles << (3 + log_s) : 4u * n_sm; }
+
 template <int D>
 void launch_attention_t(const BatchLayout& bl, const Dims& dm, int layer, const void* q, void* o, const void* kv_pool,
                         int64_t n_pages, float* part_o, float* part_ml, int tok_per_tile, int n_sm, int* status,
-                        cudaStream_t st, bool whole) {
+                        cudaStream_t st, bool whole, int tiles) {
   static bool configured[kMaxDevices] = {false};
   if (first_use_on_device(configured))
     cudaFuncSetAttribute(attention_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnSmem<D>::kTotal);
@@ -475,8 +514,9 @@ void launch_attention_t(const BatchLayout& bl, const Dims& dm, int layer, const 
   P.status = status;
   launch_pdl(attention_kernel<D>, dim3(n_sm), dim3(kAttnThreads), AttnSmem<D>::kTotal, st, P);
   if (whole) return;
-  launch_pdl(attention_combine_kernel<D>, dim3(4 * n_sm), dim3(512), 0, st, (const AttnTile*)bl.tiles, (const int*)bl.counts,
-             dm.n_q, P.group, (const float*)part_o, (const float*)part_ml, static_cast<__nv_bfloat16*>(o), 0);
+  const int log_s = combine_split(tiles, n_sm);
+  launch_pdl(log_s ? attention_combine_kernel<D, true> : attention_combine_kernel<D, false>, dim3(combine_ctas(tiles, log_s, n_sm)), dim3(512), 0, st, (const AttnTile*)bl.tiles, (const int*)bl.counts,
+             dm.n_q, P.group, (const float*)part_o, (const float*)part_ml, static_cast<__nv_bfloat16*>(o), 0, log_s);
 }
 
 }  // namespace
@@ -487,19 +527,20 @@ size_t attention_smem_bytes(int head_dim) {
 
 void launch_attention(const BatchLayout& bl, const Dims& dm, int layer, const void* q, void* o, const void* kv_pool,
                       int64_t n_pages, float* part_o, float* part_ml, int tok_per_tile, int n_sm, int* status,
-                      cudaStream_t st, bool use_tc, bool layout_settled, bool whole) {
+                      cudaStream_t st, bool use_tc, bool layout_settled, bool whole, int tiles) {
   if (use_tc && dm.head_dim == 128) {
     launch_attention_tc_main(bl, dm, layer, q, o, kv_pool, n_pages, part_o, part_ml, n_sm, status, st, layout_settled);
     if (whole) return;
-    launch_pdl(attention_combine_kernel<128>, dim3(4 * n_sm), dim3(512), 0, st, (const AttnTile*)bl.tiles,
+    const int log_s = combine_split(tiles, n_sm);
+    launch_pdl(log_s ? attention_combine_kernel<128, true> : attention_combine_kernel<128, false>, dim3(combine_ctas(tiles, log_s, n_sm)), dim3(512), 0, st, (const AttnTile*)bl.tiles,
                (const int*)bl.counts, dm.n_q, dm.n_q / dm.n_kv, (const float*)part_o, (const float*)part_ml,
-               static_cast<__nv_bfloat16*>(o), 1);    // (the kernel in front signals its dependents when the list is settled)
+               static_cast<__nv_bfloat16*>(o), 1, log_s);    // (the kernel in front signals its dependents when the list is settled)
     return;
   }
   if (dm.head_dim == 64)
-    launch_attention_t<64>(bl, dm, layer, q, o, kv_pool, n_pages, part_o, part_ml, tok_per_tile, n_sm, status, st, whole);
+    launch_attention_t<64>(bl, dm, layer, q, o, kv_pool, n_pages, part_o, part_ml, tok_per_tile, n_sm, status, st, whole, tiles);
   else
-    launch_attention_t<128>(bl, dm, layer, q, o, kv_pool, n_pages, part_o, part_ml, tok_per_tile, n_sm, status, st, whole);
+    launch_attention_t<128>(bl, dm, layer, q, o, kv_pool, n_pages, part_o, part_ml, tok_per_tile, n_sm, status, st, whole, tiles);
 }
 
 }  // namespace recg

@@ -56,6 +56,7 @@ struct recg_ctx {
   bool layout_valid = false;
   bool layout_has_pages = false;
   bool layout_whole = false;     // no attention tile was cut: no combine kernel
+  int layout_tiles = 0;          // its row tiles, all kv heads (0: the lengths are on the device)
   // An attention kernel has been enqueued behind the last layout kernel.  The first one waits for its predecessors before it
   // reads the work list, and no thread of it signals its dependents before that wait: whatever runs behind it finds the list
   // settled and may read it ahead of its own wait.
@@ -353,7 +354,13 @@ recg_status upload_and_layout(recg_ctx* ctx, const recg_batch* b, bool need_page
   if (b->page_table) {       // (a verify-only batch without pages has neither slots nor attention work)
     const int64_t n_pages = b->kv_pool ? b->kv_pool_pages : (int64_t)1 << 40;
     ctx->h_rows.resize(b->n_req);
-    for (int r = 0; r < b->n_req; ++r) ctx->h_rows[r] = request_rows(b, r);
+    long long tiles = 0;
+    for (int r = 0; r < b->n_req; ++r) {
+      ctx->h_rows[r] = request_rows(b, r);
+      tiles += (ctx->h_rows[r] + ctx->tok_per_tile - 1) / ctx->tok_per_tile;
+    }
+    tiles *= ctx->dm.n_kv;
+    ctx->layout_tiles = tiles < (1 << 20) ? (int)tiles : 1 << 20;
     ctx->layout_whole = attention_whole_tiles(b->n_req, b->ctx_len, ctx->h_rows.data(), ctx->dm.n_kv, ctx->tok_per_tile, ctx->target_items);
     launch_layout(ctx->bl, ctx->dm, ctx->tok_per_tile, ctx->target_items, ctx->layout_whole, n_pages, ctx->d_status,
                   !forward, ctx->d_desc, small ? &ctx->small_desc : nullptr, ctx->stream);
@@ -614,7 +621,7 @@ static recg_status run_forward(recg_ctx* ctx, void* kv_pool, int64_t kv_pool_pag
     // (the first layer's attention kernel may be resident while the work list is still being built: idle lanes of a projection
     // signal its dependents before the projection has waited)
     launch_attention(bl, d, l, ctx->q, ctx->o, kv_pool, kv_pool_pages, ctx->part_o, ctx->part_ml, ctx->tok_per_tile, ctx->n_sm,
-                     ctx->d_status, st, !(ctx->cfg.flags & RECG_FLAG_SIMT_ATTENTION), ctx->list_settled, ctx->layout_whole);
+                     ctx->d_status, st, !(ctx->cfg.flags & RECG_FLAG_SIMT_ATTENTION), ctx->list_settled, ctx->layout_whole, 0);
     CU(cudaGetLastError());
     ctx->list_settled = true;
     ctx->mark(3, ctx->layout_whole ? 1 : 2);
@@ -752,6 +759,7 @@ recg_status recg_step_device(recg_ctx* ctx, const recg_device_batch* b, recg_log
   bl.risk_delta = 0.5f;
   launch_pack_device(device_round(ctx, b), ctx->d_desc, ctx->d_dyn, ctx->d_status, ctx->stream);
   ctx->layout_whole = false;           // (the lengths are on the device)
+  ctx->layout_tiles = 0;
   launch_layout(bl, ctx->dm, ctx->tok_per_tile, ctx->target_items, false, b->kv_pool_pages, ctx->d_status, false, ctx->d_desc, nullptr, ctx->stream);
   ctx->list_settled = false;
   ctx->small_desc.n = 0;
@@ -915,7 +923,7 @@ recg_status recg_attention(recg_ctx* ctx, const recg_batch* batch, int32_t layer
   }
   launch_attention(ctx->bl, ctx->dm, layer, q, o, ctx->last_pool, ctx->last_pool_pages, ctx->part_o, ctx->part_ml,
                    ctx->tok_per_tile, ctx->n_sm, ctx->d_status, ctx->stream, !(ctx->cfg.flags & RECG_FLAG_SIMT_ATTENTION),
-                   ctx->list_settled, ctx->layout_whole);
+                   ctx->list_settled, ctx->layout_whole, ctx->layout_tiles);
   CU(cudaGetLastError());
   ctx->list_settled = true;
   return RECG_OK;

@@ -1,5 +1,6 @@
-"""The attention kernel's reference maximum where its paths change: scores that outgrow it in every stage or never, and rows that
-see nothing of their first stages."""
+"""The attention kernel's reference maximum and its combine kernel where their paths change: scores that outgrow the reference in
+every stage or never, rows that see nothing of their first stages, and few row tiles (their parts are merged by one, two or four
+warps a row)."""
 import numpy as np
 import pytest
 import torch
@@ -7,7 +8,7 @@ import torch
 from oracle import recg_oracle as orc
 from paper_2609_34388_b200 import binding, synth
 from tests._util import f64
-from tests.test_gpu_ops import ATTN_TOL, ops_ctx
+from tests.test_gpu_ops import ATTN_TOL, ops_ctx, run_attention_case
 
 pytestmark = pytest.mark.gpu
 
@@ -36,3 +37,16 @@ def test_scores_against_the_standing_reference(kind, L, v, b):
     # 2e-3 of a probability; P and the result are rounded to bf16, 2^-9 each)
     assert np.max(np.abs(f64(o) - ref)) <= ATTN_TOL * np.max(np.abs(ref))
     ctx.recg_free()
+
+
+@pytest.mark.parametrize("n_kv,reqs", [
+    (8, [(4096, 16, 16)]),                       # 8 tiles: four warps a row
+    (8, [(900, 20, 12), (3000, 1, 0)]),          # 16 tiles: two
+    (1, [(9000, 30, 2)]),                        # one tile in a part per CTA
+    (3, [(1200, 33, 0), (2, 1, 0), (700, 2, 9)]),   # 12 tiles, a pair among them
+    (8, [(500, 4, 4), (1500, 8, 8), (2500, 2, 30)]),    # 24 tiles: one warp
+])
+def test_parts_of_few_tiles(n_kv, reqs):
+    for d in (64, 128):
+        shape = synth.ModelShape(n_layers=1, hidden=64, n_q_heads=4 * n_kv, n_kv_heads=n_kv, head_dim=d, ffn=64, vocab=64)
+        assert run_attention_case(shape, reqs, seed=len(reqs) + n_kv) < ATTN_TOL
