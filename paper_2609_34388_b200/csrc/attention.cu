@@ -368,14 +368,16 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attention_kernel(AttnParams P
 // their way at the same time.  With few tiles (combine_split) the parts of a row are dealt out over 2^log_s warps, which merge
 // their sums through shared memory.  Measured for one request (18 parts per row), attention and combine kernel of a layer together:
 // 19.5 us with four parts fetched at a time, each with its own pair, 16.1 us like this.
-template <int D, bool SPLIT>
-__global__ void __launch_bounds__(512, 2) attention_combine_kernel(const AttnTile* __restrict__ tiles,
+enum CombineMode { kManyTiles, kSplitRows, kDeepRows };
+template <int D, CombineMode MODE>
+__global__ void __launch_bounds__(512, MODE == kDeepRows ? 1 : 2) attention_combine_kernel(const AttnTile* __restrict__ tiles,
                                                                 const int* __restrict__ counts, int n_q, int group,
                                                                 const float* __restrict__ part_o,
                                                                 const float* __restrict__ part_ml,
                                                                 __nv_bfloat16* __restrict__ o, int list_settled, int log_split) {
   constexpr int E = D / 32;
-  constexpr int kRows = 6;     // partial rows in flight
+  constexpr bool SPLIT = MODE == kSplitRows;
+  constexpr int kRows = MODE == kDeepRows ? 18 : 6;     // partial rows in flight
   // (without a split no shared memory: the next projection's CTA has room beside this one's)
   __shared__ float s_acc[SPLIT ? 16 : 1][D + 2];
   griddep_launch();
@@ -474,20 +476,29 @@ __global__ void __launch_bounds__(512, 2) attention_combine_kernel(const AttnTil
   }
 }
 
-// Few row tiles (at most `tiles`, 0: not known, or not wanted) are merged by few warps, each with many parts: a chain of dependent
-// reads while most SMs are idle.  Two or four warps share a row where the CTAs for it are resident at once, two per SM.  One
-// request over 4096 tokens (8 tiles of 18 parts), 32 layers: 479 us with one warp per row, 446 with four.  Inside a step the
-// idle SMs are worth more to the next projection, whose CTAs come in early and request weights: a round of that request 3548 us
-// with one warp per row, 3600 with four.
-int combine_split(int tiles, int n_sm) {
-  return tiles <= 0 ? 0 : (tiles * 32 <= 2 * n_sm ? 2 : (tiles * 16 <= 2 * n_sm ? 1 : 0));
+// Few row tiles (at most `tiles`, 0: not known) are merged by few warps, each with many parts: a chain of dependent reads while most
+// SMs are idle.  The line lies where two or four warps per row are resident at once, two CTAs per SM; such a tile has eight parts
+// or more.
+// By itself (recg_attention) two or four warps share a row: one request over 4096 tokens (8 tiles of 18 parts), 32 layers, 479 us
+// with one warp per row, 446 with four.  Inside a step the idle SMs are worth more to the next projection, whose CTAs come in early
+// and request weights (a round of that request 3548 us with one warp per row, 3600 with four): there a row keeps its warp, in a
+// CTA with an SM's registers to itself, and up to 18 of its parts are on their way at once (3538 -> 3506 us; as many CTAs as there
+// is work, but six parts at once: 3553).
+int combine_split(int tiles, int n_sm, bool step) {
+  return tiles <= 0 || step ? 0 : (tiles * 32 <= 2 * n_sm ? 2 : (tiles * 16 <= 2 * n_sm ? 1 : 0));
 }
-unsigned combine_ctas(int tiles, int log_s, int n_sm) { return log_s ? (unsigned)tiles << (3 + log_s) : 4u * n_sm; }
+bool few_tiles(int tiles, int n_sm) { return tiles > 0 && tiles * 16 <= 2 * n_sm; }
+unsigned combine_ctas(int tiles, int log_s, int n_sm) { return few_tiles(tiles, n_sm) ? (unsigned)tiles << (3 + log_s) : 4u * n_sm; }
+template <int D>
+auto combine_kernel(int tiles, int log_s, int n_sm) {
+  return log_s ? attention_combine_kernel<D, kSplitRows>
+               : (few_tiles(tiles, n_sm) ? attention_combine_kernel<D, kDeepRows> : attention_combine_kernel<D, kManyTiles>);
+}
 
 template <int D>
 void launch_attention_t(const BatchLayout& bl, const Dims& dm, int layer, const void* q, void* o, const void* kv_pool,
                         int64_t n_pages, float* part_o, float* part_ml, int tok_per_tile, int n_sm, int* status,
-                        cudaStream_t st, bool whole, int tiles) {
+                        cudaStream_t st, bool whole, int tiles, bool step) {
   static bool configured[kMaxDevices] = {false};
   if (first_use_on_device(configured))
     cudaFuncSetAttribute(attention_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnSmem<D>::kTotal);
@@ -514,8 +525,8 @@ void launch_attention_t(const BatchLayout& bl, const Dims& dm, int layer, const 
   P.status = status;
   launch_pdl(attention_kernel<D>, dim3(n_sm), dim3(kAttnThreads), AttnSmem<D>::kTotal, st, P);
   if (whole) return;
-  const int log_s = combine_split(tiles, n_sm);
-  launch_pdl(log_s ? attention_combine_kernel<D, true> : attention_combine_kernel<D, false>, dim3(combine_ctas(tiles, log_s, n_sm)), dim3(512), 0, st, (const AttnTile*)bl.tiles, (const int*)bl.counts,
+  const int log_s = combine_split(tiles, n_sm, step);
+  launch_pdl(combine_kernel<D>(tiles, log_s, n_sm), dim3(combine_ctas(tiles, log_s, n_sm)), dim3(512), 0, st, (const AttnTile*)bl.tiles, (const int*)bl.counts,
              dm.n_q, P.group, (const float*)part_o, (const float*)part_ml, static_cast<__nv_bfloat16*>(o), 0, log_s);
 }
 
@@ -527,20 +538,20 @@ size_t attention_smem_bytes(int head_dim) {
 
 void launch_attention(const BatchLayout& bl, const Dims& dm, int layer, const void* q, void* o, const void* kv_pool,
                       int64_t n_pages, float* part_o, float* part_ml, int tok_per_tile, int n_sm, int* status,
-                      cudaStream_t st, bool use_tc, bool layout_settled, bool whole, int tiles) {
+                      cudaStream_t st, bool use_tc, bool layout_settled, bool whole, int tiles, bool step) {
   if (use_tc && dm.head_dim == 128) {
     launch_attention_tc_main(bl, dm, layer, q, o, kv_pool, n_pages, part_o, part_ml, n_sm, status, st, layout_settled);
     if (whole) return;
-    const int log_s = combine_split(tiles, n_sm);
-    launch_pdl(log_s ? attention_combine_kernel<128, true> : attention_combine_kernel<128, false>, dim3(combine_ctas(tiles, log_s, n_sm)), dim3(512), 0, st, (const AttnTile*)bl.tiles,
+    const int log_s = combine_split(tiles, n_sm, step);
+    launch_pdl(combine_kernel<128>(tiles, log_s, n_sm), dim3(combine_ctas(tiles, log_s, n_sm)), dim3(512), 0, st, (const AttnTile*)bl.tiles,
                (const int*)bl.counts, dm.n_q, dm.n_q / dm.n_kv, (const float*)part_o, (const float*)part_ml,
                static_cast<__nv_bfloat16*>(o), 1, log_s);    // (the kernel in front signals its dependents when the list is settled)
     return;
   }
   if (dm.head_dim == 64)
-    launch_attention_t<64>(bl, dm, layer, q, o, kv_pool, n_pages, part_o, part_ml, tok_per_tile, n_sm, status, st, whole, tiles);
+    launch_attention_t<64>(bl, dm, layer, q, o, kv_pool, n_pages, part_o, part_ml, tok_per_tile, n_sm, status, st, whole, tiles, step);
   else
-    launch_attention_t<128>(bl, dm, layer, q, o, kv_pool, n_pages, part_o, part_ml, tok_per_tile, n_sm, status, st, whole, tiles);
+    launch_attention_t<128>(bl, dm, layer, q, o, kv_pool, n_pages, part_o, part_ml, tok_per_tile, n_sm, status, st, whole, tiles, step);
 }
 
 }  // namespace recg

@@ -215,10 +215,10 @@ bool launch_gemm_chain(void* s, const ChainOp* ops, int n_ops, int M, const Chai
 // layout_settled: an attention kernel has been enqueued behind the kernel that wrote the work list (and has waited for it):
 // the tcgen05 kernel then reads its work range before it waits for its predecessor
 // whole: the work list was laid out with whole tiles
-// tiles: the row tiles of all kv heads, cut or not (0: known on the device only, or a projection follows; see combine_split)
+// tiles: the row tiles of all kv heads, cut or not (0: known on the device only); step: a projection follows
 void launch_attention(const BatchLayout& bl, const Dims& dm, int layer, const void* q, void* o, const void* kv_pool,
                       int64_t n_pages, float* part_o, float* part_ml, int tok_per_tile, int n_sm, int* status,
-                      cudaStream_t st, bool use_tc, bool layout_settled, bool whole, int tiles);
+                      cudaStream_t st, bool use_tc, bool layout_settled, bool whole, int tiles, bool step);
 void launch_attention_tc_main(const BatchLayout& bl, const Dims& dm, int layer, const void* q, void* o,
                               const void* kv_pool, int64_t n_pages, float* part_o, float* part_ml, int n_sm, int* status,
                               cudaStream_t st, bool layout_settled);

@@ -621,7 +621,7 @@ static recg_status run_forward(recg_ctx* ctx, void* kv_pool, int64_t kv_pool_pag
     // (the first layer's attention kernel may be resident while the work list is still being built: idle lanes of a projection
     // signal its dependents before the projection has waited)
     launch_attention(bl, d, l, ctx->q, ctx->o, kv_pool, kv_pool_pages, ctx->part_o, ctx->part_ml, ctx->tok_per_tile, ctx->n_sm,
-                     ctx->d_status, st, !(ctx->cfg.flags & RECG_FLAG_SIMT_ATTENTION), ctx->list_settled, ctx->layout_whole, 0);
+                     ctx->d_status, st, !(ctx->cfg.flags & RECG_FLAG_SIMT_ATTENTION), ctx->list_settled, ctx->layout_whole, ctx->layout_tiles, true);
     CU(cudaGetLastError());
     ctx->list_settled = true;
     ctx->mark(3, ctx->layout_whole ? 1 : 2);
@@ -923,7 +923,7 @@ recg_status recg_attention(recg_ctx* ctx, const recg_batch* batch, int32_t layer
   }
   launch_attention(ctx->bl, ctx->dm, layer, q, o, ctx->last_pool, ctx->last_pool_pages, ctx->part_o, ctx->part_ml,
                    ctx->tok_per_tile, ctx->n_sm, ctx->d_status, ctx->stream, !(ctx->cfg.flags & RECG_FLAG_SIMT_ATTENTION),
-                   ctx->list_settled, ctx->layout_whole, ctx->layout_tiles);
+                   ctx->list_settled, ctx->layout_whole, ctx->layout_tiles, false);
   CU(cudaGetLastError());
   ctx->list_settled = true;
   return RECG_OK;

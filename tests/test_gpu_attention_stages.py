@@ -7,8 +7,9 @@ import torch
 
 from oracle import recg_oracle as orc
 from paper_2609_34388_b200 import binding, synth
-from tests._util import f64
+from tests._util import f64, oracle_cfg, oracle_weights
 from tests.test_gpu_ops import ATTN_TOL, ops_ctx, run_attention_case
+from tests.test_gpu_step import HID_TOL, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -50,3 +51,33 @@ def test_parts_of_few_tiles(n_kv, reqs):
     for d in (64, 128):
         shape = synth.ModelShape(n_layers=1, hidden=64, n_q_heads=4 * n_kv, n_kv_heads=n_kv, head_dim=d, ffn=64, vocab=64)
         assert run_attention_case(shape, reqs, seed=len(reqs) + n_kv) < ATTN_TOL
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("n_kv,reqs", [(1, [(9000, 6, 2)]), (2, [(3000, 30, 10)]), (2, [(700, 1, 3), (2600, 4, 0)]), (9, [(500, 3, 1), (1300, 2, 2)]),
+                                       (9, [(500, 3, 1), (1300, 2, 2), (90, 1, 0)])])
+def test_step_with_few_tiles(n_kv, reqs, d):
+    """Inside a step a warp keeps a row: 1 to 18 tiles with up to 148 parts (18 at a time), and 27."""
+    shape = synth.ModelShape(n_layers=1, hidden=128, n_q_heads=2 * n_kv, n_kv_heads=n_kv, head_dim=d, ffn=128, vocab=256)
+    W = synth.model_weights(shape, seed=0, dtype=torch.bfloat16)
+    L, v, b = ([r[i] for r in reqs] for i in range(3))
+    desc = synth.fixed_descriptor(L, v, b, seed=3)
+    ctx = binding.Context(binding.make_config(shape, len(reqs), desc.n_tokens, desc.page_table.shape[1]), to_dev(W))
+    pool = binding.alloc_kv_pool(ctx, desc.n_pages, fill=None)
+    pool.fill_(float("nan"))
+    kvs, ys = [], []
+    for r in range(len(reqs)):
+        ys.append(synth.token_ids(v[r], shape.vocab, seed=r + 1).tolist())
+        kvs.append(synth.kv_values(L[r], n_kv, d, seed=r))
+        ctx.recg_kv_write(pool, desc.n_pages, 0, desc.page_table[r], 0, kvs[r][0].cuda(), kvs[r][1].cuda())
+    batch = binding.Batch(desc.ctx_len, desc.verify_len, desc.block_size, [t for y in ys for t in y], desc.page_table, pool, desc.n_pages)
+    logits = f64(ctx.logits_tensor(ctx.recg_step(batch)))
+    ctx.recg_sync()
+    t0 = 0
+    for r in range(len(reqs)):
+        K, V = kvs[r]
+        ref, _, _ = orc.fused_round_cached(oracle_cfg(shape), oracle_weights(W), [(K.double().numpy(), V.double().numpy())], L[r], ys[r], b[r])
+        got = logits[t0:t0 + v[r] + b[r]]
+        assert np.max(np.abs(got - ref)) <= HID_TOL * np.max(np.abs(ref)), r
+        t0 += v[r] + b[r]
+    ctx.recg_free()
