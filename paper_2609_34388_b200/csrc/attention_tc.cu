@@ -64,6 +64,7 @@ constexpr uint32_t kSpin = 1u << 22;
 constexpr int kTmemCols = 512;                 // two S buffers of 128 columns (stage & 1); group g owns columns [64 g, 64 g + 64) of each
                                                // and overwrites the first 32 of them with its bf16 P; O of group g at 256 + 128 g
 constexpr int kTmemO = 2 * kBT;
+constexpr float kNoRef = -1e30f;               // reference maximum of a row that has seen no token yet
 
 constexpr int kOffQ = 0;                       // two Q buffers: item i uses buffer i & 1
 constexpr int kOffKV = kOffQ + 2 * kQBytes;
@@ -493,7 +494,9 @@ __global__ void __launch_bounds__(kThreads, 1) attention_tc_kernel(const __grid_
       const bool rvalid = row < R;
       const bool warp_valid = dry || quad * 32 < R;
       const int climit = nx_cl, vlo = nx_lo, vhi = nx_hi;
-      float m_ref = -1e30f, l_run = 0.f;
+      // the row's reference maximum (in powers of two), the sum of its probabilities, the score above which the reference moves
+      float m_ref = rvalid ? kNoRef : 0.f, l_run = 0.f, outgrown = INFINITY;
+      const float inv_scale = 1.f / P.scale_log2;
       bool first = true;
 
       for (int n = 0; n < nblk; ++n, ++cs) {
@@ -526,7 +529,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_tc_kernel(const __grid_
           }
           // (a row's first stage, or the first one in which it sees any of this group's tokens; what it has summed up until
           // then is nothing)
-          if (__any_sync(0xffffffffu, rvalid && m_ref < -1e29f)) {     // four independent chains instead of one long dependent one
+          if (__any_sync(0xffffffffu, m_ref == kNoRef)) {     // four independent chains instead of one long dependent one
             float mxa[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
             for (int c = 0; c < 2; ++c)
@@ -535,37 +538,42 @@ __global__ void __launch_bounds__(kThreads, 1) attention_tc_kernel(const __grid_
                 mxa[2 * c] = fmaxf(mxa[2 * c], fmaxf(__uint_as_float(sr[c][i]), __uint_as_float(sr[c][i + 1])));
                 mxa[2 * c + 1] = fmaxf(mxa[2 * c + 1], fmaxf(__uint_as_float(sr[c][i + 2]), __uint_as_float(sr[c][i + 3])));
               }
-            const float m_blk = fmaxf(fmaxf(mxa[0], mxa[1]), fmaxf(mxa[2], mxa[3])) * P.scale_log2;
-            if (rvalid && m_ref < -1e29f && m_blk > m_ref) m_ref = m_blk;
+            const float m_blk = __fmul_rn(fmaxf(fmaxf(mxa[0], mxa[1]), fmaxf(mxa[2], mxa[3])), P.scale_log2);
+            if (m_ref == kNoRef && m_blk > m_ref) {
+              m_ref = m_blk;
+              outgrown = (m_blk + 8.f) * inv_scale;
+            }
           }
           // The probabilities are taken relative to the reference maximum as it stands, and only then compared with it: the
           // reference moves when the row maximum outgrows it by more than 2^8 (probabilities stay well inside bf16 and fp32
-          // range), which is rare, and the stage is then done again.  (Once: where scores are so large that the reference cannot
-          // be met exactly the result has no meaning anyway.)  The search for the maximum thus runs beside the exponentials
-          // instead of in front of them: rounds of 16 requests 8352 -> 8255 us, 2000 prompt tokens 29.6 -> 29.2 ms.  A quarter
-          // or half of the exponentials as polynomials on the FMA units gave nothing on top (8270, 8262 us): the chain of
-          // products, not the 2^x unit, bounds a stage.
+          // range), which is rare, and the stage is then done again.  The search for the maximum thus runs beside the
+          // exponentials instead of in front of them: rounds of 16 requests 8352 -> 8255 us, 2000 prompt tokens 29.6 -> 29.2 ms.
+          // A quarter or half of the exponentials as polynomials on the FMA units gave nothing on top (8270, 8262 us): the chain
+          // of products, not the 2^x unit, bounds a stage.
 #pragma unroll 1
           for (int pass = 0; pass < 2; ++pass) {
             const float2 scale2 = make_float2(P.scale_log2, P.scale_log2), neg_ref2 = make_float2(-m_ref, -m_ref);
             float2 lsa[4] = {};
-            float ymx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+            float mxa[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
               uint32_t pk[16];     // 32 tokens -> 16 packed columns over the start of this S buffer
 #pragma unroll
               for (int i = 0; i < 32; i += 2) {
                 const int k = (i >> 1) & 3;
-                const float2 y = fma2(make_float2(__uint_as_float(sr[c][i]), __uint_as_float(sr[c][i + 1])), scale2, neg_ref2);
-                ymx[k] = fmaxf(ymx[k], fmaxf(y.x, y.y));
+                const float2 t = make_float2(__uint_as_float(sr[c][i]), __uint_as_float(sr[c][i + 1])), y = fma2(t, scale2, neg_ref2);
+                mxa[k] = fmaxf(mxa[k], fmaxf(t.x, t.y));
                 const float2 p = make_float2(exp2f(y.x), exp2f(y.y));   // exp2(-inf) = 0 for masked
                 lsa[k] = add2(lsa[k], p);
                 pk[i >> 1] = pack_bf16(p.x, p.y);
               }
               tmem_st16(s_buf + c * 16, pk);
             }
-            const float m_over = fmaxf(fmaxf(ymx[0], ymx[1]), fmaxf(ymx[2], ymx[3]));     // row maximum over the reference
-            const bool grow = n > 0 && rvalid && m_over > 8.f;
+            // (A reference is always a scaled maximum of scores itself: their excess over the old one is rounded as coarsely as that
+            // is, and a masked first stage may have left -1e11.  Compared are the scores: scaling the maximum of every stage first
+            // took 451 us instead of 445 for the attention of one request over 4096 tokens, 32 layers.)
+            const float s_max = fmaxf(fmaxf(mxa[0], mxa[1]), fmaxf(mxa[2], mxa[3]));
+            const bool grow = n > 0 && s_max > outgrown;
             if (pass == 1 || !__any_sync(0xffffffffu, grow)) {
               const float2 ls = add2(add2(lsa[0], lsa[1]), add2(lsa[2], lsa[3]));
               l_run += ls.x + ls.y;
@@ -574,8 +582,10 @@ __global__ void __launch_bounds__(kThreads, 1) attention_tc_kernel(const __grid_
             // O is rescaled in TMEM, once the group's P V of the previous stage has completed
             bwait(pv_done, (cs - 1) & 1, DEV_TIMEOUT_MMA);
             tc_fence_after();
-            const float f = grow ? exp2f(-m_over) : 1.f;
-            if (grow) m_ref += m_over;
+            const float m_new = grow ? fmaxf(m_ref, __fmul_rn(s_max, P.scale_log2)) : m_ref;
+            if (grow) outgrown = (m_new + 8.f) * inv_scale;
+            const float f = exp2f(m_ref - m_new);
+            m_ref = m_new;
             l_run *= f;
 #pragma unroll 1
             for (int c = 0; c < D / 32; ++c) {

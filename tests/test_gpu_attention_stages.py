@@ -40,6 +40,89 @@ def test_scores_against_the_standing_reference(kind, L, v, b):
     ctx.recg_free()
 
 
+def cut_of_single_tiles(kv_len, n_kv, n_ctas=148):
+    """The KV ranges [first, end) of every request (per kv head, in tokens) where each request has one row tile: the work list's
+    rule, restated (a segment costs its 64-token blocks and four more, and the CTAs share the sum evenly)."""
+    blocks = [-(-n // 64) for n in kv_len for _ in range(n_kv)]
+    per = -(-sum(n + 4 for n in blocks) // n_ctas)
+    cut, at = [], 0
+    for n in blocks:
+        g0 = at + 4
+        at = g0 + n
+        ends = [min(g0 + n, (c + 1) * per) - g0 for c in range(g0 // per, (g0 + n - 1) // per + 1)]
+        cut.append([(64 * a, 64 * e) for a, e in zip([0] + ends, ends)])
+    return cut
+
+
+def stages_done_again(scores, cut):
+    """Stage numbers of every item and softmax group in which a row of `scores` (in powers of two) outgrows its reference."""
+    out = []
+    for first, end in cut:
+        for g in (0, 64):
+            ref, again = None, []
+            for n, t in enumerate(range(first + g, min(end, len(scores)), 128)):
+                top = scores[t:min(t + 64, end)].max()
+                if ref is None:
+                    ref = top
+                elif top > ref + 8:
+                    ref = top
+                    again.append(n)
+            out.append(again)
+    return out
+
+
+@pytest.mark.parametrize("profile,base,low", [("late", 2.0 ** 20, 0), ("late", 2.0 ** 24, 0), ("late", 2.0 ** 26, 0), ("every", 0.0, 0),
+                                              ("every", 2.0 ** 24, 0), ("late", 2.0 ** 13, -2.0 ** 40), ("every", 2.0 ** 13, -2.0 ** 40)])
+def test_reference_follows_the_scores_exactly(profile, base, low):
+    """Scores that outgrow the reference late in an item, or in every stage of it, on top of a common value `base`, and (low) a third
+    of the context with scores as of a mask.  Every score is a sum of at most two products and exact in fp32, so nothing but the
+    probabilities' and the result's rounding to bf16 stands between the kernel and float64, however large the scores are."""
+    n_kv, n_req, v, b = 8, 16, 2, 2
+    lens = [1900 + 13 * r for r in range(n_req)]
+    shape = synth.ModelShape(n_layers=1, hidden=64, n_q_heads=4 * n_kv, n_kv_heads=n_kv, head_dim=128, ffn=64, vocab=64)
+    desc = synth.fixed_descriptor(lens, [v] * n_req, [b] * n_req, seed=1)
+    ctx = ops_ctx(shape, n_req, desc.n_tokens, desc.page_table.shape[1])
+    pool = binding.alloc_kv_pool(ctx, desc.n_pages, fill=None)
+    pool.fill_(float("nan"))
+    side = 2.0 ** (np.log2(base) // 2) if base else 0.0
+    q = torch.zeros((desc.n_tokens, 4 * n_kv, 128))
+    q[..., 0], q[..., 1] = 2.0 ** 20, side
+    q[:, ::2, 2] = 8.0                   # (every other head sees the steps, the others a plain mean of what is not masked)
+    q = q.to(torch.bfloat16)
+    cut = cut_of_single_tiles([n + v + b for n in lens], n_kv)
+    kvs, again = [], []
+    for r, L in enumerate(lens):
+        n = L + v + b
+        pos = torch.arange(n)
+        step = (pos == 1200 + 40 * r).float() if profile == "late" else (pos // 128 + (pos % 64 == 5)).float()
+        masked = (pos < n // 3) if low else torch.zeros(n, dtype=torch.bool)
+        k = torch.zeros((n, n_kv, 128))
+        k[:, :, 0] = (masked * low / 2.0 ** 20)[:, None]
+        k[:, :, 1] = (~masked * (base / side if base else 0.0))[:, None]
+        k[:, :, 2] = (~masked * 9.0 * step)[:, None]
+        k = k.to(torch.bfloat16)
+        _, vals = synth.kv_values(n, n_kv, 128, seed=r)
+        vals = (0.25 * vals.float() + 1.0 - 2.0 * (step % 2)[:, None, None]).to(torch.bfloat16)
+        kvs.append((k, vals))
+        ctx.recg_kv_write(pool, desc.n_pages, 0, desc.page_table[r], 0, k.cuda(), vals.cuda())
+        scores = (f64(q[0, 0]) @ f64(k[:, 0]).T) / (np.sqrt(128.0) * np.log(2.0))
+        again += [a for h in range(n_kv) for a in stages_done_again(scores, cut[r * n_kv + h])]
+    # a stage is done again behind the second one, and (steps in every stage) one right behind the other
+    assert any(a and a[-1] >= 2 for a in again)
+    assert profile == "late" or any(len(a) >= 3 and a[2] == a[0] + 2 for a in again)
+    batch = binding.Batch(desc.ctx_len, desc.verify_len, desc.block_size, None, desc.page_table, pool, desc.n_pages)
+    o = torch.full((desc.n_tokens, 4 * n_kv, 128), float("nan"), dtype=torch.bfloat16, device="cuda")
+    ctx.recg_attention(batch, 0, q.cuda(), o)
+    ctx.recg_sync()
+    got = f64(o)
+    for r, L in enumerate(lens):
+        rows = slice(4 * r, 4 * r + 4)
+        ref = orc.hybrid_attention(f64(q[rows]), f64(kvs[r][0]), f64(kvs[r][1]), L, v, b)
+        # (P and the result are rounded to bf16, 2^-9 each, against values of at most 2.2)
+        assert np.max(np.abs(got[rows] - ref)) <= ATTN_TOL * np.max(np.abs(ref)), r
+    ctx.recg_free()
+
+
 @pytest.mark.parametrize("n_kv,reqs", [
     (8, [(4096, 16, 16)]),                       # 8 tiles: four warps a row
     (8, [(900, 20, 12), (3000, 1, 0)]),          # 16 tiles: two
