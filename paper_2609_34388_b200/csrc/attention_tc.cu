@@ -210,8 +210,9 @@ __global__ void __launch_bounds__(kThreads, 1) attention_tc_kernel(const __grid_
   // A wait that runs out records why and raises this flag; from then on no wait in this CTA blocks any more, so
   // every warp still walks through its loops (and meets the others at the named barriers) and the kernel ends.
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  // (the first look at the barrier does not wait either: try_wait may suspend the thread, test_wait does not)
   auto bwait = [&](uint64_t* bar, uint32_t parity, int code) {
-    if (mbar_try_wait(bar, parity) || *abort_flag) return;
+    if (mbar_test_wait(bar, parity) || *abort_flag) return;
     if (!mbar_wait(bar, parity, kSpin)) {
       set_status(P.status, code);
       *abort_flag = 1;
