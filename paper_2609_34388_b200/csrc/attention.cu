@@ -360,15 +360,17 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attention_kernel(AttnParams P
   }
 }
 
+// How many warps merge a row and how many of its partial rows are on their way at once (see combine_split and few_tiles):
+// kManyTiles one warp, six rows; kSplitRows two or four warps, which merge their sums through shared memory; kDeepRows one warp,
+// 18 rows, for which a CTA has the registers of an SM to itself (117 of 128 a thread at head_dim 128).
+enum CombineMode { kManyTiles, kSplitRows, kDeepRows };
 // Merges the KV-range partials of the tiles that were split (`tiles` lists no others: tiles with a single part were written by
-// the attention kernel itself).  Work unit = 16 rows of a tile, one warp per query row, each lane D/32
+// the attention kernel itself).  Work unit = 16 rows of a tile (8 or 4 where rows are split), each lane D/32
 // consecutive dims.  Bound by latency, not by its bytes (a tile entry, the (max, sum) pairs and the partial rows are
 // dependent reads): the tile entry is read ahead of the wait where the work list is settled, lane p fetches the pair of part
 // p, so that one read and a few shuffles give all weights of up to 32 parts, and the rows of the first kRows parts are on
-// their way at the same time.  With few tiles (combine_split) the parts of a row are dealt out over 2^log_s warps, which merge
-// their sums through shared memory.  Measured for one request (18 parts per row), attention and combine kernel of a layer together:
-// 19.5 us with four parts fetched at a time, each with its own pair, 16.1 us like this.
-enum CombineMode { kManyTiles, kSplitRows, kDeepRows };
+// their way at the same time.  Attention and combine kernel of a layer together, one request of 18 parts per row: 19.5 us with
+// four parts fetched at a time, each with its own pair, 16.1 with six and one read for all pairs; 13.9 now, with four warps a row.
 template <int D, CombineMode MODE>
 __global__ void __launch_bounds__(512, MODE == kDeepRows ? 1 : 2) attention_combine_kernel(const AttnTile* __restrict__ tiles,
                                                                 const int* __restrict__ counts, int n_q, int group,
@@ -378,7 +380,6 @@ __global__ void __launch_bounds__(512, MODE == kDeepRows ? 1 : 2) attention_comb
   constexpr int E = D / 32;
   constexpr bool SPLIT = MODE == kSplitRows;
   constexpr int kRows = MODE == kDeepRows ? 18 : 6;     // partial rows in flight
-  // (without a split no shared memory: the next projection's CTA has room beside this one's)
   __shared__ float s_acc[SPLIT ? 16 : 1][D + 2];
   griddep_launch();
   if (!list_settled) griddep_wait();
@@ -477,13 +478,18 @@ __global__ void __launch_bounds__(512, MODE == kDeepRows ? 1 : 2) attention_comb
 }
 
 // Few row tiles (at most `tiles`, 0: not known) are merged by few warps, each with many parts: a chain of dependent reads while most
-// SMs are idle.  The line lies where two or four warps per row are resident at once, two CTAs per SM; such a tile has eight parts
-// or more.
+// SMs are idle.
 // By itself (recg_attention) two or four warps share a row: one request over 4096 tokens (8 tiles of 18 parts), 32 layers, 479 us
-// with one warp per row, 446 with four.  Inside a step the idle SMs are worth more to the next projection, whose CTAs come in early
-// and request weights (a round of that request 3548 us with one warp per row, 3600 with four): there a row keeps its warp, in a
-// CTA with an SM's registers to itself, and up to 18 of its parts are on their way at once (3538 -> 3506 us; as many CTAs as there
-// is work, but six parts at once: 3553).
+// with one warp per row, 446 with four.  The line lies where that many warps per row are resident at once, two CTAs per SM.
+// Inside a step the idle SMs are worth more to the next projection, whose CTAs come in early and request weights (a round of that
+// request 3548 us with one warp per row, 3600 with four): there a row keeps its warp, in as many CTAs as there is work, and up to
+// 18 of its parts are on their way at once (six at once: 3553).  18 are the parts of a row where one request's 8 tiles share all
+// CTAs; fewer tiles have more parts and take more turns.  Rounds with kManyTiles and with kDeepRows, us (runs differ by up to 0.4 %):
+//   8 tiles: contexts of 900, 4096 and 8192 tokens 3415 -> 3382, 3555 -> 3515, 3686 -> 3641; 14B class, 3000 tokens, 5533 -> 5424
+//   16 tiles: two requests of 4096 tokens 3888 -> 3882, one of 64 rows 3826 -> 3820; two of 1000 3697 -> 3698 (4.7 %), two of 200
+//     to 8000 3756 -> 3655 (6 %), two of the 14B class 5781 -> 5609 (3.4 %)
+//   2 layers of hidden size 512, 4000 tokens: 2, 10 and 18 tiles 124 -> 116, 130 -> 125 (6 %), 148 -> 134 (24 %)
+// The line lies where all CTAs of kDeepRows are resident at once, one per SM (18 tiles: 144); nothing below it is slower.
 int combine_split(int tiles, int n_sm, bool step) {
   return tiles <= 0 || step ? 0 : (tiles * 32 <= 2 * n_sm ? 2 : (tiles * 16 <= 2 * n_sm ? 1 : 0));
 }
@@ -526,8 +532,9 @@ void launch_attention_t(const BatchLayout& bl, const Dims& dm, int layer, const 
   launch_pdl(attention_kernel<D>, dim3(n_sm), dim3(kAttnThreads), AttnSmem<D>::kTotal, st, P);
   if (whole) return;
   const int log_s = combine_split(tiles, n_sm, step);
-  launch_pdl(combine_kernel<D>(tiles, log_s, n_sm), dim3(combine_ctas(tiles, log_s, n_sm)), dim3(512), 0, st, (const AttnTile*)bl.tiles, (const int*)bl.counts,
-             dm.n_q, P.group, (const float*)part_o, (const float*)part_ml, static_cast<__nv_bfloat16*>(o), 0, log_s);
+  launch_pdl(combine_kernel<D>(tiles, log_s, n_sm), dim3(combine_ctas(tiles, log_s, n_sm)), dim3(512), 0, st,
+             (const AttnTile*)bl.tiles, (const int*)bl.counts, dm.n_q, P.group, (const float*)part_o, (const float*)part_ml,
+             static_cast<__nv_bfloat16*>(o), 0, log_s);
 }
 
 }  // namespace
@@ -543,8 +550,8 @@ void launch_attention(const BatchLayout& bl, const Dims& dm, int layer, const vo
     launch_attention_tc_main(bl, dm, layer, q, o, kv_pool, n_pages, part_o, part_ml, n_sm, status, st, layout_settled);
     if (whole) return;
     const int log_s = combine_split(tiles, n_sm, step);
-    launch_pdl(combine_kernel<128>(tiles, log_s, n_sm), dim3(combine_ctas(tiles, log_s, n_sm)), dim3(512), 0, st, (const AttnTile*)bl.tiles,
-               (const int*)bl.counts, dm.n_q, dm.n_q / dm.n_kv, (const float*)part_o, (const float*)part_ml,
+    launch_pdl(combine_kernel<128>(tiles, log_s, n_sm), dim3(combine_ctas(tiles, log_s, n_sm)), dim3(512), 0, st,
+               (const AttnTile*)bl.tiles, (const int*)bl.counts, dm.n_q, dm.n_q / dm.n_kv, (const float*)part_o, (const float*)part_ml,
                static_cast<__nv_bfloat16*>(o), 1, log_s);    // (the kernel in front signals its dependents when the list is settled)
     return;
   }
